@@ -204,7 +204,7 @@ img_status prepare(img_ctx *c) {
     const Range range_("img.prepare");
     if (!c->has_cov) return IMG_EINVAL;
     if (c->prepared) return (img_status)c->prep_status;
-    CK(img::launch_factor(c->djp, 1, c->stream));
+    CK(img::launch_factor(c->djp, 1, c->prm.p, c->stream));
     if (items_bounds(c)) {
         img_status st = wide_ready(c);
         if (st != IMG_OK) return st;
@@ -948,7 +948,7 @@ img_status launch_prepare(img_ctx *const *ctxs, const Groups &g, cudaStream_t s,
         const int nb = g.end[m] - g.begin[m];
         if (!nb) continue;
         JobDev *const *jp = g_ws.jobs + g.begin[m];
-        CK(img::launch_factor(jp, nb, s));
+        CK(img::launch_factor(jp, nb, g.max_p[m], s));
         if (m == kItemsGroup) {
             for (int q = g.begin[m]; q < g.end[m]; ++q) {
                 img_ctx *c = ctxs[g.order[q]];
@@ -1328,7 +1328,7 @@ struct img_server {
                 CK(img::launch_job(jp, nb, max_p, md, sl.infos + q0, nullptr, sl.s));
             } else {
                 CK(img::launch_tables(jp, nb, sl.s));
-                CK(img::launch_factor(jp, nb, sl.s));
+                CK(img::launch_factor(jp, nb, max_p, sl.s));
                 CK(img::launch_bounds(jp, nb, max_tiles, max_p, Groups::bounds_mode(md), sl.s));
                 CK(img::launch_finalize(jp, nb, sl.s, nullptr));
                 CK(img::launch_solve(jp, nb, max_p, Groups::solve_mode(md), sl.infos + q0, nullptr, sl.s));
@@ -1350,7 +1350,7 @@ struct img_server {
                 img_status wst = wide_ready(c);
                 if (wst != IMG_OK) return wst;
                 CK(img::launch_tables(jp, 1, sl.s));
-                CK(img::launch_factor(jp, 1, sl.s));
+                CK(img::launch_factor(jp, 1, c->prm.p, sl.s));
                 if (items_bounds(c)) CK(img::ws_bounds(c->ws, c->hj, sl.s));
                 else CK(img::launch_bounds(jp, 1, tiles, c->prm.p, op_mode_of(c), sl.s));
                 CK(img::launch_finalize(jp, 1, sl.s, nullptr));

@@ -45,7 +45,7 @@ struct JobDev {
     const double *mg;      // n_m
     // covariance and factors (column-major p x p)
     double2 *R64;          // R_hat
-    double2 *L64;          // Cholesky factor, lower
+    double2 *L64;          // Cholesky factor, lower (workspace of the factorisation)
     double2 *Li64;         // L^-1, lower
     float2 *R32;           // R_hat
     float2 *Ri32;          // R_hat^-1
@@ -87,13 +87,14 @@ struct JobDev {
     int *ev_count;
     // status and report
     DevInfo *info;
-    int *flags;            // [0]: factor status, [1]: bounds valid
+    int *flags;            // [0]: factor status, [1]: bounds valid, [2]: timeout, [3]: bad pivot
 };
 
 // Kernel launchers (defined in the .cu files, called by the host API).
 // `jobs` is a device array of n job pointers.
 cudaError_t launch_tables(JobDev *const *jobs, int n, cudaStream_t st);
-cudaError_t launch_factor(JobDev *const *jobs, int n, cudaStream_t st);
+// Cholesky factor, L^-1, R^-1 (factor.cu); max_p: most antennas of any job.
+cudaError_t launch_factor(JobDev *const *jobs, int n, int max_p, cudaStream_t st);
 // mode 1/2 use tensor cores: the shared-memory operator for p <= 64, the
 // streamed (wide) operator for 64 < p <= 256.
 cudaError_t launch_bounds(JobDev *const *jobs, int n, int max_tiles, int max_p, int mode,

@@ -1,7 +1,8 @@
 // Kernels of the bounded least-squares imager (SIMT FP32 operator path).
 //
 //   k_tables    separable steering tables (FP64 phase reduction + sincospi)
-//   k_factor    Cholesky R = L L^H, L^-1 and R^-1 in FP64 (one CTA per job)
+//   factor_job  Cholesky R = L L^H, L^-1 and R^-1 in FP64 by one CTA (the
+//               fused server kernel; all other paths: factor.cu)
 //   k_bounds    dirty image a^H R a and a^H R^-1 a over all pixels (many CTAs
 //               per job), the adjoint operator with U = R_hat and R_hat^-1
 //   k_finalize  MVDR bound, D, thresholds (Sec. III-D, Appendix A)
@@ -130,8 +131,6 @@ __device__ void factor_job(const JobDev &J) {
     }
     if (threadIdx.x == 0) J.flags[0] = 0;
 }
-
-__global__ void k_factor(JobDev *const *jobs) { factor_job(*jobs[blockIdx.x]); }
 
 // ---------------------------------------------------------------- bounds
 // dirty_i = Re(a_i^H R a_i) and h_i = a_i^H R^-1 a_i = ||L^-1 a_i||^2 for
@@ -1416,11 +1415,6 @@ static int num_sms() {
 
 cudaError_t launch_tables(JobDev *const *jobs, int n, cudaStream_t st) {
     k_tables<<<dim3(16, n), kThreads, 0, st>>>(jobs);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_factor(JobDev *const *jobs, int n, cudaStream_t st) {
-    k_factor<<<n, kThreads, 0, st>>>(jobs);
     return cudaGetLastError();
 }
 
