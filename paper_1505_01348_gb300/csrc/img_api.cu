@@ -137,6 +137,7 @@ size_t carve(img_ctx *c, char *base) {
     J.Bimg = p <= img::kMaxWideP ? cv.take<unsigned char>(2 * img::wide_B_bytes(p)) : nullptr;
     J.Bscale = cv.take<float>(2);
     J.Bmax = cv.take<unsigned>(2);           // also the forward's max |w| word at every p
+    J.vmax = cv.take<unsigned long long>(1);
     J.info = cv.take<DevInfo>(1);
     J.flags = cv.take<int>(4);
     c->dj = cv.take<JobDev>(1);
@@ -205,15 +206,15 @@ img_status prepare(img_ctx *c) {
     if (!c->has_cov) return IMG_EINVAL;
     if (c->prepared) return (img_status)c->prep_status;
     CK(img::launch_factor(c->djp, 1, c->prm.p, c->stream));
+    const int ntiles = (c->hj.Q + img::kTile - 1) / img::kTile;
     if (items_bounds(c)) {
         img_status st = wide_ready(c);
         if (st != IMG_OK) return st;
         CK(img::ws_bounds(c->ws, c->hj, c->stream));
     } else {
-        const int ntiles = (c->hj.Q + img::kTile - 1) / img::kTile;
         CK(img::launch_bounds(c->djp, 1, ntiles, c->prm.p, op_mode_of(c), c->stream));
     }
-    CK(img::launch_finalize(c->djp, 1, c->stream, nullptr));
+    CK(img::launch_finalize(c->djp, 1, ntiles, c->stream, nullptr));
     int flag = 0;
     CK(cudaMemcpyAsync(&flag, c->hj.flags, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
@@ -959,7 +960,7 @@ img_status launch_prepare(img_ctx *const *ctxs, const Groups &g, cudaStream_t s,
         } else {
             CK(img::launch_bounds(jp, nb, g.max_tiles[m], g.max_p[m], Groups::bounds_mode(m), s));
         }
-        CK(img::launch_finalize(jp, nb, s, status_out ? status_out + g.begin[m] : nullptr));
+        CK(img::launch_finalize(jp, nb, g.max_tiles[m], s, status_out ? status_out + g.begin[m] : nullptr));
     }
     return IMG_OK;
 }
@@ -1330,7 +1331,7 @@ struct img_server {
                 CK(img::launch_tables(jp, nb, sl.s));
                 CK(img::launch_factor(jp, nb, max_p, sl.s));
                 CK(img::launch_bounds(jp, nb, max_tiles, max_p, Groups::bounds_mode(md), sl.s));
-                CK(img::launch_finalize(jp, nb, sl.s, nullptr));
+                CK(img::launch_finalize(jp, nb, max_tiles, sl.s, nullptr));
                 CK(img::launch_solve(jp, nb, max_p, Groups::solve_mode(md), sl.infos + q0, nullptr, sl.s));
             }
             return IMG_OK;
@@ -1353,7 +1354,7 @@ struct img_server {
                 CK(img::launch_factor(jp, 1, c->prm.p, sl.s));
                 if (items_bounds(c)) CK(img::ws_bounds(c->ws, c->hj, sl.s));
                 else CK(img::launch_bounds(jp, 1, tiles, c->prm.p, op_mode_of(c), sl.s));
-                CK(img::launch_finalize(jp, 1, sl.s, nullptr));
+                CK(img::launch_finalize(jp, 1, tiles, sl.s, nullptr));
                 CK(img::ws_launch(c->ws, sl.s));
                 CK(cudaMemcpyAsync(sl.infos + q, c->hj.info, sizeof(DevInfo), cudaMemcpyDeviceToDevice, sl.s));
             }

@@ -80,6 +80,7 @@ struct JobDev {
     unsigned char *Bimg;
     float *Bscale;
     unsigned *Bmax;      // max |entry| bits of the operators being imaged (atomicMax)
+    unsigned long long *vmax;  // bits of the cost's largest dirty-image value (atomicMax)
     // decision log (Table I order): kind << 24 | pixel, and lambda or mu
     int *ev;
     float *evv;
@@ -99,7 +100,8 @@ cudaError_t launch_factor(JobDev *const *jobs, int n, int max_p, cudaStream_t st
 // streamed (wide) operator for 64 < p <= 256.
 cudaError_t launch_bounds(JobDev *const *jobs, int n, int max_tiles, int max_p, int mode,
                           cudaStream_t st);
-cudaError_t launch_finalize(JobDev *const *jobs, int n, cudaStream_t st, int *batch_status);
+// max_tiles: most 64-pixel tiles of any job
+cudaError_t launch_finalize(JobDev *const *jobs, int n, int max_tiles, cudaStream_t st, int *batch_status);
 // mode: 0 CUDA-core FP32 operators, 1 tensor cores FP16x3, 2 tensor cores BF16x3
 cudaError_t launch_solve(JobDev *const *jobs, int n, int max_p, int mode, DevInfo *batch_info,
                          double *const *sigma_out, cudaStream_t st);

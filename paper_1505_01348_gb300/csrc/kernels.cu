@@ -569,55 +569,88 @@ cudaError_t launch_wait_selftest(unsigned polls, int arrive, int *status, cudaSt
     return cudaGetLastError();
 }
 
-// Bounds, preconditioner and thresholds (one CTA per job):
+// Bounds, preconditioner and thresholds:
 //   C = N/(N-p) or 1; mvdr = C/h; D = h^2/C; std_MF = dirty/sqrt(N);
 //   std_MVDR = mvdr/sqrt(N-p-1); gamma = chosen image, optionally inflated;
 //   PWLS: x = D sigma (scale 1/D, upper D gamma); eps = kappa std with a floor.
-__device__ void finalize_job(const JobDev &J) {
-    __shared__ double sbuf[kThreads / 32];
-    const double C = J.bias_c ? (double)J.N / (double)(J.N - J.p) : 1.0;
-    const double sqN = sqrt((double)J.N);
-    const double dof = (double)(J.N - J.p - 1);
-    const bool pwls = J.cost == IMG_COST_PWLS;
-    double mx = 0.0;
-    for (int i = threadIdx.x; i < J.Q; i += blockDim.x) {
-        const double h = J.h[i];
-        const double d = J.dirty[i];
-        const double mv = C / h;
-        const double base = J.bound == IMG_BOUND_MF ? d : mv;
-        const double sd = J.bound == IMG_BOUND_MF ? d / sqN : (dof > 0 ? mv / sqrt(dof) : INFINITY);
-        double g = base;
-        if (J.inflate == IMG_INFLATE_RATIO) g = (1.0 + J.alpha) * base;
-        else if (J.inflate == IMG_INFLATE_STD) g = base + J.alpha * sd;
-        const double D = h * h / C;
-        double mb = mv;
-        if (J.inflate == IMG_INFLATE_RATIO) mb = (1.0 + J.alpha) * mv;
-        else if (J.inflate == IMG_INFLATE_STD) mb = mv + J.alpha * (dof > 0 ? mv / sqrt(dof) : INFINITY);
-        J.mvb[i] = mb;
-        J.gamma[i] = g;
-        J.upper[i] = pwls ? D * g : g;
-        J.scale[i] = pwls ? (float)(1.0 / D) : 1.0f;
-        const double sdc = pwls ? (dof > 0 ? mv / sqrt(dof) : INFINITY) : d / sqN;
-        J.eps[i] = (float)(J.kappa * sdc);
-        mx = fmax(mx, pwls ? mv : d);
-    }
-    // max over the CTA (all values positive)
+struct FinalizeConsts {
+    double C, sqN, dof, sqdof;
+    bool pwls;
+    __device__ explicit FinalizeConsts(const JobDev &J)
+        : C(J.bias_c ? (double)J.N / (double)(J.N - J.p) : 1.0), sqN(sqrt((double)J.N)),
+          dof((double)(J.N - J.p - 1)), sqdof(sqrt(dof)), pwls(J.cost == IMG_COST_PWLS) {}
+};
+
+// Pixel i; returns its value of the cost's dirty image (for the eps floor).
+__device__ __forceinline__ double finalize_pixel(const JobDev &J, const FinalizeConsts &k, int i) {
+    const double h = J.h[i];
+    const double d = J.dirty[i];
+    const double mv = k.C / h;
+    const double mvsd = k.dof > 0 ? mv / k.sqdof : INFINITY;
+    const double base = J.bound == IMG_BOUND_MF ? d : mv;
+    const double sd = J.bound == IMG_BOUND_MF ? d / k.sqN : mvsd;
+    double g = base;
+    if (J.inflate == IMG_INFLATE_RATIO) g = (1.0 + J.alpha) * base;
+    else if (J.inflate == IMG_INFLATE_STD) g = base + J.alpha * sd;
+    const double D = h * h / k.C;
+    double mb = mv;
+    if (J.inflate == IMG_INFLATE_RATIO) mb = (1.0 + J.alpha) * mv;
+    else if (J.inflate == IMG_INFLATE_STD) mb = mv + J.alpha * mvsd;
+    J.mvb[i] = mb;
+    J.gamma[i] = g;
+    J.upper[i] = k.pwls ? D * g : g;
+    J.scale[i] = k.pwls ? (float)(1.0 / D) : 1.0f;
+    const double sdc = k.pwls ? mvsd : d / k.sqN;
+    J.eps[i] = (float)(J.kappa * sdc);
+    return k.pwls ? mv : d;
+}
+
+// Largest v > 0 over the CTA (0 when there is none; NaN is never larger).
+__device__ __forceinline__ double block_max_pos(double mx, double *sbuf) {
     for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if ((threadIdx.x & 31) == 0) sbuf[threadIdx.x >> 5] = mx;
     __syncthreads();
     mx = 0.0;
     for (int w = 0; w < kThreads / 32; ++w) mx = fmax(mx, sbuf[w]);
+    return mx;
+}
+
+// All pixels by one CTA (the fused server kernel).
+__device__ void finalize_job(const JobDev &J) {
+    __shared__ double sbuf[kThreads / 32];
+    const FinalizeConsts k(J);
+    double mx = 0.0;
+    for (int i = threadIdx.x; i < J.Q; i += blockDim.x) mx = fmax(mx, finalize_pixel(J, k, i));
+    mx = block_max_pos(mx, sbuf);
     const float fl = (float)(J.eps_floor * mx);
     for (int i = threadIdx.x; i < J.Q; i += blockDim.x) J.eps[i] = fmaxf(J.eps[i], fl);
     if (threadIdx.x == 0) J.flags[1] = 1;
     __syncthreads();
 }
 
+// The same over the GPU (blockIdx.x = job): four FP64 divisions per pixel are
+// bound by the FP64 pipe, 865 us for 256x256 pixels on one SM.  The maximum
+// of the non-negative values goes through an integer atomicMax on their bits
+// (zeroed with the factor), and the floor is a second launch.
 __global__ void k_finalize(JobDev *const *jobs, int *batch_status) {
     const JobDev &J = *jobs[blockIdx.x];
-    if (batch_status && threadIdx.x == 0) batch_status[blockIdx.x] = J.flags[0];
+    __shared__ double sbuf[kThreads / 32];
+    if (batch_status && blockIdx.y == 0 && threadIdx.x == 0) batch_status[blockIdx.x] = J.flags[0];
     if (J.flags[0] != 0) return;
-    finalize_job(J);
+    const FinalizeConsts k(J);
+    double mx = 0.0;
+    for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < J.Q; i += gridDim.y * blockDim.x)
+        mx = fmax(mx, finalize_pixel(J, k, i));
+    mx = block_max_pos(mx, sbuf);
+    if (threadIdx.x == 0 && mx > 0.0) atomicMax(J.vmax, (unsigned long long)__double_as_longlong(mx));
+}
+__global__ void k_eps_floor(JobDev *const *jobs) {
+    const JobDev &J = *jobs[blockIdx.x];
+    if (J.flags[0] != 0) return;
+    const float fl = (float)(J.eps_floor * __longlong_as_double((long long)*J.vmax));
+    for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < J.Q; i += gridDim.y * blockDim.x)
+        J.eps[i] = fmaxf(J.eps[i], fl);
+    if (blockIdx.y == 0 && threadIdx.x == 0) J.flags[1] = 1;
 }
 
 // ---------------------------------------------------------------- solver
@@ -1460,8 +1493,12 @@ cudaError_t launch_bounds(JobDev *const *jobs, int n, int max_tiles, int max_p, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(JobDev *const *jobs, int n, cudaStream_t st, int *batch_status) {
-    k_finalize<<<n, kThreads, 0, st>>>(jobs, batch_status);
+cudaError_t launch_finalize(JobDev *const *jobs, int n, int max_tiles, cudaStream_t st, int *batch_status) {
+    // one pixel per thread while the CTAs of all jobs stay within a few waves
+    const int need = (max_tiles * kTile + kThreads - 1) / kThreads;
+    const dim3 grid(n, max(1, min(need, 8 * num_sms() / n)));
+    k_finalize<<<grid, kThreads, 0, st>>>(jobs, batch_status);
+    k_eps_floor<<<grid, kThreads, 0, st>>>(jobs);
     return cudaGetLastError();
 }
 
