@@ -47,6 +47,33 @@ __device__ __forceinline__ double block_sum(double v, double *sbuf) {
     return t;
 }
 
+// The same sum, in the same order, for the threads of warp 0 (0 elsewhere).
+// sbuf may be written again after the caller's next __syncthreads.
+__device__ __forceinline__ double block_sum_w0(double v, double *sbuf) {
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sbuf[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x < 32)
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w) t += sbuf[w];
+    return t;
+}
+
+// Largest value >= 0 over the CTA, in every thread.  FP32 throughout: through
+// FP64 entries the conversions alone took 1,000 cycles of the FP64 pipe.
+__device__ __forceinline__ float block_max_f(float mx, double *sbuf) {
+    float *fbuf = reinterpret_cast<float *>(sbuf);
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0) fbuf[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    mx = 0.f;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) mx = fmaxf(mx, fbuf[w]);
+    __syncthreads();
+    return mx;
+}
+
 // Lexicographic (value, index) minimum over the CTA; ties go to the smaller
 // index.  Every thread receives the result.
 __device__ __forceinline__ void block_argmin(double &v, int &idx, double *sv, int *si) {

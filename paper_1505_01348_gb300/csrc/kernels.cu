@@ -661,6 +661,13 @@ struct SolveShared {
     int cbuf[kThreads / 32];
     float wsm[kTile];
     float red[kTile + 16 * kTile];
+    float ls[8];          // LSQR: coefficients that warp 0 hands to the CTA
+    int lsi;
+};
+
+// Clock cycles of a solve's phases (one thread's view; reported as doubles).
+struct SolveCycles {
+    long long gradient = 0, lsqr = 0, fwd = 0, adj = 0, aux[6] = {};
 };
 
 // c = T a_i for the support cache (T = L^-1 for PWLS, identity for LS), and
@@ -681,14 +688,8 @@ __device__ void cache_vector(const JobDev &J, int i, int slot, double *sbuf) {
         c[k] = s;
         mx = fmaxf(mx, fmaxf(fabsf(s.x), fabsf(s.y)));
     }
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) sbuf[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float m = 0.f;
-        for (int w = 0; w < kThreads / 32; ++w) m = fmaxf(m, (float)sbuf[w]);
-        J.cmax[slot] = m;
-    }
+    mx = block_max_f(mx, sbuf);
+    if (threadIdx.x == 0) J.cmax[slot] = mx;
     __syncthreads();
 }
 
@@ -697,12 +698,7 @@ __device__ void cache_vector(const JobDev &J, int i, int slot, double *sbuf) {
 __device__ float list_scale(const JobDev &J, const int *pos, int n, double *sbuf) {
     float mx = 0.f;
     for (int j = threadIdx.x; j < n; j += blockDim.x) mx = fmaxf(mx, J.cmax[pos ? pos[j] : j]);
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) sbuf[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    mx = 0.f;
-    for (int w = 0; w < kThreads / 32; ++w) mx = fmaxf(mx, (float)sbuf[w]);
-    __syncthreads();
+    mx = block_max_f(mx, sbuf);
     return (mx > 0.f ? exp2f(-ceilf(log2f(mx))) : 1.f) * kLift;
 }
 
@@ -825,8 +821,14 @@ __device__ void adjoint_full(const JobDev &J, const float2 *U, float2 *A, TcWork
 // FP64.  The u-space vector is kept unnormalised: W0 holds t with u = t * us
 // (us = 1/beta), which saves a normalisation pass per iteration.  Returns the
 // iteration count; the solution is in J.xs[0..f).
+//
+// The FP64 scalars are computed by warp 0 alone, independent divisions and
+// roots in neighbouring lanes, and handed to the CTA as the FP32 coefficients
+// it uses: the FP64 pipe takes a warp instruction per 16 cycles and SM, so the
+// same scalars in all 8 warps cost 25,000 of the 50,000 cycles of an
+// iteration at p = 48 (f <= 256).
 template <int MODE>
-__device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShared &S, DevInfo &info) {
+__device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShared &S, SolveCycles &cyc) {
     constexpr bool BF = MODE == 2;
     const int p = J.p, pp = p * p;
     const int *__restrict__ fpos = J.fpos;
@@ -860,46 +862,65 @@ __device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShare
     }
     float acc = 0.f;     // per-thread partial (<= 16 terms), reduced in FP64
     for (int e = threadIdx.x; e < pp; e += blockDim.x) acc = fmaf(t[e].x, t[e].x, fmaf(t[e].y, t[e].y, acc));
-    double beta = sqrt(block_sum((double)acc, S.dbuf));
-    const double bnorm = beta;
+    const bool w0 = threadIdx.x < 32;
+    const int lane = threadIdx.x & 31;
+    // scalars of the recurrence, valid in warp 0
+    double alpha = 0.0, beta = 0.0, bnorm = 0.0, us = 0.0, phibar = 0.0, rhobar = 0.0, anorm2 = 0.0;
+    {
+        const double ss = block_sum_w0((double)acc, S.dbuf);
+        if (w0) {
+            beta = bnorm = phibar = sqrt(ss);
+            us = 1.0 / beta;
+            S.ls[0] = (float)us;
+            S.lsi = beta == 0.0;
+        }
+    }
     for (int j = threadIdx.x; j < f; j += blockDim.x) xs[j] = 0.f;
-    if (beta == 0.0) {
+    __syncthreads();
+    if (S.lsi) {
         for (int j = threadIdx.x; j < f; j += blockDim.x) J.xs[j] = 0.f;
         __syncthreads();
         return 0;
     }
-    double us = 1.0 / beta;
     auto adjoint = [&](auto epi) {
         if constexpr (MODE != 0) {
             if (resident) {
-                tc_adjoint_resident<BF>(T, t, p, f, sXr, S.red, S.dbuf, epi, info.cyc_aux);
+                tc_adjoint_resident<BF>(T, t, p, f, sXr, S.red, S.dbuf, epi, cyc.aux);
                 return;
             }
         }
         adjoint_list<MODE>(J, t, fpos, f, A, T, S.red, S.dbuf, epi);
     };
     {
-        const float fus = (float)us;
+        const float fus = S.ls[0];
         adjoint([&](int j, float y) { v[j] = sF[j] * (y * fus); });
     }
     acc = 0.f;
     for (int j = threadIdx.x; j < f; j += blockDim.x) acc = fmaf(v[j], v[j], acc);
-    double alpha = sqrt(block_sum((double)acc, S.dbuf));
+    {
+        const double ss = block_sum_w0((double)acc, S.dbuf);
+        if (w0) {
+            alpha = rhobar = sqrt(ss);
+            S.ls[5] = (float)(1.0 / alpha);
+            S.ls[0] = (float)(alpha * us);
+            S.lsi = alpha == 0.0;
+        }
+    }
+    __syncthreads();
     int it = 0;
-    if (alpha == 0.0) {
+    if (S.lsi) {
         for (int j = threadIdx.x; j < f; j += blockDim.x) J.xs[j] = 0.f;
         __syncthreads();
         return 0;
     }
     {
-        const float ia = (float)(1.0 / alpha);
+        const float ia = S.ls[5];
         for (int j = threadIdx.x; j < f; j += blockDim.x) {
             v[j] *= ia;
             w[j] = v[j];
         }
     }
     __syncthreads();
-    double phibar = beta, rhobar = alpha, anorm2 = 0.0;
     const int maxit = J.lsqr_maxit > 0 ? J.lsqr_maxit : 4 * f + 20;
     const double atol = J.lsqr_atol, btol = J.lsqr_btol;
     for (it = 1; it <= maxit; ++it) {
@@ -907,13 +928,13 @@ __device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShare
         for (int j = threadIdx.x; j < f; j += blockDim.x) wt[j] = sF[j] * v[j];
         __syncthreads();
         long long tc0 = clock64();
-        const float fa = (float)(alpha * us);
+        const float fa = S.ls[0];
         acc = 0.f;
         bool done = false;
         if constexpr (MODE != 0) {
             if (resident) {
                 float inv;
-                const float *G = tc_forward_resident<BF>(T, stage, f, wt, sXr, &inv, S.dbuf, info.cyc_aux);
+                const float *G = tc_forward_resident<BF>(T, stage, f, wt, sXr, &inv, S.dbuf, cyc.aux);
                 const long long cu = clock64();
                 for (int e = threadIdx.x; e < pp; e += blockDim.x) {
                     const int bcol = e / p, a = e - bcol * p;
@@ -923,7 +944,7 @@ __device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShare
                     t[e] = tn;
                     acc = fmaf(tn.x, tn.x, fmaf(tn.y, tn.y, acc));
                 }
-                info.cyc_aux[2] += (double)(clock64() - cu);
+                cyc.aux[2] += clock64() - cu;
                 done = true;
             }
         }
@@ -938,27 +959,43 @@ __device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShare
                 acc = fmaf(tn.x, tn.x, fmaf(tn.y, tn.y, acc));
             }
         }
-        info.cyc_lsqr_fwd += (double)(clock64() - tc0);
-        beta = sqrt(block_sum((double)acc, S.dbuf));
-        us = beta > 0.0 ? 1.0 / beta : 0.0;
-        anorm2 += alpha * alpha + beta * beta;
+        cyc.fwd += clock64() - tc0;
+        double ss = block_sum_w0((double)acc, S.dbuf);
+        if (w0) {
+            beta = sqrt(ss);
+            us = beta > 0.0 ? 1.0 / beta : 0.0;
+            anorm2 += alpha * alpha + beta * beta;
+            S.ls[1] = (float)beta;
+            S.ls[2] = (float)us;
+        }
+        __syncthreads();
         // v <- M^H u - beta v
-        const float fb = (float)beta, fus = (float)us;
+        const float fb = S.ls[1], fus = S.ls[2];
         tc0 = clock64();
         adjoint([&](int j, float y) { v[j] = sF[j] * (y * fus) - fb * v[j]; });
-        info.cyc_lsqr_adj += (double)(clock64() - tc0);
+        cyc.adj += clock64() - tc0;
         acc = 0.f;
         for (int j = threadIdx.x; j < f; j += blockDim.x) acc = fmaf(v[j], v[j], acc);
-        alpha = sqrt(block_sum((double)acc, S.dbuf));
-        // plane rotation (scalars in FP64, the same in every thread)
-        const double rho = hypot(rhobar, beta);
-        const double c = rhobar / rho, s = beta / rho;
-        const double theta = s * alpha;
-        rhobar = -c * alpha;
-        const double phi = c * phibar;
-        phibar = s * phibar;
-        const float t1 = (float)(phi / rho), t2 = (float)(-theta / rho);
-        const float ia = alpha > 0.0 ? (float)(1.0 / alpha) : 1.f;
+        ss = block_sum_w0((double)acc, S.dbuf);
+        double absc = 0.0;
+        if (w0) {
+            // plane rotation; lanes 0..2: c, s, 1/alpha, then lanes 0, 1: the coefficients
+            alpha = sqrt(ss);
+            const double rho = hypot(rhobar, beta);
+            const double q = (lane == 0 ? rhobar : lane == 1 ? beta : 1.0) / (lane == 2 ? alpha : rho);
+            const double c = __shfl_sync(0xffffffffu, q, 0), sn = __shfl_sync(0xffffffffu, q, 1);
+            const double ialpha = __shfl_sync(0xffffffffu, q, 2);
+            const double theta = sn * alpha;
+            rhobar = -c * alpha;
+            const double phi = c * phibar;
+            phibar = sn * phibar;
+            absc = fabs(c);
+            const double t = (lane == 0 ? phi : -theta) / rho;
+            if (lane < 2) S.ls[3 + lane] = (float)t;
+            if (lane == 0) S.ls[5] = alpha > 0.0 ? (float)ialpha : 1.f;
+        }
+        __syncthreads();
+        const float t1 = S.ls[3], t2 = S.ls[4], ia = S.ls[5];
         acc = 0.f;
         for (int j = threadIdx.x; j < f; j += blockDim.x) {
             const float vj = v[j] * ia;                 // v <- v / alpha
@@ -968,12 +1005,17 @@ __device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShare
             w[j] = vj + t2 * w[j];
             acc = fmaf(xj, xj, acc);
         }
-        const double xnorm = sqrt(block_sum((double)acc, S.dbuf));
-        const double rnorm = phibar;
-        const double arnorm = phibar * alpha * fabs(c);
-        const double anorm = sqrt(anorm2);
-        if (rnorm <= btol * bnorm + atol * anorm * xnorm) break;
-        if (arnorm <= atol * anorm * rnorm) break;
+        ss = block_sum_w0((double)acc, S.dbuf);
+        if (w0) {
+            const double q = sqrt(lane == 0 ? ss : anorm2);
+            const double xnorm = __shfl_sync(0xffffffffu, q, 0), anorm = __shfl_sync(0xffffffffu, q, 1);
+            const double rnorm = phibar;
+            const double arnorm = phibar * alpha * absc;
+            S.lsi = rnorm <= btol * bnorm + atol * anorm * xnorm || arnorm <= atol * anorm * rnorm;
+            S.ls[0] = (float)(alpha * us);
+        }
+        __syncthreads();
+        if (S.lsi) break;
     }
     if (xs != J.xs)
         for (int j = threadIdx.x; j < f; j += blockDim.x) J.xs[j] = xs[j];
@@ -1019,6 +1061,7 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
     __shared__ uint64_t tc_bar[2];
     __shared__ uint32_t tc_slot;
     DevInfo info{};
+    SolveCycles cyc;
     info.status = IMG_OK;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(info.t_begin_ns));
     const int p = J.p, Q = J.Q;
@@ -1096,8 +1139,8 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
                                     S.dbuf);
                 info.op_flops += flops_fwd(p, nu);
                 const long long t0 = clock64();
-                const int its = lsqr_cta<MODE>(J, f, A, T, S, info);
-                info.cyc_lsqr += (double)(clock64() - t0);
+                const int its = lsqr_cta<MODE>(J, f, A, T, S, cyc);
+                cyc.lsqr += clock64() - t0;
                 info.lsqr_iters += its;
                 info.op_flops += (its + 1) * (flops_fwd(p, f) + flops_adj(p, f));
                 // feasibility with the relative tolerance tau, non-strict
@@ -1168,7 +1211,7 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
                 best = bestf;
                 info.op_flops += flops_adj(p, Q);
                 block_argmin(best, bidx, S.vbuf, S.ibuf);
-                info.cyc_gradient += (double)(clock64() - tg);
+                cyc.gradient += clock64() - tg;
                 lam_min = best;
                 if (bidx == 0x7fffffff) {
                     converged = true;
@@ -1255,6 +1298,11 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
         info.converged = converged ? 1 : 0;
         info.lambda_min = lam_min;
         info.cyc_total = (double)(clock64() - t_start);
+        info.cyc_gradient = (double)cyc.gradient;
+        info.cyc_lsqr = (double)cyc.lsqr;
+        info.cyc_lsqr_fwd = (double)cyc.fwd;
+        info.cyc_lsqr_adj = (double)cyc.adj;
+        for (int q = 0; q < 6; ++q) info.cyc_aux[q] = (double)cyc.aux[q];
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(info.t_end_ns));
         *J.ev_count = nev;
         *J.info = info;

@@ -306,12 +306,7 @@ __device__ float tc_build_B(const float2 *U, int p, TcWork &T, double *sbuf) {
             for (int e = 0; e < 8; ++e) mx = fmaxf(mx, fmaxf(fabsf(v[q][e].x), fabsf(v[q][e].y)));
         }
     }
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) sbuf[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    mx = 0.f;
-    for (int w = 0; w < kThreads / 32; ++w) mx = fmaxf(mx, (float)sbuf[w]);
-    __syncthreads();
+    mx = block_max_f(mx, sbuf);
     const float sc = (mx > 0.f ? exp2f(-ceilf(log2f(mx))) : 1.f) * kLift;
 #pragma unroll
     for (int q = 0; q < kMaxItems; ++q) {
@@ -726,12 +721,7 @@ __device__ inline float *tc_read_fwd(const TcWork &T, float *G) {
 __device__ inline float pow2_scale_of(const float *w, int n, double *sbuf) {
     float mx = 0.f;
     for (int j = threadIdx.x; j < n; j += blockDim.x) mx = fmaxf(mx, fabsf(w[j]));
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) sbuf[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    mx = 0.f;
-    for (int w2 = 0; w2 < kThreads / 32; ++w2) mx = fmaxf(mx, (float)sbuf[w2]);
-    __syncthreads();
+    mx = block_max_f(mx, sbuf);
     return mx > 0.f ? exp2f(-ceilf(log2f(mx))) : 1.f;
 }
 
@@ -880,7 +870,7 @@ __device__ inline void tc_issue_fwd_chunk(const TcWork &T, const unsigned char *
 // that read it completed.  Returns G (scaled by sX^2 sW; *scale = 1/that).
 template <bool BF16>
 __device__ const float *tc_forward_resident(TcWork &T, unsigned char *stage, int f, const float *w,
-                                            float sX, float *scale, double *dbuf, double *cyc = nullptr) {
+                                            float sX, float *scale, double *dbuf, long long *cyc = nullptr) {
     long long c0 = clock64();
     const float sW = pow2_scale_of(w, f, dbuf);
     const uint32_t idesc = idesc_f16_mn(2 * T.Kp, BF16 ? 1 : 0);
@@ -910,8 +900,8 @@ __device__ const float *tc_forward_resident(TcWork &T, unsigned char *stage, int
     *scale = 1.f / (sX * sX * sW);
     const float *G = nchunks ? tc_read_fwd(T, reinterpret_cast<float *>(T.Bhi)) : nullptr;
     if (cyc) {
-        cyc[0] += (double)(c1 - c0);
-        cyc[1] += (double)(clock64() - c1);
+        cyc[0] += c1 - c0;
+        cyc[1] += clock64() - c1;
     }
     return G;
 }
@@ -919,7 +909,7 @@ __device__ const float *tc_forward_resident(TcWork &T, unsigned char *stage, int
 // Adjoint over the resident tiles: epi(j, Re(c_j^H U c_j)) for j < f.
 template <bool BF16, class Epi>
 __device__ void tc_adjoint_resident(TcWork &T, const float2 *U, int p, int f, float sX, float *red,
-                                    double *dbuf, Epi epi, double *cyc = nullptr) {
+                                    double *dbuf, Epi epi, long long *cyc = nullptr) {
     long long c0 = clock64();
     const float sB = tc_build_B<BF16>(U, p, T, dbuf);
     const uint32_t idesc = idesc_f16(2 * T.Kp, BF16 ? 1 : 0);
@@ -945,9 +935,9 @@ __device__ void tc_adjoint_resident(TcWork &T, const float2 *U, int p, int f, fl
         ce += clock64() - a1;
     }
     if (cyc) {
-        cyc[3] += (double)(c1 - c0);
-        cyc[4] += (double)cw;
-        cyc[5] += (double)ce;
+        cyc[3] += c1 - c0;
+        cyc[4] += cw;
+        cyc[5] += ce;
     }
 }
 
