@@ -714,18 +714,14 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_ws_adj(const JobDev *Jp, Ws
 //   the plane rotation (FP64); v <- v / alpha; init: w = v, x = 0; else
 //   x += t1 w, w = v + t2 w; the weights s_F v of the next forward and their
 //   maximum; ||x|| and the Paige-Saunders stopping tests; h_lsqr := continue.
-constexpr int kVxThreads = 256;
-
-__device__ __forceinline__ double vx_sum(double v, double *sb) {
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) sb[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double t = 0.0;
-#pragma unroll 8
-    for (int w = 0; w < kVxThreads / 32; ++w) t += sb[w];
-    __syncthreads();
-    return t;
-}
+//
+// Latency bound (one CTA, a few hundred rows).  The FP64 scalars run in warp
+// 0 alone, independent divisions and roots in neighbouring lanes (the FP64
+// pipe takes a warp instruction per 16 cycles: in all 8 warps they cost
+// most of the 15.5 us the kernel took), and the first kVxReg rows of a thread stay in
+// registers from one phase to the next, loaded before the first reduction.
+constexpr int kVxThreads = kThreads;
+constexpr int kVxReg = 4;               // rows per thread held in registers (f <= 1024)
 
 __global__ void __launch_bounds__(kVxThreads) k_ws_vx(const JobDev *Jp, WsBufs B, int init,
                                                        cudaGraphConditionalHandle h_lsqr) {
@@ -734,94 +730,154 @@ __global__ void __launch_bounds__(kVxThreads) k_ws_vx(const JobDev *Jp, WsBufs B
     WsCtl *ctl = B.ctl;
     __shared__ double sb[kVxThreads / 32];
     __shared__ float swm[kVxThreads / 32];
+    __shared__ float s_c[5];                // us, beta, then 1/alpha, t1, t2
     if (ctl->stop) {
         if (threadIdx.x == 0) ws_cond(ctl, kCondLsqr, h_lsqr, 0u);
         return;
     }
+    const bool w0 = threadIdx.x < 32;
+    const int lane = threadIdx.x & 31;
     const int f = ctl->f, ld = B.ld_adj, rows = ctl->adj_rows;
-    // beta from the reduction's CTA shares
-    double part = 0.0;
-    for (int b = threadIdx.x; b < ctl->nsums; b += blockDim.x) part += ctl->sums[b];
-    const double beta = sqrt(vx_sum(part, sb));
-    const double us = beta > 0.0 ? 1.0 / beta : 0.0;
-    const double alpha_prev = ctl->alpha;
-    const float sc = 1.f / (ctl->sXF * ctl->sB);
-    const float fus = (float)us, fb = (float)beta;
-    float ss = 0.f;
     const int r4 = rows >> 2;
     float *__restrict__ vv = J.v;
+    float *__restrict__ ww = J.w;
+    float *__restrict__ xx = J.xs;
     const float *__restrict__ sF = J.sF;
+    const float *__restrict__ padj = B.padj;
+    float vr[kVxReg], wr[kVxReg], xr[kVxReg], fr[kVxReg];
+#pragma unroll
+    for (int q = 0; q < kVxReg; ++q) {
+        const int j = threadIdx.x + q * kVxThreads;
+        const bool ok = j < f, old = ok && !init;
+        fr[q] = ok ? sF[j] : 0.f;
+        vr[q] = old ? vv[j] : 0.f;
+        wr[q] = old ? ww[j] : 0.f;
+        xr[q] = old ? xx[j] : 0.f;
+    }
     // two rows per thread per step: every load of both rows is in flight
     // before the sums (rows <= nu nk <= 36 partial dots, 9 float4)
-    for (int j0 = threadIdx.x; j0 < f; j0 += 2 * blockDim.x) {
-        float4 s4[2][9];
-        float vo[2], sf[2];
+    float4 s4[2][9];
+    auto load = [&](int j0) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int j = j0 + h * blockDim.x;
+            const int j = j0 + h * kVxThreads;
             const bool ok = j < f;
-            const float4 *pr = reinterpret_cast<const float4 *>(B.padj + (size_t)(ok ? j : 0) * ld);
+            const float4 *pr = reinterpret_cast<const float4 *>(padj + (size_t)(ok ? j : 0) * ld);
 #pragma unroll
             for (int q = 0; q < 9; ++q) s4[h][q] = (ok && q < r4) ? pr[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-            sf[h] = ok ? sF[j] : 0.f;
-            vo[h] = (ok && !init) ? vv[j] : 0.f;
         }
+    };
+    load(threadIdx.x);
+    // beta from the reduction's CTA shares
+    double part = 0.0;
+    for (int b = threadIdx.x; b < ctl->nsums; b += kVxThreads) part += ctl->sums[b];
+    const double alpha_prev = ctl->alpha;
+    double beta = 0.0, us = 0.0;
+    {
+        const double t = block_sum_w0(part, sb);
+        if (w0) {
+            beta = sqrt(t);
+            us = beta > 0.0 ? 1.0 / beta : 0.0;
+            s_c[0] = (float)us;
+            s_c[1] = (float)beta;
+        }
+    }
+    const float sc = 1.f / (ctl->sXF * ctl->sB);
+    __syncthreads();
+    const float fus = s_c[0], fb = s_c[1];
+    float ss = 0.f;
+    // one row: its new v (before normalisation) from the loaded partial dots
+    auto row = [&](int h, int j, float sf, float vo) {
+        float y = 0.f;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) y += (s4[h][q].x + s4[h][q].y) + (s4[h][q].z + s4[h][q].w);
+        for (int u = 4 * r4; u < rows; ++u) y += padj[(size_t)j * ld + u];
+        y *= sc;
+        const float vn = init ? sf * (y * fus) : sf * (y * fus) - fb * vo;
+        ss = fmaf(vn, vn, ss);
+        return vn;
+    };
+#pragma unroll
+    for (int q = 0; q < kVxReg; q += 2) {
+        const int j0 = threadIdx.x + q * kVxThreads;
+        if (q > 0 && j0 < f) load(j0);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (j0 + h * kVxThreads < f) vr[q + h] = row(h, j0 + h * kVxThreads, fr[q + h], vr[q + h]);
+    }
+    for (int j0 = threadIdx.x + kVxReg * kVxThreads; j0 < f; j0 += 2 * kVxThreads) {
+        load(j0);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int j = j0 + h * blockDim.x;
-            if (j >= f) continue;
-            float y = 0.f;
-#pragma unroll
-            for (int q = 0; q < 9; ++q) y += (s4[h][q].x + s4[h][q].y) + (s4[h][q].z + s4[h][q].w);
-            for (int u = 4 * r4; u < rows; ++u) y += B.padj[(size_t)j * ld + u];
-            y *= sc;
-            const float vn = init ? sf[h] * (y * fus) : sf[h] * (y * fus) - fb * vo[h];
-            vv[j] = vn;
-            ss = fmaf(vn, vn, ss);
+            const int j = j0 + h * kVxThreads;
+            if (j < f) vv[j] = row(h, j, sF[j], init ? 0.f : vv[j]);
         }
     }
-    const double alpha = sqrt(vx_sum((double)ss, sb));
-    double rhobar = ctl->rhobar, phibar = ctl->phibar, anorm2 = ctl->anorm2, t1 = 0.0, t2 = 0.0, absc = 0.0;
-    if (init) {
-        phibar = beta;
-        rhobar = alpha;
-        anorm2 = 0.0;
-    } else {
-        anorm2 += alpha_prev * alpha_prev + beta * beta;
-        const double rho = hypot(rhobar, beta);
-        const double c = rhobar / rho, sn = beta / rho;
-        const double theta = sn * alpha;
-        rhobar = -c * alpha;
-        const double phi = c * phibar;
-        phibar = sn * phibar;
-        t1 = phi / rho;
-        t2 = -theta / rho;
-        absc = fabs(c);
+    double alpha = 0.0, rhobar = ctl->rhobar, phibar = ctl->phibar, anorm2 = ctl->anorm2, absc = 0.0;
+    {
+        const double t = block_sum_w0((double)ss, sb);
+        if (w0) {
+            alpha = sqrt(t);
+            if (init) {
+                phibar = beta;
+                rhobar = alpha;
+                anorm2 = 0.0;
+                const double ialpha = 1.0 / alpha;
+                if (lane == 0) s_c[2] = alpha > 0.0 ? (float)ialpha : 1.f;
+                if (lane == 0) s_c[3] = s_c[4] = 0.f;
+            } else {
+                // plane rotation; lanes 0..2: c, s, 1/alpha, then lanes 0, 1: the coefficients
+                anorm2 += alpha_prev * alpha_prev + beta * beta;
+                const double rho = hypot(rhobar, beta);
+                const double q = (lane == 0 ? rhobar : lane == 1 ? beta : 1.0) / (lane == 2 ? alpha : rho);
+                const double c = __shfl_sync(0xffffffffu, q, 0), sn = __shfl_sync(0xffffffffu, q, 1);
+                const double ialpha = __shfl_sync(0xffffffffu, q, 2);
+                const double theta = sn * alpha;
+                rhobar = -c * alpha;
+                const double phi = c * phibar;
+                phibar = sn * phibar;
+                absc = fabs(c);
+                const double t12 = (lane == 0 ? phi : -theta) / rho;
+                if (lane < 2) s_c[3 + lane] = (float)t12;
+                if (lane == 0) s_c[2] = alpha > 0.0 ? (float)ialpha : 1.f;
+            }
+        }
+        __syncthreads();
     }
-    const float ia = alpha > 0.0 ? (float)(1.0 / alpha) : 1.f, ft1 = (float)t1, ft2 = (float)t2;
+    const float ia = s_c[2], ft1 = s_c[3], ft2 = s_c[4];
     float xs2 = 0.f, wm = 0.f;
-#pragma unroll 4
-    for (int j = threadIdx.x; j < f; j += blockDim.x) {
-        const float vj = J.v[j] * ia;
-        J.v[j] = vj;
+    auto update = [&](int j, float vn, float wo, float xo, float sf) {
+        const float vj = vn * ia;
+        vv[j] = vj;
         if (init) {
-            J.w[j] = vj;
-            J.xs[j] = 0.f;
+            ww[j] = vj;
+            xx[j] = 0.f;
         } else {
-            const float xj = J.xs[j] + ft1 * J.w[j];
-            J.xs[j] = xj;
-            J.w[j] = vj + ft2 * J.w[j];
+            const float xj = xo + ft1 * wo;
+            xx[j] = xj;
+            ww[j] = vj + ft2 * wo;
             xs2 = fmaf(xj, xj, xs2);
         }
-        const float wv = J.sF[j] * vj;
+        const float wv = sf * vj;
         B.wl[j] = wv;
         wm = fmaxf(wm, fabsf(wv));
+    };
+#pragma unroll
+    for (int q = 0; q < kVxReg; ++q) {
+        const int j = threadIdx.x + q * kVxThreads;
+        if (j < f) update(j, vr[q], wr[q], xr[q], fr[q]);
     }
-    const double xnorm2 = vx_sum((double)xs2, sb);
+#pragma unroll 4
+    for (int j = threadIdx.x + kVxReg * kVxThreads; j < f; j += kVxThreads)
+        update(j, vv[j], init ? 0.f : ww[j], init ? 0.f : xx[j], sF[j]);
     for (int o = 16; o; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
-    if ((threadIdx.x & 31) == 0) swm[threadIdx.x >> 5] = wm;
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    if (lane == 0) swm[threadIdx.x >> 5] = wm;
+    const double xnorm2 = block_sum_w0((double)xs2, sb);     // its barrier publishes swm too
+    if (!w0) return;
+    // lanes 0, 1: ||x||, ||B||
+    const double q = sqrt(lane == 0 ? xnorm2 : anorm2);
+    const double xnorm = __shfl_sync(0xffffffffu, q, 0), anorm = __shfl_sync(0xffffffffu, q, 1);
+    if (lane == 0) {
         for (int w = 0; w < kVxThreads / 32; ++w) wm = fmaxf(wm, swm[w]);
         ctl->mx_w = __float_as_uint(wm);
         ctl->mx_t = 0u;                       // the image of t is consumed
@@ -837,10 +893,8 @@ __global__ void __launch_bounds__(kVxThreads) k_ws_vx(const JobDev *Jp, WsBufs B
             more = alpha > 0.0 && beta > 0.0 && ctl->maxit >= 1;
         } else {
             ctl->it++;
-            const double xnorm = sqrt(xnorm2);
             const double rnorm = phibar;
             const double arnorm = phibar * alpha * absc;
-            const double anorm = sqrt(anorm2);
             more = ctl->it < ctl->maxit;
             if (rnorm <= J.lsqr_btol * ctl->bnorm + J.lsqr_atol * anorm * xnorm) more = false;
             if (arnorm <= J.lsqr_atol * anorm * rnorm) more = false;
