@@ -167,9 +167,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bounds_tc(JobDev *const *jobs) 
     const JobDev &J = *jobs[blockIdx.y];
     if (J.flags[0] != 0) return;
     constexpr bool BF = MODE == 2;
-    extern __shared__ float4 smem4[];
-    unsigned char *dyn = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem4) + 1023) & ~uintptr_t(1023));
+    unsigned char *dyn = dyn_smem();
     __shared__ uint64_t bars[2];
     __shared__ uint32_t slot;
     __shared__ double dbuf[kThreads / 32];
@@ -208,9 +206,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_psi_adj_tc(const JobDev *Jp, co
                                                            double *out) {
     const JobDev &J = *Jp;
     constexpr bool BF = MODE == 2;
-    extern __shared__ float4 smem4[];
-    unsigned char *dyn = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem4) + 1023) & ~uintptr_t(1023));
+    unsigned char *dyn = dyn_smem();
     __shared__ uint64_t bars[2];
     __shared__ uint32_t slot;
     __shared__ double dbuf[kThreads / 32];
@@ -268,9 +264,7 @@ template <int MODE>
 __global__ void __launch_bounds__(kWideThreads, 1) k_bounds_wide(JobDev *const *jobs) {
     const JobDev &J = *jobs[blockIdx.y];
     if (J.flags[0] != 0) return;
-    extern __shared__ float4 smem4[];
-    unsigned char *dyn = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem4) + 1023) & ~uintptr_t(1023));
+    unsigned char *dyn = dyn_smem();
     __shared__ uint64_t bars[kWideBars];
     __shared__ uint32_t slot;
     const int ntiles = tc_num_tiles(J.n_l, J.n_m);
@@ -297,9 +291,7 @@ __global__ void k_emb_one(const JobDev *Jp, const TC *U) {
 template <int MODE>
 __global__ void __launch_bounds__(kWideThreads, 1) k_psi_adj_wide(const JobDev *Jp, double *out) {
     const JobDev &J = *Jp;
-    extern __shared__ float4 smem4[];
-    unsigned char *dyn = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem4) + 1023) & ~uintptr_t(1023));
+    unsigned char *dyn = dyn_smem();
     __shared__ uint64_t bars[kWideBars];
     __shared__ uint32_t slot;
     const int ntiles = tc_num_tiles(J.n_l, J.n_m);
@@ -323,9 +315,7 @@ template <int MODE>
 __global__ void __launch_bounds__(kFwdThreads, 1) k_fwd_wide(const JobDev *Jp, const float *w, const unsigned *wbits,
                                                             FwdMap map, float *part) {
     const JobDev &J = *Jp;
-    extern __shared__ float4 smem4[];
-    unsigned char *dyn = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem4) + 1023) & ~uintptr_t(1023));
+    unsigned char *dyn = dyn_smem();
     __shared__ uint64_t bars[5];
     __shared__ uint32_t slot;
     const int pr = blockIdx.y, S = gridDim.x;
@@ -662,8 +652,12 @@ struct SolveShared {
     float wsm[kTile];
     float red[kTile + 16 * kTile];
     float ls[8];          // LSQR: coefficients that warp 0 hands to the CTA
+    float fm[kThreads / 32];
     int lsi;
 };
+// At namespace scope, so that the solver's out-of-line functions address it
+// (and the operand tiles, through dyn_smem) as shared memory.
+__shared__ SolveShared g_solve;
 
 // Clock cycles of a solve's phases (one thread's view; reported as doubles).
 struct SolveCycles {
@@ -746,13 +740,13 @@ __device__ void adjoint_list(const JobDev &J, const float2 *U, const int *pos, i
             [&](int t, int b) {
                 const int j0 = t * kTcM;
                 tc_gen_X_cache<BF>(J, T, b, pos, j0, min(kTcM, n - j0), sXl);
-                T.sX[b] = sXl;
+                
             },
             [&](int t, int b) {
                 const int j0 = t * kTcM;
                 const int np = min(kTcM, n - j0);
                 tc_epilogue<BF>(T, b, red);
-                const float inv = 1.f / (T.sX[b] * T.sX[b] * sB);
+                const float inv = 1.f / (sXl * sXl * sB);
                 if (threadIdx.x < np) epi(j0 + threadIdx.x, red[threadIdx.x] * inv);
                 __syncthreads();
             });
@@ -829,32 +823,10 @@ __device__ void adjoint_full(const JobDev &J, const float2 *U, float2 *A, TcWork
 // iteration at p = 48 (f <= 256).
 template <int MODE>
 __device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShared &S, SolveCycles &cyc) {
-    constexpr bool BF = MODE == 2;
     const int p = J.p, pp = p * p;
     const int *__restrict__ fpos = J.fpos;
     float2 *__restrict__ t = J.W0;
-    // free-set tiles resident in shared memory for the whole solve (tensor
-    // cores, Kp = 64, at most two 128-pixel tiles); the f-vectors then live
-    // in shared memory too
-    bool resident = false;
-    float sXr = 1.f;
-    unsigned char *stage = nullptr;
     float *v = J.v, *w = J.w, *xs = J.xs, *sF = J.sF, *wt = J.xs + J.cap;
-    if constexpr (MODE != 0) {
-        resident = T.Kp == 64 && f <= 2 * kTcM;
-        if (resident) {
-            stage = T.Blo + (T.Blo - T.Bhi);
-            float *fv = reinterpret_cast<float *>(stage + tc_stage_bytes(p));
-            v = fv;
-            w = fv + 2 * kTcM;
-            xs = fv + 4 * kTcM;
-            sF = fv + 6 * kTcM;
-            wt = fv + 8 * kTcM;
-            sXr = list_scale(J, fpos, f, S.dbuf);
-            tc_gen_X_cache<BF>(J, T, 0, fpos, 0, min(kTcM, f), sXr);
-            if (f > kTcM) tc_gen_X_cache<BF>(J, T, 1, fpos, kTcM, f - kTcM, sXr);
-        }
-    }
     {
         const int *__restrict__ supp = J.supp;
         const float *__restrict__ scale = J.scale;
@@ -883,12 +855,6 @@ __device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShare
         return 0;
     }
     auto adjoint = [&](auto epi) {
-        if constexpr (MODE != 0) {
-            if (resident) {
-                tc_adjoint_resident<BF>(T, t, p, f, sXr, S.red, S.dbuf, epi, cyc.aux);
-                return;
-            }
-        }
         adjoint_list<MODE>(J, t, fpos, f, A, T, S.red, S.dbuf, epi);
     };
     {
@@ -930,34 +896,14 @@ __device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShare
         long long tc0 = clock64();
         const float fa = S.ls[0];
         acc = 0.f;
-        bool done = false;
-        if constexpr (MODE != 0) {
-            if (resident) {
-                float inv;
-                const float *G = tc_forward_resident<BF>(T, stage, f, wt, sXr, &inv, S.dbuf, cyc.aux);
-                const long long cu = clock64();
-                for (int e = threadIdx.x; e < pp; e += blockDim.x) {
-                    const int bcol = e / p, a = e - bcol * p;
-                    float2 kv = G ? tc_k_entry(G, T.Kp, a, bcol) : make_float2(0.f, 0.f);
-                    const float2 to = t[e];
-                    const float2 tn = make_float2(kv.x * inv - fa * to.x, kv.y * inv - fa * to.y);
-                    t[e] = tn;
-                    acc = fmaf(tn.x, tn.x, fmaf(tn.y, tn.y, acc));
-                }
-                cyc.aux[2] += clock64() - cu;
-                done = true;
-            }
-        }
-        if (!done) {
-            forward_cache<MODE>(J, T, fpos, wt, f, nullptr, false, J.W1, A, S.wsm, S.dbuf);
-            const float2 *__restrict__ W1 = J.W1;
-            for (int e = threadIdx.x; e < pp; e += blockDim.x) {
-                const float2 mv = W1[e];
-                const float2 to = t[e];
-                const float2 tn = make_float2(mv.x - fa * to.x, mv.y - fa * to.y);
-                t[e] = tn;
-                acc = fmaf(tn.x, tn.x, fmaf(tn.y, tn.y, acc));
-            }
+        forward_cache<MODE>(J, T, fpos, wt, f, nullptr, false, J.W1, A, S.wsm, S.dbuf);
+        const float2 *__restrict__ W1 = J.W1;
+        for (int e = threadIdx.x; e < pp; e += blockDim.x) {
+            const float2 mv = W1[e];
+            const float2 to = t[e];
+            const float2 tn = make_float2(mv.x - fa * to.x, mv.y - fa * to.y);
+            t[e] = tn;
+            acc = fmaf(tn.x, tn.x, fmaf(tn.y, tn.y, acc));
         }
         cyc.fwd += clock64() - tc0;
         double ss = block_sum_w0((double)acc, S.dbuf);
@@ -1017,10 +963,453 @@ __device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShare
         __syncthreads();
         if (S.lsi) break;
     }
-    if (xs != J.xs)
-        for (int j = threadIdx.x; j < f; j += blockDim.x) J.xs[j] = xs[j];
     __syncthreads();
     return min(it, maxit);
+}
+
+// ---------------------------------------------------------------- resident LSQR
+// LSQR on the free set for f <= 256 on tensor cores (Kp = 32 or 64), with
+// everything that an iteration touches on the SM: the free-set tiles in
+// shared memory (tile 0 in buffer 0, tile 1 in buffer 1), the p x p vector t
+// in registers (thread tid: entries tid + 256 k), v, w, x, s_F of free pixel
+// j in the registers of thread j.  Same arithmetic and the same order of
+// every sum as lsqr_cta's; the fused multiply-adds are written out, so that
+// the rounding does not depend on what the compiler contracts where.
+//
+// Bound by latency: a chain of small phases in one CTA, so what counts is
+// the barriers and the exposed scalars.  An iteration has 8 barriers (f <=
+// 64); the weighted rows of the forward are staged 64 at a time into the B
+// region, which is free until the B image of t is rebuilt; the norm of t and
+// its largest entry share a reduction, so that warp 0 forms beta while the
+// others build B; the rotation runs behind the issued MMAs, the stopping
+// tests behind the next iteration's staging.
+//
+// Forward: Kp = 64 as the Gram matrix of the tiles on tensor cores, Kp = 32
+// in FP32 from the free vectors themselves (shared memory), thread-owned
+// entries of t directly: at p <= 32 the Gram matrix's read-out costs more
+// than the sums, and the products keep lsqr_cta's FP32 bits.
+constexpr int kResF = 2 * kTcM;         // most free pixels
+constexpr int kResRows = 64;            // weighted rows staged at a time
+
+// Bytes behind the operand tiles: Kp = 64: the Gram read-out's overhang over
+// the B region; Kp = 32: the free vectors.  Then the weights (kResF floats).
+__host__ __device__ inline size_t res_extra_bytes(int p) {
+    return ((p + 31) / 32 * 32 == 32 ? (size_t)kResF * p * sizeof(float2) : 1024) + kResF * sizeof(float);
+}
+
+// The split B image of the matrix whose entries e = tid + 256 k (e = n p + a:
+// row a, column n) are tr[k]: entry (a, n) appears at (n, a) and (Kp + n, Kp +
+// a) as Re, at (n, Kp + a) as Im, at (Kp + n, a) as -Im.  Even p: neighbouring
+// lanes hold a and a + 1 and share the work, the even lane writing the Re
+// pairs, the odd lane the Im pairs.
+template <bool BF16>
+__device__ __forceinline__ void res_build_B(const TcWork &T, int p, const float2 *tr, float sc) {
+    const int Kp = T.Kp, N = 2 * Kp, nc8 = Kp / 8, pp = p * p;
+    const bool even = (p & 1) == 0;
+    const bool odd_lane = threadIdx.x & 1;
+    unsigned char *bh = T.Bhi(), *bl = T.Blo();
+    // padding: whole 16-byte chunks
+    if (p < Kp) {
+        const int live = (p + 7) / 8;
+        for (int it = threadIdx.x; it < N * 2 * nc8; it += kThreads) {
+            const int n = it / (2 * nc8), c = it - n * (2 * nc8);
+            if ((n >= Kp ? n - Kp : n) >= p || (c >= nc8 ? c - nc8 : c) >= live) {
+                const uint32_t off = sw128_off(n, c, N);
+                *reinterpret_cast<uint4 *>(bh + off) = make_uint4(0u, 0u, 0u, 0u);
+                *reinterpret_cast<uint4 *>(bl + off) = make_uint4(0u, 0u, 0u, 0u);
+            }
+        }
+    }
+    const int da = kThreads % p, dn = kThreads / p;
+    int a = threadIdx.x % p, n = threadIdx.x / p;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        if (k * kThreads >= pp) break;
+        const bool ok = threadIdx.x + k * kThreads < pp;
+        const float2 t = tr[k];
+        const float other = __shfl_xor_sync(0xffffffffu, odd_lane ? t.x : t.y, 1);
+        if (ok) {
+            if (even) {
+                const int a0 = a & ~1, c8 = a0 >> 3, ao = (a0 & 7) * 2;
+                uint32_t hi, lo;
+                auto put = [&](int row, int ch) {
+                    const uint32_t off = sw128_off(row, ch, N) + ao;
+                    *reinterpret_cast<uint32_t *>(bh + off) = hi;
+                    *reinterpret_cast<uint32_t *>(bl + off) = lo;
+                    // the rest of the last live chunk is padding
+                    if (a0 + 2 == p)
+                        for (int q = ao + 4; q < 16; q += 4) {
+                            *reinterpret_cast<uint32_t *>(bh + off - ao + q) = 0u;
+                            *reinterpret_cast<uint32_t *>(bl + off - ao + q) = 0u;
+                        }
+                };
+                if (!odd_lane) {
+                    split2<BF16>(t.x * sc, other * sc, hi, lo);
+                    put(n, c8);
+                    put(Kp + n, nc8 + c8);
+                } else {
+                    split2<BF16>(other * sc, t.y * sc, hi, lo);
+                    put(n, nc8 + c8);
+                    split2<BF16>(-other * sc, -t.y * sc, hi, lo);
+                    put(Kp + n, c8);
+                }
+            } else {
+                const int c8 = a >> 3, ao = (a & 7) * 2;
+                auto put = [&](int row, int ch, float v) {
+                    uint32_t hi, lo;
+                    split2<BF16>(v, 0.f, hi, lo);
+                    const uint32_t off = sw128_off(row, ch, N) + ao;
+                    *reinterpret_cast<uint16_t *>(bh + off) = (uint16_t)hi;
+                    *reinterpret_cast<uint16_t *>(bl + off) = (uint16_t)lo;
+                    if (a + 1 == p)
+                        for (int q = ao + 2; q < 16; q += 2) {
+                            *reinterpret_cast<uint16_t *>(bh + off - ao + q) = 0;
+                            *reinterpret_cast<uint16_t *>(bl + off - ao + q) = 0;
+                        }
+                };
+                put(n, c8, t.x * sc);
+                put(Kp + n, nc8 + c8, t.x * sc);
+                put(n, nc8 + c8, t.y * sc);
+                put(Kp + n, c8, -t.y * sc);
+            }
+        }
+        a += da;
+        n += dn;
+        if (a >= p) {
+            a -= p;
+            ++n;
+        }
+    }
+}
+
+// Rows r0 .. r0 + nst - 1 of the resident tiles times sW w[row] (zero from
+// row f on) as an MN-major operand of kResRows rows per feature block at dst
+// (hi, then lo), re-split.
+template <bool BF16>
+__device__ __forceinline__ void res_stage_rows(const TcWork &T, unsigned char *dst, int r0, int nst, int f,
+                                               const float *w, float sW) {
+    const int nch = 2 * T.Kp / 8;
+    const size_t half_bytes = (size_t)(2 * T.Kp / 64) * kResRows * 128;
+    const int tile = r0 / kTcM, rt = r0 % kTcM;
+#pragma unroll 2
+    for (int it = threadIdx.x; it < nst * nch; it += kThreads) {
+        const int rr = it / nch, c = it - rr * nch;
+        const uint32_t src = sw128_off(rt + rr, c, kTcM);
+        const uint32_t off = sw128_off(rr, c, kResRows);
+        const float wr = r0 + rr < f ? sW * w[r0 + rr] : 0.f;
+        const uint4 h4 = *reinterpret_cast<const uint4 *>(T.Xhi(tile) + src);
+        const uint4 l4 = *reinterpret_cast<const uint4 *>(T.Xlo(tile) + src);
+        const uint32_t hw[4] = {h4.x, h4.y, h4.z, h4.w}, lw[4] = {l4.x, l4.y, l4.z, l4.w};
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float2 h = unpack2<BF16>(hw[q]), l = unpack2<BF16>(lw[q]);
+            split2<BF16>(__fmul_rn(wr, h.x + l.x), __fmul_rn(wr, h.y + l.y), hi[q], lo[q]);
+        }
+        *reinterpret_cast<uint4 *>(dst + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        *reinterpret_cast<uint4 *>(dst + half_bytes + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    }
+}
+
+//
+// Out of line: inlined into k_solve the two spilled 2.5 KB per thread.
+template <int MODE>
+__device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, SolveCycles &cio) {
+    constexpr bool BF = MODE == 2;
+    TcWork T = Tio;
+    T.base = dyn_smem();
+    SolveCycles cyc;
+    const int p = J.p, pp = p * p, Kp = T.Kp, N = 2 * Kp;
+    const bool gram = Kp == 64;
+    SolveShared &S = g_solve;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool w0 = warp == 0;
+    const int j = threadIdx.x;                    // this thread's free pixel
+    const bool mine = j < f;
+    const int ntiles = f > kTcM ? 2 : 1;
+    const int *__restrict__ fpos = J.fpos;
+    unsigned char *extra = T.Blo() + (T.Blo() - T.Bhi());
+    float2 *C = reinterpret_cast<float2 *>(extra);                              // Kp = 32: free vectors
+    float *wt = reinterpret_cast<float *>(extra + res_extra_bytes(p)) - kResF;
+    const float sX = list_scale(J, fpos, f, S.dbuf);
+    for (int t = 0; t < ntiles; ++t) tc_gen_X_cache<BF>(J, T, t, fpos, t * kTcM, min(kTcM, f - t * kTcM), sX);
+    if (!gram)
+        for (int e = threadIdx.x; e < f * p; e += kThreads) {
+            const int r = e / p;
+            C[e] = J.cvec[(size_t)fpos[r] * p + e - r * p];
+        }
+    const float sF = mine ? J.scale[J.supp[fpos[j]]] : 0.f;
+    float v = 0.f, w = 0.f, x = 0.f;
+    float2 tr[16];
+    const int da = kThreads % p, dn = kThreads / p;
+    const int a_first = threadIdx.x % p, n_first = threadIdx.x / p;
+    float acc = 0.f, mx = 0.f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const int e = threadIdx.x + k * kThreads;
+        tr[k] = e < pp ? J.W0[e] : make_float2(0.f, 0.f);
+        acc = fmaf(tr[k].x, tr[k].x, fmaf(tr[k].y, tr[k].y, acc));
+        mx = fmaxf(mx, fmaxf(fabsf(tr[k].x), fabsf(tr[k].y)));
+    }
+    // CTA sum (FP64, warp 0) and maximum (every thread) after one barrier
+    auto reduce = [&](float sum, float m) -> double {
+        double d = (double)sum;
+        for (int o = 16; o; o >>= 1) {
+            d += __shfl_xor_sync(0xffffffffu, d, o);
+            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        }
+        if (lane == 0) {
+            S.dbuf[warp] = d;
+            S.fm[warp] = m;
+        }
+        __syncthreads();
+        double t = 0.0;
+        if (w0)
+#pragma unroll
+            for (int q = 0; q < kThreads / 32; ++q) t += S.dbuf[q];
+        return t;
+    };
+    auto cta_max = [&]() {
+        float m = S.fm[0];
+#pragma unroll
+        for (int q = 1; q < kThreads / 32; ++q) m = fmaxf(m, S.fm[q]);
+        return m;
+    };
+    auto pow2_of = [](float m) { return m > 0.f ? exp2f(-ceilf(log2f(m))) : 1.f; };
+    // scalars of the recurrence, valid in warp 0
+    double alpha = 0.0, beta = 0.0, bnorm = 0.0, us = 0.0, phibar = 0.0, rhobar = 0.0, anorm2 = 0.0, absc = 0.0;
+    double rho = 0.0, cs = 0.0, sn = 0.0, phi = 0.0;
+    // y_j = Re(c_j^H t c_j) (scaled back), thread j; warp 0 runs `behind`
+    // while the MMAs of the first tile are in flight
+    const uint32_t idesc = idesc_f16(N, BF ? 1 : 0);
+    auto adjoint = [&](auto behind) -> float {
+        const long long c0 = clock64();
+        const float sB = pow2_of(cta_max()) * kLift;
+        res_build_B<BF>(T, p, tr, sB);
+        fence_async_smem();
+        __syncthreads();
+        if (w0) {
+            if (lane == 0)
+                for (int t = 0; t < ntiles; ++t) tc_issue(T, t, idesc);
+            __syncwarp();
+            behind();
+        }
+        const long long c1 = clock64();
+        for (int t = 0; t < ntiles; ++t) {
+            T.wait(t);
+            tc_fence_after();
+            S.red[t * 2 * kTcM + (warp >> 2) * kTcM + 32 * (warp & 3) + lane] = tc_row_dot<BF>(T, t);
+        }
+        tc_fence_before();
+        __syncthreads();
+        cyc.aux[3] += c1 - c0;
+        cyc.aux[5] += clock64() - c1;
+        const float *r = S.red + (j >> 7) * 2 * kTcM + (j & (kTcM - 1));
+        return mine ? (r[0] + r[kTcM]) * (1.f / (sX * sX * sB)) : 0.f;
+    };
+    // write the solution and hand back the barriers' phases and the counters
+    auto leave = [&](int its) {
+        if (mine) J.xs[j] = x;
+        Tio.phase = T.phase;
+        Tio.timeouts = T.timeouts;
+        cio.fwd += cyc.fwd;
+        cio.adj += cyc.adj;
+        for (int q = 0; q < 6; ++q) cio.aux[q] += cyc.aux[q];
+        __syncthreads();
+        return its;
+    };
+    {
+        const double ss = reduce(acc, mx);
+        if (w0) {
+            beta = bnorm = phibar = sqrt(ss);
+            us = 1.0 / beta;
+            S.ls[2] = (float)us;
+            S.lsi = beta == 0.0;
+        }
+    }
+    {
+        const float y = adjoint([]() {});
+        if (S.lsi) return leave(0);
+        if (mine) v = sF * (y * S.ls[2]);
+    }
+    {
+        const double ss = reduce(fmaf(v, v, 0.f), 0.f);
+        if (w0) {
+            alpha = rhobar = sqrt(ss);
+            S.ls[5] = (float)(1.0 / alpha);
+            S.ls[0] = (float)(alpha * us);
+            S.lsi = alpha == 0.0;
+        }
+        __syncthreads();
+        if (S.lsi) return leave(0);
+        v *= S.ls[5];
+        w = v;
+        const float wj = sF * v;
+        wt[j] = wj;
+        reduce(0.f, fabsf(wj));
+    }
+    const int maxit = J.lsqr_maxit > 0 ? J.lsqr_maxit : 4 * f + 20;
+    const double atol = J.lsqr_atol, btol = J.lsqr_btol;
+    const uint32_t fdesc = idesc_f16_mn(N, BF ? 1 : 0);
+    int it = 0;
+    for (it = 1; it <= maxit; ++it) {
+        // t <- M v - alpha u  (u = t us), beta = ||t||; the stopping tests of
+        // the iteration before arrive with the first barrier
+        const long long c0 = clock64();
+        bool stop = false;
+        float fa = 0.f, inv = 0.f;
+        const float *G = nullptr;
+        if (gram) {
+            const float sW = pow2_of(cta_max());
+            const int ngrp = (f + kResRows - 1) / kResRows;
+            for (int g = 0; g < ngrp; ++g) {
+                const int b = g & 1, r0 = g * kResRows, ks = (min(kResRows, f - r0) + 15) / 16;
+                unsigned char *st = T.Bhi() + b * (2 * 2 * kResRows * 128);
+                if (g >= 2) {
+                    T.wait(b);
+                    tc_fence_after();
+                }
+                res_stage_rows<BF>(T, st, r0, 16 * ks, f, wt, sW);
+                fence_async_smem();
+                __syncthreads();
+                if (g == 0) {
+                    fa = S.ls[0];
+                    stop = it > 1 && S.lsi;
+                    if (stop) break;
+                }
+                if (threadIdx.x == 0) {
+                    tc_fence_after();
+                    const uint32_t ah = smem_u32(st), al = ah + 2 * kResRows * 128;
+                    const int tile = r0 / kTcM;
+                    const uint32_t bo = (uint32_t)((r0 % kTcM) / 8) * 1024;
+                    const uint32_t bh = smem_u32(T.Xhi(tile)) + bo, bl = smem_u32(T.Xlo(tile)) + bo;
+                    const uint32_t d = T.tmem + (uint32_t)(2 * N);
+                    constexpr uint32_t alb = kResRows * 128, blb = kTcM * 128;
+                    for (int s = 0; s < ks; ++s) {
+                        const uint32_t o = s * 2048;
+                        mma_f16(d, sw128_desc_mn(ah + o, alb, 1024), sw128_desc_mn(bh + o, blb, 1024), fdesc,
+                                (g > 0 || s > 0) ? 1u : 0u);
+                        mma_f16(d, sw128_desc_mn(ah + o, alb, 1024), sw128_desc_mn(bl + o, blb, 1024), fdesc, 1u);
+                        mma_f16(d, sw128_desc_mn(al + o, alb, 1024), sw128_desc_mn(bh + o, blb, 1024), fdesc, 1u);
+                    }
+                    mma_commit(&T.bar[b]);
+                }
+            }
+            if (stop) break;
+            for (int g = max(0, ngrp - 2); g < ngrp; ++g) {
+                const int b = g & 1;
+                T.wait(b);
+            }
+            tc_fence_after();
+            inv = 1.f / (sX * sX * sW);
+            const long long c1 = clock64();
+            G = tc_read_fwd(T, reinterpret_cast<float *>(T.Bhi()));
+            cyc.aux[0] += c1 - c0;
+            cyc.aux[1] += clock64() - c1;
+        } else {
+            __syncthreads();
+            fa = S.ls[0];
+            if (it > 1 && S.lsi) break;
+        }
+        const long long c2 = clock64();
+        acc = 0.f;
+        mx = 0.f;
+        {
+            int a = a_first, n = n_first;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                if (k * kThreads >= pp) break;
+                if (threadIdx.x + k * kThreads < pp) {
+                    float2 kv;
+                    if (gram) {
+                        kv = tc_k_entry(G, Kp, a, n);
+                        kv = make_float2(__fmaf_rn(kv.x, inv, -__fmul_rn(fa, tr[k].x)),
+                                         __fmaf_rn(kv.y, inv, -__fmul_rn(fa, tr[k].y)));
+                    } else {
+                        float2 s = make_float2(0.f, 0.f);
+                        const float2 *ca = C + a, *cn = C + n;
+#pragma unroll 4
+                        for (int q = 0; q < f; ++q) {
+                            const float wq = wt[q];
+                            const float2 u = ca[q * p], z = cn[q * p];
+                            cfma(s, make_float2(wq * u.x, wq * u.y), make_float2(z.x, -z.y));
+                        }
+                        kv = make_float2(__fmaf_rn(-fa, tr[k].x, 0.f + s.x), __fmaf_rn(-fa, tr[k].y, 0.f + s.y));
+                    }
+                    tr[k] = kv;
+                    acc = fmaf(kv.x, kv.x, fmaf(kv.y, kv.y, acc));
+                    mx = fmaxf(mx, fmaxf(fabsf(kv.x), fabsf(kv.y)));
+                }
+                a += da;
+                n += dn;
+                if (a >= p) {
+                    a -= p;
+                    ++n;
+                }
+            }
+        }
+        double ss = reduce(acc, mx);
+        if (w0) {
+            beta = sqrt(ss);
+            us = beta > 0.0 ? 1.0 / beta : 0.0;
+            anorm2 += alpha * alpha + beta * beta;
+            S.ls[1] = (float)beta;
+            S.ls[2] = (float)us;
+        }
+        const long long c3 = clock64();
+        cyc.aux[2] += c3 - c2;
+        cyc.fwd += c3 - c0;
+        // v <- M^H u - beta v
+        const float y = adjoint([&]() {
+            // the rotation's part that does not need alpha; lanes 0, 1: c, s
+            rho = hypot(rhobar, beta);
+            const double q = (lane == 0 ? rhobar : beta) / rho;
+            const double c = __shfl_sync(0xffffffffu, q, 0);
+            sn = __shfl_sync(0xffffffffu, q, 1);
+            phi = c * phibar;
+            phibar = sn * phibar;
+            cs = c;
+        });
+        if (mine) v = __fmaf_rn(sF, __fmul_rn(y, S.ls[2]), -__fmul_rn(S.ls[1], v));
+        cyc.adj += clock64() - c3;
+        ss = reduce(mine ? fmaf(v, v, 0.f) : 0.f, 0.f);
+        if (w0) {
+            // lanes 0..2: the coefficients of x and w, 1/alpha
+            alpha = sqrt(ss);
+            const double theta = sn * alpha;
+            rhobar = -cs * alpha;
+            absc = fabs(cs);
+            const double q = (lane == 0 ? phi : lane == 1 ? -theta : 1.0) / (lane == 2 ? alpha : rho);
+            if (lane < 2) S.ls[3 + lane] = (float)q;
+            if (lane == 2) S.ls[5] = alpha > 0.0 ? (float)q : 1.f;
+        }
+        __syncthreads();
+        acc = 0.f;
+        mx = 0.f;
+        if (mine) {
+            const float t1 = S.ls[3], t2 = S.ls[4], ia = S.ls[5];
+            const float vj = __fmul_rn(v, ia);          // v <- v / alpha
+            v = vj;
+            const float xj = __fmaf_rn(t1, w, x);
+            x = xj;
+            w = __fmaf_rn(t2, w, vj);
+            acc = fmaf(xj, xj, 0.f);
+            const float wj = sF * vj;
+            wt[j] = wj;
+            mx = fabsf(wj);
+        }
+        ss = reduce(acc, mx);
+        if (w0) {
+            const double q = sqrt(lane == 0 ? ss : anorm2);
+            const double xnorm = __shfl_sync(0xffffffffu, q, 0), anorm = __shfl_sync(0xffffffffu, q, 1);
+            const double rnorm = phibar;
+            const double arnorm = phibar * alpha * absc;
+            S.lsi = rnorm <= btol * bnorm + atol * anorm * xnorm || arnorm <= atol * anorm * rnorm;
+            S.ls[0] = (float)(alpha * us);
+        }
+    }
+    // a stop is seen by the iteration after the one that caused it
+    return leave(it <= maxit ? it - 1 : maxit);
 }
 
 __device__ __forceinline__ double flops_fwd(int p, int n) { return 4.0 * p * (double)p * n; }
@@ -1052,12 +1441,10 @@ template <int MODE, bool PREP>
 __global__ void __launch_bounds__(kThreads, 1)
 k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
     const JobDev &J = *jobs[blockIdx.x];
-    extern __shared__ float4 smem4[];
     // one 1024-aligned region serves the CUDA-core chunk or the tensor tiles
-    unsigned char *dyn = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem4) + 1023) & ~uintptr_t(1023));
+    unsigned char *dyn = dyn_smem();
     float2 *A = reinterpret_cast<float2 *>(dyn);
-    __shared__ SolveShared S;
+    SolveShared &S = g_solve;
     __shared__ uint64_t tc_bar[2];
     __shared__ uint32_t tc_slot;
     DevInfo info{};
@@ -1139,7 +1526,17 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
                                     S.dbuf);
                 info.op_flops += flops_fwd(p, nu);
                 const long long t0 = clock64();
-                const int its = lsqr_cta<MODE>(J, f, A, T, S, cyc);
+                int its;
+                if (MODE != 0 && f <= kResF) {
+                    TcWork Tl = T;            // by reference only here: T stays in registers
+                    SolveCycles cl;
+                    its = lsqr_resident<MODE>(J, f, Tl, cl);
+                    T.phase = Tl.phase;
+                    T.timeouts = Tl.timeouts;
+                    cyc.fwd += cl.fwd;
+                    cyc.adj += cl.adj;
+                    for (int q = 0; q < 6; ++q) cyc.aux[q] += cl.aux[q];
+                } else its = lsqr_cta<MODE>(J, f, A, T, S, cyc);
                 cyc.lsqr += clock64() - t0;
                 info.lsqr_iters += its;
                 info.op_flops += (its + 1) * (flops_fwd(p, f) + flops_adj(p, f));
@@ -1386,9 +1783,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_psi_partial_tc(const JobDev *Jp
                                                                int per) {
     const JobDev &J = *Jp;
     constexpr bool BF = MODE == 2;
-    extern __shared__ float4 smem4[];
-    unsigned char *dyn = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem4) + 1023) & ~uintptr_t(1023));
+    unsigned char *dyn = dyn_smem();
     __shared__ uint64_t bars[2];
     __shared__ uint32_t slot;
     __shared__ double dbuf[kThreads / 32];
@@ -1454,8 +1849,7 @@ __global__ void k_d2f(const double *src, float *dst, int n) {
 // ---------------------------------------------------------------- launchers
 size_t solve_smem_bytes(int p, int mode) {
     size_t b = (size_t)p * kTile * sizeof(float2);
-    // tensor tiles + forward staging + five LSQR f-vectors of 256 floats
-    const size_t tc = tc_smem_bytes(p) + tc_stage_bytes(p) + 10 * kTcM * sizeof(float);
+    const size_t tc = tc_smem_bytes(p) + res_extra_bytes(p);
     if (mode != 0) b = b > tc ? b : tc;
     return b + 1024;
 }

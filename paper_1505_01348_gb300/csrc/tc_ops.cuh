@@ -31,6 +31,13 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
+// The dynamic shared memory from its first 1024-byte boundary (computed by
+// pointer arithmetic, so that accesses keep the shared address space).
+__device__ __forceinline__ unsigned char *dyn_smem() {
+    extern __shared__ float4 smem4[];
+    return reinterpret_cast<unsigned char *>(smem4) + ((1024u - (smem_u32(smem4) & 1023u)) & 1023u);
+}
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
@@ -187,6 +194,14 @@ __device__ __forceinline__ void split2(float v0, float v1, uint32_t &hi, uint32_
     }
 }
 
+// The two values of a packed 16-bit pair.
+template <bool BF16>
+__device__ __forceinline__ float2 unpack2(uint32_t w) {
+    if (BF16) return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+    return make_float2(__half2float(__ushort_as_half((unsigned short)(w & 0xffffu))),
+                       __half2float(__ushort_as_half((unsigned short)(w >> 16))));
+}
+
 // Byte offset of 16-byte chunk c (8 elements, covering K = 8c .. 8c+7) of
 // row r in a swizzled K-major tile with R rows.
 __device__ __forceinline__ uint32_t sw128_off(int r, int c, int R) {
@@ -197,14 +212,25 @@ __device__ __forceinline__ uint32_t sw128_off(int r, int c, int R) {
 // Tensor-core workspace of one CTA: two X tiles and two accumulators so that
 // generating tile t+1 and the epilogue of tile t overlap the MMAs.
 struct TcWork {
-    unsigned char *Xhi[2], *Xlo[2];  // 1024-aligned operand tiles (pixels x 2Kp)
-    unsigned char *Bhi, *Blo;        // (2Kp x 2Kp)
+    unsigned char *base;             // 1024-aligned shared memory: X tiles, then B
     uint64_t *bar;                   // two MMA completion barriers
     uint32_t tmem;                   // accumulator base (lane 0, column 0)
-    uint32_t phase[2];               // parity of each barrier's next completion
-    float sX[2];                     // scale of the X tile in each buffer
+    uint32_t phase;                  // parity of barrier b's next completion in bit b
     int Kp;                          // p rounded up to 32
     int timeouts;                    // bounded waits that ran out
+
+    // operand tiles: X (pixels x 2Kp) of buffer b, B (2Kp x 2Kp)
+    __device__ __forceinline__ uint32_t x_bytes() const { return (uint32_t)(kTcM * 4 * Kp); }
+    __device__ __forceinline__ uint32_t b_bytes() const { return (uint32_t)(8 * Kp * Kp); }
+    __device__ __forceinline__ unsigned char *Xhi(int b) const { return base + 2 * b * x_bytes(); }
+    __device__ __forceinline__ unsigned char *Xlo(int b) const { return base + (2 * b + 1) * x_bytes(); }
+    __device__ __forceinline__ unsigned char *Bhi() const { return base + 4 * x_bytes(); }
+    __device__ __forceinline__ unsigned char *Blo() const { return base + 4 * x_bytes() + b_bytes(); }
+    // Wait for the next completion of barrier b.
+    __device__ __forceinline__ void wait(int b) {
+        if (!mbar_wait(&bar[b], (phase >> b) & 1u)) timeouts++;
+        phase ^= 1u << b;
+    }
 };
 
 // Bytes of shared memory the operand tiles need for p (plus 1024 alignment).
@@ -225,16 +251,9 @@ __host__ __device__ inline uint32_t tc_tmem_cols(int p) {
 
 // Carve the operand tiles from a 1024-aligned shared-memory region.
 __device__ inline void tc_carve(TcWork &T, unsigned char *base, int p) {
+    T.base = base;
     T.Kp = (p + 31) / 32 * 32;
-    const size_t x = (size_t)kTcM * 2 * T.Kp * 2;
-    const size_t b = (size_t)2 * T.Kp * 2 * T.Kp * 2;
-    T.Xhi[0] = base;
-    T.Xlo[0] = base + x;
-    T.Xhi[1] = base + 2 * x;
-    T.Xlo[1] = base + 3 * x;
-    T.Bhi = base + 4 * x;
-    T.Blo = base + 4 * x + b;
-    T.phase[0] = T.phase[1] = 0;
+    T.phase = 0;
     T.timeouts = 0;
 }
 
@@ -324,19 +343,19 @@ __device__ float tc_build_B(const float2 *U, int p, TcWork &T, double *sbuf) {
         uint4 hi, lo;
         split8<BF16>(re, hi, lo);                       // (re row, re col): Re V
         uint32_t off = sw128_off(n, c8, N);
-        *reinterpret_cast<uint4 *>(T.Bhi + off) = hi;
-        *reinterpret_cast<uint4 *>(T.Blo + off) = lo;
+        *reinterpret_cast<uint4 *>(T.Bhi() + off) = hi;
+        *reinterpret_cast<uint4 *>(T.Blo() + off) = lo;
         off = sw128_off(Kp + n, nc8 + c8, N);           // (im row, im col): Re V
-        *reinterpret_cast<uint4 *>(T.Bhi + off) = hi;
-        *reinterpret_cast<uint4 *>(T.Blo + off) = lo;
+        *reinterpret_cast<uint4 *>(T.Bhi() + off) = hi;
+        *reinterpret_cast<uint4 *>(T.Blo() + off) = lo;
         split8<BF16>(nim, hi, lo);                      // (re row, im col): -Im V
         off = sw128_off(n, nc8 + c8, N);
-        *reinterpret_cast<uint4 *>(T.Bhi + off) = hi;
-        *reinterpret_cast<uint4 *>(T.Blo + off) = lo;
+        *reinterpret_cast<uint4 *>(T.Bhi() + off) = hi;
+        *reinterpret_cast<uint4 *>(T.Blo() + off) = lo;
         split8<BF16>(im, hi, lo);                       // (im row, re col): Im V
         off = sw128_off(Kp + n, c8, N);
-        *reinterpret_cast<uint4 *>(T.Bhi + off) = hi;
-        *reinterpret_cast<uint4 *>(T.Blo + off) = lo;
+        *reinterpret_cast<uint4 *>(T.Bhi() + off) = hi;
+        *reinterpret_cast<uint4 *>(T.Blo() + off) = lo;
     }
     return sc;
 }
@@ -346,8 +365,8 @@ __device__ float tc_build_B(const float2 *U, int p, TcWork &T, double *sbuf) {
 __device__ inline void tc_issue(const TcWork &T, int b, uint32_t idesc) {
     const int Kp = T.Kp, N = 2 * Kp, nks = (2 * Kp) / 16;
     tc_fence_after();
-    const uint32_t xh = smem_u32(T.Xhi[b]), xl = smem_u32(T.Xlo[b]);
-    const uint32_t bh = smem_u32(T.Bhi), bl = smem_u32(T.Blo);
+    const uint32_t xh = smem_u32(T.Xhi(b)), xl = smem_u32(T.Xlo(b));
+    const uint32_t bh = smem_u32(T.Bhi()), bl = smem_u32(T.Blo());
     const uint32_t d = T.tmem + (uint32_t)(b * N);
     for (int s = 0; s < nks; ++s) {
         const uint32_t kb = s >> 2, off = (s & 3) * 32;
@@ -377,8 +396,7 @@ __device__ inline void tc_run_tiles(TcWork &T, int ntiles, uint32_t idesc, Gen g
         pre(t);
         if (t + 1 < ntiles) gen(t + 1, b ^ 1);
         fence_async_smem();
-        if (!mbar_wait(&T.bar[b], T.phase[b])) T.timeouts++;
-        T.phase[b] ^= 1u;
+        T.wait(b);
         tc_fence_after();
         __syncthreads();
         if (t + 1 < ntiles && threadIdx.x == 0) tc_issue(T, b ^ 1, idesc);
@@ -421,7 +439,7 @@ __device__ inline void tc_gen_X_steer(const JobDev &J, TcWork &T, int b, int t, 
     const int p = J.p, Kp = T.Kp, nc8 = Kp / 8, nl = J.n_l;
     const float2 *__restrict__ El = J.El;
     const float2 *__restrict__ Em = J.Em;
-    unsigned char *xh = T.Xhi[b], *xl = T.Xlo[b];
+    unsigned char *xh = T.Xhi(b), *xl = T.Xlo(b);
     const bool vec = (p & 7) == 0;       // 64-byte aligned antenna chunks
     for (int it = threadIdx.x; it < kTcM * nc8; it += blockDim.x) {
         const int r = it / nc8, c8 = it - r * nc8;
@@ -474,7 +492,7 @@ __device__ inline void tc_gen_X_steer(const JobDev &J, TcWork &T, int b, int t, 
 template <bool BF16>
 __device__ inline void tc_gen_X_range(const JobDev &J, TcWork &T, int b, int pix0, int np, float sX) {
     const int p = J.p, Kp = T.Kp, nc8 = Kp / 8, nl = J.n_l;
-    unsigned char *xh = T.Xhi[b], *xl = T.Xlo[b];
+    unsigned char *xh = T.Xhi(b), *xl = T.Xlo(b);
     for (int it = threadIdx.x; it < kTcM * nc8; it += blockDim.x) {
         const int r = it / nc8, c8 = it - r * nc8;
         float re[8], im[8];
@@ -506,7 +524,7 @@ template <bool BF16>
 __device__ inline void tc_gen_X_cache(const JobDev &J, TcWork &T, int b, const int *pos, int j0, int np,
                                       float sX) {
     const int p = J.p, Kp = T.Kp, nc8 = Kp / 8;
-    unsigned char *xh = T.Xhi[b], *xl = T.Xlo[b];
+    unsigned char *xh = T.Xhi(b), *xl = T.Xlo(b);
     const bool vec = (p & 7) == 0;
     for (int it = threadIdx.x; it < kTcM * nc8; it += blockDim.x) {
         const int r = it / nc8, c8 = it - r * nc8;
@@ -548,15 +566,12 @@ __device__ inline void tc_gen_X_cache(const JobDev &J, TcWork &T, int b, const i
     }
 }
 
-// Epilogue of one tile: thread (row r = pixel, half h = real / imaginary
-// columns) forms sum_k xs_k D[r][h Kp + k], with xs = hi + lo rebuilt from the
-// operand tile in shared memory (the scaled x the MMA consumed; conflict-free
-// 16-byte reads).  red[r] (r < 128) holds the tile's sums after the call; the
-// caller multiplies by 1/(sX^2 sB).  SQ: the sum of squares of the row's
-// accumulator, ||D[r]||^2 (B built from V = L^-1: the whitened MVDR
-// denominator); the caller multiplies by 1/(sX sB)^2.
+// One tile's dot on thread (row r = pixel, half h = real / imaginary columns):
+// sum_k xs_k D[r][h Kp + k], with xs = hi + lo rebuilt from the operand tile in
+// shared memory (the scaled x the MMA consumed; conflict-free 16-byte reads).
+// SQ: the sum of squares of the row's accumulator instead.
 template <bool BF16, bool SQ = false>
-__device__ inline void tc_epilogue(const TcWork &T, int b, float *red) {
+__device__ __forceinline__ float tc_row_dot(const TcWork &T, int b) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int half = warp >> 2, r = 32 * (warp & 3) + lane;
     const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
@@ -566,44 +581,39 @@ __device__ inline void tc_epilogue(const TcWork &T, int b, float *red) {
         float dd[2][16];
         const uint32_t ta = T.tmem + lane_base + (uint32_t)(b * 2 * T.Kp + half * T.Kp + c00);
         tmem_ld16x2(ta, ta + 16, dd[0], dd[1]);
-        if (SQ) {
 #pragma unroll
-            for (int g = 0; g < 2; ++g)
-#pragma unroll
-                for (int q = 0; q < 16; ++q) acc = fmaf(dd[g][q], dd[g][q], acc);
-        } else {
-#pragma unroll
-            for (int g = 0; g < 2; ++g) {
-            const int c0 = c00 + 16 * g;
+        for (int g = 0; g < 2; ++g) {
             const float *d = dd[g];
+            if constexpr (SQ) {
+#pragma unroll
+                for (int q = 0; q < 16; ++q) acc = fmaf(d[q], d[q], acc);
+            } else {
 #pragma unroll
             for (int s8 = 0; s8 < 2; ++s8) {
-                const uint32_t off = sw128_off(r, half * nc8 + c0 / 8 + s8, kTcM);
-                const uint4 h4 = *reinterpret_cast<const uint4 *>(T.Xhi[b] + off);
-                const uint4 l4 = *reinterpret_cast<const uint4 *>(T.Xlo[b] + off);
+                const uint32_t off = sw128_off(r, half * nc8 + (c00 + 16 * g) / 8 + s8, kTcM);
+                const uint4 h4 = *reinterpret_cast<const uint4 *>(T.Xhi(b) + off);
+                const uint4 l4 = *reinterpret_cast<const uint4 *>(T.Xlo(b) + off);
                 const uint32_t hw[4] = {h4.x, h4.y, h4.z, h4.w}, lw[4] = {l4.x, l4.y, l4.z, l4.w};
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    float h0, h1, l0, l1;
-                    if (BF16) {
-                        h0 = __uint_as_float(hw[q] << 16);
-                        h1 = __uint_as_float(hw[q] & 0xffff0000u);
-                        l0 = __uint_as_float(lw[q] << 16);
-                        l1 = __uint_as_float(lw[q] & 0xffff0000u);
-                    } else {
-                        h0 = __half2float(__ushort_as_half((unsigned short)(hw[q] & 0xffffu)));
-                        h1 = __half2float(__ushort_as_half((unsigned short)(hw[q] >> 16)));
-                        l0 = __half2float(__ushort_as_half((unsigned short)(lw[q] & 0xffffu)));
-                        l1 = __half2float(__ushort_as_half((unsigned short)(lw[q] >> 16)));
-                    }
-                    acc = fmaf(h0 + l0, d[s8 * 8 + 2 * q], acc);
-                    acc = fmaf(h1 + l1, d[s8 * 8 + 2 * q + 1], acc);
+                    const float2 h = unpack2<BF16>(hw[q]), l = unpack2<BF16>(lw[q]);
+                    acc = fmaf(h.x + l.x, d[s8 * 8 + 2 * q], acc);
+                    acc = fmaf(h.y + l.y, d[s8 * 8 + 2 * q + 1], acc);
                 }
             }
             }
         }
     }
-    red[half * kTcM + r] = acc;
+    return acc;
+}
+
+// Epilogue of one tile: red[r] (r < 128) holds the tile's sums after the call;
+// the caller multiplies by 1/(sX^2 sB).  SQ: ||D[r]||^2 (B built from V =
+// L^-1: the whitened MVDR denominator); the caller multiplies by 1/(sX sB)^2.
+template <bool BF16, bool SQ = false>
+__device__ inline void tc_epilogue(const TcWork &T, int b, float *red) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    red[(warp >> 2) * kTcM + 32 * (warp & 3) + lane] = tc_row_dot<BF16, SQ>(T, b);
     __syncthreads();
     if (threadIdx.x < kTcM) red[threadIdx.x] = red[threadIdx.x] + red[kTcM + threadIdx.x];
     tc_fence_before();
@@ -650,32 +660,21 @@ __device__ inline void tc_weight_rows(TcWork &T, const float *w, int np, float s
     for (int it = threadIdx.x; it < kTcM * nch; it += blockDim.x) {
         const int r = it / nch, c = it - r * nch;
         const uint32_t off = sw128_off(r, c, kTcM);
-        const uint4 h4 = *reinterpret_cast<const uint4 *>(T.Xhi[0] + off);
-        const uint4 l4 = *reinterpret_cast<const uint4 *>(T.Xlo[0] + off);
+        const uint4 h4 = *reinterpret_cast<const uint4 *>(T.Xhi(0) + off);
+        const uint4 l4 = *reinterpret_cast<const uint4 *>(T.Xlo(0) + off);
         const uint32_t hw[4] = {h4.x, h4.y, h4.z, h4.w}, lw[4] = {l4.x, l4.y, l4.z, l4.w};
         const float wr = r < np ? sW * w[r] : 0.f;
         float v[8];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            float h0, h1, l0, l1;
-            if (BF16) {
-                h0 = __uint_as_float(hw[q] << 16);
-                h1 = __uint_as_float(hw[q] & 0xffff0000u);
-                l0 = __uint_as_float(lw[q] << 16);
-                l1 = __uint_as_float(lw[q] & 0xffff0000u);
-            } else {
-                h0 = __half2float(__ushort_as_half((unsigned short)(hw[q] & 0xffffu)));
-                h1 = __half2float(__ushort_as_half((unsigned short)(hw[q] >> 16)));
-                l0 = __half2float(__ushort_as_half((unsigned short)(lw[q] & 0xffffu)));
-                l1 = __half2float(__ushort_as_half((unsigned short)(lw[q] >> 16)));
-            }
-            v[2 * q] = wr * (h0 + l0);
-            v[2 * q + 1] = wr * (h1 + l1);
+            const float2 h = unpack2<BF16>(hw[q]), l = unpack2<BF16>(lw[q]);
+            v[2 * q] = wr * (h.x + l.x);
+            v[2 * q + 1] = wr * (h.y + l.y);
         }
         uint4 hi, lo;
         split8<BF16>(v, hi, lo);
-        *reinterpret_cast<uint4 *>(T.Xhi[1] + off) = hi;
-        *reinterpret_cast<uint4 *>(T.Xlo[1] + off) = lo;
+        *reinterpret_cast<uint4 *>(T.Xhi(1) + off) = hi;
+        *reinterpret_cast<uint4 *>(T.Xlo(1) + off) = lo;
     }
 }
 
@@ -684,8 +683,8 @@ __device__ inline void tc_weight_rows(TcWork &T, const float *w, int np, float s
 __device__ inline void tc_issue_fwd(const TcWork &T, uint32_t idesc, bool first) {
     const int N = 2 * T.Kp;
     tc_fence_after();
-    const uint32_t ah = smem_u32(T.Xhi[1]), al = smem_u32(T.Xlo[1]);
-    const uint32_t bh = smem_u32(T.Xhi[0]), bl = smem_u32(T.Xlo[0]);
+    const uint32_t ah = smem_u32(T.Xhi(1)), al = smem_u32(T.Xlo(1));
+    const uint32_t bh = smem_u32(T.Xhi(0)), bl = smem_u32(T.Xlo(0));
     const uint32_t d = T.tmem + (uint32_t)(2 * N);
     const uint32_t lbo = kTcM * 128, sbo = 1024;
     for (int s = 0; s < kTcM / 16; ++s) {
@@ -706,11 +705,16 @@ __device__ inline float *tc_read_fwd(const TcWork &T, float *G) {
     const int half = warp >> 2, m = 32 * (warp & 3) + lane;
     const int N = 2 * T.Kp;
     const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
-    for (int c0 = 0; c0 < T.Kp; c0 += 16) {
-        float d[16];
-        tmem_ld16(T.tmem + lane_base + (uint32_t)(2 * N + half * T.Kp + c0), d);
+    for (int c0 = 0; c0 < T.Kp; c0 += 32) {
+        float d[2][16];
+        const uint32_t ta = T.tmem + lane_base + (uint32_t)(2 * N + half * T.Kp + c0);
+        tmem_ld16x2(ta, ta + 16, d[0], d[1]);
+        float *g = G + m * (N + 1) + half * T.Kp + c0;
 #pragma unroll
-        for (int q = 0; q < 16; ++q) G[m * (N + 1) + half * T.Kp + c0 + q] = d[q];
+        for (int q = 0; q < 16; ++q) {
+            g[q] = d[0][q];
+            g[16 + q] = d[1][q];
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -756,12 +760,11 @@ __device__ void tc_forward(TcWork &T, int p, int n, const float *wt, float sX, G
         fence_async_smem();
         __syncthreads();
         if (threadIdx.x == 0) tc_issue_fwd(T, idesc, t == 0);
-        if (!mbar_wait(&T.bar[0], T.phase[0])) T.timeouts++;
-        T.phase[0] ^= 1u;
+        T.wait(0);
         tc_fence_after();
         __syncthreads();
     }
-    const float *G = ntiles ? tc_read_fwd(T, reinterpret_cast<float *>(T.Xhi[0])) : nullptr;
+    const float *G = ntiles ? tc_read_fwd(T, reinterpret_cast<float *>(T.Xhi(0))) : nullptr;
     tc_combine_fwd(T, p, G, 1.f / (sX * sX * sW), base, base_identity, K);
 }
 
@@ -783,162 +786,6 @@ __device__ inline void tc_combine_fwd(const TcWork &T, int p, const float *G, fl
         K[e] = make_float2(bb.x + kr, bb.y + ki);
     }
     __syncthreads();
-}
-
-}  // namespace img
-
-namespace img {
-
-// ---------------------------------------------------------------- resident LSQR
-// During one LSQR solve the free set is fixed, so (for f <= 256 and Kp = 64)
-// its X tiles stay in shared memory for every iteration: tile 0 in buffer 0,
-// tile 1 in buffer 1.  The forward product stages only the weighted K-chunks
-// (32 pixels, both MN blocks) in a 16 KB region after the B tiles.
-constexpr int kChunk = 16;              // pixels per forward K-chunk (one MMA K-step)
-
-// Two staging buffers (hi + lo, MN blocks x 16 rows x 128 bytes each).
-__host__ __device__ inline size_t tc_stage_bytes(int p) {
-    const int Kp = (p + 31) / 32 * 32;
-    return (size_t)2 * 2 * (2 * Kp / 64) * kChunk * 128;
-}
-
-// Weighted chunk rows r0 .. r0+31 of resident tile `tile` into the staging
-// region (MN blocks of 32 rows x 128 bytes), rows j >= nrow zero.
-template <bool BF16>
-__device__ inline void tc_weight_chunk(TcWork &T, unsigned char *stage, int tile, int r0, int nrow,
-                                       const float *w, float sW) {
-    const int nch = 2 * T.Kp / 8;
-    const size_t half_bytes = (size_t)(2 * T.Kp / 64) * kChunk * 128;
-    for (int it = threadIdx.x; it < kChunk * nch; it += blockDim.x) {
-        const int rr = it / nch, c = it - rr * nch;
-        const uint32_t src = sw128_off(r0 + rr, c, kTcM);
-        const uint32_t dst = sw128_off(rr, c, kChunk);
-        const float wr = rr < nrow ? sW * w[rr] : 0.f;
-        const uint4 h4 = *reinterpret_cast<const uint4 *>(T.Xhi[tile] + src);
-        const uint4 l4 = *reinterpret_cast<const uint4 *>(T.Xlo[tile] + src);
-        const uint32_t hw[4] = {h4.x, h4.y, h4.z, h4.w}, lw[4] = {l4.x, l4.y, l4.z, l4.w};
-        float v[8];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            float h0, h1, l0, l1;
-            if (BF16) {
-                h0 = __uint_as_float(hw[q] << 16);
-                h1 = __uint_as_float(hw[q] & 0xffff0000u);
-                l0 = __uint_as_float(lw[q] << 16);
-                l1 = __uint_as_float(lw[q] & 0xffff0000u);
-            } else {
-                h0 = __half2float(__ushort_as_half((unsigned short)(hw[q] & 0xffffu)));
-                h1 = __half2float(__ushort_as_half((unsigned short)(hw[q] >> 16)));
-                l0 = __half2float(__ushort_as_half((unsigned short)(lw[q] & 0xffffu)));
-                l1 = __half2float(__ushort_as_half((unsigned short)(lw[q] >> 16)));
-            }
-            v[2 * q] = wr * (h0 + l0);
-            v[2 * q + 1] = wr * (h1 + l1);
-        }
-        uint4 hi, lo;
-        split8<BF16>(v, hi, lo);
-        *reinterpret_cast<uint4 *>(stage + dst) = hi;
-        *reinterpret_cast<uint4 *>(stage + half_bytes + dst) = lo;
-    }
-}
-
-// MMAs of one staged chunk against resident rows r0 .. r0+31 of `tile`,
-// accumulating into the forward accumulator; commits to barrier 0.
-__device__ inline void tc_issue_fwd_chunk(const TcWork &T, const unsigned char *stage, int tile, int r0,
-                                          uint32_t idesc, bool first, int bar) {
-    const int N = 2 * T.Kp;
-    tc_fence_after();
-    const size_t half_bytes = (size_t)(N / 64) * kChunk * 128;
-    const uint32_t ah = smem_u32(stage), al = smem_u32(stage + half_bytes);
-    const uint32_t bh = smem_u32(T.Xhi[tile]), bl = smem_u32(T.Xlo[tile]);
-    const uint32_t d = T.tmem + (uint32_t)(2 * N);
-    for (int s = 0; s < kChunk / 16; ++s) {
-        const uint32_t ao = s * 2048, bo = (uint32_t)((r0 + 16 * s) / 8) * 1024;
-        const uint32_t alb = kChunk * 128, blb = kTcM * 128;
-        mma_f16(d, sw128_desc_mn(ah + ao, alb, 1024), sw128_desc_mn(bh + bo, blb, 1024), idesc,
-                (first && s == 0) ? 0u : 1u);
-        mma_f16(d, sw128_desc_mn(ah + ao, alb, 1024), sw128_desc_mn(bl + bo, blb, 1024), idesc, 1u);
-        mma_f16(d, sw128_desc_mn(al + ao, alb, 1024), sw128_desc_mn(bh + bo, blb, 1024), idesc, 1u);
-    }
-    mma_commit(&T.bar[bar]);
-}
-
-// Forward over the resident free-set tiles: G = sum_j w_j x_j x_j^T read out
-// into the B + staging region (the B tile is rebuilt later).  Weighted
-// 16-pixel chunks alternate between two staging buffers, so weighting chunk
-// c+1 overlaps the MMAs of chunk c; a buffer is reused only after the MMAs
-// that read it completed.  Returns G (scaled by sX^2 sW; *scale = 1/that).
-template <bool BF16>
-__device__ const float *tc_forward_resident(TcWork &T, unsigned char *stage, int f, const float *w,
-                                            float sX, float *scale, double *dbuf, long long *cyc = nullptr) {
-    long long c0 = clock64();
-    const float sW = pow2_scale_of(w, f, dbuf);
-    const uint32_t idesc = idesc_f16_mn(2 * T.Kp, BF16 ? 1 : 0);
-    const int nchunks = (f + kChunk - 1) / kChunk;
-    const size_t buf = (size_t)2 * (2 * T.Kp / 64) * kChunk * 128;   // one staging buffer (hi + lo)
-    for (int c = 0; c < nchunks; ++c) {
-        const int b = c & 1;
-        if (c >= 2) {
-            if (!mbar_wait(&T.bar[b], T.phase[b])) T.timeouts++;
-            T.phase[b] ^= 1u;
-            tc_fence_after();
-        }
-        const int j0 = c * kChunk, tile = j0 / kTcM, r0 = j0 % kTcM;
-        tc_weight_chunk<BF16>(T, stage + b * buf, tile, r0, min(kChunk, f - j0), w + j0, sW);
-        fence_async_smem();
-        __syncthreads();
-        if (threadIdx.x == 0) tc_issue_fwd_chunk(T, stage + b * buf, tile, r0, idesc, c == 0, b);
-    }
-    for (int c = max(0, nchunks - 2); c < nchunks; ++c) {
-        const int b = c & 1;
-        if (!mbar_wait(&T.bar[b], T.phase[b])) T.timeouts++;
-        T.phase[b] ^= 1u;
-    }
-    tc_fence_after();
-    __syncthreads();
-    long long c1 = clock64();
-    *scale = 1.f / (sX * sX * sW);
-    const float *G = nchunks ? tc_read_fwd(T, reinterpret_cast<float *>(T.Bhi)) : nullptr;
-    if (cyc) {
-        cyc[0] += c1 - c0;
-        cyc[1] += clock64() - c1;
-    }
-    return G;
-}
-
-// Adjoint over the resident tiles: epi(j, Re(c_j^H U c_j)) for j < f.
-template <bool BF16, class Epi>
-__device__ void tc_adjoint_resident(TcWork &T, const float2 *U, int p, int f, float sX, float *red,
-                                    double *dbuf, Epi epi, long long *cyc = nullptr) {
-    long long c0 = clock64();
-    const float sB = tc_build_B<BF16>(U, p, T, dbuf);
-    const uint32_t idesc = idesc_f16(2 * T.Kp, BF16 ? 1 : 0);
-    const int ntiles = (f + kTcM - 1) / kTcM;
-    fence_async_smem();
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int t = 0; t < ntiles; ++t) tc_issue(T, t, idesc);
-    const float inv = 1.f / (sX * sX * sB);
-    long long c1 = clock64(), cw = 0, ce = 0;
-    for (int t = 0; t < ntiles; ++t) {
-        long long a0 = clock64();
-        if (!mbar_wait(&T.bar[t], T.phase[t])) T.timeouts++;
-        T.phase[t] ^= 1u;
-        tc_fence_after();
-        __syncthreads();
-        long long a1 = clock64();
-        tc_epilogue<BF16>(T, t, red);
-        const int j = t * kTcM + threadIdx.x;
-        if (threadIdx.x < kTcM && j < f) epi(j, red[threadIdx.x] * inv);
-        __syncthreads();
-        cw += a1 - a0;
-        ce += clock64() - a1;
-    }
-    if (cyc) {
-        cyc[3] += c1 - c0;
-        cyc[4] += cw;
-        cyc[5] += ce;
-    }
 }
 
 }  // namespace img

@@ -506,8 +506,7 @@ __global__ void __launch_bounds__(kItemsFwdThreads, 1) k_ws_fwd(const JobDev *Jp
     if (n <= 0) return;
     const int nsplit = ctl->nsplit;
     const int tasks = B.npairs * nsplit;
-    extern __shared__ float4 smem4[];
-    unsigned char *dyn = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem4) + 1023) & ~uintptr_t(1023));
+    unsigned char *dyn = dyn_smem();
     __shared__ uint64_t bars[6];
     __shared__ uint32_t tslot;
     if (blockIdx.x >= tasks) return;
@@ -680,8 +679,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_ws_adj(const JobDev *Jp, Ws
     const int ntiles = LIST ? (n + kTcM - 1) / kTcM : tc_num_tiles(J.n_l, J.n_m);
     const int nkg = LIST ? ws_nkg(ntiles * g.nu, g.nk, gridDim.x) : 1;
     if (LIST && blockIdx.x == 0 && threadIdx.x == 0) ctl->adj_rows = g.nu * nkg;
-    extern __shared__ float4 smem4[];
-    unsigned char *dyn = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem4) + 1023) & ~uintptr_t(1023));
+    unsigned char *dyn = dyn_smem();
     __shared__ uint64_t bars[kWideBars];
     __shared__ uint32_t tslot;
     float *out = B.padj;
