@@ -74,60 +74,117 @@ __host__ __device__ inline uint32_t sw_row_off(int r, int c16) {
 }
 
 // ---------------------------------------------------------------- B unit image
-// One 16-byte chunk (8 K columns) of row n of unit block (u, kc) of the
-// embedding of U (p x p column-major FP32 complex, Hermitian):
+// One 16-byte chunk (8 K columns) of an image: its 8 source vectors' entries,
+// `part` chosen and scaled, split and stored at off (hi) and off + lo_off (lo).
+// The image kernels load several chunks before they store any: one chunk at a
+// time they are a chain of L2 latencies.
+struct ImgChunk {
+    float2 w[8];
+    // 8 consecutive entries from src (null: zeros), the first n of them live.
+    // Through L2: inside the cluster LSQR other CTAs have just written U.
+    __device__ __forceinline__ void load(const float2 *src, int n, bool vec) {
+        if (src && vec && n >= 8) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 x = __ldcg(reinterpret_cast<const float4 *>(src) + q);
+                w[2 * q] = make_float2(x.x, x.y);
+                w[2 * q + 1] = make_float2(x.z, x.w);
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) w[e] = src && e < n ? __ldcg(src + e) : make_float2(0.f, 0.f);
+        }
+    }
+    template <bool BF16>
+    __device__ __forceinline__ void store(const float *v, unsigned char *at, size_t lo_off) const {
+        uint4 hi, lo;
+        split8<BF16>(v, hi, lo);
+        *reinterpret_cast<uint4 *>(at) = hi;
+        *reinterpret_cast<uint4 *>(at + lo_off) = lo;
+    }
+};
+constexpr int kImgUnroll = 4;
+
+// B unit image of U (p x p column-major FP32 complex, Hermitian), scaled by
+// sc, by threads t0, t0 + nt, ... of the launch:
 //   B[(Re, kr), (Re, kc)] = B[(Im, kr), (Im, kc)] = Re U(kc, kr)
 //   B[(Re, kr), (Im, kc)] = Im U(kc, kr),  B[(Im, kr), (Re, kc)] = -Im U(kc, kr)
-// so that x^T B x = Re(a^H U a) for x = [Re a; Im a].  sc: power-of-two scale.
+// so that x^T B x = Re(a^H U a) for x = [Re a; Im a].
 template <bool BF16>
-__device__ inline void unit_image_chunk(const float2 *__restrict__ U, int p, const UnitGeom &g, float sc,
-                                        unsigned char *img, int u, int kc, int n, int c16) {
-    const int ku = g.ku, rows = unit_rows(g);
-    const int rpart = n >= ku, kr = u * ku + n - rpart * ku;
-    const int col0 = kc * kChunkK + c16 * 8;
-    const int cpart = col0 >= g.Kp, k0 = col0 - cpart * g.Kp;
-    float v[8];
+__device__ inline void unit_image(const float2 *U, int p, const UnitGeom &g, float sc, unsigned char *img, int t0,
+                                  int nt) {
+    const int ku = g.ku, rows = unit_rows(g), total = g.nu * g.nk * rows * 8;
+    const bool vec = (p & 1) == 0;
+    for (int e0 = t0; e0 < total; e0 += kImgUnroll * nt) {
+        ImgChunk c[kImgUnroll];
+        unsigned char *at[kImgUnroll];
+        int kind[kImgUnroll];                       // 0: Re U, 1: Im U, 2: -Im U
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        float2 w = make_float2(0.f, 0.f);
-        if (kr < p && k0 + e < p) w = U[(size_t)kr * p + k0 + e];
-        v[e] = sc * ((rpart == cpart) ? w.x : (rpart == 0 ? w.y : -w.y));
+        for (int q = 0; q < kImgUnroll; ++q) {
+            const int e = e0 + q * nt;
+            at[q] = nullptr;
+            if (e >= total) continue;
+            const int c16 = e & 7, n = (e >> 3) % rows, r2 = (e >> 3) / rows;
+            const int kc = r2 % g.nk, u = r2 / g.nk;
+            const int rpart = n >= ku, kr = u * ku + n - rpart * ku;
+            const int col0 = kc * kChunkK + c16 * 8;
+            const int cpart = col0 >= g.Kp, k0 = col0 - cpart * g.Kp;
+            kind[q] = rpart == cpart ? 0 : 1 + rpart;
+            c[q].load(kr < p ? U + (size_t)kr * p + k0 : nullptr, p - k0, vec);
+            at[q] = img + (size_t)(u * g.nk + kc) * unit_block_bytes(g) + sw_row_off(n, c16);
+        }
+#pragma unroll
+        for (int q = 0; q < kImgUnroll; ++q) {
+            if (!at[q]) continue;
+            float v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                v[e] = sc * (kind[q] == 0 ? c[q].w[e].x : (kind[q] == 1 ? c[q].w[e].y : -c[q].w[e].y));
+            c[q].store<BF16>(v, at[q], (size_t)rows * 128);
+        }
     }
-    uint4 hi, lo;
-    split8<BF16>(v, hi, lo);
-    unsigned char *blk = img + (size_t)(u * g.nk + kc) * unit_block_bytes(g);
-    const uint32_t off = sw_row_off(n, c16);
-    *reinterpret_cast<uint4 *>(blk + off) = hi;
-    *reinterpret_cast<uint4 *>(blk + (size_t)rows * 128 + off) = lo;
 }
 
 // ---------------------------------------------------------------- list image
-// One 16-byte chunk of row r of tile block (t, kc) of the list image of the
-// vectors vec[pos[j] * p + k] (j = 128 t + r < n; zero beyond), scaled by sX
-// and, when wgt is given, by the row weight wgt[j].
+// List image of the n vectors vec[pos[j] * p + k] (row j of the tiles; rows
+// beyond n and the padding chunks are zero), scaled by sX and, when wgt is
+// given, by the row weight wgt[j]; by threads t0, t0 + nt, ... of the launch.
 template <bool BF16>
-__device__ inline void list_image_chunk(const float2 *__restrict__ vec, const int *__restrict__ pos,
-                                        const float *__restrict__ wgt, int n, int p, const UnitGeom &g, float sX,
-                                        unsigned char *img, int t, int kc, int r, int c16) {
-    const int j = t * kTcM + r;
-    const int col0 = kc * kChunkK + c16 * 8;
-    const int part = col0 >= g.Kp, k0 = col0 - part * g.Kp;
-    float v[8];
-    const bool live = j < n && kc < g.nk;
-    const float2 *src = live ? vec + (size_t)pos[j] * p : nullptr;
-    const float sw = live ? (wgt ? wgt[j] * sX : sX) : 0.f;
+__device__ inline void list_image(const float2 *vec, const int *pos, const float *wgt, int n, int p, const UnitGeom &g,
+                                  float sX, unsigned char *img, int t0, int nt) {
+    const int total = (n + kTcM - 1) / kTcM * g.nkA * kTcM * 8;
+    const bool v4 = (p & 1) == 0;
+    for (int e0 = t0; e0 < total; e0 += kImgUnroll * nt) {
+        ImgChunk c[kImgUnroll];
+        int sl[kImgUnroll];
+        float sw[kImgUnroll];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        float2 w = make_float2(0.f, 0.f);
-        if (src && k0 + e < p) w = src[k0 + e];
-        v[e] = sw * (part ? w.y : w.x);
+        for (int q = 0; q < kImgUnroll; ++q) {
+            const int e = e0 + q * nt;
+            const int r = (e >> 3) % kTcM, r2 = (e >> 3) / kTcM, kc = r2 % g.nkA, j = r2 / g.nkA * kTcM + r;
+            const bool live = e < total && j < n && kc < g.nk;
+            sl[q] = live ? pos[j] : -1;
+            sw[q] = live ? (wgt ? __ldcg(wgt + j) * sX : sX) : 0.f;
+        }
+#pragma unroll
+        for (int q = 0; q < kImgUnroll; ++q) {
+            const int e = e0 + q * nt;
+            const int kc = (e >> 3) / kTcM % g.nkA, col0 = kc * kChunkK + (e & 7) * 8;
+            const int k0 = col0 >= g.Kp ? col0 - g.Kp : col0;
+            c[q].load(sl[q] >= 0 ? vec + (size_t)sl[q] * p + k0 : nullptr, p - k0, v4);
+        }
+#pragma unroll
+        for (int q = 0; q < kImgUnroll; ++q) {
+            const int e = e0 + q * nt;
+            if (e >= total) break;
+            const int r = (e >> 3) % kTcM, r2 = (e >> 3) / kTcM, kc = r2 % g.nkA, t = r2 / g.nkA;
+            const bool im = kc * kChunkK + (e & 7) * 8 >= g.Kp;
+            float v[8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) v[x] = __fmul_rn(sw[q], im ? c[q].w[x].y : c[q].w[x].x);
+            c[q].store<BF16>(v, img + (size_t)(t * g.nkA + kc) * kListBlock + sw_row_off(r, e & 7), (size_t)kTcM * 128);
+        }
     }
-    uint4 hi, lo;
-    split8<BF16>(v, hi, lo);
-    unsigned char *blk = img + (size_t)(t * g.nkA + kc) * kListBlock;
-    const uint32_t off = sw_row_off(r, c16);
-    *reinterpret_cast<uint4 *>(blk + off) = hi;
-    *reinterpret_cast<uint4 *>(blk + (size_t)kTcM * 128 + off) = lo;
 }
 
 // ---------------------------------------------------------------- item adjoint
@@ -147,15 +204,18 @@ __host__ __device__ inline size_t items_smem_bytes() { return 2 * kWideXStage + 
 // epi(q, t, r, v) receives, on the epilogue thread of row r, the partial dot
 // of unit u and K group kg, q = u nkg + kg (still scaled by the X and B
 // scales; a steering tile's scale is steer_scale(p) kLift).  Needs kWideThreads
-// threads, kWideBars mbarriers and the 1024-aligned dynamic shared memory of
-// items_smem_bytes() - 1024 bytes.  Returns the number of waits that timed out.
+// threads (LIST: at least 160, the copies and MMAs then run in warp 4),
+// kWideBars mbarriers, the 1024-aligned dynamic shared memory of
+// items_smem_bytes() - 1024 bytes and 512 columns of tensor memory at tmem.
+// LIST: warps 5 and up have no part; each calls idle(warp) once meanwhile.
+// Returns the number of waits that timed out.
 // sq (nkg = 1 only): the partial is the unit's sum of squares ||D[r]||^2
 // instead of the dot (B from V = L^-1: the whitened MVDR denominator
 // ||L^-1 a_i||^2 as the sum of the units' partials, scaled twice).
-template <bool BF16, bool LIST, class Epi>
-__device__ int items_adjoint(const JobDev &J, const UnitGeom &g, unsigned char *dyn, uint64_t *bars, uint32_t *slot,
+template <bool BF16, bool LIST, class Epi, class Idle>
+__device__ int items_adjoint(const JobDev &J, const UnitGeom &g, unsigned char *dyn, uint64_t *bars, uint32_t tmem,
                              const unsigned char *Bimg, const unsigned char *Ximg, const float2 *vec, const int *pos,
-                             int nrows, int ntiles, int nkg, int first, int stride, bool sq, Epi epi) {
+                             int nrows, int ntiles, int nkg, int first, int stride, bool sq, Epi epi, Idle idle) {
     const int p = J.p, Kp = g.Kp, nk = g.nk, ku = g.ku, rows_u = unit_rows(g);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned char *Xs = dyn, *Bs = dyn + 2 * kWideXStage;
@@ -174,11 +234,9 @@ __device__ int items_adjoint(const JobDev &J, const UnitGeom &g, unsigned char *
             mbar_init(&bars[kAEmpty + q], 4);
         }
     }
-    if (warp == 0) tmem_alloc(slot, 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *slot;
     int timeouts = 0;
     auto item_of = [&](int k, int &u, int &t, int &kg) {
         const int it = first + k * stride;
@@ -194,7 +252,7 @@ __device__ int items_adjoint(const JobDev &J, const UnitGeom &g, unsigned char *
         kc = kg * nkc + c % nkc;
     };
 
-    if (warp == 8) {
+    if (warp == (LIST ? 4 : 8)) {
         // ---------------- bulk copies and MMAs (lane 0 issues, the warp waits)
         if (total > 0) {
             const bool leader = lane == 0;
@@ -243,6 +301,7 @@ __device__ int items_adjoint(const JobDev &J, const UnitGeom &g, unsigned char *
             }
         }
     } else if (warp >= 4) {
+        if (LIST) idle(warp);
         // ---------------- steering producers (2-D tiles only): chunk c into X
         // stage c & 1.  Warp w fills rows 32w + 8b + a (l offset a, m offset
         // 4w + b), lane j columns 2j, 2j + 1 of the chunk.
@@ -422,7 +481,6 @@ __device__ int items_adjoint(const JobDev &J, const UnitGeom &g, unsigned char *
     if (timeouts) atomicAdd(&s_timeouts, timeouts);
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, 512);
     return s_timeouts;
 }
 
@@ -450,8 +508,9 @@ __host__ __device__ inline int items_fwd_pairs(const UnitGeom &g, int *pm, int *
 }
 constexpr int kItemsFwdMaxPairs = 24;
 
-// One CTA: block (m, nb) over list stages s0, s0 + S, ... (64 entries each);
-// writes the FP32 block (128 x 256 column-major: entry (r, c) at c 128 + r,
+// One CTA: B chunks [q0, q0 + nq) (64 columns each) of block (m, nb) over list
+// stages s0, s0 + S, ... (64 entries each); writes their columns of the FP32
+// block (128 x 256 column-major: entry (r, c) at c 128 + r,
 // still scaled by the images' scales) to out.  XA: unweighted list image
 // (rows features 128 m ..), XB: weighted list image (columns features
 // 256 nb ..); every operand arrives by bulk copy: per stage, chunks 2m, 2m+1
@@ -467,15 +526,15 @@ __host__ __device__ inline size_t items_fwd_smem_bytes() { return 2 * kFwdStage 
 
 template <bool BF16>
 __device__ int items_forward(const UnitGeom &g, unsigned char *dyn, uint64_t *bars, uint32_t tmem,
-                             const unsigned char *XA, const unsigned char *XB, int n, int m, int nb, int s0, int S,
-                             float *out) {
-    const int N = items_fwd_n(g, nb);
+                             const unsigned char *XA, const unsigned char *XB, int n, int m, int nb, int q0, int nq,
+                             int s0, int S, float *out) {
+    const int N = min(items_fwd_n(g, nb) - 64 * q0, 64 * nq);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nstages = (n + kFwdPix - 1) / kFwdPix;
     const int mine = nstages > s0 ? (nstages - 1 - s0) / S + 1 : 0;
     // B chunks 4nb + q that exist in the image: the last block may be short,
     // and an MMA of N columns reads only its first N / 64 chunks (N / 64 <= nbq)
-    const int nbq = min(4, g.nkA - 4 * nb);
+    const int nbq = min(nq, g.nkA - 4 * nb - q0);
     enum { kFull = 0, kEmpty = 2, kAcc = 4 };
     __shared__ int s_timeouts;
     if (threadIdx.x == 0) {
@@ -512,7 +571,7 @@ __device__ int items_forward(const UnitGeom &g, unsigned char *dyn, uint64_t *ba
                 }
                 for (int q = 0; q < nbq; ++q) {
                     const unsigned char *src =
-                        XB + (size_t)(tile * g.nkA + 4 * nb + q) * kListBlock + (size_t)half * kFwdChunk;
+                        XB + (size_t)(tile * g.nkA + 4 * nb + q0 + q) * kListBlock + (size_t)half * kFwdChunk;
                     tma_bulk_g2s(dst + (4 + q) * kFwdChunk, src, (uint32_t)kFwdChunk, &bars[kFull + sg]);
                     tma_bulk_g2s(dst + (8 + q) * kFwdChunk, src + (size_t)kTcM * 128, (uint32_t)kFwdChunk,
                                  &bars[kFull + sg]);
@@ -554,7 +613,7 @@ __device__ int items_forward(const UnitGeom &g, unsigned char *dyn, uint64_t *ba
         // ---------------- accumulator -> out: lanes hold consecutive rows, so
         // each column's 32 rows are one 128-byte store
         const int r = 32 * warp + lane;
-        float *col = out + r;
+        float *col = out + (size_t)64 * q0 * kTcM + r;
         if (mine > 0) {
             wide_wait(bars, kAcc, ph, timeouts);
             tc_fence_after();

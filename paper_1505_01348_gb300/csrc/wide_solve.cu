@@ -3,11 +3,11 @@
 //
 // The Table I loop is a graph WHILE node whose body is one pass (or two:
 // freeing the pixel chosen by the last gradient, then the next subproblem).
-// The subproblem's LSQR is an IF node holding the initialisation and a WHILE
-// node of Golub-Kahan iterations; the feasible / infeasible branch is an
-// IF/ELSE node.  Kernels set the conditions from device memory, so a whole
-// solve runs without a host round trip.  Every kernel has a fixed grid and
-// reads the sizes of the moment (|F|, |U|, support) from the control block.
+// The subproblem's LSQR is an IF node holding one kernel, whose thread-block
+// cluster iterates until the stopping tests hold; the feasible / infeasible
+// branch is an IF/ELSE node.  Kernels set the conditions from device memory, so
+// a whole solve runs without a host round trip.  Every kernel has a fixed grid
+// and reads the sizes of the moment (|F|, |U|, support) from the control block.
 //
 // Operators (tc_items.cuh): the adjoint over the free set or over every pixel
 // runs in (tile, unit) work items from a B image of U; the forward over a
@@ -29,11 +29,10 @@
 namespace img {
 
 constexpr int kWsThreads = 256;
-// Grid of the list kernels (forward, free-list adjoint): a share of the SMs,
-// so that the kernels of several solves in flight pack next to each other;
-// the full-image adjoint of the gradient takes every SM.  32 measured best
-// for 16 solves of 256x256, p = 288 in flight (0.54 images/s; 64 CTAs:
-// 0.48, 48: 0.51, 16: 0.53); fewer CTAs also mean fewer forward splits.
+// CTAs that the list operators' work is split for: the gradient's forward
+// runs on that many, and the K groups of the free-list adjoint and the
+// capacity of the forward's partial blocks - parts of the sums' order - follow
+// from it whatever number of CTAs runs them.
 constexpr int kListGrid = 32;
 constexpr int kWsSums = 2048;           // per-CTA partial sums of the reductions
 // 64-pixel stages per forward task (at least).  Fewer, longer tasks write
@@ -45,6 +44,13 @@ constexpr int kWsSums = 2048;           // per-CTA partial sums of the reduction
 // falls the other way).
 constexpr int kFwdPerTask = 4;
 
+// Scalars of the LSQR recurrence: in the control block, or in CTA 0's shared
+// memory when a cluster runs the whole subproblem.
+struct VxState {
+    double alpha, beta, us, bnorm, rhobar, phibar, anorm2, rho, c, sn, phi, xnorm2;
+    float fus, fb, ia, t1, t2;
+};
+
 // Device control block of one wide solve.
 struct WsCtl {
     int f, nu, ns;              // |F|, |U|, |F u U| of the current subproblem
@@ -54,14 +60,14 @@ struct WsCtl {
     int converged, status, feasible, nev, timeouts;
     int it, maxit, lsqr_total;  // LSQR iterations of this subproblem / cap / sum
     int nsplit;                 // forward split of the current list
-    int nlist;                  // length of the current forward list
     int adj_rows;               // unit x K-group partial rows of the free-list adjoint
     float sXF, sXS;             // power-of-two scales of the F and support list images
     float sW;                   // weight scale used by the last forward
     float sB;                   // scale of the current B image
     unsigned mx_t, mx_w;        // max |entry| bits of the matrix being imaged / the weights
     unsigned long long key;     // argmin key of the multiplier test
-    double alpha, beta, us, bnorm, anorm2, rhobar, phibar, fa;
+    VxState vx;
+    double fa;
     double lam_min, op_flops;
     unsigned long long t_begin;
     unsigned cond[4];           // last value of each loop / branch condition (host-driven mode)
@@ -93,6 +99,7 @@ struct WsBufs {
     unsigned char *ximgF, *ximgS, *ximgW, *bimg;   // list images: F, U or support, weighted; B image
     int npairs, pm[kItemsFwdMaxPairs], pnb[kItemsFwdMaxPairs];
     int max_tasks;              // capacity of pfwd in blocks
+    int list_grid;              // CTAs that the free-list adjoint's K groups are chosen for
     int fwd_per;                // 64-pixel stages per forward task (at least)
     int nrows_adj;              // rows of padj (max(Q, cap))
     int ld_adj;                 // partial dots per row of padj (nu nk)
@@ -154,7 +161,6 @@ __global__ void k_ws_start(const JobDev *Jp, WsBufs B, cudaGraphConditionalHandl
         ctl->timeouts = 0;
         ctl->it = ctl->maxit = ctl->lsqr_total = 0;
         ctl->nsplit = 1;
-        ctl->nlist = 0;
         ctl->mx_t = ctl->mx_w = 0;
         ctl->lam_min = 0.0;
         ctl->op_flops = 0.0;
@@ -414,7 +420,6 @@ __global__ void k_ws_pass(const JobDev *Jp, WsBufs B, cudaGraphConditionalHandle
         ctl->outer++;
         ctl->f = f;
         ctl->nu = nu;
-        ctl->nlist = nu;
         ctl->sXF = pow2_scale(mF) * kLift;
         ctl->sXS = pow2_scale(mU) * kLift;
         ctl->mx_w = __float_as_uint(wm);
@@ -433,13 +438,11 @@ __global__ void k_ws_pass(const JobDev *Jp, WsBufs B, cudaGraphConditionalHandle
 // weighted: the image of the rows times their weights wl (the second
 // operand of a forward) into ximgW, scaled by sX sW with sW the power of two
 // of max |wl| (stored for the reduction).
+// CTA `rank` of `ctas` does its share.
 template <bool BF16>
-__global__ void k_ws_listimg(const JobDev *Jp, WsBufs B, int which, int weighted) {
-    ws_count(B.ctl);
-    const JobDev &J = *Jp;
+__device__ void ws_listimg(const JobDev &J, const WsBufs &B, const UnitGeom &g, int which, int weighted, int rank,
+                           int ctas) {
     WsCtl *ctl = B.ctl;
-    if (ctl->stop) return;
-    const UnitGeom g = unit_geom(J.p);
     const bool S = which == kListS, Ul = which == kListU;
     const int n = S ? ctl->ns : (Ul ? ctl->nu : ctl->f);
     const int *pos = S ? B.iota : (Ul ? J.fpos + ctl->f : J.fpos);
@@ -448,89 +451,91 @@ __global__ void k_ws_listimg(const JobDev *Jp, WsBufs B, int which, int weighted
     unsigned char *img = weighted ? B.ximgW : ((S || Ul) ? B.ximgS : B.ximgF);
     if (weighted) {
         const float sW = pow2_scale(__uint_as_float(ctl->mx_w));
-        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->sW = sW;
+        if (rank == 0 && threadIdx.x == 0) ctl->sW = sW;
         sX *= sW;
     }
     const float *wgt = weighted ? B.wl : nullptr;
-    const int ntl = (n + kTcM - 1) / kTcM;
-    const long long total = (long long)ntl * g.nkA * kTcM * 8;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int c16 = (int)(e & 7);
-        long long r2 = e >> 3;
-        const int r = (int)(r2 % kTcM);
-        r2 /= kTcM;
-        const int kc = (int)(r2 % g.nkA), t = (int)(r2 / g.nkA);
-        list_image_chunk<BF16>(vec, pos, wgt, n, J.p, g, sX, img, t, kc, r, c16);
-    }
+    list_image<BF16>(vec, pos, wgt, n, J.p, g, sX, img, rank * blockDim.x + threadIdx.x, ctas * blockDim.x);
+}
+template <bool BF16>
+__global__ void k_ws_listimg(const JobDev *Jp, WsBufs B, int which, int weighted) {
+    ws_count(B.ctl);
+    if (B.ctl->stop) return;
+    ws_listimg<BF16>(*Jp, B, unit_geom(Jp->p), which, weighted, blockIdx.x, gridDim.x);
 }
 
 // B unit image of the matrix U (W0 for LSQR, W1 for the gradient) with the
 // power-of-two scale of ctl->mx_t.
 template <bool BF16>
+__device__ void ws_emb(const JobDev &J, const WsBufs &B, const UnitGeom &g, const float2 *U, int rank, int ctas) {
+    WsCtl *ctl = B.ctl;
+    const float sc = pow2_scale(__uint_as_float(ctl->mx_t)) * kLift;
+    if (rank == 0 && threadIdx.x == 0) ctl->sB = sc;
+    unit_image<BF16>(U, J.p, g, sc, B.bimg, rank * blockDim.x + threadIdx.x, ctas * blockDim.x);
+}
+template <bool BF16>
 __global__ void k_ws_emb(const JobDev *Jp, WsBufs B, int grad, const float2 *Um) {
     ws_count(B.ctl);
     const JobDev &J = *Jp;
-    WsCtl *ctl = B.ctl;
-    if (ctl->stop) return;
-    const UnitGeom g = unit_geom(J.p);
-    const float sc = pow2_scale(__uint_as_float(ctl->mx_t)) * kLift;
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->sB = sc;
-    const float2 *U = Um ? Um : (grad ? J.W1 : J.W0);
-    const int rows = unit_rows(g);
-    const long long total = (long long)g.nu * g.nk * rows * 8;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int c16 = (int)(e & 7);
-        long long r2 = e >> 3;
-        const int n = (int)(r2 % rows);
-        r2 /= rows;
-        const int kc = (int)(r2 % g.nk), u = (int)(r2 / g.nk);
-        unit_image_chunk<BF16>(U, J.p, g, sc, B.bimg, u, kc, n, c16);
-    }
+    if (B.ctl->stop) return;
+    ws_emb<BF16>(J, B, unit_geom(J.p), Um ? Um : (grad ? J.W1 : J.W0), blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------- operators
 // Forward over the current list: F (weights wl = s_j v_j, cvec), U (weights
 // -s_i x_i, cvec) or the support S (weights -s_i x_i, dvec / cvec): Gram
-// blocks from the list's image and its weighted image.
+// blocks from the list's image and its weighted image.  The list's split over
+// tasks (nsplit) fixes the order of the sums; how many of a block's 64-column
+// chunks one task takes does not, so blocks are cut into slices while there
+// are fewer tasks than CTAs.  dyn, bars, tmem: as items_forward.
+template <bool BF16>
+__device__ int ws_forward(const WsBufs &B, const UnitGeom &g, int which, int rank, int ctas, unsigned char *dyn,
+                          uint64_t *bars, uint32_t tmem) {
+    const WsCtl *ctl = B.ctl;
+    const int n = which == kListF ? ctl->f : (which == kListU ? ctl->nu : ctl->ns);
+    const unsigned char *XA = which == kListF ? B.ximgF : B.ximgS;
+    if (n <= 0) return 0;
+    const int nsplit = ctl->nsplit;
+    const int blocks = B.npairs * nsplit;
+    const int slices = blocks >= 2 * ctas ? 1 : (2 * blocks >= ctas ? 2 : 4), nq = 4 / slices;
+    int to = 0;
+    for (int task = rank; task < blocks * slices; task += ctas) {
+        const int blk = task / slices, q0 = (task - blk * slices) * nq;
+        const int pr = blk / nsplit, s = blk - pr * nsplit;
+        if (64 * q0 >= items_fwd_n(g, B.pnb[pr])) continue;
+        to += items_forward<BF16>(g, dyn, bars, tmem, XA, B.ximgW, n, B.pm[pr], B.pnb[pr], q0, nq, s, nsplit,
+                                  B.pfwd + (size_t)blk * kTcM * 256);
+        __syncthreads();
+    }
+    return to;
+}
+
+// A broken pipeline ends the solve: every later kernel sees stop.
+__device__ __forceinline__ void ws_timeouts(WsCtl *ctl, int to) {
+    if (to && threadIdx.x == 0) {
+        atomicAdd(&ctl->timeouts, to);
+        ctl->stop = 1;
+    }
+}
+
 template <bool BF16>
 __global__ void __launch_bounds__(kItemsFwdThreads, 1) k_ws_fwd(const JobDev *Jp, WsBufs B, int which) {
     ws_count(B.ctl);
-    const JobDev &J = *Jp;
-    WsCtl *ctl = B.ctl;
-    if (ctl->stop) return;
-    const UnitGeom g = unit_geom(J.p);
-    const int n = which == kListF ? ctl->f : (which == kListU ? ctl->nu : ctl->ns);
-    const unsigned char *XA = which == kListF ? B.ximgF : B.ximgS;
-    if (n <= 0) return;
-    const int nsplit = ctl->nsplit;
-    const int tasks = B.npairs * nsplit;
+    if (B.ctl->stop) return;
     unsigned char *dyn = dyn_smem();
     __shared__ uint64_t bars[6];
     __shared__ uint32_t tslot;
-    if (blockIdx.x >= tasks) return;
     // one tensor-memory allocation for all of this CTA's tasks
     if (threadIdx.x < 32) tmem_alloc(&tslot, 256);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tslot;
-    int to = 0;
-    for (int task = blockIdx.x; task < tasks; task += gridDim.x) {
-        const int pr = task / nsplit, s = task - pr * nsplit;
-        to += items_forward<BF16>(g, dyn, bars, tmem, XA, B.ximgW, n, B.pm[pr], B.pnb[pr], s, nsplit,
-                                  B.pfwd + (size_t)task * kTcM * 256);
-        __syncthreads();
-    }
+    const int to = ws_forward<BF16>(B, unit_geom(Jp->p), which, blockIdx.x, gridDim.x, dyn, bars, tmem);
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x < 32) tmem_dealloc(tmem, 256);
-    if (to && threadIdx.x == 0) {
-        // a broken pipeline ends the solve: every later kernel sees stop
-        atomicAdd(&ctl->timeouts, to);
-        ctl->stop = 1;
-    }
+    ws_timeouts(B.ctl, to);
 }
 
 // Sum the forward partial blocks in a fixed order into K and form
@@ -553,13 +558,9 @@ __device__ __forceinline__ const float *fred_at(const WsBufs &B, const int *pidx
     return B.pfwd + (size_t)pidx[m * 4 + nb] * nsplit * kTcM * 256 + (size_t)(c - 256 * nb) * kTcM + (r - 128 * m);
 }
 
-__global__ void __launch_bounds__(kWsThreads) k_ws_fred(const JobDev *Jp, WsBufs B, int mode) {
-    ws_count(B.ctl);
-    const JobDev &J = *Jp;
+__device__ void ws_fred(const JobDev &J, const WsBufs &B, const UnitGeom &g, int mode, int rank, int ctas) {
     WsCtl *ctl = B.ctl;
-    if (ctl->stop) return;
     const int p = J.p;
-    const UnitGeom g = unit_geom(p);
     const int Kp = g.Kp;
     const bool pwls = J.cost == IMG_COST_PWLS;
     const int n = mode == kRedT ? ctl->f : (mode == kRedB ? ctl->nu : ctl->ns);
@@ -568,8 +569,9 @@ __global__ void __launch_bounds__(kWsThreads) k_ws_fred(const JobDev *Jp, WsBufs
     const float inv = n > 0 ? 1.f / (sX * sX * ctl->sW) : 0.f;
     const float fa = (float)ctl->fa;
     float2 *dst = mode == kRedG ? J.W1 : J.W0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->mx_w = 0u;     // the weights are consumed
+    if (rank == 0 && threadIdx.x == 0) ctl->mx_w = 0u;     // the weights are consumed
     __shared__ int pidx[6 * 4];
+    __shared__ double sbuf[kWsThreads / 32];
     __shared__ float T[4][kRedTile][kRedTile + 1];   // G(a,b), G(Kp+a,Kp+b), G(a,Kp+b), G(b,Kp+a), as [a][b]
     if (threadIdx.x < 24) pidx[threadIdx.x] = 0;
     __syncthreads();
@@ -577,8 +579,9 @@ __global__ void __launch_bounds__(kWsThreads) k_ws_fred(const JobDev *Jp, WsBufs
     __syncthreads();
     const int nt = (p + kRedTile - 1) / kRedTile;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;      // 32 x 8
-    float mx = 0.f, ss = 0.f;
-    for (int tile = blockIdx.x; tile < nt * nt; tile += gridDim.x) {
+    float mx = 0.f;
+    for (int tile = rank; tile < nt * nt; tile += ctas) {
+        float ss = 0.f;
         const int a0 = (tile % nt) * kRedTile, b0 = (tile / nt) * kRedTile;
         if (n > 0) {
             // the stored blocks are column-major: lanes run along the stored
@@ -609,7 +612,7 @@ __global__ void __launch_bounds__(kWsThreads) k_ws_fred(const JobDev *Jp, WsBufs
 #pragma unroll
                 for (int ii = 0; ii < 4; ++ii)
 #pragma unroll
-                    for (int e = 0; e < 6; ++e) v[ii][e] = src[ii][e] ? src[ii][e][off] : 0.f;
+                    for (int e = 0; e < 6; ++e) v[ii][e] = src[ii][e] ? __ldcg(src[ii][e] + off) : 0.f;
 #pragma unroll
                 for (int ii = 0; ii < 4; ++ii)
 #pragma unroll
@@ -653,207 +656,237 @@ __global__ void __launch_bounds__(kWsThreads) k_ws_fred(const JobDev *Jp, WsBufs
                 ss = fmaf(out.x, out.x, fmaf(out.y, out.y, ss));
             }
         }
+        // this tile's share of ||W0||^2 (FP64); the vector step adds the
+        // shares in tile order
+        const double cs = mode == kRedG ? 0.0 : block_sum_w0((double)ss, sbuf);
+        if (mode != kRedG && threadIdx.x == 0) ctl->sums[tile] = cs;
         __syncthreads();
     }
     for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if ((threadIdx.x & 31) == 0) atomicMax(&ctl->mx_t, __float_as_uint(mx));
-    if (mode == kRedG) return;
-    // this CTA's share of ||W0||^2 (FP64); k_ws_vx adds the shares in CTA order
-    __shared__ double sbuf[kWsThreads / 32];
-    const double cs = block_sum((double)ss, sbuf);
-    if (threadIdx.x == 0) ctl->sums[blockIdx.x] = cs;
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->nsums = gridDim.x;
+    if (mode != kRedG && rank == 0 && threadIdx.x == 0) ctl->nsums = nt * nt;
+}
+__global__ void __launch_bounds__(kWsThreads) k_ws_fred(const JobDev *Jp, WsBufs B, int mode) {
+    ws_count(B.ctl);
+    if (B.ctl->stop) return;
+    ws_fred(*Jp, B, unit_geom(Jp->p), mode, blockIdx.x, gridDim.x);
 }
 
-// Adjoint over the free list (LIST) or over every pixel (gradient): unit
-// partial dots into padj[row * ld_adj + u] (u: unit, or unit x K group).
-template <bool BF16, bool LIST>
+// Adjoint over every pixel (gradient, bounds): unit partial dots into
+// padj[row * ld_adj + u].
+template <bool BF16>
 __global__ void __launch_bounds__(kWideThreads, 1) k_ws_adj(const JobDev *Jp, WsBufs B) {
     ws_count(B.ctl);
     const JobDev &J = *Jp;
     WsCtl *ctl = B.ctl;
     if (ctl->stop) return;
-    const UnitGeom g = unit_geom(J.p);
-    const int n = LIST ? ctl->f : J.Q;
-    if (n <= 0) return;
-    const int ntiles = LIST ? (n + kTcM - 1) / kTcM : tc_num_tiles(J.n_l, J.n_m);
-    const int nkg = LIST ? ws_nkg(ntiles * g.nu, g.nk, gridDim.x) : 1;
-    if (LIST && blockIdx.x == 0 && threadIdx.x == 0) ctl->adj_rows = g.nu * nkg;
     unsigned char *dyn = dyn_smem();
     __shared__ uint64_t bars[kWideBars];
     __shared__ uint32_t tslot;
+    if (threadIdx.x < 32) tmem_alloc(&tslot, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tslot;
     float *out = B.padj;
     const int ld = B.ld_adj;
-    const bool sq = !LIST && ctl->adj_sq;
-    const int to = items_adjoint<BF16, LIST>(
-        J, g, dyn, bars, &tslot, B.bimg, B.ximgF, J.cvec, J.fpos, n, ntiles, nkg, blockIdx.x, gridDim.x, sq,
-        [&](int u, int t, int r, float v) {
-            if (LIST) {
-                const int j = t * kTcM + r;
-                if (j < n) out[(size_t)j * ld + u] = v;
-            } else {
-                const int i = tc_tile_pixel(t, r, J.n_l, J.n_m);
-                if (i >= 0) out[(size_t)i * ld + u] = v;
-            }
-        });
-    if (to && threadIdx.x == 0) {
-        // a broken pipeline ends the solve: every later kernel sees stop
-        atomicAdd(&ctl->timeouts, to);
-        ctl->stop = 1;
+    const int to = items_adjoint<BF16, false>(
+        J, unit_geom(J.p), dyn, bars, tmem, B.bimg, nullptr, nullptr, nullptr, J.Q, tc_num_tiles(J.n_l, J.n_m), 1,
+        blockIdx.x, gridDim.x, ctl->adj_sq, [&](int u, int t, int r, float v) {
+            const int i = tc_tile_pixel(t, r, J.n_l, J.n_m);
+            if (i >= 0) out[(size_t)i * ld + u] = v;
+        }, [](int) {});
+    if (threadIdx.x < 32) tmem_dealloc(tmem, 512);
+    ws_timeouts(ctl, to);
+}
+
+// Adjoint over the free list: (unit, K group) partial dots into padj.  The
+// number of K groups - part of the order of the sums - is that of a grid of
+// `list_grid` CTAs.  idle(warp): as items_adjoint.
+template <bool BF16, class Idle>
+__device__ int ws_adj_list(const JobDev &J, const WsBufs &B, const UnitGeom &g, int rank, int ctas,
+                           unsigned char *dyn, uint64_t *bars, uint32_t tmem, Idle idle) {
+    WsCtl *ctl = B.ctl;
+    const int n = ctl->f;
+    const int ntiles = (n + kTcM - 1) / kTcM;
+    const int nkg = ws_nkg(ntiles * g.nu, g.nk, B.list_grid);
+    if (rank == 0 && threadIdx.x == 0) ctl->adj_rows = g.nu * nkg;
+    float *out = B.padj;
+    const int ld = B.ld_adj;
+    return items_adjoint<BF16, true>(J, g, dyn, bars, tmem, B.bimg, B.ximgF, J.cvec, J.fpos, n, ntiles, nkg, rank,
+                                     ctas, false, [&](int u, int t, int r, float v) {
+                                         const int j = t * kTcM + r;
+                                         if (j < n) out[(size_t)j * ld + u] = v;
+                                     }, idle);
+}
+
+// ---------------------------------------------------------------- LSQR
+// One subproblem's LSQR (Sec. V-A): the phases of a Golub-Kahan iteration are
+//
+//   weighted list image | forward blocks | reduction t = M v - alpha u |
+//   B image of t | free-list adjoint | vectors (one CTA)
+//
+// each a few microseconds of work for a list of some hundred pixels.  Two
+// forms of the same phases, chosen by ws_clustered:
+//
+// * small operands: one kernel, a cluster of kLsqrCtas CTAs that walks the
+//   phases, separated by cluster barriers, until the stopping tests hold.
+//   As kernels of the solve's graph most of an iteration's ~45 us at p = 100
+//   is launch, ramp and drain between the phases.  Eight CTAs are one portable
+//   cluster: the hardware places them together, so no phase waits for another
+//   solve's CTAs, and 16 solves in flight leave SMs for their gradients.
+// * large operands: a graph WHILE node of one kernel per phase, whose grids
+//   spread the images and the reduction over every SM.
+//
+// Shares and splits follow the list alone (not the CTA count), so every sum
+// has the same order in both.
+//
+// The vector step's FP64 scalars hide where they can (a dependent FP64
+// instruction takes 67 cycles, a division 550, hypot 1,050): ||t|| and the
+// rotation's part that needs no alpha run in an idle warp of the adjoint
+// phase, in the cluster the stopping tests during the next weighted image.
+constexpr int kLsqrCtas = 8;
+constexpr int kVxReg = 4;               // rows per thread held in registers (f <= 1024)
+
+// beta = ||t|| from the reduction's shares (added as a CTA of 256 threads
+// would: 32 shares at a time, butterfly, then in order), u's scale, and the
+// rotation up to alpha.  One warp.
+__device__ void vx_beta(const WsCtl *ctl, VxState &S, bool init) {
+    const int lane = threadIdx.x & 31, n = ctl->nsums;
+    double t = 0.0;
+    for (int w = 0; w * 32 < n; ++w) {
+        double d = w * 32 + lane < n ? ctl->sums[w * 32 + lane] : 0.0;
+        for (int o = 16; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        t += d;
+    }
+    const double beta = sqrt(t);
+    const double us = beta > 0.0 ? 1.0 / beta : 0.0;
+    if (lane == 0) {
+        S.beta = beta;
+        S.us = us;
+        S.fus = (float)us;
+        S.fb = (float)beta;
+    }
+    if (init) {
+        if (lane == 0) {
+            S.bnorm = S.phibar = beta;
+            S.anorm2 = 0.0;
+        }
+    } else {
+        const double alpha = S.alpha, phibar = S.phibar, rhobar = S.rhobar;
+        double anorm2 = S.anorm2;
+        anorm2 += alpha * alpha + beta * beta;
+        const double rho = hypot(rhobar, beta);
+        const double q = (lane == 0 ? rhobar : beta) / rho;
+        const double c = __shfl_sync(0xffffffffu, q, 0), sn = __shfl_sync(0xffffffffu, q, 1);
+        __syncwarp();
+        if (lane == 0) {
+            S.anorm2 = anorm2;
+            S.rho = rho;
+            S.c = c;
+            S.sn = sn;
+            S.phi = c * phibar;
+            S.phibar = sn * phibar;
+        }
     }
 }
 
-// ---------------------------------------------------------------- LSQR vectors
-// One CTA of kVxThreads threads per Golub-Kahan half step on the f-vectors:
-//   beta = ||t|| from the CTA shares of the reduction (FP64, in CTA order),
-//   us = 1/beta; (init: ||b|| = beta; else ||B||^2 += alpha^2 + beta^2);
-//   v <- s_F (M^H u) - beta v  (init: v <- s_F M^H u), M^H u = us times the
-//   adjoint's unit (x K group) partial dots;  alpha = ||v||;
-//   the plane rotation (FP64); v <- v / alpha; init: w = v, x = 0; else
-//   x += t1 w, w = v + t2 w; the weights s_F v of the next forward and their
-//   maximum; ||x|| and the Paige-Saunders stopping tests; h_lsqr := continue.
-//
-// Latency bound (one CTA, a few hundred rows).  The FP64 scalars run in warp
-// 0 alone, independent divisions and roots in neighbouring lanes (the FP64
-// pipe takes a warp instruction per 16 cycles: in all 8 warps they cost
-// most of the 15.5 us the kernel took), and the first kVxReg rows of a thread stay in
-// registers from one phase to the next, loaded before the first reduction.
-constexpr int kVxThreads = kThreads;
-constexpr int kVxReg = 4;               // rows per thread held in registers (f <= 1024)
-
-__global__ void __launch_bounds__(kVxThreads) k_ws_vx(const JobDev *Jp, WsBufs B, int init,
-                                                       cudaGraphConditionalHandle h_lsqr) {
-    ws_count(B.ctl);
-    const JobDev &J = *Jp;
+// The f-vectors (one CTA): v <- s_F (M^H u) - beta v (init: v <- s_F M^H u),
+// M^H u = us times the adjoint's partial dots; alpha = ||v||; v <- v / alpha;
+// init: w = v, x = 0, else x += t1 w, w = v + t2 w; the weights s_F v of the
+// next forward and their maximum; ||x||^2.
+__device__ void vx_step(const JobDev &J, const WsBufs &B, VxState &S, double *sb, float *swm, bool init) {
     WsCtl *ctl = B.ctl;
-    __shared__ double sb[kVxThreads / 32];
-    __shared__ float swm[kVxThreads / 32];
-    __shared__ float s_c[5];                // us, beta, then 1/alpha, t1, t2
-    if (ctl->stop) {
-        if (threadIdx.x == 0) ws_cond(ctl, kCondLsqr, h_lsqr, 0u);
-        return;
-    }
     const bool w0 = threadIdx.x < 32;
     const int lane = threadIdx.x & 31;
     const int f = ctl->f, ld = B.ld_adj, rows = ctl->adj_rows;
     const int r4 = rows >> 2;
-    float *__restrict__ vv = J.v;
-    float *__restrict__ ww = J.w;
-    float *__restrict__ xx = J.xs;
-    const float *__restrict__ sF = J.sF;
-    const float *__restrict__ padj = B.padj;
+    float *vv = J.v, *ww = J.w, *xx = J.xs;
+    const float *sF = J.sF;
     float vr[kVxReg], wr[kVxReg], xr[kVxReg], fr[kVxReg];
 #pragma unroll
     for (int q = 0; q < kVxReg; ++q) {
-        const int j = threadIdx.x + q * kVxThreads;
+        const int j = threadIdx.x + q * kThreads;
         const bool ok = j < f, old = ok && !init;
         fr[q] = ok ? sF[j] : 0.f;
         vr[q] = old ? vv[j] : 0.f;
         wr[q] = old ? ww[j] : 0.f;
         xr[q] = old ? xx[j] : 0.f;
     }
+    const float sc = 1.f / (ctl->sXF * ctl->sB);
+    const float fus = S.fus, fb = S.fb;
+    float ss = 0.f;
     // two rows per thread per step: every load of both rows is in flight
     // before the sums (rows <= nu nk <= 36 partial dots, 9 float4)
     float4 s4[2][9];
     auto load = [&](int j0) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int j = j0 + h * kVxThreads;
+            const int j = j0 + h * kThreads;
             const bool ok = j < f;
-            const float4 *pr = reinterpret_cast<const float4 *>(padj + (size_t)(ok ? j : 0) * ld);
+            const float4 *pr = reinterpret_cast<const float4 *>(B.padj + (size_t)(ok ? j : 0) * ld);
 #pragma unroll
-            for (int q = 0; q < 9; ++q) s4[h][q] = (ok && q < r4) ? pr[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int q = 0; q < 9; ++q) s4[h][q] = (ok && q < r4) ? __ldcg(pr + q) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
-    load(threadIdx.x);
-    // beta from the reduction's CTA shares
-    double part = 0.0;
-    for (int b = threadIdx.x; b < ctl->nsums; b += kVxThreads) part += ctl->sums[b];
-    const double alpha_prev = ctl->alpha;
-    double beta = 0.0, us = 0.0;
-    {
-        const double t = block_sum_w0(part, sb);
-        if (w0) {
-            beta = sqrt(t);
-            us = beta > 0.0 ? 1.0 / beta : 0.0;
-            s_c[0] = (float)us;
-            s_c[1] = (float)beta;
-        }
-    }
-    const float sc = 1.f / (ctl->sXF * ctl->sB);
-    __syncthreads();
-    const float fus = s_c[0], fb = s_c[1];
-    float ss = 0.f;
     // one row: its new v (before normalisation) from the loaded partial dots
     auto row = [&](int h, int j, float sf, float vo) {
         float y = 0.f;
 #pragma unroll
         for (int q = 0; q < 9; ++q) y += (s4[h][q].x + s4[h][q].y) + (s4[h][q].z + s4[h][q].w);
-        for (int u = 4 * r4; u < rows; ++u) y += padj[(size_t)j * ld + u];
+        for (int u = 4 * r4; u < rows; ++u) y += __ldcg(B.padj + (size_t)j * ld + u);
         y *= sc;
-        const float vn = init ? sf * (y * fus) : sf * (y * fus) - fb * vo;
+        const float yf = __fmul_rn(y, fus);
+        const float vn = init ? __fmul_rn(sf, yf) : __fmaf_rn(sf, yf, -__fmul_rn(fb, vo));
         ss = fmaf(vn, vn, ss);
         return vn;
     };
 #pragma unroll
     for (int q = 0; q < kVxReg; q += 2) {
-        const int j0 = threadIdx.x + q * kVxThreads;
-        if (q > 0 && j0 < f) load(j0);
+        const int j0 = threadIdx.x + q * kThreads;
+        if (j0 < f) load(j0);
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-            if (j0 + h * kVxThreads < f) vr[q + h] = row(h, j0 + h * kVxThreads, fr[q + h], vr[q + h]);
+            if (j0 + h * kThreads < f) vr[q + h] = row(h, j0 + h * kThreads, fr[q + h], vr[q + h]);
     }
-    for (int j0 = threadIdx.x + kVxReg * kVxThreads; j0 < f; j0 += 2 * kVxThreads) {
+    for (int j0 = threadIdx.x + kVxReg * kThreads; j0 < f; j0 += 2 * kThreads) {
         load(j0);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int j = j0 + h * kVxThreads;
+            const int j = j0 + h * kThreads;
             if (j < f) vv[j] = row(h, j, sF[j], init ? 0.f : vv[j]);
         }
     }
-    double alpha = 0.0, rhobar = ctl->rhobar, phibar = ctl->phibar, anorm2 = ctl->anorm2, absc = 0.0;
     {
         const double t = block_sum_w0((double)ss, sb);
         if (w0) {
-            alpha = sqrt(t);
-            if (init) {
-                phibar = beta;
-                rhobar = alpha;
-                anorm2 = 0.0;
-                const double ialpha = 1.0 / alpha;
-                if (lane == 0) s_c[2] = alpha > 0.0 ? (float)ialpha : 1.f;
-                if (lane == 0) s_c[3] = s_c[4] = 0.f;
-            } else {
-                // plane rotation; lanes 0..2: c, s, 1/alpha, then lanes 0, 1: the coefficients
-                anorm2 += alpha_prev * alpha_prev + beta * beta;
-                const double rho = hypot(rhobar, beta);
-                const double q = (lane == 0 ? rhobar : lane == 1 ? beta : 1.0) / (lane == 2 ? alpha : rho);
-                const double c = __shfl_sync(0xffffffffu, q, 0), sn = __shfl_sync(0xffffffffu, q, 1);
-                const double ialpha = __shfl_sync(0xffffffffu, q, 2);
-                const double theta = sn * alpha;
-                rhobar = -c * alpha;
-                const double phi = c * phibar;
-                phibar = sn * phibar;
-                absc = fabs(c);
-                const double t12 = (lane == 0 ? phi : -theta) / rho;
-                if (lane < 2) s_c[3 + lane] = (float)t12;
-                if (lane == 0) s_c[2] = alpha > 0.0 ? (float)ialpha : 1.f;
+            // lanes 0..2: the coefficients of x and w, 1/alpha
+            const double alpha = sqrt(t);
+            const double rho = init ? 1.0 : S.rho, c = S.c, sn = S.sn, phi = S.phi;
+            const double theta = sn * alpha;
+            const double q = (lane == 0 ? phi : lane == 1 ? -theta : 1.0) / (lane == 2 ? alpha : rho);
+            if (lane == 0) {
+                S.alpha = alpha;
+                S.rhobar = init ? alpha : -c * alpha;
+                S.t1 = init ? 0.f : (float)q;
             }
+            if (lane == 1) S.t2 = init ? 0.f : (float)q;
+            if (lane == 2) S.ia = alpha > 0.0 ? (float)q : 1.f;
         }
         __syncthreads();
     }
-    const float ia = s_c[2], ft1 = s_c[3], ft2 = s_c[4];
+    const float ia = S.ia, ft1 = S.t1, ft2 = S.t2;
     float xs2 = 0.f, wm = 0.f;
     auto update = [&](int j, float vn, float wo, float xo, float sf) {
-        const float vj = vn * ia;
+        const float vj = __fmul_rn(vn, ia);
         vv[j] = vj;
         if (init) {
             ww[j] = vj;
             xx[j] = 0.f;
         } else {
-            const float xj = xo + ft1 * wo;
+            const float xj = __fmaf_rn(ft1, wo, xo);
             xx[j] = xj;
-            ww[j] = vj + ft2 * wo;
+            ww[j] = __fmaf_rn(ft2, wo, vj);
             xs2 = fmaf(xj, xj, xs2);
         }
         const float wv = sf * vj;
@@ -862,47 +895,154 @@ __global__ void __launch_bounds__(kVxThreads) k_ws_vx(const JobDev *Jp, WsBufs B
     };
 #pragma unroll
     for (int q = 0; q < kVxReg; ++q) {
-        const int j = threadIdx.x + q * kVxThreads;
+        const int j = threadIdx.x + q * kThreads;
         if (j < f) update(j, vr[q], wr[q], xr[q], fr[q]);
     }
 #pragma unroll 4
-    for (int j = threadIdx.x + kVxReg * kVxThreads; j < f; j += kVxThreads)
+    for (int j = threadIdx.x + kVxReg * kThreads; j < f; j += kThreads)
         update(j, vv[j], init ? 0.f : ww[j], init ? 0.f : xx[j], sF[j]);
     for (int o = 16; o; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
     if (lane == 0) swm[threadIdx.x >> 5] = wm;
     const double xnorm2 = block_sum_w0((double)xs2, sb);     // its barrier publishes swm too
-    if (!w0) return;
-    // lanes 0, 1: ||x||, ||B||
-    const double q = sqrt(lane == 0 ? xnorm2 : anorm2);
-    const double xnorm = __shfl_sync(0xffffffffu, q, 0), anorm = __shfl_sync(0xffffffffu, q, 1);
-    if (lane == 0) {
-        for (int w = 0; w < kVxThreads / 32; ++w) wm = fmaxf(wm, swm[w]);
+    if (threadIdx.x == 0) {
+        for (int w = 0; w < kThreads / 32; ++w) wm = fmaxf(wm, swm[w]);
         ctl->mx_w = __float_as_uint(wm);
         ctl->mx_t = 0u;                       // the image of t is consumed
-        ctl->beta = beta;
-        ctl->us = us;
-        ctl->alpha = alpha;
-        ctl->rhobar = rhobar;
-        ctl->phibar = phibar;
-        ctl->anorm2 = anorm2;
-        bool more;
-        if (init) {
-            ctl->bnorm = beta;
-            more = alpha > 0.0 && beta > 0.0 && ctl->maxit >= 1;
-        } else {
-            ctl->it++;
-            const double rnorm = phibar;
-            const double arnorm = phibar * alpha * absc;
-            more = ctl->it < ctl->maxit;
-            if (rnorm <= J.lsqr_btol * ctl->bnorm + J.lsqr_atol * anorm * xnorm) more = false;
-            if (arnorm <= J.lsqr_atol * anorm * rnorm) more = false;
-        }
+        S.xnorm2 = xnorm2;
         // the next forward: t <- M v - alpha u with u = t us, so fa = alpha us
-        ctl->fa = alpha * us;
-        ctl->nlist = f;
-        ctl->nsplit = ws_nsplit(f, B.npairs, B.max_tasks, B.fwd_per);
+        ctl->fa = S.alpha * S.us;
+        if (init) ctl->nsplit = ws_nsplit(f, B.npairs, B.max_tasks, B.fwd_per);
+    }
+}
+
+// Paige-Saunders stopping tests after `it` iterations (0: after the
+// initialisation); one warp, the same answer in every lane.
+__device__ bool vx_more(const JobDev &J, const WsCtl *ctl, const VxState &S, int it) {
+    const int lane = threadIdx.x & 31;
+    if (it == 0) return S.alpha > 0.0 && S.beta > 0.0 && ctl->maxit >= 1;
+    const double q = sqrt(lane == 0 ? S.xnorm2 : S.anorm2);
+    const double xnorm = __shfl_sync(0xffffffffu, q, 0), anorm = __shfl_sync(0xffffffffu, q, 1);
+    const double rnorm = S.phibar;
+    const double arnorm = S.phibar * S.alpha * fabs(S.c);
+    bool more = it < ctl->maxit;
+    if (rnorm <= J.lsqr_btol * S.bnorm + J.lsqr_atol * anorm * xnorm) more = false;
+    if (arnorm <= J.lsqr_atol * anorm * rnorm) more = false;
+    return more;
+}
+
+// All CTAs' writes before, generic or by bulk copies' operands, visible after.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("fence.proxy.async;" ::: "memory");
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("fence.proxy.async;" ::: "memory");
+}
+
+// The phases as kernels: the adjoint with the scalars in an idle warp of CTA
+// 0, and the vector step with the stopping tests.
+template <bool BF16>
+__global__ void __launch_bounds__(kThreads, 1) k_ws_adj_list(const JobDev *Jp, WsBufs B, int init) {
+    ws_count(B.ctl);
+    const JobDev &J = *Jp;
+    WsCtl *ctl = B.ctl;
+    if (ctl->stop) return;
+    unsigned char *dyn = dyn_smem();
+    __shared__ uint64_t bars[kWideBars];
+    __shared__ uint32_t tslot;
+    if (threadIdx.x < 32) tmem_alloc(&tslot, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tslot;
+    const int to = ws_adj_list<BF16>(J, B, unit_geom(J.p), blockIdx.x, gridDim.x, dyn, bars, tmem, [&](int warp) {
+        if (blockIdx.x == 0 && warp == 7) vx_beta(ctl, ctl->vx, init);
+    });
+    if (threadIdx.x < 32) tmem_dealloc(tmem, 512);
+    ws_timeouts(ctl, to);
+}
+
+__global__ void __launch_bounds__(kThreads) k_ws_vx(const JobDev *Jp, WsBufs B, int init,
+                                                    cudaGraphConditionalHandle h_lsqr) {
+    ws_count(B.ctl);
+    const JobDev &J = *Jp;
+    WsCtl *ctl = B.ctl;
+    __shared__ double sb[kThreads / 32];
+    __shared__ float swm[kThreads / 32];
+    __shared__ VxState S;
+    if (ctl->stop) {
+        if (threadIdx.x == 0) ws_cond(ctl, kCondLsqr, h_lsqr, 0u);
+        return;
+    }
+    if (threadIdx.x == 0) S = ctl->vx;
+    __syncthreads();
+    vx_step(J, B, S, sb, swm, init);
+    __syncwarp();
+    if (threadIdx.x >= 32) return;
+    const int it = init ? 0 : ctl->it + 1;
+    const bool more = vx_more(J, ctl, S, it);
+    if (threadIdx.x == 0) {
+        ctl->it = it;
+        ctl->vx = S;
         ws_cond(ctl, kCondLsqr, h_lsqr, more ? 1u : 0u);
     }
+}
+
+template <bool BF16>
+__global__ void __cluster_dims__(kLsqrCtas, 1, 1) __launch_bounds__(kThreads, 1)
+k_ws_lsqr(const JobDev *Jp, WsBufs B) {
+    ws_count(B.ctl);
+    const JobDev &J = *Jp;
+    WsCtl *ctl = B.ctl;
+    if (ctl->stop) return;
+    unsigned char *dyn = dyn_smem();
+    __shared__ uint64_t bars[kWideBars];
+    __shared__ uint32_t tslot;
+    __shared__ double sb[kThreads / 32];
+    __shared__ float swm[kThreads / 32];
+    __shared__ VxState S;
+    const int rank = blockIdx.x;
+    const UnitGeom g = unit_geom(J.p);
+    if (threadIdx.x < 32) tmem_alloc(&tslot, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tslot;
+    // data b = base - sum_U s x c c^H, then M^H b
+    ws_listimg<BF16>(J, B, g, kListF, 0, rank, kLsqrCtas);
+    ws_listimg<BF16>(J, B, g, kListU, 0, rank, kLsqrCtas);
+    ws_listimg<BF16>(J, B, g, kListU, 1, rank, kLsqrCtas);
+    cluster_sync();
+    for (int it = 0;; ++it) {
+        const bool init = it == 0;
+        if (!init) {
+            // the tests of the iteration before run beside the weighted image
+            if (rank == 0 && threadIdx.x < 32) {
+                const bool more = vx_more(J, ctl, S, it - 1) && !*(volatile int *)&ctl->stop;
+                if (threadIdx.x == 0) ctl->cond[kCondLsqr] = more;
+            }
+            ws_listimg<BF16>(J, B, g, kListF, 1, rank, kLsqrCtas);
+            cluster_sync();
+            if (!*(volatile unsigned *)&ctl->cond[kCondLsqr]) {
+                if (rank == 0 && threadIdx.x == 0) ctl->it = it - 1;
+                break;
+            }
+        }
+        ws_timeouts(ctl, ws_forward<BF16>(B, g, init ? kListU : kListF, rank, kLsqrCtas, dyn, bars, tmem));
+        cluster_sync();
+        ws_fred(J, B, g, init ? kRedB : kRedT, rank, kLsqrCtas);
+        cluster_sync();
+        ws_emb<BF16>(J, B, g, J.W0, rank, kLsqrCtas);
+        cluster_sync();
+        ws_timeouts(ctl, ws_adj_list<BF16>(J, B, g, rank, kLsqrCtas, dyn, bars, tmem, [&](int warp) {
+                        if (rank == 0 && warp == 7) vx_beta(ctl, S, init);
+                    }));
+        cluster_sync();
+        if (rank == 0) vx_step(J, B, S, sb, swm, init);
+        cluster_sync();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x < 32) tmem_dealloc(tmem, 512);
 }
 
 // ---------------------------------------------------------------- feasibility
@@ -969,7 +1109,6 @@ __global__ void k_ws_accept(const JobDev *Jp, WsBufs B) {
         for (int w = 0; w < kWsThreads / 32; ++w) wm = fmaxf(wm, swm[w]);
         ctl->mx_w = __float_as_uint(wm);
         ctl->sXS = pow2_scale(mS) * kLift;
-        ctl->nlist = ns;
         ctl->nsplit = ws_nsplit(ns, B.npairs, B.max_tasks, B.fwd_per);
         ctl->key = ~0ull;
         ctl->op_flops += ws_flops_fwd(J.p, ns) + ws_flops_adj(J.p, J.Q);
@@ -1197,10 +1336,12 @@ struct WsHost {
     int device = 0;
     int bf16 = 0;
     int direct = 0;             // host-driven loop instead of the graph
+    int cluster = 0;            // LSQR as one cluster kernel
     int sms = 1;
     unsigned *h_cond = nullptr; // pinned mirror of the conditions
     const JobDev *dj = nullptr;
     int p = 0, cap = 0, Q = 0;
+    int g_red = 1;              // CTAs of the forward reduction (one tile each)
     UnitGeom g{};
     void *mem = nullptr;
     WsBufs B{};
@@ -1221,6 +1362,7 @@ size_t ws_bytes(const JobDev &hj, int sms, WsBufs *B, char *base) {
     WsBufs b{};
     b.npairs = items_fwd_pairs(g, b.pm, b.pnb);
     b.max_tasks = std::max(b.npairs, 2 * std::min(sms, kListGrid));
+    b.list_grid = std::min(sms, kListGrid);
     b.fwd_per = kFwdPerTask;
     b.nrows_adj = std::max(hj.Q, cap);
     b.ld_adj = (g.nu * g.nk + 3) / 4 * 4;    // a multiple of 4: rows read as float4
@@ -1239,6 +1381,41 @@ size_t ws_bytes(const JobDev &hj, int sms, WsBufs *B, char *base) {
     return off + 1024;
 }
 
+// LSQR as one cluster kernel (see there) when the B image has one unit, p <=
+// 128.  Time per iteration, 64x64 pixels, 300 passes (f <= 150), cluster /
+// kernels: p = 70: 34.7 / 40.4 us, 100: 38.3 / 41.2, 128: 39.5 / 42.9, but 130:
+// 54.0 / 40.7, 288: 104 / 48 (the reduction and the B image of 81 and 27 tiles
+// need more than 8 SMs).  16 solves in flight: p = 100: 41 / 61 us each.
+static bool ws_clustered(const UnitGeom &g) { return g.nu == 1; }
+
+// The launches of LSQR's initialisation and of one iteration as kernels.
+template <bool BF>
+static void ws_lsqr_begin(WsHost *w, cudaStream_t s, cudaGraphConditionalHandle h_lsqr) {
+    const WsBufs &B = w->B;
+    const JobDev *dj = w->dj;
+    const size_t fsm = items_fwd_smem_bytes(), asm_ = items_smem_bytes();
+    k_ws_listimg<BF><<<w->sms, kWsThreads, 0, s>>>(dj, B, kListF, 0);
+    k_ws_listimg<BF><<<w->sms, kWsThreads, 0, s>>>(dj, B, kListU, 0);
+    k_ws_listimg<BF><<<w->sms, kWsThreads, 0, s>>>(dj, B, kListU, 1);
+    k_ws_fwd<BF><<<B.list_grid, kItemsFwdThreads, fsm, s>>>(dj, B, kListU);
+    k_ws_fred<<<w->g_red, kWsThreads, 0, s>>>(dj, B, kRedB);
+    k_ws_emb<BF><<<w->sms, kWsThreads, 0, s>>>(dj, B, 0, nullptr);
+    k_ws_adj_list<BF><<<B.list_grid, kThreads, asm_, s>>>(dj, B, 1);
+    k_ws_vx<<<1, kThreads, 0, s>>>(dj, B, 1, h_lsqr);
+}
+template <bool BF>
+static void ws_lsqr_iterate(WsHost *w, cudaStream_t s, cudaGraphConditionalHandle h_lsqr) {
+    const WsBufs &B = w->B;
+    const JobDev *dj = w->dj;
+    const size_t fsm = items_fwd_smem_bytes(), asm_ = items_smem_bytes();
+    k_ws_listimg<BF><<<w->sms, kWsThreads, 0, s>>>(dj, B, kListF, 1);
+    k_ws_fwd<BF><<<B.list_grid, kItemsFwdThreads, fsm, s>>>(dj, B, kListF);
+    k_ws_fred<<<w->g_red, kWsThreads, 0, s>>>(dj, B, kRedT);
+    k_ws_emb<BF><<<w->sms, kWsThreads, 0, s>>>(dj, B, 0, nullptr);
+    k_ws_adj_list<BF><<<B.list_grid, kThreads, asm_, s>>>(dj, B, 0);
+    k_ws_vx<<<1, kThreads, 0, s>>>(dj, B, 0, h_lsqr);
+}
+
 template <bool BF>
 static cudaError_t ws_capture(WsHost *w, const JobDev *dj, const JobDev &hj, int sms) {
     const WsBufs &B = w->B;
@@ -1249,18 +1426,17 @@ static cudaError_t ws_capture(WsHost *w, const JobDev *dj, const JobDev &hj, int
     cudaGraphConditionalHandle h_outer = 0, h_lif = 0, h_lsqr = 0, h_feas = 0;
     if (c.err == cudaSuccess) c.err = cudaGraphConditionalHandleCreate(&h_outer, G, 1, cudaGraphCondAssignDefault);
     if (c.err == cudaSuccess) c.err = cudaGraphConditionalHandleCreate(&h_lif, G, 0, 0);
-    if (c.err == cudaSuccess) c.err = cudaGraphConditionalHandleCreate(&h_lsqr, G, 0, 0);
+    if (c.err == cudaSuccess && !w->cluster) c.err = cudaGraphConditionalHandleCreate(&h_lsqr, G, 0, 0);
     if (c.err == cudaSuccess) c.err = cudaGraphConditionalHandleCreate(&h_feas, G, 0, 0);
     const size_t fsm = items_fwd_smem_bytes(), asm_ = items_smem_bytes();
     if (c.err == cudaSuccess) c.err = set_smem(k_ws_fwd<BF>, fsm);
-    if (c.err == cudaSuccess) c.err = set_smem(k_ws_adj<BF, true>, asm_);
-    if (c.err == cudaSuccess) c.err = set_smem(k_ws_adj<BF, false>, asm_);
-    const int ntr = (hj.p + kRedTile - 1) / kRedTile;
-    const int g_red = std::min(ntr * ntr, kWsSums);
+    if (c.err == cudaSuccess) c.err = set_smem(k_ws_lsqr<BF>, asm_);
+    if (c.err == cudaSuccess) c.err = set_smem(k_ws_adj_list<BF>, asm_);
+    if (c.err == cudaSuccess) c.err = set_smem(k_ws_adj<BF>, asm_);
     const int g_grad = std::min((hj.Q + kWsThreads - 1) / kWsThreads, 4 * sms);
     const int g_img = sms;
     const int g_cache = (hj.p + kCacheRows - 1) / kCacheRows;
-    const int g_fwd = std::min(sms, kListGrid), g_adj = std::min(sms, kListGrid);
+    const int g_fwd = std::min(sms, kListGrid);
     cudaStream_t s = c.st;
     // top level: start, the Table I loop, finish
     c.begin(G, nullptr);
@@ -1282,29 +1458,23 @@ static cudaError_t ws_capture(WsHost *w, const JobDev *dj, const JobDev &hj, int
     cudaGraphNode_t n1 = c.end();
     cudaGraph_t lb[1] = {};
     cudaGraphNode_t nif = add_cond(c, ob[0], h_lif, cudaGraphCondTypeIf, 1, n1, lb);
-    // LSQR on F (Sec. V-A): data b, initialisation, iterations
+    // LSQR on F (Sec. V-A)
     c.begin(lb[0], nullptr);
-    k_ws_listimg<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, kListF, 0);
-    k_ws_listimg<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, kListU, 0);
-    k_ws_listimg<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, kListU, 1);
-    k_ws_fwd<BF><<<g_fwd, kItemsFwdThreads, fsm, s>>>(dj, B, kListU);
-    k_ws_fred<<<g_red, kWsThreads, 0, s>>>(dj, B, kRedB);
-    k_ws_emb<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, 0, nullptr);
-    k_ws_adj<BF, true><<<g_adj, kWideThreads, asm_, s>>>(dj, B);
-    k_ws_vx<<<1, kVxThreads, 0, s>>>(dj, B, 1, h_lsqr);
-    c.check();
-    cudaGraphNode_t n2 = c.end();
-    cudaGraph_t wb[1] = {};
-    add_cond(c, lb[0], h_lsqr, cudaGraphCondTypeWhile, 1, n2, wb);
-    c.begin(wb[0], nullptr);
-    k_ws_listimg<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, kListF, 1);
-    k_ws_fwd<BF><<<g_fwd, kItemsFwdThreads, fsm, s>>>(dj, B, kListF);
-    k_ws_fred<<<g_red, kWsThreads, 0, s>>>(dj, B, kRedT);
-    k_ws_emb<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, 0, nullptr);
-    k_ws_adj<BF, true><<<g_adj, kWideThreads, asm_, s>>>(dj, B);
-    k_ws_vx<<<1, kVxThreads, 0, s>>>(dj, B, 0, h_lsqr);
-    c.check();
-    c.end();
+    if (w->cluster) {
+        k_ws_lsqr<BF><<<kLsqrCtas, kThreads, asm_, s>>>(dj, B);
+        c.check();
+        c.end();
+    } else {
+        ws_lsqr_begin<BF>(w, s, h_lsqr);
+        c.check();
+        cudaGraphNode_t n2 = c.end();
+        cudaGraph_t wb[1] = {};
+        add_cond(c, lb[0], h_lsqr, cudaGraphCondTypeWhile, 1, n2, wb);
+        c.begin(wb[0], nullptr);
+        ws_lsqr_iterate<BF>(w, s, h_lsqr);
+        c.check();
+        c.end();
+    }
     // feasibility, then the gradient (feasible) or the step (infeasible)
     c.begin(ob[0], nif);
     k_ws_feas<<<1, kWsThreads, 0, s>>>(dj, B, h_feas);
@@ -1317,9 +1487,9 @@ static cudaError_t ws_capture(WsHost *w, const JobDev *dj, const JobDev &hj, int
     k_ws_listimg<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, kListS, 0);
     k_ws_listimg<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, kListS, 1);
     k_ws_fwd<BF><<<g_fwd, kItemsFwdThreads, fsm, s>>>(dj, B, kListS);
-    k_ws_fred<<<g_red, kWsThreads, 0, s>>>(dj, B, kRedG);
+    k_ws_fred<<<w->g_red, kWsThreads, 0, s>>>(dj, B, kRedG);
     k_ws_emb<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, 1, nullptr);
-    k_ws_adj<BF, false><<<sms, kWideThreads, asm_, s>>>(dj, B);
+    k_ws_adj<BF><<<sms, kWideThreads, asm_, s>>>(dj, B);
     k_ws_grad<<<g_grad, kWsThreads, 0, s>>>(dj, B);
     k_ws_decide<<<1, 32, 0, s>>>(dj, B);
     c.check();
@@ -1348,12 +1518,10 @@ static cudaError_t ws_direct(WsHost *w, cudaStream_t s) {
     const JobDev *dj = w->dj;
     const int sms = w->sms;
     const size_t fsm = items_fwd_smem_bytes(), asm_ = items_smem_bytes();
-    const int ntr = (w->p + kRedTile - 1) / kRedTile;
-    const int g_red = std::min(ntr * ntr, kWsSums);
     const int g_grad = std::min((w->Q + kWsThreads - 1) / kWsThreads, 4 * sms);
     const int g_img = sms;
     const int g_cache = (w->p + kCacheRows - 1) / kCacheRows;
-    const int g_fwd = std::min(sms, kListGrid), g_adj = std::min(sms, kListGrid);
+    const int g_fwd = std::min(sms, kListGrid);
     cudaError_t e = cudaSuccess;
     auto cond = [&](int which) -> unsigned {
         if (e == cudaSuccess) e = cudaMemcpyAsync(w->h_cond, &B.ctl->cond[0], 4 * sizeof(unsigned),
@@ -1367,21 +1535,11 @@ static cudaError_t ws_direct(WsHost *w, cudaStream_t s) {
         k_ws_cache<<<g_cache, kWsThreads, 0, s>>>(dj, B);
         k_ws_pass<<<1, kWsThreads, 0, s>>>(dj, B, 0);
         if (cond(kCondLsqrIf)) {
-            k_ws_listimg<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, kListF, 0);
-            k_ws_listimg<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, kListU, 0);
-            k_ws_listimg<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, kListU, 1);
-            k_ws_fwd<BF><<<g_fwd, kItemsFwdThreads, fsm, s>>>(dj, B, kListU);
-            k_ws_fred<<<g_red, kWsThreads, 0, s>>>(dj, B, kRedB);
-            k_ws_emb<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, 0, nullptr);
-            k_ws_adj<BF, true><<<g_adj, kWideThreads, asm_, s>>>(dj, B);
-            k_ws_vx<<<1, kVxThreads, 0, s>>>(dj, B, 1, 0);
-            while (cond(kCondLsqr)) {
-                k_ws_listimg<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, kListF, 1);
-                k_ws_fwd<BF><<<g_fwd, kItemsFwdThreads, fsm, s>>>(dj, B, kListF);
-                k_ws_fred<<<g_red, kWsThreads, 0, s>>>(dj, B, kRedT);
-                k_ws_emb<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, 0, nullptr);
-                k_ws_adj<BF, true><<<g_adj, kWideThreads, asm_, s>>>(dj, B);
-                k_ws_vx<<<1, kVxThreads, 0, s>>>(dj, B, 0, 0);
+            if (w->cluster) {
+                k_ws_lsqr<BF><<<kLsqrCtas, kThreads, asm_, s>>>(dj, B);
+            } else {
+                ws_lsqr_begin<BF>(w, s, 0);
+                while (cond(kCondLsqr)) ws_lsqr_iterate<BF>(w, s, 0);
             }
         }
         k_ws_feas<<<1, kWsThreads, 0, s>>>(dj, B, 0);
@@ -1390,9 +1548,9 @@ static cudaError_t ws_direct(WsHost *w, cudaStream_t s) {
             k_ws_listimg<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, kListS, 0);
             k_ws_listimg<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, kListS, 1);
             k_ws_fwd<BF><<<g_fwd, kItemsFwdThreads, fsm, s>>>(dj, B, kListS);
-            k_ws_fred<<<g_red, kWsThreads, 0, s>>>(dj, B, kRedG);
+            k_ws_fred<<<w->g_red, kWsThreads, 0, s>>>(dj, B, kRedG);
             k_ws_emb<BF><<<g_img, kWsThreads, 0, s>>>(dj, B, 1, nullptr);
-            k_ws_adj<BF, false><<<sms, kWideThreads, asm_, s>>>(dj, B);
+            k_ws_adj<BF><<<sms, kWideThreads, asm_, s>>>(dj, B);
             k_ws_grad<<<g_grad, kWsThreads, 0, s>>>(dj, B);
             k_ws_decide<<<1, 32, 0, s>>>(dj, B);
         } else {
@@ -1416,8 +1574,8 @@ static cudaError_t ws_carveout() {
     const void *ks[] = {(const void *)k_ws_start, (const void *)k_ws_end, (const void *)k_ws_finish,
                         (const void *)k_ws_free, (const void *)k_ws_cache,
                         (const void *)k_ws_pass, (const void *)k_ws_listimg<BF>, (const void *)k_ws_emb<BF>,
-                        (const void *)k_ws_fwd<BF>, (const void *)k_ws_fred, (const void *)k_ws_adj<BF, true>,
-                        (const void *)k_ws_adj<BF, false>, (const void *)k_ws_vx, (const void *)k_ws_feas,
+                        (const void *)k_ws_fwd<BF>, (const void *)k_ws_fred, (const void *)k_ws_lsqr<BF>, (const void *)k_ws_adj_list<BF>, (const void *)k_ws_vx,
+                        (const void *)k_ws_adj<BF>, (const void *)k_ws_feas,
                         (const void *)k_ws_accept, (const void *)k_ws_grad, (const void *)k_ws_decide,
                         (const void *)k_ws_step};
     for (const void *k : ks) {
@@ -1441,6 +1599,11 @@ cudaError_t ws_create(const JobDev &hj, const JobDev *dj, int mode, WsHost **out
     w->p = hj.p;
     w->cap = hj.cap;
     w->Q = hj.Q;
+    w->cluster = ws_clustered(w->g);
+    {
+        const int ntr = (hj.p + kRedTile - 1) / kRedTile;
+        w->g_red = std::min(ntr * ntr, kWsSums);
+    }
     {
         const char *env = getenv("IMG_SOLVE_GRAPH");
         w->direct = env && env[0] == '0';
@@ -1454,8 +1617,8 @@ cudaError_t ws_create(const JobDev &hj, const JobDev *dj, int mode, WsHost **out
     char *base = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(w->mem) + 1023) & ~uintptr_t(1023));
     ws_bytes(hj, sms, &w->B, base);
     e = w->bf16 ? ws_carveout<true>() : ws_carveout<false>();
-    if (e == cudaSuccess) e = set_smem(k_ws_adj<true, false>, items_smem_bytes());
-    if (e == cudaSuccess) e = set_smem(k_ws_adj<false, false>, items_smem_bytes());
+    if (e == cudaSuccess) e = set_smem(k_ws_adj<true>, items_smem_bytes());
+    if (e == cudaSuccess) e = set_smem(k_ws_adj<false>, items_smem_bytes());
     if (e != cudaSuccess) {
         ws_destroy(w);
         return e;
@@ -1466,10 +1629,12 @@ cudaError_t ws_create(const JobDev &hj, const JobDev *dj, int mode, WsHost **out
             // the attributes the graph build would set
             e = set_smem(k_ws_fwd<true>, items_fwd_smem_bytes());
             if (e == cudaSuccess) e = set_smem(k_ws_fwd<false>, items_fwd_smem_bytes());
-            if (e == cudaSuccess) e = set_smem(k_ws_adj<true, true>, items_smem_bytes());
-            if (e == cudaSuccess) e = set_smem(k_ws_adj<true, false>, items_smem_bytes());
-            if (e == cudaSuccess) e = set_smem(k_ws_adj<false, true>, items_smem_bytes());
-            if (e == cudaSuccess) e = set_smem(k_ws_adj<false, false>, items_smem_bytes());
+            if (e == cudaSuccess) e = set_smem(k_ws_lsqr<true>, items_smem_bytes());
+            if (e == cudaSuccess) e = set_smem(k_ws_adj_list<true>, items_smem_bytes());
+            if (e == cudaSuccess) e = set_smem(k_ws_adj<true>, items_smem_bytes());
+            if (e == cudaSuccess) e = set_smem(k_ws_lsqr<false>, items_smem_bytes());
+            if (e == cudaSuccess) e = set_smem(k_ws_adj_list<false>, items_smem_bytes());
+            if (e == cudaSuccess) e = set_smem(k_ws_adj<false>, items_smem_bytes());
         }
     } else {
         e = w->bf16 ? ws_capture<true>(w, dj, hj, sms) : ws_capture<false>(w, dj, hj, sms);
@@ -1496,10 +1661,10 @@ cudaError_t ws_bounds(WsHost *w, const JobDev &hj, cudaStream_t st) {
         k_ws_bnd_max<<<sms, kWsThreads, 0, st>>>(dj, B, U, k == 0, k);
         if (w->bf16) {
             k_ws_emb<true><<<sms, kWsThreads, 0, st>>>(dj, B, 0, U);
-            k_ws_adj<true, false><<<sms, kWideThreads, asm_, st>>>(dj, B);
+            k_ws_adj<true><<<sms, kWideThreads, asm_, st>>>(dj, B);
         } else {
             k_ws_emb<false><<<sms, kWsThreads, 0, st>>>(dj, B, 0, U);
-            k_ws_adj<false, false><<<sms, kWideThreads, asm_, st>>>(dj, B);
+            k_ws_adj<false><<<sms, kWideThreads, asm_, st>>>(dj, B);
         }
         k_ws_bnd_out<<<gq, kWsThreads, 0, st>>>(dj, B, k == 0 ? hj.dirty : hj.h);
     }
@@ -1517,10 +1682,10 @@ cudaError_t ws_psi_adj(WsHost *w, const JobDev &hj, const float2 *U, double *out
     k_ws_bnd_max<<<sms, kWsThreads, 0, st>>>(dj, B, U, 2, 0);
     if (w->bf16) {
         k_ws_emb<true><<<sms, kWsThreads, 0, st>>>(dj, B, 0, U);
-        k_ws_adj<true, false><<<sms, kWideThreads, asm_, st>>>(dj, B);
+        k_ws_adj<true><<<sms, kWideThreads, asm_, st>>>(dj, B);
     } else {
         k_ws_emb<false><<<sms, kWsThreads, 0, st>>>(dj, B, 0, U);
-        k_ws_adj<false, false><<<sms, kWideThreads, asm_, st>>>(dj, B);
+        k_ws_adj<false><<<sms, kWideThreads, asm_, st>>>(dj, B);
     }
     k_ws_adj_out<<<gq, kWsThreads, 0, st>>>(dj, B, out);
     k_ws_bnd_reset<<<1, 32, 0, st>>>(B);
