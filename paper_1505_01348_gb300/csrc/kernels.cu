@@ -977,12 +977,12 @@ __device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShare
 // the rounding does not depend on what the compiler contracts where.
 //
 // Bound by latency: a chain of small phases in one CTA, so what counts is
-// the barriers and the exposed scalars.  An iteration has 8 barriers (f <=
-// 64); the weighted rows of the forward are staged 64 at a time into the B
-// region, which is free until the B image of t is rebuilt; the norm of t and
-// its largest entry share a reduction, so that warp 0 forms beta while the
-// others build B; the rotation runs behind the issued MMAs, the stopping
-// tests behind the next iteration's staging.
+// the barriers and the exposed scalars (a dependent FP64 instruction takes 67
+// cycles, a division 550, hypot 1,050).  The weighted rows of the forward are
+// staged 64 at a time into the B region, which is free until the B image of
+// t is rebuilt; the norm of t and its largest entry share a reduction, so
+// that warp 0 forms beta and the rotation while the others build B and the
+// MMAs run; the stopping tests run behind the next iteration's staging.
 //
 // Forward: Kp = 64 as the Gram matrix of the tiles on tensor cores, Kp = 32
 // in FP32 from the free vectors themselves (shared memory), thread-owned
@@ -997,89 +997,50 @@ __host__ __device__ inline size_t res_extra_bytes(int p) {
     return ((p + 31) / 32 * 32 == 32 ? (size_t)kResF * p * sizeof(float2) : 1024) + kResF * sizeof(float);
 }
 
-// The split B image of the matrix whose entries e = tid + 256 k (e = n p + a:
-// row a, column n) are tr[k]: entry (a, n) appears at (n, a) and (Kp + n, Kp +
-// a) as Re, at (n, Kp + a) as Im, at (Kp + n, a) as -Im.  Even p: neighbouring
-// lanes hold a and a + 1 and share the work, the even lane writing the Re
-// pairs, the odd lane the Im pairs.
+// Named barriers of the resident LSQR (0 is __syncthreads).
+__device__ __forceinline__ void bar_sync(int id, int n) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int n) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
+// The split B image of t, which lies (p x p, column-major) at the start of the
+// B region itself: each of warps 1 .. 7 takes its chunks of t to registers
+// before any of them writes.  As tc_build_B, scaled by sc.
 template <bool BF16>
-__device__ __forceinline__ void res_build_B(const TcWork &T, int p, const float2 *tr, float sc) {
-    const int Kp = T.Kp, N = 2 * Kp, nc8 = Kp / 8, pp = p * p;
-    const bool even = (p & 1) == 0;
-    const bool odd_lane = threadIdx.x & 1;
-    unsigned char *bh = T.Bhi(), *bl = T.Blo();
-    // padding: whole 16-byte chunks
-    if (p < Kp) {
-        const int live = (p + 7) / 8;
-        for (int it = threadIdx.x; it < N * 2 * nc8; it += kThreads) {
-            const int n = it / (2 * nc8), c = it - n * (2 * nc8);
-            if ((n >= Kp ? n - Kp : n) >= p || (c >= nc8 ? c - nc8 : c) >= live) {
-                const uint32_t off = sw128_off(n, c, N);
-                *reinterpret_cast<uint4 *>(bh + off) = make_uint4(0u, 0u, 0u, 0u);
-                *reinterpret_cast<uint4 *>(bl + off) = make_uint4(0u, 0u, 0u, 0u);
-            }
-        }
-    }
-    const int da = kThreads % p, dn = kThreads / p;
-    int a = threadIdx.x % p, n = threadIdx.x / p;
+__device__ __forceinline__ void res_build_B(const TcWork &T, int p, float sc) {
+    constexpr int kNt = kThreads - 32, kMax = 3;             // 64 x 8 chunks over 224 threads
+    const int Kp = T.Kp, N = 2 * Kp, nc8 = Kp / 8, items = Kp * nc8;
+    const float2 *t = reinterpret_cast<const float2 *>(T.Bhi());
+    const int tid = threadIdx.x - 32;
+    const bool vec = (p & 1) == 0;
+    float2 v[kMax][8];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        if (k * kThreads >= pp) break;
-        const bool ok = threadIdx.x + k * kThreads < pp;
-        const float2 t = tr[k];
-        const float other = __shfl_xor_sync(0xffffffffu, odd_lane ? t.x : t.y, 1);
-        if (ok) {
-            if (even) {
-                const int a0 = a & ~1, c8 = a0 >> 3, ao = (a0 & 7) * 2;
-                uint32_t hi, lo;
-                auto put = [&](int row, int ch) {
-                    const uint32_t off = sw128_off(row, ch, N) + ao;
-                    *reinterpret_cast<uint32_t *>(bh + off) = hi;
-                    *reinterpret_cast<uint32_t *>(bl + off) = lo;
-                    // the rest of the last live chunk is padding
-                    if (a0 + 2 == p)
-                        for (int q = ao + 4; q < 16; q += 4) {
-                            *reinterpret_cast<uint32_t *>(bh + off - ao + q) = 0u;
-                            *reinterpret_cast<uint32_t *>(bl + off - ao + q) = 0u;
-                        }
-                };
-                if (!odd_lane) {
-                    split2<BF16>(t.x * sc, other * sc, hi, lo);
-                    put(n, c8);
-                    put(Kp + n, nc8 + c8);
-                } else {
-                    split2<BF16>(other * sc, t.y * sc, hi, lo);
-                    put(n, nc8 + c8);
-                    split2<BF16>(-other * sc, -t.y * sc, hi, lo);
-                    put(Kp + n, c8);
-                }
-            } else {
-                const int c8 = a >> 3, ao = (a & 7) * 2;
-                auto put = [&](int row, int ch, float v) {
-                    uint32_t hi, lo;
-                    split2<BF16>(v, 0.f, hi, lo);
-                    const uint32_t off = sw128_off(row, ch, N) + ao;
-                    *reinterpret_cast<uint16_t *>(bh + off) = (uint16_t)hi;
-                    *reinterpret_cast<uint16_t *>(bl + off) = (uint16_t)lo;
-                    if (a + 1 == p)
-                        for (int q = ao + 2; q < 16; q += 2) {
-                            *reinterpret_cast<uint16_t *>(bh + off - ao + q) = 0;
-                            *reinterpret_cast<uint16_t *>(bl + off - ao + q) = 0;
-                        }
-                };
-                put(n, c8, t.x * sc);
-                put(Kp + n, nc8 + c8, t.x * sc);
-                put(n, nc8 + c8, t.y * sc);
-                put(Kp + n, c8, -t.y * sc);
+    for (int q = 0; q < kMax; ++q) {
+        const int it = tid + q * kNt, n = it / nc8, k0 = (it - n * nc8) * 8;
+        const float2 *src = t + n * p + k0;
+        if (vec && n < p && k0 + 8 <= p) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float4 x = reinterpret_cast<const float4 *>(src)[e];
+                v[q][2 * e] = make_float2(x.x, x.y);
+                v[q][2 * e + 1] = make_float2(x.z, x.w);
             }
-        }
-        a += da;
-        n += dn;
-        if (a >= p) {
-            a -= p;
-            ++n;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[q][e] = n < p && k0 + e < p ? src[e] : make_float2(0.f, 0.f);
         }
     }
+    bar_sync(2, kNt);
+#pragma unroll
+    for (int q = 0; q < kMax; ++q) {
+        const int it = tid + q * kNt, n = it / nc8, c8 = it - n * nc8;
+        if (it >= items) break;
+        tc_put_B<BF16>(T, n, c8, v[q], sc);
+    }
+    fence_async_smem();
+    bar_sync(2, kNt);
 }
 
 // Rows r0 .. r0 + nst - 1 of the resident tiles times sW w[row] (zero from
@@ -1151,8 +1112,9 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
         acc = fmaf(tr[k].x, tr[k].x, fmaf(tr[k].y, tr[k].y, acc));
         mx = fmaxf(mx, fmaxf(fabsf(tr[k].x), fabsf(tr[k].y)));
     }
-    // CTA sum (FP64, warp 0) and maximum (every thread) after one barrier
-    auto reduce = [&](float sum, float m) -> double {
+    // CTA sum (FP64, for cta_sum in warp 0) and maximum (for cta_max), up to
+    // and including their barrier
+    auto reduce = [&](float sum, float m) {
         double d = (double)sum;
         for (int o = 16; o; o >>= 1) {
             d += __shfl_xor_sync(0xffffffffu, d, o);
@@ -1163,10 +1125,11 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
             S.fm[warp] = m;
         }
         __syncthreads();
+    };
+    auto cta_sum = [&]() {
         double t = 0.0;
-        if (w0)
 #pragma unroll
-            for (int q = 0; q < kThreads / 32; ++q) t += S.dbuf[q];
+        for (int q = 0; q < kThreads / 32; ++q) t += S.dbuf[q];
         return t;
     };
     auto cta_max = [&]() {
@@ -1177,22 +1140,27 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
     };
     auto pow2_of = [](float m) { return m > 0.f ? exp2f(-ceilf(log2f(m))) : 1.f; };
     // scalars of the recurrence, valid in warp 0
-    double alpha = 0.0, beta = 0.0, bnorm = 0.0, us = 0.0, phibar = 0.0, rhobar = 0.0, anorm2 = 0.0, absc = 0.0;
+    double alpha = 0.0, beta = 0.0, bnorm = 0.0, us = 0.0, phibar = 0.0, rhobar = 0.0, anorm2 = 0.0;
     double rho = 0.0, cs = 0.0, sn = 0.0, phi = 0.0;
-    // y_j = Re(c_j^H t c_j) (scaled back), thread j; warp 0 runs `behind`
-    // while the MMAs of the first tile are in flight
+    // y_j = Re(c_j^H t c_j) (scaled back), thread j.  Warps 1 .. 7 build the B
+    // image of t and issue the MMAs while warp 0 runs scalars().
     const uint32_t idesc = idesc_f16(N, BF ? 1 : 0);
-    auto adjoint = [&](auto behind) -> float {
+    auto adjoint = [&](auto scalars) -> float {
         const long long c0 = clock64();
         const float sB = pow2_of(cta_max()) * kLift;
-        res_build_B<BF>(T, p, tr, sB);
-        fence_async_smem();
-        __syncthreads();
+        float2 *ts = reinterpret_cast<float2 *>(T.Bhi());
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            if (threadIdx.x + k * kThreads < pp) ts[threadIdx.x + k * kThreads] = tr[k];
         if (w0) {
-            if (lane == 0)
+            bar_arrive(1, kThreads);
+            scalars();
+        } else {
+            bar_sync(1, kThreads);
+            res_build_B<BF>(T, p, sB);
+            if (threadIdx.x == 32)
                 for (int t = 0; t < ntiles; ++t) tc_issue(T, t, idesc);
             __syncwarp();
-            behind();
         }
         const long long c1 = clock64();
         for (int t = 0; t < ntiles; ++t) {
@@ -1218,36 +1186,30 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
         __syncthreads();
         return its;
     };
+    reduce(acc, mx);
     {
-        const double ss = reduce(acc, mx);
-        if (w0) {
-            beta = bnorm = phibar = sqrt(ss);
+        const float y = adjoint([&]() {
+            beta = bnorm = phibar = sqrt(cta_sum());
             us = 1.0 / beta;
             S.ls[2] = (float)us;
             S.lsi = beta == 0.0;
-        }
-    }
-    {
-        const float y = adjoint([]() {});
+        });
         if (S.lsi) return leave(0);
         if (mine) v = sF * (y * S.ls[2]);
     }
-    {
-        const double ss = reduce(fmaf(v, v, 0.f), 0.f);
-        if (w0) {
-            alpha = rhobar = sqrt(ss);
-            S.ls[5] = (float)(1.0 / alpha);
-            S.ls[0] = (float)(alpha * us);
-            S.lsi = alpha == 0.0;
-        }
-        __syncthreads();
-        if (S.lsi) return leave(0);
-        v *= S.ls[5];
-        w = v;
-        const float wj = sF * v;
-        wt[j] = wj;
-        reduce(0.f, fabsf(wj));
+    reduce(fmaf(v, v, 0.f), 0.f);
+    if (w0) {
+        alpha = rhobar = sqrt(cta_sum());
+        S.ls[5] = (float)(1.0 / alpha);
+        S.ls[0] = (float)(alpha * us);
+        S.lsi = alpha == 0.0;
     }
+    __syncthreads();
+    if (S.lsi) return leave(0);
+    v *= S.ls[5];
+    w = v;
+    wt[j] = sF * v;
+    reduce(0.f, fabsf(sF * v));
     const int maxit = J.lsqr_maxit > 0 ? J.lsqr_maxit : 4 * f + 20;
     const double atol = J.lsqr_atol, btol = J.lsqr_btol;
     const uint32_t fdesc = idesc_f16_mn(N, BF ? 1 : 0);
@@ -1317,68 +1279,72 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
         {
             int a = a_first, n = n_first;
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                if (k * kThreads >= pp) break;
-                if (threadIdx.x + k * kThreads < pp) {
-                    float2 kv;
+            for (int k0 = 0; k0 < 16; k0 += 4) {
+                if (k0 * kThreads >= pp) break;
+                // four entries at a time, their reads in flight together
+                float2 kv[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const bool in = threadIdx.x + (k0 + q) * kThreads < pp;
+                    kv[q] = make_float2(0.f, 0.f);
                     if (gram) {
-                        kv = tc_k_entry(G, Kp, a, n);
-                        kv = make_float2(__fmaf_rn(kv.x, inv, -__fmul_rn(fa, tr[k].x)),
-                                         __fmaf_rn(kv.y, inv, -__fmul_rn(fa, tr[k].y)));
-                    } else {
-                        float2 s = make_float2(0.f, 0.f);
+                        if (in) kv[q] = tc_k_entry(G, Kp, a, n);
+                    } else if (in) {
                         const float2 *ca = C + a, *cn = C + n;
 #pragma unroll 4
-                        for (int q = 0; q < f; ++q) {
-                            const float wq = wt[q];
-                            const float2 u = ca[q * p], z = cn[q * p];
-                            cfma(s, make_float2(wq * u.x, wq * u.y), make_float2(z.x, -z.y));
+                        for (int r = 0; r < f; ++r) {
+                            const float wq = wt[r];
+                            const float2 u = ca[r * p], z = cn[r * p];
+                            cfma(kv[q], make_float2(wq * u.x, wq * u.y), make_float2(z.x, -z.y));
                         }
-                        kv = make_float2(__fmaf_rn(-fa, tr[k].x, 0.f + s.x), __fmaf_rn(-fa, tr[k].y, 0.f + s.y));
                     }
-                    tr[k] = kv;
-                    acc = fmaf(kv.x, kv.x, fmaf(kv.y, kv.y, acc));
-                    mx = fmaxf(mx, fmaxf(fabsf(kv.x), fabsf(kv.y)));
+                    a += da;
+                    n += dn;
+                    if (a >= p) {
+                        a -= p;
+                        ++n;
+                    }
                 }
-                a += da;
-                n += dn;
-                if (a >= p) {
-                    a -= p;
-                    ++n;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    float2 &t = tr[k0 + q];
+                    if (gram)
+                        t = make_float2(__fmaf_rn(kv[q].x, inv, -__fmul_rn(fa, t.x)),
+                                        __fmaf_rn(kv[q].y, inv, -__fmul_rn(fa, t.y)));
+                    else
+                        t = make_float2(__fmaf_rn(-fa, t.x, 0.f + kv[q].x), __fmaf_rn(-fa, t.y, 0.f + kv[q].y));
+                    acc = fmaf(t.x, t.x, fmaf(t.y, t.y, acc));
+                    mx = fmaxf(mx, fmaxf(fabsf(t.x), fabsf(t.y)));
                 }
             }
         }
-        double ss = reduce(acc, mx);
-        if (w0) {
-            beta = sqrt(ss);
-            us = beta > 0.0 ? 1.0 / beta : 0.0;
-            anorm2 += alpha * alpha + beta * beta;
-            S.ls[1] = (float)beta;
-            S.ls[2] = (float)us;
-        }
+        reduce(acc, mx);
         const long long c3 = clock64();
         cyc.aux[2] += c3 - c2;
         cyc.fwd += c3 - c0;
         // v <- M^H u - beta v
         const float y = adjoint([&]() {
+            beta = sqrt(cta_sum());
+            us = beta > 0.0 ? 1.0 / beta : 0.0;
+            S.ls[1] = (float)beta;
+            S.ls[2] = (float)us;
+            anorm2 += alpha * alpha + beta * beta;
             // the rotation's part that does not need alpha; lanes 0, 1: c, s
             rho = hypot(rhobar, beta);
             const double q = (lane == 0 ? rhobar : beta) / rho;
-            const double c = __shfl_sync(0xffffffffu, q, 0);
+            cs = __shfl_sync(0xffffffffu, q, 0);
             sn = __shfl_sync(0xffffffffu, q, 1);
-            phi = c * phibar;
+            phi = cs * phibar;
             phibar = sn * phibar;
-            cs = c;
         });
         if (mine) v = __fmaf_rn(sF, __fmul_rn(y, S.ls[2]), -__fmul_rn(S.ls[1], v));
         cyc.adj += clock64() - c3;
-        ss = reduce(mine ? fmaf(v, v, 0.f) : 0.f, 0.f);
+        reduce(mine ? fmaf(v, v, 0.f) : 0.f, 0.f);
         if (w0) {
             // lanes 0..2: the coefficients of x and w, 1/alpha
-            alpha = sqrt(ss);
+            alpha = sqrt(cta_sum());
             const double theta = sn * alpha;
             rhobar = -cs * alpha;
-            absc = fabs(cs);
             const double q = (lane == 0 ? phi : lane == 1 ? -theta : 1.0) / (lane == 2 ? alpha : rho);
             if (lane < 2) S.ls[3 + lane] = (float)q;
             if (lane == 2) S.ls[5] = alpha > 0.0 ? (float)q : 1.f;
@@ -1398,12 +1364,13 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
             wt[j] = wj;
             mx = fabsf(wj);
         }
-        ss = reduce(acc, mx);
+        reduce(acc, mx);
         if (w0) {
+            const double ss = cta_sum();
             const double q = sqrt(lane == 0 ? ss : anorm2);
             const double xnorm = __shfl_sync(0xffffffffu, q, 0), anorm = __shfl_sync(0xffffffffu, q, 1);
             const double rnorm = phibar;
-            const double arnorm = phibar * alpha * absc;
+            const double arnorm = phibar * alpha * fabs(cs);
             S.lsi = rnorm <= btol * bnorm + atol * anorm * xnorm || arnorm <= atol * anorm * rnorm;
             S.ls[0] = (float)(alpha * us);
         }

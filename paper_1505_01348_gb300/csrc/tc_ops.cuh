@@ -287,6 +287,34 @@ __device__ inline void tc_teardown(TcWork &T, int p) {
 // the lift is harmless there.)
 constexpr float kLift = 8192.f;
 
+// The four blocks of B that the entries u[e] = U(8 c8 + e, n) = conj(V(n, k))
+// make, V = U^H: Re V = u.x at (n, k) and (Kp+n, Kp+k), -Im V = u.y at (n, Kp+k),
+// Im V at (Kp+n, k); scaled by sc and split.
+template <bool BF16>
+__device__ __forceinline__ void tc_put_B(const TcWork &T, int n, int c8, const float2 *u, float sc) {
+    const int Kp = T.Kp, N = 2 * Kp, nc8 = Kp / 8;
+    float re[8], nim[8], im[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        re[e] = u[e].x * sc;
+        im[e] = -u[e].y * sc;
+        nim[e] = u[e].y * sc;
+    }
+    auto put = [&](int row, int c, const uint4 &hi, const uint4 &lo) {
+        const uint32_t off = sw128_off(row, c, N);
+        *reinterpret_cast<uint4 *>(T.Bhi() + off) = hi;
+        *reinterpret_cast<uint4 *>(T.Blo() + off) = lo;
+    };
+    uint4 hi, lo;
+    split8<BF16>(re, hi, lo);
+    put(n, c8, hi, lo);
+    put(Kp + n, nc8 + c8, hi, lo);
+    split8<BF16>(nim, hi, lo);
+    put(n, nc8 + c8, hi, lo);
+    split8<BF16>(im, hi, lo);
+    put(Kp + n, c8, hi, lo);
+}
+
 // B = real embedding of U, scaled by a power of two to max |entry| <= 1,
 // lifted by kLift and split into hi/lo 16-bit tiles.  Row n of B^T (N index) holds, for
 // n < p: [Re V(n,:), -Im V(n,:)], for Kp <= n < Kp+p: [Im V(n,:), Re V(n,:)]
@@ -295,7 +323,7 @@ constexpr float kLift = 8192.f;
 // column chunks of U in registers while the CTA finds the scale.
 template <bool BF16>
 __device__ float tc_build_B(const float2 *U, int p, TcWork &T, double *sbuf) {
-    const int Kp = T.Kp, N = 2 * Kp, nc8 = Kp / 8;
+    const int Kp = T.Kp, nc8 = Kp / 8;
     constexpr int kMaxItems = 4;          // (Kp/8) * Kp / kThreads <= 4 for Kp <= 128
     const int items = Kp * nc8;           // (row n < Kp, chunk of 8 columns)
     float2 v[kMaxItems][8];
@@ -332,30 +360,7 @@ __device__ float tc_build_B(const float2 *U, int p, TcWork &T, double *sbuf) {
         const int it = threadIdx.x + q * kThreads;
         if (it >= items) break;
         const int n = it / nc8, c8 = it - n * nc8;
-        // u = U(k, n) = conj(V(n, k)):  Re V = u.x, Im V = -u.y
-        float re[8], nim[8], im[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            re[e] = v[q][e].x * sc;
-            im[e] = -v[q][e].y * sc;
-            nim[e] = v[q][e].y * sc;
-        }
-        uint4 hi, lo;
-        split8<BF16>(re, hi, lo);                       // (re row, re col): Re V
-        uint32_t off = sw128_off(n, c8, N);
-        *reinterpret_cast<uint4 *>(T.Bhi() + off) = hi;
-        *reinterpret_cast<uint4 *>(T.Blo() + off) = lo;
-        off = sw128_off(Kp + n, nc8 + c8, N);           // (im row, im col): Re V
-        *reinterpret_cast<uint4 *>(T.Bhi() + off) = hi;
-        *reinterpret_cast<uint4 *>(T.Blo() + off) = lo;
-        split8<BF16>(nim, hi, lo);                      // (re row, im col): -Im V
-        off = sw128_off(n, nc8 + c8, N);
-        *reinterpret_cast<uint4 *>(T.Bhi() + off) = hi;
-        *reinterpret_cast<uint4 *>(T.Blo() + off) = lo;
-        split8<BF16>(im, hi, lo);                       // (im row, re col): Im V
-        off = sw128_off(Kp + n, c8, N);
-        *reinterpret_cast<uint4 *>(T.Bhi() + off) = hi;
-        *reinterpret_cast<uint4 *>(T.Blo() + off) = lo;
+        tc_put_B<BF16>(T, n, c8, v[q], sc);
     }
     return sc;
 }
