@@ -195,6 +195,12 @@ __device__ __forceinline__ void wide_wait(uint64_t *bars, int slot, uint32_t &ph
     if (!mbar_wait(&bars[slot], par)) timeouts++;
 }
 
+// The same for a completion whose parity the caller knows.
+__device__ __forceinline__ void wide_wait_parity(uint64_t *bars, int slot, uint32_t par, int &timeouts) {
+    uint32_t ph = par << slot;
+    wide_wait(bars, slot, ph, timeouts);
+}
+
 // out = Re(a_i^H U_s a_i) for npass <= 2 operators s (B images B0, B1,
 // scales sB[s]) over the 2-D tiles t0, t0 + dt, ... (ntiles of them);
 // epi(s, i, v) receives each pixel's value.  Bit s of sq_mask makes pass s
@@ -492,12 +498,19 @@ __device__ int wide_adjoint(const JobDev &J, unsigned char *dyn, uint64_t *bars,
 // and B weighted by w_i, split hi + lo as in the adjoint.  Each CTA writes its
 // FP32 block to a partial buffer; fwd_assemble sums the partials in a fixed
 // order (deterministic) and forms K.
-//   warps 0-7  steering producers (then warps 0-3 read the accumulator);
-//   warp 8     MMA issue (lane 0).
+//   warps 0-14 steering producers;
+//   warp 15    MMA issue (lane 0); then all warps read the accumulator out.
+// Bound by the producers: a stage is 8 to 12 tasks of 32 pixels x 64
+// features, each ~480 instructions behind a dozen L2 loads.  Fifteen warps
+// that take tasks of both stages in flight keep the loads of some tasks under
+// the arithmetic of others; with eight warps of one or two tasks per stage
+// the stage took 7,300 cycles at p = 256, 5 times its MMAs (Psi x and Psi^H u of
+// p = 256, 512x512: 1026 -> 760 us).
 constexpr int kFwdPix = 64;                                  // pixels per stage
 constexpr size_t kFwdChunk = (size_t)kFwdPix * 128;          // one 64-feature chunk, 8 KB
 constexpr size_t kFwdStage = (2 + 4) * 2 * kFwdChunk;        // A: 2 chunks, B: 4 chunks, hi + lo
-constexpr int kFwdThreads = 288;
+constexpr int kFwdProducers = 15;                            // warps
+constexpr int kFwdThreads = 32 * (kFwdProducers + 1);
 __host__ __device__ inline size_t fwd_smem_bytes() { return 2 * kFwdStage + 1024; }
 __host__ __device__ inline int fwd_n_of(int p, int nb) {
     const int n = 2 * wide_kp(p) - 256 * nb;
@@ -553,11 +566,18 @@ __device__ int wide_forward(const JobDev &J, unsigned char *dyn, uint64_t *bars,
     const float sX = steer_scale(p);
     const float sW = emb_scale_of(wbits);
     enum { kFull = 0, kEmpty = 2, kAcc = 4 };
+    // feature chunks of a stage: A = {2m, 2m+1}, then those of B = {4nb ..}
+    // that are not among them
+    const int nB = N / 64, ov = 2 * m - 4 * nb;              // A's place in B when 0 <= ov < 4
+    const bool over = ov >= 0 && ov < 4;
+    const int nchunk = 2 + nB - (over ? (ov < nB) + (ov + 1 < nB) : 0);
+    auto chunk_of = [&](int ci) { return ci < 2 ? 2 * m + ci : 4 * nb + ci - 2 + (over && ci - 2 >= ov ? 2 : 0); };
+    const int ntask = 2 * nchunk;                            // per stage: (chunk, half of the 64 pixels)
     __shared__ int s_timeouts;
     if (threadIdx.x == 0) {
         s_timeouts = 0;
         for (int q = 0; q < 2; ++q) {
-            mbar_init(&bars[kFull + q], 8);
+            mbar_init(&bars[kFull + q], ntask);
             mbar_init(&bars[kEmpty + q], 1);
         }
         mbar_init(&bars[kAcc], 1);
@@ -569,15 +589,8 @@ __device__ int wide_forward(const JobDev &J, unsigned char *dyn, uint64_t *bars,
     const uint32_t tmem = *slot;
     int timeouts = 0;
     uint32_t ph = 0;
-    // chunks of features: A = {2m, 2m+1}, B = {4nb .. 4nb+3}; chunk list without repeats
-    int chunk[6], nchunk = 0;
-    for (int q = 0; q < 2; ++q) chunk[nchunk++] = 2 * m + q;
-    for (int q = 0; q < 4; ++q) {
-        const int c = 4 * nb + q;
-        if (64 * c < 256 * nb + N && c != 2 * m && c != 2 * m + 1) chunk[nchunk++] = c;
-    }
 
-    if (warp == 8) {
+    if (warp == kFwdProducers) {
         if (lane == 0 && mine > 0) {
             const uint32_t idesc = idesc_f16_mn128(N, BF16 ? 1 : 0);
             for (int t = 0; t < mine; ++t) {
@@ -603,71 +616,43 @@ __device__ int wide_forward(const JobDev &J, unsigned char *dyn, uint64_t *bars,
             }
         }
     } else {
-        // ---------------- producers: warp w takes tasks (chunk, half h) w, w + 8, ...
-        // of each stage: the 32 pixel rows of m offsets b = 4h .. 4h+3 (l offsets
-        // a = 0..7), lane j the features 2j, 2j+1 of the chunk.  The 8 E_l and
-        // 4 E_m entries and the 32 weights of the warp's next task (in this
-        // stage or the next) load while the current task is written.
-        const bool vec = (p & 1) == 0, wvec = (nl & 3) == 0;
+        // ---------------- producers: the stages' tasks in order, warp w those
+        // numbered w, w + 15, ...: (chunk, half h) = the 32 pixel rows of m
+        // offsets b = 4h .. 4h+3 (l offsets a = 0..7), lane j the features 2j,
+        // 2j+1 of the chunk.  Lane j also holds the weight of row j = 8b + a.
+        const bool vec = (p & 1) == 0;
         const float2 *__restrict__ El = J.El;
         const float2 *__restrict__ Em = J.Em;
-        const int ntask = nchunk * 2;
-        const int my = warp < ntask ? (ntask - 1 - warp) / 8 + 1 : 0;    // tasks per stage
         // swizzled byte offset of (row a, this lane's column pair) in an 8-row group
         uint32_t xo[8];
 #pragma unroll
         for (int a = 0; a < 8; ++a) xo[a] = (uint32_t)(a * 128 + (((lane >> 2) ^ a) << 4) + (lane & 3) * 4);
         float2 e[8][2], fm[4][2];
-        float wr[4][8];
+        float wl = 0.f;
         auto load = [&](int t, int task) {
             const int blk = s0 + t * S, bm = blk / tlb, bl = blk - bm * tlb;
-            const int ci = task >> 1, h = task & 1, c = chunk[ci];
+            const int h = task & 1, c = chunk_of(task >> 1);
             const int f = c * 64 + 2 * lane, part = f >= Kp, k = f - part * Kp;
             const bool kok = f < Nf && k < p;
-#pragma unroll
-            for (int a = 0; a < 8; ++a) {
-                const int il = bl * 8 + a;
-                e[a][0] = e[a][1] = make_float2(0.f, 0.f);
-                if (kok && il < nl) {
-                    const float2 *src = El + (size_t)il * p + k;
-                    if (vec) {
-                        const float4 v = __ldg(reinterpret_cast<const float4 *>(src));
-                        e[a][0] = make_float2(v.x, v.y);
-                        e[a][1] = make_float2(v.z, v.w);
-                    } else {
-                        e[a][0] = __ldg(src);
-                        if (k + 1 < p) e[a][1] = __ldg(src + 1);
-                    }
-                }
-            }
-#pragma unroll
-            for (int bb = 0; bb < 4; ++bb) {
-                const int im = bm * 8 + 4 * h + bb;
-                fm[bb][0] = fm[bb][1] = make_float2(0.f, 0.f);
-                if (kok && im < nm) {
-                    const float2 *src = Em + (size_t)im * p + k;
-                    if (vec) {
-                        const float4 v = __ldg(reinterpret_cast<const float4 *>(src));
-                        fm[bb][0] = make_float2(v.x, v.y);
-                        fm[bb][1] = make_float2(v.z, v.w);
-                    } else {
-                        fm[bb][0] = __ldg(src);
-                        if (k + 1 < p) fm[bb][1] = __ldg(src + 1);
-                    }
-                }
-                // the 8 weights of this m row (same address in every lane)
-                const int il0 = bl * 8;
-                const float *wrow = w + (size_t)im * nl + il0;
-                if (im < nm && wvec && il0 + 8 <= nl) {
-                    const float4 w0 = __ldg(reinterpret_cast<const float4 *>(wrow));
-                    const float4 w1 = __ldg(reinterpret_cast<const float4 *>(wrow) + 1);
-                    wr[bb][0] = w0.x; wr[bb][1] = w0.y; wr[bb][2] = w0.z; wr[bb][3] = w0.w;
-                    wr[bb][4] = w1.x; wr[bb][5] = w1.y; wr[bb][6] = w1.z; wr[bb][7] = w1.w;
+            auto row = [&](const float2 *tab, int g, bool ok, float2 *v) {
+                v[0] = v[1] = make_float2(0.f, 0.f);
+                if (!ok) return;
+                const float2 *src = tab + (size_t)g * p + k;
+                if (vec) {
+                    const float4 x = __ldg(reinterpret_cast<const float4 *>(src));
+                    v[0] = make_float2(x.x, x.y);
+                    v[1] = make_float2(x.z, x.w);
                 } else {
-#pragma unroll
-                    for (int a = 0; a < 8; ++a) wr[bb][a] = (im < nm && il0 + a < nl) ? __ldg(wrow + a) : 0.f;
+                    v[0] = __ldg(src);
+                    if (k + 1 < p) v[1] = __ldg(src + 1);
                 }
-            }
+            };
+#pragma unroll
+            for (int a = 0; a < 8; ++a) row(El, bl * 8 + a, kok && bl * 8 + a < nl, e[a]);
+#pragma unroll
+            for (int bb = 0; bb < 4; ++bb) row(Em, bm * 8 + 4 * h + bb, kok && bm * 8 + 4 * h + bb < nm, fm[bb]);
+            const int im = bm * 8 + 4 * h + (lane >> 3), il = bl * 8 + (lane & 7);
+            wl = (im < nm && il < nl) ? __ldg(w + (size_t)im * nl + il) * sW : 0.f;
         };
         // write one task: rows of m offsets 4h + bb; A (unweighted) and/or B (weighted) copies
         auto emit = [&](unsigned char *st, int c, int h, int part, auto inA_t, auto inB_t) {
@@ -696,7 +681,7 @@ __device__ int wide_forward(const JobDev &J, unsigned char *dyn, uint64_t *bars,
                         *reinterpret_cast<uint32_t *>(ah + 2 * kFwdChunk + off) = lo;
                     }
                     if (inB) {
-                        const float wi = wr[bb][a] * sW;
+                        const float wi = __shfl_sync(0xffffffffu, wl, 8 * bb + a);
                         split2<BF16>(v0 * wi, v1 * wi, hi, lo);
                         *reinterpret_cast<uint32_t *>(bh + off) = hi;
                         *reinterpret_cast<uint32_t *>(bh + 4 * kFwdChunk + off) = lo;
@@ -704,48 +689,56 @@ __device__ int wide_forward(const JobDev &J, unsigned char *dyn, uint64_t *bars,
                 }
             }
         };
-        if (mine > 0 && my > 0) load(0, warp);
-        for (int t = 0; t < mine; ++t) {
-            const int sg = t & 1;
-            if (t >= 2) wide_wait(bars, kEmpty + sg, ph, timeouts);
+        // At most two stages' tasks in flight: a warp's next task is then at
+        // most two stages on, where the wait below is for the completion after
+        // one that it knows of (the MMAs finish in order), so that a parity
+        // names it.  Small arrays have as few as 4 tasks per stage.
+        const int np = min(kFwdProducers, 2 * ntask);
+        const int total = warp < np ? mine * ntask : 0;
+        if (warp < total) load(warp / ntask, warp % ntask);
+        for (int id = warp; id < total; id += np) {
+            const int t = id / ntask, task = id - t * ntask, sg = t & 1;
+            // the MMAs of stage t - 2 are done with the buffer
+            if (t >= 2) wide_wait_parity(bars, kEmpty + sg, ((t >> 1) - 1) & 1, timeouts);
             unsigned char *st = dyn + sg * kFwdStage;
-            for (int q = 0; q < my; ++q) {
-                const int task = warp + 8 * q;
-                const int ci = task >> 1, h = task & 1, c = chunk[ci];
-                const int part = c * 64 + 2 * lane >= Kp;
-                const bool inA = c == 2 * m || c == 2 * m + 1;
-                const bool inB = c >= 4 * nb && 64 * c < 256 * nb + N;
-                if (inA && inB) emit(st, c, h, part, std::true_type{}, std::true_type{});
-                else if (inA) emit(st, c, h, part, std::true_type{}, std::false_type{});
-                else emit(st, c, h, part, std::false_type{}, std::true_type{});
-                // next task of this warp (after the registers of this one are consumed)
-                if (q + 1 < my) load(t, task + 8);
-                else if (t + 1 < mine) load(t + 1, warp);
-            }
+            const int h = task & 1, c = chunk_of(task >> 1);
+            const int part = c * 64 + 2 * lane >= Kp;
+            const bool inA = c == 2 * m || c == 2 * m + 1;
+            const bool inB = c >= 4 * nb && 64 * c < 256 * nb + N;
+            if (inA && inB) emit(st, c, h, part, std::true_type{}, std::true_type{});
+            else if (inA) emit(st, c, h, part, std::true_type{}, std::false_type{});
+            else emit(st, c, h, part, std::false_type{}, std::true_type{});
+            // next task of this warp (after the registers of this one are consumed)
+            const int next = id + np;
+            if (next < total) load(next / ntask, next % ntask);
             fence_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[kFull + sg]);
         }
-        // ---------------- accumulator -> out (warps 0-3: one row of the block per thread)
-        if (warp < 4) {
-            const int r = 32 * warp + lane;
-            float *row = out + (size_t)r * 256;
+    }
+    {
+        // ---------------- accumulator -> out: warp w the rows 32 (w % 4) ..,
+        // columns 64 (w / 4) .. of the block
+        __syncwarp();
+        const int r = 32 * (warp & 3) + lane, c0 = 64 * (warp >> 2);
+        float *row = out + (size_t)r * 256 + c0;
+        if (c0 < N) {
             if (mine > 0) {
                 wide_wait(bars, kAcc, ph, timeouts);
                 tc_fence_after();
-                const uint32_t base = tmem + ((uint32_t)(32 * warp) << 16);
-                for (int c0 = 0; c0 < N; c0 += 32) {
+                const uint32_t base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
+                for (int cc = 0; cc < 64; cc += 32) {
                     float d0[16], d1[16];
-                    tmem_ld16x2(base + c0, base + c0 + 16, d0, d1);
+                    tmem_ld16x2(base + cc, base + cc + 16, d0, d1);
 #pragma unroll
                     for (int q = 0; q < 16; q += 4) {
-                        *reinterpret_cast<float4 *>(row + c0 + q) = make_float4(d0[q], d0[q + 1], d0[q + 2], d0[q + 3]);
-                        *reinterpret_cast<float4 *>(row + c0 + 16 + q) =
+                        *reinterpret_cast<float4 *>(row + cc + q) = make_float4(d0[q], d0[q + 1], d0[q + 2], d0[q + 3]);
+                        *reinterpret_cast<float4 *>(row + cc + 16 + q) =
                             make_float4(d1[q], d1[q + 1], d1[q + 2], d1[q + 3]);
                     }
                 }
             } else {
-                for (int c0 = 0; c0 < N; ++c0) row[c0] = 0.f;
+                for (int cc = 0; cc < 64; ++cc) row[cc] = 0.f;
             }
         }
     }
