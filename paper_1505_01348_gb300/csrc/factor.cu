@@ -48,7 +48,6 @@ __global__ void k_fac_init(JobDev *const *jobs) {
     if (blockIdx.y == 0 && threadIdx.x == 0) {
         J.flags[3] = 0;                              // no bad pivot yet
         *J.vmax = 0ull;                              // (k_finalize)
-        if (J.Bmax) J.Bmax[0] = J.Bmax[1] = 0u;      // max |R|, |L^-1| of the wide bounds start at zero
     }
     for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < p * p; e += gridDim.y * blockDim.x) {
         const int col = e / p, row = e - col * p;

@@ -136,7 +136,7 @@ size_t carve(img_ctx *c, char *base) {
     J.ev_count = cv.take<int>(1);
     J.Bimg = p <= img::kMaxWideP ? cv.take<unsigned char>(2 * img::wide_B_bytes(p)) : nullptr;
     J.Bscale = cv.take<float>(2);
-    J.Bmax = cv.take<unsigned>(2);           // also the forward's max |w| word at every p
+    J.opmax = cv.take<float>(2 * img::kOpMax);
     J.vmax = cv.take<unsigned long long>(1);
     J.info = cv.take<DevInfo>(1);
     J.flags = cv.take<int>(4);
@@ -545,15 +545,13 @@ img_status img_psi(img_ctx *c, const double *x, double *Kout, int on_device) {
     const Range range_("img.psi");
     if (!c || !x || !Kout) return IMG_EINVAL;
     const int Q = c->hj.Q, p = c->prm.p;
-    if (on_device) {
-        CK(img::launch_d2f(x, c->wx, Q, c->stream));
-    } else {
+    const int om = fwd_mode_of(c);
+    if (!on_device) {
         std::vector<float> f(Q);
         for (int i = 0; i < Q; ++i) f[i] = (float)x[i];
         CK(cudaMemcpyAsync(c->wx, f.data(), Q * sizeof(float), cudaMemcpyHostToDevice, c->stream));
         CK(cudaStreamSynchronize(c->stream));
     }
-    const int om = fwd_mode_of(c);
     if (om != 0) {
         // tensor-core Gram blocks; their partial sums need a scratch buffer
         if (!c->fwd_part) {
@@ -561,13 +559,16 @@ img_status img_psi(img_ctx *c, const double *x, double *Kout, int on_device) {
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
             CK(cudaMalloc(&c->fwd_part, img::psi_wide_part_floats(sms) * sizeof(float)));
         }
-        CK(img::launch_psi_wide(c->dj, c->hj.Bmax + 1, c->wx, c->fwd_part, Q, p, c->prm.n_l, c->prm.n_m, om, c->Z,
-                                c->stream));
+        const img::FwdIn in{on_device ? x : nullptr, nullptr, nullptr, c->wx, c->hj.opmax + img::kOpMax};
+        CK(img::launch_psi_wide(c->dj, in, c->fwd_part, Q, p, c->prm.n_l, c->prm.n_m, om,
+                                on_device ? Kout : reinterpret_cast<double *>(c->Z), nullptr, c->stream));
     } else {
+        if (on_device) CK(img::launch_d2f(x, c->wx, Q, c->stream));
         CK(img::launch_psi(c->dj, c->wx, c->part, c->nparts, Q, p, mode_of(c), c->Z, c->stream));
     }
-    CK(cudaMemcpyAsync(Kout, c->Z, (size_t)p * p * sizeof(double2),
-                       on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
+    if (om == 0 || !on_device)
+        CK(cudaMemcpyAsync(Kout, c->Z, (size_t)p * p * sizeof(double2),
+                           on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
     if (on_device == 2) return IMG_OK;           // stream-ordered, no host wait
     return sync(c);
 }
@@ -585,7 +586,7 @@ img_status img_psi_adj(img_ctx *c, const double *U, double *out, int on_device) 
             CK(cudaMemcpyAsync(c->Z, U, (size_t)p * p * sizeof(double2), cudaMemcpyHostToDevice, c->stream));
             Ud = c->Z;
         }
-        CK(img::launch_psi_adj_wide(c->dj, c->hj.Bmax, Ud, true, on_device ? out : c->outd, Q, p, om,
+        CK(img::launch_psi_adj_wide(c->dj, Ud, true, on_device ? out : c->outd, Q, p, om,
                                     c->stream));
         if (on_device == 2) return IMG_OK;
         if (on_device) return sync(c);

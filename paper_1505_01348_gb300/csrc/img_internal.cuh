@@ -79,7 +79,7 @@ struct JobDev {
     // operators (64 < p <= 256), and their scales
     unsigned char *Bimg;
     float *Bscale;
-    unsigned *Bmax;      // max |entry| bits of the operators being imaged (atomicMax)
+    float *opmax;        // per-CTA maxima: kOpMax of the adjoint's operands, kOpMax of the forward's weights
     unsigned long long *vmax;  // bits of the cost's largest dirty-image value (atomicMax)
     // decision log (Table I order): kind << 24 | pixel, and lambda or mu
     int *ev;
@@ -162,17 +162,25 @@ cudaError_t ls_snap_begin(const LsSnap &s, LsBufs &b, cudaStream_t st);
 cudaError_t ls_snap_iterate(const LsSnap &s, LsBufs &b, cudaStream_t st);
 cudaError_t launch_snap_scale(const SnapPtrs &sp, int K, int Q, int pwls, double C, float *scale, cudaStream_t st);
 
-// Wide tensor-core forward K = Psi w (64 < p <= 256, mode 1 or 2): wbits is
-// a device word (cleared here), part a scratch of psi_wide_part_floats(SMs)
-// floats; Kout p x p complex128.
+// Tensor-core forward K = Psi w (p <= 384, mode 1 or 2).  The pixel weights w
+// (Q floats) are made here from x (FP64), or as sc o xf (FP32), or taken as
+// they are (x and sc null); wmax: kOpMax floats of scratch.  part: a scratch of
+// psi_wide_part_floats(SMs) floats; K (p x p, interleaved complex) to K64 or,
+// when that is null, K32.
+constexpr int kOpMax = 256;
+struct FwdIn {
+    const double *x;
+    const float *sc, *xf;
+    float *w, *wmax;
+};
 size_t psi_wide_part_floats(int sms);
-cudaError_t launch_psi_wide(const JobDev *job_dev, unsigned *wbits, const float *wx, float *part, int Q, int p,
-                            int n_l, int n_m, int mode, double2 *Kout, cudaStream_t st);
+cudaError_t launch_psi_wide(const JobDev *job_dev, const FwdIn &in, float *part, int Q, int p, int n_l, int n_m, int mode,
+                            double *K64, float *K32, cudaStream_t st);
 // Wide tensor-core adjoint (64 < p <= 256, mode 1 or 2) from U in FP32
 // (u64 false) or FP64 complex (converted while the operand image is
-// written); bmax is the job's Bmax (device), cleared here.
-cudaError_t launch_psi_adj_wide(const JobDev *job_dev, unsigned *bmax, const void *U, bool u64, double *out,
-                                int Q, int p, int mode, cudaStream_t st);
+// written).
+cudaError_t launch_psi_adj_wide(const JobDev *job_dev, const void *U, bool u64, double *out, int Q, int p, int mode,
+                                cudaStream_t st);
 cudaError_t launch_psi_adj(const JobDev *job_dev, const float2 *U, double *out, int Q, int p,
                            int mode, cudaStream_t st);
 cudaError_t launch_z2c(const double2 *src, float2 *dst, int n, cudaStream_t st);

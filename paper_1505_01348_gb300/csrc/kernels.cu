@@ -55,7 +55,6 @@ __device__ void factor_job(const JobDev &J) {
     __shared__ int bad;
     if (threadIdx.x == 0) {
         bad = 0;
-        if (J.Bmax) J.Bmax[0] = J.Bmax[1] = 0u;   // max |R|, |R^-1| of the wide bounds start at zero
     }
     for (int e = threadIdx.x; e < p * p; e += blockDim.x) L[e] = J.R64[e];
     __syncthreads();
@@ -235,12 +234,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_psi_adj_tc(const JobDev *Jp, co
 }
 
 // max |entry| of R_hat (blockIdx.y = 0) and L^-H (1) per job, 8 blocks
-// each (J.Bmax was zeroed by the factor kernel).
+// each, into J.opmax[8 w + block].
+constexpr int kBoundsMaxBlocks = 8;
 __global__ void k_emb_max_bounds(JobDev *const *jobs) {
     const JobDev &J = *jobs[blockIdx.x];
     if (J.flags[0] != 0) return;
     const int w = blockIdx.y;
-    emb_absmax(w ? J.LiH32 : J.R32, J.p, blockIdx.z, gridDim.z, J.Bmax + w);
+    const float mx = emb_absmax(w ? J.LiH32 : J.R32, J.p, blockIdx.z, gridDim.z);
+    if (threadIdx.x == 0) J.opmax[w * gridDim.z + blockIdx.z] = mx;
 }
 
 // Chunked B images of R_hat (blockIdx.y = 0) and L^-H (1) per job; one
@@ -253,8 +254,8 @@ __global__ void k_emb_bounds(JobDev *const *jobs) {
     const int kc = blockIdx.z / kRB, rb = blockIdx.z - kc * kRB;
     if (J.flags[0] != 0 || kc >= wide_nk(J.p) || rb * kEmbRows >= 2 * wide_kp(J.p)) return;
     const int w = blockIdx.y;
-    emb_B_chunk<MODE == 2>(w ? J.LiH32 : J.R32, J.p, J.Bimg + (size_t)w * wide_B_bytes(J.p), J.Bmax[w],
-                           J.Bscale + w, kc, rb);
+    emb_B_chunk<MODE == 2>(w ? J.LiH32 : J.R32, J.p, J.Bimg + (size_t)w * wide_B_bytes(J.p),
+                           warp_max_of(J.opmax + w * kBoundsMaxBlocks, kBoundsMaxBlocks), J.Bscale + w, kc, rb);
 }
 
 // Wide tensor-core bounds for 64 < p <= 256: dirty image (B = R_hat) and
@@ -276,15 +277,17 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bounds_wide(JobDev *const *
     if (to && threadIdx.x == 0) J.flags[2] = IMG_ETIMEOUT;
 }
 
-// max |entry| of one operator U (Jp->Bmax[0] zeroed before), and its B
-// image for k_psi_adj_wide (grid: chunks x row blocks).
+// max |entry| of one operator U, one value per CTA into the job's opmax, and
+// its B image for k_psi_adj_wide (grid: chunks x row blocks).  Plain values
+// per CTA need no cleared word before and no atomics.
 template <class TC>
 __global__ void k_emb_max_one(const JobDev *Jp, const TC *U) {
-    emb_absmax(U, Jp->p, blockIdx.x, gridDim.x, Jp->Bmax);
+    const float mx = emb_absmax(U, Jp->p, blockIdx.x, gridDim.x);
+    if (threadIdx.x == 0) Jp->opmax[blockIdx.x] = mx;
 }
 template <int MODE, class TC>
-__global__ void k_emb_one(const JobDev *Jp, const TC *U) {
-    emb_B_chunk<MODE == 2>(U, Jp->p, Jp->Bimg, Jp->Bmax[0], Jp->Bscale, blockIdx.x, blockIdx.y);
+__global__ void k_emb_one(const JobDev *Jp, const TC *U, int nmax) {
+    emb_B_chunk<MODE == 2>(U, Jp->p, Jp->Bimg, warp_max_of(Jp->opmax, nmax), Jp->Bscale, blockIdx.x, blockIdx.y);
 }
 
 // Wide tensor-core Psi^H vect(U) over all pixels of one job.
@@ -309,60 +312,85 @@ struct FwdMap {
     int idx[6][3];      // 2 Kp <= 768 features: 6 row blocks of 128, 3 column blocks of 256
 };
 
-__global__ void k_fwd_wmax(const float *w, int Q, unsigned *wbits) { fwd_wmax(w, Q, wbits); }
+// Pixel weights of a forward as FP32, w = x (FP64), w = s o x (FP32), or w as
+// it is (x null), and their maximum, one value per CTA.
+__global__ void k_fwd_weights(const double *x, const float *sc, const float *xf, float *w, int Q, float *wmax) {
+    float mx = 0.f;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Q; i += gridDim.x * blockDim.x) {
+        float v;
+        if (x) w[i] = v = (float)x[i];
+        else if (sc) w[i] = v = sc[i] * xf[i];
+        else v = w[i];
+        mx = fmaxf(mx, fabsf(v));
+    }
+    mx = cta_max_t0(mx);
+    if (threadIdx.x == 0) wmax[blockIdx.x] = mx;
+}
 
 template <int MODE>
-__global__ void __launch_bounds__(kFwdThreads, 1) k_fwd_wide(const JobDev *Jp, const float *w, const unsigned *wbits,
+__global__ void __launch_bounds__(kFwdThreads, 1) k_fwd_wide(const JobDev *Jp, const float *w, const float *wmax, int nmax,
                                                             FwdMap map, float *part) {
     const JobDev &J = *Jp;
     unsigned char *dyn = dyn_smem();
     __shared__ uint64_t bars[5];
     __shared__ uint32_t slot;
     const int pr = blockIdx.y, S = gridDim.x;
-    wide_forward<MODE == 2>(J, dyn, bars, &slot, w, *wbits, map.m[pr], map.nb[pr], blockIdx.x, S,
+    wide_forward<MODE == 2>(J, dyn, bars, &slot, w, wmax, nmax, map.m[pr], map.nb[pr], blockIdx.x, S,
                             part + ((size_t)pr * S + blockIdx.x) * (kTcM * 256));
 }
 
-// Sum of the S partials of every formed block, in a fixed order: 4 groups
-// of threads take s = g, g + 4, ... for 64 consecutive entries, then the 4
-// group sums are added in group order.  Ub: np blocks of 128 x 256 doubles.
-__global__ void k_fwd_reduce(const float *part, int S, int nent, double *Ub) {
-    __shared__ double red[4][64];
-    const int j = threadIdx.x & 63, g = threadIdx.x >> 6;
-    const int e = blockIdx.x * 64 + j;
+// K (p x p, column-major, interleaved; FP64 or FP32) from the S partials of the
+// formed blocks.  With U(a, b) the sum of entry (a, b) of G, on or above the
+// diagonal: K_kl = U(k,l) + U(Kp+k,Kp+l) + j (U(l,Kp+k) - U(k,Kp+l)) for k <=
+// l, scaled back by 1 / (sX^2 sW); K_lk = conj(K_kl).  Every sum in a fixed
+// order: group g of 4 takes s = g, g + 4, ..., then the groups in order.
+//
+// One CTA per 4 x 4 tile of (k, l): 4 entry kinds x 16 entries x 4 groups of
+// threads.  Bound by the FP64 pipe (a conversion and an addition per
+// partial), so only the entries that K takes are summed - about half of what
+// the blocks hold - and small tiles keep every SM at it for small arrays.
+constexpr int kAsmT = 4;
+template <class Out>
+__global__ void __launch_bounds__(256) k_fwd_assemble(int p, const float *part, int S, FwdMap map, const float *wmax,
+                                                      int nmax, Out *K) {
+    __shared__ double red[4][4][kAsmT * kAsmT];              // [group][kind][entry]
+    __shared__ double s_inv;
+    const int k0 = blockIdx.x * kAsmT, l0 = blockIdx.y * kAsmT;
+    if (k0 > l0) return;
+    const int Kp = wide_kp(p);
     constexpr size_t kBlk = (size_t)kTcM * 256;
+    const int e = threadIdx.x & 15, kind = (threadIdx.x >> 4) & 3, g = threadIdx.x >> 6;
+    const int hi = e >> 2, lo = e & 3;                       // lo runs along the stored rows
+    // kinds: U(k, l), U(Kp+k, Kp+l), U(k, Kp+l) with k = k0 + hi, l = l0 + lo;
+    // U(l, Kp+k) with l = l0 + hi, k = k0 + lo
+    int a = (kind == 3 ? l0 : k0) + hi, b = (kind == 3 ? k0 : l0) + lo;
+    const int ka = kind == 3 ? b : a, la = kind == 3 ? a : b;
+    a += kind == 1 ? Kp : 0;
+    b += kind >= 1 ? Kp : 0;
     double acc = 0.0;
-    if (e < nent) {
-        const int pr = e / (int)kBlk, off = e - pr * (int)kBlk;
-        const float *q = part + (size_t)pr * S * kBlk + off;
-#pragma unroll 4
+    if (ka <= la && la < p) {
+        const int m = a >> 7, nb = b >> 8;
+        const float *q = part + (size_t)map.idx[m][nb] * S * kBlk + (size_t)(a - 128 * m) * 256 + (b - 256 * nb);
+#pragma unroll 8
         for (int s = g; s < S; s += 4) acc += q[(size_t)s * kBlk];
     }
-    red[g][j] = acc;
-    __syncthreads();
-    if (g == 0 && e < nent) Ub[e] = ((red[0][j] + red[1][j]) + red[2][j]) + red[3][j];
-}
-
-// K (p x p complex128, column-major) from the summed blocks: entries of G on
-// or above the diagonal, U(a, b); K_kl = U(k,l) + U(Kp+k,Kp+l) + j (U(l,Kp+k)
-// - U(k,Kp+l)) for k <= l, scaled back by 1 / (sX^2 sW); K_lk = conj(K_kl).
-__global__ void k_fwd_assemble(int p, const double *Ub, FwdMap map, const unsigned *wbits, double2 *K) {
-    const int Kp = wide_kp(p);
-    const float sX = steer_scale(p);
-    const double inv = 1.0 / ((double)sX * sX * emb_scale_of(*wbits));
-    constexpr size_t kBlk = (size_t)kTcM * 256;
-    auto U = [&](int a, int b) {
-        const int m = a >> 7, nb = b >> 8, pr = map.idx[m][nb];
-        return Ub[(size_t)pr * kBlk + (size_t)(a - 128 * m) * 256 + (b - 256 * nb)];
-    };
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < p * p; e += gridDim.x * blockDim.x) {
-        const int l = e / p, k = e - l * p;
-        if (k > l) continue;
-        const double re = (U(k, l) + U(Kp + k, Kp + l)) * inv;
-        const double im = k == l ? 0.0 : (U(l, Kp + k) - U(k, Kp + l)) * inv;
-        K[(size_t)l * p + k] = make_double2(re, im);
-        K[(size_t)k * p + l] = make_double2(re, -im);
+    red[g][kind][kind == 3 ? lo * kAsmT + hi : e] = acc;     // entry (k, l) at 4 (k - k0) + l - l0
+    if (threadIdx.x < 32) {
+        const float sX = steer_scale(p);
+        const double inv = 1.0 / ((double)sX * sX * emb_scale_of(warp_max_of(wmax, nmax)));
+        if (threadIdx.x == 0) s_inv = inv;
     }
+    __syncthreads();
+    const int k = k0 + (threadIdx.x >> 2), l = l0 + (threadIdx.x & 3);
+    if (threadIdx.x >= kAsmT * kAsmT || k > l || l >= p) return;
+    auto U = [&](int q) { return ((red[0][q][e] + red[1][q][e]) + red[2][q][e]) + red[3][q][e]; };
+    const double re = (U(0) + U(1)) * s_inv;
+    const double im = k == l ? 0.0 : (U(3) - U(2)) * s_inv;
+    // component stores: a caller's FP64 matrix may be 8-byte aligned only
+    Out *u = K + 2 * ((size_t)l * p + k), *v = K + 2 * ((size_t)k * p + l);
+    u[0] = v[0] = (Out)re;
+    u[1] = (Out)im;
+    v[1] = (Out)-im;
 }
 
 // ---------------------------------------------------------------- full-image LSQR
@@ -1873,7 +1901,7 @@ static cudaError_t launch_bounds_tc_t(JobDev *const *jobs, int n, int max_tiles,
 
 template <int MODE>
 static cudaError_t launch_bounds_wide_t(JobDev *const *jobs, int n, int max_tiles, int max_p, cudaStream_t st) {
-    k_emb_max_bounds<<<dim3(n, 2, 8), kThreads, 0, st>>>(jobs);
+    k_emb_max_bounds<<<dim3(n, 2, kBoundsMaxBlocks), kThreads, 0, st>>>(jobs);
     k_emb_bounds<MODE><<<dim3(n, 2, wide_nk(max_p) * (2 * kWideMaxP / kEmbRows)), kThreads, 0, st>>>(jobs);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1976,12 +2004,11 @@ cudaError_t launch_psi(const JobDev *job_dev, const float *wx, float2 *part, int
     return cudaGetLastError();
 }
 
-// Partial blocks (one per CTA, at most one CTA per SM) followed by the
-// summed blocks (at most 12 at Kp = 384, in doubles; room for 16).
-size_t psi_wide_part_floats(int sms) { return (size_t)sms * kTcM * 256 + (size_t)2 * 16 * kTcM * 256; }
+// Partial blocks, one per CTA, at most one CTA per SM.
+size_t psi_wide_part_floats(int sms) { return (size_t)sms * kTcM * 256; }
 
-cudaError_t launch_psi_wide(const JobDev *job_dev, unsigned *wbits, const float *wx, float *part, int Q, int p,
-                            int n_l, int n_m, int mode, double2 *Kout, cudaStream_t st) {
+cudaError_t launch_psi_wide(const JobDev *job_dev, const FwdIn &in, float *part, int Q, int p, int n_l, int n_m, int mode,
+                            double *K64, float *K32, cudaStream_t st) {
     if (p < 1 || p > kMaxWideFwdP || (mode != 1 && mode != 2)) return cudaErrorInvalidValue;
     if (fwd_pairs(p, nullptr, nullptr) > 16) return cudaErrorInvalidValue;
     FwdMap map{};
@@ -1992,22 +2019,18 @@ cudaError_t launch_psi_wide(const JobDev *job_dev, unsigned *wbits, const float 
     const int sms = num_sms();
     const int nblk = fwd_nblocks(n_l, n_m);
     const int S = max(1, min(nblk, sms / map.np));
-    cudaError_t e = cudaMemsetAsync(wbits, 0, sizeof(unsigned), st);
-    if (e != cudaSuccess) return e;
-    k_fwd_wmax<<<max(1, min(2 * sms, (Q + 4 * kThreads - 1) / (4 * kThreads))), kThreads, 0, st>>>(wx, Q, wbits);
+    const int nmax = max(1, min(min(sms, kOpMax), (Q + 4 * kThreads - 1) / (4 * kThreads)));
+    k_fwd_weights<<<nmax, kThreads, 0, st>>>(in.x, in.sc, in.xf, in.w, Q, in.wmax);
     const size_t sm = fwd_smem_bytes();
-    e = (mode == 1) ? ensure_smem((const void *)k_fwd_wide<1>, sm) : ensure_smem((const void *)k_fwd_wide<2>, sm);
+    cudaError_t e = (mode == 1) ? ensure_smem((const void *)k_fwd_wide<1>, sm) : ensure_smem((const void *)k_fwd_wide<2>, sm);
     if (e != cudaSuccess) return e;
     if (mode == 1)
-        k_fwd_wide<1><<<dim3(S, map.np), kFwdThreads, sm, st>>>(job_dev, wx, wbits, map, part);
+        k_fwd_wide<1><<<dim3(S, map.np), kFwdThreads, sm, st>>>(job_dev, in.w, in.wmax, nmax, map, part);
     else
-        k_fwd_wide<2><<<dim3(S, map.np), kFwdThreads, sm, st>>>(job_dev, wx, wbits, map, part);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    double *Ub = reinterpret_cast<double *>(part + (size_t)sms * kTcM * 256);
-    const int nent = map.np * kTcM * 256;
-    k_fwd_reduce<<<(nent + 63) / 64, 256, 0, st>>>(part, S, nent, Ub);
-    k_fwd_assemble<<<(p * p + kThreads - 1) / kThreads, kThreads, 0, st>>>(p, Ub, map, wbits, Kout);
+        k_fwd_wide<2><<<dim3(S, map.np), kFwdThreads, sm, st>>>(job_dev, in.w, in.wmax, nmax, map, part);
+    const int nt = (p + kAsmT - 1) / kAsmT;
+    if (K64) k_fwd_assemble<double><<<dim3(nt, nt), 256, 0, st>>>(p, part, S, map, in.wmax, nmax, K64);
+    else k_fwd_assemble<float><<<dim3(nt, nt), 256, 0, st>>>(p, part, S, map, in.wmax, nmax, K32);
     return cudaGetLastError();
 }
 
@@ -2017,11 +2040,17 @@ static inline int ls_grid(int n) { return max(1, min(4 * num_sms(), (n + kThread
 cudaError_t ls_forward(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, float *fwd_part, float2 *part,
                        int nparts, cudaStream_t st) {
     const int Q = hj.Q, p = hj.p, pp = p * p;
-    k_ls_weights<<<ls_grid(Q), kThreads, 0, st>>>(hj.scale, b.v, b.wx, Q);
-    cudaError_t e = mode != 0 ? launch_psi_wide(jd, hj.Bmax + 1, b.wx, fwd_part, Q, p, hj.n_l, hj.n_m, mode, b.Kd, st)
-                              : launch_psi(jd, b.wx, part, nparts, Q, p, 0, b.Kd, st);
+    cudaError_t e;
+    if (mode != 0) {
+        // pixel weights D^-1 v; K straight to FP32
+        const FwdIn in{nullptr, hj.scale, b.v, b.wx, hj.opmax + kOpMax};
+        e = launch_psi_wide(jd, in, fwd_part, Q, p, hj.n_l, hj.n_m, mode, nullptr, reinterpret_cast<float *>(b.Mv), st);
+    } else {
+        k_ls_weights<<<ls_grid(Q), kThreads, 0, st>>>(hj.scale, b.v, b.wx, Q);
+        e = launch_psi(jd, b.wx, part, nparts, Q, p, 0, b.Kd, st);
+        if (e == cudaSuccess) k_d2c<<<ls_grid(pp), kThreads, 0, st>>>(b.Kd, b.Mv, pp);
+    }
     if (e != cudaSuccess) return e;
-    k_d2c<<<ls_grid(pp), kThreads, 0, st>>>(b.Kd, b.Mv, pp);
     if (hj.cost == IMG_COST_PWLS) {
         // W vect(K) = vect(L^-1 K L^-H)
         const dim3 g((p + 31) / 32, (p + 31) / 32);
@@ -2041,7 +2070,7 @@ cudaError_t ls_adjoint(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, 
         k_cgemm<<<g, kThreads, 0, st>>>(p, hj.Li32, 1, b.T1, 0, b.Uw);
         U = b.Uw;
     }
-    cudaError_t e = mode != 0 ? launch_psi_adj_wide(jd, hj.Bmax, U, false, b.y, Q, p, mode, st)
+    cudaError_t e = mode != 0 ? launch_psi_adj_wide(jd, U, false, b.y, Q, p, mode, st)
                               : launch_psi_adj(jd, U, b.y, Q, p, 0, st);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
@@ -2194,20 +2223,18 @@ static cudaError_t launch_psi_adj_tc_t(const JobDev *job_dev, const float2 *U, d
 }
 
 template <int MODE>
-static cudaError_t launch_psi_adj_wide_t(const JobDev *job_dev, unsigned *bmax, const void *U, bool u64,
-                                         double *out, int Q, int p, cudaStream_t st) {
+static cudaError_t launch_psi_adj_wide_t(const JobDev *job_dev, const void *U, bool u64, double *out, int Q, int p,
+                                         cudaStream_t st) {
     const dim3 eg(wide_nk(p), 2 * wide_kp(p) / kEmbRows);
-    cudaError_t e = cudaMemsetAsync(bmax, 0, sizeof(unsigned), st);
-    if (e != cudaSuccess) return e;
     const int nmax = min(16, (p * p + kThreads - 1) / kThreads);
     if (u64) {
         k_emb_max_one<double2><<<nmax, kThreads, 0, st>>>(job_dev, static_cast<const double2 *>(U));
-        k_emb_one<MODE, double2><<<eg, kThreads, 0, st>>>(job_dev, static_cast<const double2 *>(U));
+        k_emb_one<MODE, double2><<<eg, kThreads, 0, st>>>(job_dev, static_cast<const double2 *>(U), nmax);
     } else {
         k_emb_max_one<float2><<<nmax, kThreads, 0, st>>>(job_dev, static_cast<const float2 *>(U));
-        k_emb_one<MODE, float2><<<eg, kThreads, 0, st>>>(job_dev, static_cast<const float2 *>(U));
+        k_emb_one<MODE, float2><<<eg, kThreads, 0, st>>>(job_dev, static_cast<const float2 *>(U), nmax);
     }
-    e = cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const size_t sm = wide_smem_bytes(p);
     e = ensure_smem((const void *)k_psi_adj_wide<MODE>, sm);
@@ -2217,11 +2244,11 @@ static cudaError_t launch_psi_adj_wide_t(const JobDev *job_dev, unsigned *bmax, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_psi_adj_wide(const JobDev *job_dev, unsigned *bmax, const void *U, bool u64, double *out,
-                                int Q, int p, int mode, cudaStream_t st) {
+cudaError_t launch_psi_adj_wide(const JobDev *job_dev, const void *U, bool u64, double *out, int Q, int p, int mode,
+                                cudaStream_t st) {
     if (p < 1 || p > kMaxWideP || (mode != 1 && mode != 2)) return cudaErrorInvalidValue;
-    if (mode == 1) return launch_psi_adj_wide_t<1>(job_dev, bmax, U, u64, out, Q, p, st);
-    return launch_psi_adj_wide_t<2>(job_dev, bmax, U, u64, out, Q, p, st);
+    if (mode == 1) return launch_psi_adj_wide_t<1>(job_dev, U, u64, out, Q, p, st);
+    return launch_psi_adj_wide_t<2>(job_dev, U, u64, out, Q, p, st);
 }
 
 cudaError_t launch_psi_adj(const JobDev *job_dev, const float2 *U, double *out, int Q, int p, int mode,

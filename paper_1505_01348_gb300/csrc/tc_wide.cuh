@@ -94,12 +94,21 @@ __device__ __forceinline__ void cp_async_wait2() { asm volatile("cp.async.wait_g
 __device__ __forceinline__ float2 to_f2(float2 v) { return v; }
 __device__ __forceinline__ float2 to_f2(double2 v) { return make_float2((float)v.x, (float)v.y); }
 
+// Largest value >= 0 over the CTA, in thread 0 (any number of warps).
+__device__ __forceinline__ float cta_max_t0(float mx) {
+    __shared__ float sred[32];
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < (int)(blockDim.x + 31) / 32; ++w) mx = fmaxf(mx, sred[w]);
+    return mx;
+}
+
 // max |Re|, |Im| over the p^2 entries of U (rounded to FP32), one block's
-// share (grid-stride over blocks `b` of `nb`), folded into *mx as the bit
-// pattern of a non-negative float (atomicMax on the bits is monotonic).
-// *mx must be zero before the first block adds to it.
+// share (grid-stride over blocks `b` of `nb`); thread 0 has the result.
 template <class TC>
-__device__ inline void emb_absmax(const TC *U, int p, int b, int nb, unsigned *mx_bits) {
+__device__ inline float emb_absmax(const TC *U, int p, int b, int nb) {
     __shared__ float sred[32];
     const int n2 = p * p, stride = nb * blockDim.x;
     float mx = 0.f;
@@ -115,19 +124,19 @@ __device__ inline void emb_absmax(const TC *U, int p, int b, int nb, unsigned *m
         const float2 v = to_f2(U[e]);
         mx = fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.y)));
     }
+    return cta_max_t0(mx);
+}
+
+// Largest of the per-CTA maxima m[0 .. n) (one warp, every lane).
+__device__ __forceinline__ float warp_max_of(const float *m, int n) {
+    float mx = 0.f;
+    for (int i = threadIdx.x & 31; i < n; i += 32) mx = fmaxf(mx, m[i]);
     for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x + 31) / 32; ++w) mx = fmaxf(mx, sred[w]);
-        mx = fmaxf(mx, sred[0]);
-        atomicMax(mx_bits, __float_as_uint(mx));
-    }
+    return mx;
 }
 
 // Power-of-two scale that brings max |U| to (1/2, 1].
-__device__ __forceinline__ float emb_scale_of(unsigned mx_bits) {
-    const float mx = __uint_as_float(mx_bits);
+__device__ __forceinline__ float emb_scale_of(float mx) {
     return mx > 0.f ? exp2f(-ceilf(log2f(mx))) : 1.f;
 }
 
@@ -138,13 +147,13 @@ constexpr int kEmbRows = 64;
 // (column-major p x p, FP32 or FP64 complex, used as FP32): B = emb(V), V = U^H, whose quadratic form equals
 // that of emb(U).  With u = U[k_row * p + k_col] (= conj V(k_row, k_col)):
 // blocks (Re, Re) and (Im, Im) hold u.x, (Re, Im) holds u.y, (Im, Re) holds
-// -u.y; scaled by the power of two of emb_scale_of(mx_bits) (max |U| from
+// -u.y; scaled by the power of two of emb_scale_of(mx) (mx = max |U| from
 // emb_absmax).  The CTA of chunk 0, row block 0 stores the scale.
 template <bool BF16, class TC>
-__device__ void emb_B_chunk(const TC *U, int p, unsigned char *img, unsigned mx_bits, float *scale, int kc,
+__device__ void emb_B_chunk(const TC *U, int p, unsigned char *img, float mx, float *scale, int kc,
                             int rb) {
     const int Kp = wide_kp(p), nc8 = Kp / 8, nu = wide_units(p), rows_u = wide_unit_rows(p);
-    const float sc = emb_scale_of(mx_bits);
+    const float sc = emb_scale_of(mx);
     if (kc == 0 && rb == 0 && threadIdx.x == 0) *scale = sc;
     unsigned char *chunk = img + (size_t)kc * wide_chunk_bytes(p);
     const size_t ub = wide_unit_bytes(p);
@@ -538,33 +547,18 @@ __host__ __device__ constexpr uint32_t idesc_f16_mn128(int n, int ab_fmt) {
            ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTcM >> 4) << 24);
 }
 
-// max |w| over Q weights (block share of a grid-stride pass), into *mx_bits.
-__device__ inline void fwd_wmax(const float *w, int Q, unsigned *mx_bits) {
-    __shared__ float sred[32];
-    float mx = 0.f;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Q; i += gridDim.x * blockDim.x) mx = fmaxf(mx, fabsf(w[i]));
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int q = 1; q < (int)(blockDim.x + 31) / 32; ++q) mx = fmaxf(mx, sred[q]);
-        mx = fmaxf(mx, sred[0]);
-        atomicMax(mx_bits, __float_as_uint(mx));
-    }
-}
-
 // One CTA: block `pair` of G over the pixel blocks s, s + S, ... of the grid;
 // writes the FP32 block (128 x 256, row-major) to out.  w: pixel weights;
-// wbits: max |w| bits.  Returns the number of waits that timed out.
+// wmax[0 .. nmax): their per-CTA maxima.  Returns the number of waits that timed out.
 template <bool BF16>
 __device__ int wide_forward(const JobDev &J, unsigned char *dyn, uint64_t *bars, uint32_t *slot, const float *w,
-                            unsigned wbits, int m, int nb, int s0, int S, float *out) {
+                            const float *wmax, int nmax, int m, int nb, int s0, int S, float *out) {
     const int p = J.p, Kp = wide_kp(p), Nf = 2 * Kp, N = fwd_n_of(p, nb);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nl = J.n_l, nm = J.n_m, tlb = (nl + 7) / 8, nblk = fwd_nblocks(nl, nm);
     const int mine = nblk > s0 ? (nblk - 1 - s0) / S + 1 : 0;
     const float sX = steer_scale(p);
-    const float sW = emb_scale_of(wbits);
+    const float sW = emb_scale_of(warp_max_of(wmax, nmax));
     enum { kFull = 0, kEmpty = 2, kAcc = 4 };
     // feature chunks of a stage: A = {2m, 2m+1}, then those of B = {4nb ..}
     // that are not among them
