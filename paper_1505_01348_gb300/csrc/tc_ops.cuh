@@ -438,47 +438,55 @@ __device__ __forceinline__ int tc_tile_pixel(int t, int r, int n_l, int n_m) {
 }
 
 // X tile (128 rows) of steering vectors for the pixels of 2-D tile t
-// (rows outside the grid are zero), scaled by sX (a power of two).
+// (rows outside the grid are zero), scaled by sX (a power of two).  p <= 64.
+// A thread makes the same 8 antennas of 2 (Kp = 32) or 4 (Kp = 64) rows that
+// share their l offset: one E_l chunk and 2 or 4 E_m chunks, all loaded before
+// the first product.  (Row by row the loads were a chain of L2 latencies:
+// with the largest shared-memory carve-out the tables do not stay in L1.)
 template <bool BF16>
 __device__ inline void tc_gen_X_steer(const JobDev &J, TcWork &T, int b, int t, float sX) {
-    const int p = J.p, Kp = T.Kp, nc8 = Kp / 8, nl = J.n_l;
-    const float2 *__restrict__ El = J.El;
-    const float2 *__restrict__ Em = J.Em;
-    unsigned char *xh = T.Xhi(b), *xl = T.Xlo(b);
-    const bool vec = (p & 7) == 0;       // 64-byte aligned antenna chunks
-    for (int it = threadIdx.x; it < kTcM * nc8; it += blockDim.x) {
-        const int r = it / nc8, c8 = it - r * nc8;
-        float re[8], im[8];
-        const int k0 = c8 * 8;
-        const int i = tc_tile_pixel(t, r, nl, J.n_m);
-        if (i >= 0 && k0 < p) {
-            const int mm = i / nl, ll = i - mm * nl;
-            if (vec) {
-                const float4 *e = reinterpret_cast<const float4 *>(El + (size_t)ll * p + k0);
-                const float4 *f = reinterpret_cast<const float4 *>(Em + (size_t)mm * p + k0);
+    const int p = J.p, nc8 = T.Kp / 8, nl = J.n_l, nm = J.n_m, tl = (nl + kTileL - 1) / kTileL;
+    const int bm = t / tl, bl = t - bm * tl;
+    const int c8 = threadIdx.x & (nc8 - 1), r0 = threadIdx.x / nc8, rstep = kThreads / nc8;
+    const int k0 = c8 * 8, il = bl * kTileL + (r0 & 7);
+    const bool vec = (p & 1) == 0;
+    auto load = [&](const float2 *row, bool ok, float2 *v) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float4 x = __ldg(e + q), y = __ldg(f + q);
-                    const float2 a0 = cmul(make_float2(x.x, x.y), make_float2(y.x, y.y));
-                    const float2 a1 = cmul(make_float2(x.z, x.w), make_float2(y.z, y.w));
-                    re[2 * q] = a0.x * sX;
-                    im[2 * q] = a0.y * sX;
-                    re[2 * q + 1] = a1.x * sX;
-                    im[2 * q + 1] = a1.y * sX;
-                }
-            } else {
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int k = k0 + q;
-                    float2 a = make_float2(0.f, 0.f);
-                    if (k < p) a = cmul(__ldg(El + (size_t)ll * p + k), __ldg(Em + (size_t)mm * p + k));
-                    re[q] = a.x * sX;
-                    im[q] = a.y * sX;
+        for (int q = 0; q < 4; ++q) {
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (ok && k0 + 2 * q < p) {
+                if (vec) {
+                    x = __ldg(reinterpret_cast<const float4 *>(row + k0 + 2 * q));
+                } else {
+                    const float2 x0 = __ldg(row + k0 + 2 * q);
+                    const float2 x1 = k0 + 2 * q + 1 < p ? __ldg(row + k0 + 2 * q + 1) : make_float2(0.f, 0.f);
+                    x = make_float4(x0.x, x0.y, x1.x, x1.y);
                 }
             }
-        } else {
+            v[2 * q] = make_float2(x.x, x.y);
+            v[2 * q + 1] = make_float2(x.z, x.w);
+        }
+    };
+    float2 e[8], f[4][8];
+    load(J.El + (size_t)il * p, il < nl, e);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) re[q] = im[q] = 0.f;
+    for (int q = 0; q < 4; ++q) {
+        const int im = bm * kTileM + ((r0 + q * rstep) >> 3);
+        load(J.Em + (size_t)im * p, r0 + q * rstep < kTcM && im < nm, f[q]);
+    }
+    unsigned char *xh = T.Xhi(b), *xl = T.Xlo(b);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int r = r0 + q * rstep;
+        if (r >= kTcM) break;
+        float re[8], im[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            // cmul with its fused operations written out
+            const float2 a = make_float2(__fmaf_rn(e[k].x, f[q][k].x, -__fmul_rn(e[k].y, f[q][k].y)),
+                                         __fmaf_rn(e[k].x, f[q][k].y, __fmul_rn(e[k].y, f[q][k].x)));
+            re[k] = a.x * sX;
+            im[k] = a.y * sX;
         }
         uint4 hi, lo;
         split8<BF16>(re, hi, lo);
