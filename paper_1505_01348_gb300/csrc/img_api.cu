@@ -131,6 +131,9 @@ size_t carve(img_ctx *c, char *base) {
     J.W0 = cv.take<float2>(pp);
     J.W1 = cv.take<float2>(pp);
     J.W2 = cv.take<float2>(pp);
+    // 128 rows x 2 x 64 columns, hi + lo, per tile; at every arithmetic (a
+    // pooled context may get jobs of another)
+    J.ximg = p > 32 && p <= img::kMaxTcP ? cv.take<unsigned char>(4 * 65536) : nullptr;
     J.ev = cv.take<int>(J.ev_cap);
     J.evv = cv.take<float>(J.ev_cap);
     J.ev_count = cv.take<int>(1);

@@ -75,6 +75,7 @@ struct JobDev {
     float *v, *w, *xs;     // cap, LSQR vectors indexed by F position
     float *sF;             // cap, s_i of the free pixels in F order (per LSQR solve)
     float2 *W0, *W1, *W2;  // p*p scratch matrices
+    unsigned char *ximg;   // 32 < p <= 64: four split free-set tiles of the one-CTA solver's LSQR
     // chunked B images of R_hat and R_hat^-1 for the wide tensor-core
     // operators (64 < p <= 256), and their scales
     unsigned char *Bimg;

@@ -681,6 +681,8 @@ struct SolveShared {
     float red[kTile + 16 * kTile];
     float ls[8];          // LSQR: coefficients that warp 0 hands to the CTA
     float fm[kThreads / 32];
+    uint64_t ldbar[2];    // tile loads into the two X buffers, and their parities
+    uint32_t ldph;
     int lsi;
 };
 // At namespace scope, so that the solver's out-of-line functions address it
@@ -996,11 +998,15 @@ __device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShare
 }
 
 // ---------------------------------------------------------------- resident LSQR
-// LSQR on the free set for f <= 256 on tensor cores (Kp = 32 or 64), with
-// everything that an iteration touches on the SM: the free-set tiles in
-// shared memory (tile 0 in buffer 0, tile 1 in buffer 1), the p x p vector t
-// in registers (thread tid: entries tid + 256 k), v, w, x, s_F of free pixel
-// j in the registers of thread j.  Same arithmetic and the same order of
+// LSQR on the free set on tensor cores, f <= 256 (Kp = 32) or 512 (Kp = 64),
+// with everything that an iteration touches on the SM: the free-set tiles in
+// shared memory (tile t in buffer t & 1; tiles beyond the second are kept
+// split in global memory and brought in by bulk copies, two tiles' worth
+// fewer than there are per product, because the products walk the tiles in
+// opposite directions), the p x p vector t in registers (thread tid: entries
+// tid + 256 k), v, w, x, s_F of free pixels tid and tid + 256 in registers.
+// Above that lsqr_cta regenerates the tiles from the cached vectors for every
+// product (99,000 cycles per iteration at p = 48, f = 256 .. 349).  Same arithmetic and the same order of
 // every sum as lsqr_cta's; the fused multiply-adds are written out, so that
 // the rounding does not depend on what the compiler contracts where.
 //
@@ -1016,13 +1022,14 @@ __device__ int lsqr_cta(const JobDev &J, int f, float2 *A, TcWork &T, SolveShare
 // in FP32 from the free vectors themselves (shared memory), thread-owned
 // entries of t directly: at p <= 32 the Gram matrix's read-out costs more
 // than the sums, and the products keep lsqr_cta's FP32 bits.
-constexpr int kResF = 2 * kTcM;         // most free pixels
+constexpr int kResF = 2 * kTcM;         // most free pixels, Kp = 32
+constexpr int kResMaxF = 4 * kTcM;      // and Kp = 64
 constexpr int kResRows = 64;            // weighted rows staged at a time
 
 // Bytes behind the operand tiles: Kp = 64: the Gram read-out's overhang over
-// the B region; Kp = 32: the free vectors.  Then the weights (kResF floats).
+// the B region; Kp = 32: the free vectors.  Then the weights (kResMaxF floats).
 __host__ __device__ inline size_t res_extra_bytes(int p) {
-    return ((p + 31) / 32 * 32 == 32 ? (size_t)kResF * p * sizeof(float2) : 1024) + kResF * sizeof(float);
+    return ((p + 31) / 32 * 32 == 32 ? (size_t)kResF * p * sizeof(float2) : 1024) + kResMaxF * sizeof(float);
 }
 
 // Named barriers of the resident LSQR (0 is __syncthreads).
@@ -1071,23 +1078,23 @@ __device__ __forceinline__ void res_build_B(const TcWork &T, int p, float sc) {
     bar_sync(2, kNt);
 }
 
-// Rows r0 .. r0 + nst - 1 of the resident tiles times sW w[row] (zero from
-// row f on) as an MN-major operand of kResRows rows per feature block at dst
+// Rows r0 .. r0 + nst - 1 of the free set, whose tile is in buffer xb, times
+// sW w[row] (zero from row f on) as an MN-major operand of kResRows rows per feature block at dst
 // (hi, then lo), re-split.
 template <bool BF16>
-__device__ __forceinline__ void res_stage_rows(const TcWork &T, unsigned char *dst, int r0, int nst, int f,
+__device__ __forceinline__ void res_stage_rows(const TcWork &T, unsigned char *dst, int xb, int r0, int nst, int f,
                                                const float *w, float sW) {
     const int nch = 2 * T.Kp / 8;
     const size_t half_bytes = (size_t)(2 * T.Kp / 64) * kResRows * 128;
-    const int tile = r0 / kTcM, rt = r0 % kTcM;
+    const int rt = r0 % kTcM;
 #pragma unroll 2
     for (int it = threadIdx.x; it < nst * nch; it += kThreads) {
         const int rr = it / nch, c = it - rr * nch;
         const uint32_t src = sw128_off(rt + rr, c, kTcM);
         const uint32_t off = sw128_off(rr, c, kResRows);
         const float wr = r0 + rr < f ? sW * w[r0 + rr] : 0.f;
-        const uint4 h4 = *reinterpret_cast<const uint4 *>(T.Xhi(tile) + src);
-        const uint4 l4 = *reinterpret_cast<const uint4 *>(T.Xlo(tile) + src);
+        const uint4 h4 = *reinterpret_cast<const uint4 *>(T.Xhi(xb) + src);
+        const uint4 l4 = *reinterpret_cast<const uint4 *>(T.Xlo(xb) + src);
         const uint32_t hw[4] = {h4.x, h4.y, h4.z, h4.w}, lw[4] = {l4.x, l4.y, l4.z, l4.w};
         uint32_t hi[4], lo[4];
 #pragma unroll
@@ -1102,7 +1109,8 @@ __device__ __forceinline__ void res_stage_rows(const TcWork &T, unsigned char *d
 
 //
 // Out of line: inlined into k_solve the two spilled 2.5 KB per thread.
-template <int MODE>
+// NP: free pixels per thread (1: f <= 256, at most two tiles).
+template <int MODE, int NP>
 __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, SolveCycles &cio) {
     constexpr bool BF = MODE == 2;
     TcWork T = Tio;
@@ -1113,22 +1121,50 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
     SolveShared &S = g_solve;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool w0 = warp == 0;
-    const int j = threadIdx.x;                    // this thread's free pixel
-    const bool mine = j < f;
-    const int ntiles = f > kTcM ? 2 : 1;
+    const int ntiles = (f + kTcM - 1) / kTcM;
+    const bool stream = NP > 1 && ntiles > 2;     // tiles beyond two come and go through the image
     const int *__restrict__ fpos = J.fpos;
     unsigned char *extra = T.Blo() + (T.Blo() - T.Bhi());
     float2 *C = reinterpret_cast<float2 *>(extra);                              // Kp = 32: free vectors
-    float *wt = reinterpret_cast<float *>(extra + res_extra_bytes(p)) - kResF;
+    float *wt = reinterpret_cast<float *>(extra + res_extra_bytes(p)) - kResMaxF;
     const float sX = list_scale(J, fpos, f, S.dbuf);
-    for (int t = 0; t < ntiles; ++t) tc_gen_X_cache<BF>(J, T, t, fpos, t * kTcM, min(kTcM, f - t * kTcM), sX);
+    const uint32_t tile_bytes = 2 * T.x_bytes();
+    for (int t = 0; t < ntiles; ++t) {
+        if (t >= 2) __syncthreads();              // the buffer's last tile is in the image
+        tc_gen_X_cache<BF>(J, T, t & 1, fpos, t * kTcM, min(kTcM, f - t * kTcM), sX);
+        if (stream) {
+            __syncthreads();
+            const uint4 *src = reinterpret_cast<const uint4 *>(T.Xhi(t & 1));
+            uint4 *dst = reinterpret_cast<uint4 *>(J.ximg + (size_t)t * tile_bytes);
+            for (uint32_t e = threadIdx.x; e < tile_bytes / 16; e += kThreads) dst[e] = src[e];
+        }
+    }
+    if (stream) asm volatile("fence.proxy.async;" ::: "memory");
+    uint32_t ldph = S.ldph;                       // parities of the tile loads
+    // tile t from the image into its buffer (thread 32, after a barrier that
+    // ended every use of the buffer)
+    auto load_tile = [&](int t) {
+        uint64_t *bar = &S.ldbar[t & 1];
+        mbar_expect_tx(bar, tile_bytes);
+        tma_bulk_g2s(T.Xhi(t & 1), J.ximg + (size_t)t * tile_bytes, tile_bytes, bar);
+    };
+    auto wait_tile = [&](int b) {
+        if (!mbar_wait(&S.ldbar[b], (ldph >> b) & 1u)) T.timeouts++;
+    };
     if (!gram)
         for (int e = threadIdx.x; e < f * p; e += kThreads) {
             const int r = e / p;
             C[e] = J.cvec[(size_t)fpos[r] * p + e - r * p];
         }
-    const float sF = mine ? J.scale[J.supp[fpos[j]]] : 0.f;
-    float v = 0.f, w = 0.f, x = 0.f;
+    // free pixels tid + 256 m
+    float sF[NP], v[NP] = {}, w[NP] = {}, x[NP] = {};
+    bool mine[NP];
+#pragma unroll
+    for (int m = 0; m < NP; ++m) {
+        const int j = threadIdx.x + m * kThreads;
+        mine[m] = j < f;
+        sF[m] = mine[m] ? J.scale[J.supp[fpos[j]]] : 0.f;
+    }
     float2 tr[16];
     const int da = kThreads % p, dn = kThreads / p;
     const int a_first = threadIdx.x % p, n_first = threadIdx.x / p;
@@ -1170,10 +1206,12 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
     // scalars of the recurrence, valid in warp 0
     double alpha = 0.0, beta = 0.0, bnorm = 0.0, us = 0.0, phibar = 0.0, rhobar = 0.0, anorm2 = 0.0;
     double rho = 0.0, cs = 0.0, sn = 0.0, phi = 0.0;
-    // y_j = Re(c_j^H t c_j) (scaled back), thread j.  Warps 1 .. 7 build the B
-    // image of t and issue the MMAs while warp 0 runs scalars().
+    // y[m] = Re(c_j^H t c_j) (scaled back), j = tid + 256 m.  Warps 1 .. 7 build
+    // the B image of t and issue the MMAs while warp 0 runs scalars().  Tiles in
+    // descending order: the forward, ascending, then finds tiles 0 and 1 in the
+    // buffers, and this finds the last two.
     const uint32_t idesc = idesc_f16(N, BF ? 1 : 0);
-    auto adjoint = [&](auto scalars) -> float {
+    auto adjoint = [&](float *y, auto scalars) {
         const long long c0 = clock64();
         const float sB = pow2_of(cta_max()) * kLift;
         float2 *ts = reinterpret_cast<float2 *>(T.Bhi());
@@ -1187,45 +1225,71 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
             bar_sync(1, kThreads);
             res_build_B<BF>(T, p, sB);
             if (threadIdx.x == 32)
-                for (int t = 0; t < ntiles; ++t) tc_issue(T, t, idesc);
+                for (int t = ntiles - 1; t >= max(0, ntiles - 2); --t) tc_issue(T, t & 1, idesc);
             __syncwarp();
         }
         const long long c1 = clock64();
-        for (int t = 0; t < ntiles; ++t) {
-            T.wait(t);
+        for (int t = ntiles - 1; t >= 0; --t) {
+            T.wait(t & 1);
             tc_fence_after();
-            S.red[t * 2 * kTcM + (warp >> 2) * kTcM + 32 * (warp & 3) + lane] = tc_row_dot<BF>(T, t);
+            S.red[t * 2 * kTcM + (warp >> 2) * kTcM + 32 * (warp & 3) + lane] = tc_row_dot<BF>(T, t & 1);
+            if (NP > 1 && t >= 2) {
+                // buffer and accumulator to tile t - 2
+                tc_fence_before();
+                __syncthreads();
+                if (threadIdx.x == 32) {
+                    load_tile(t - 2);
+                    wait_tile(t & 1);
+                    tc_issue(T, t & 1, idesc);
+                }
+                __syncwarp();
+                ldph ^= 1u << (t & 1);
+            }
         }
         tc_fence_before();
         __syncthreads();
         cyc.aux[3] += c1 - c0;
         cyc.aux[5] += clock64() - c1;
-        const float *r = S.red + (j >> 7) * 2 * kTcM + (j & (kTcM - 1));
-        return mine ? (r[0] + r[kTcM]) * (1.f / (sX * sX * sB)) : 0.f;
+#pragma unroll
+        for (int m = 0; m < NP; ++m) {
+            const int j = threadIdx.x + m * kThreads;
+            const float *r = S.red + (j >> 7) * 2 * kTcM + (j & (kTcM - 1));
+            y[m] = mine[m] ? (r[0] + r[kTcM]) * (1.f / (sX * sX * sB)) : 0.f;
+        }
     };
     // write the solution and hand back the barriers' phases and the counters
     auto leave = [&](int its) {
-        if (mine) J.xs[j] = x;
+#pragma unroll
+        for (int m = 0; m < NP; ++m)
+            if (mine[m]) J.xs[threadIdx.x + m * kThreads] = x[m];
         Tio.phase = T.phase;
         Tio.timeouts = T.timeouts;
+        if (threadIdx.x == 0) S.ldph = ldph;
         cio.fwd += cyc.fwd;
         cio.adj += cyc.adj;
         for (int q = 0; q < 6; ++q) cio.aux[q] += cyc.aux[q];
         __syncthreads();
         return its;
     };
+    auto norm_v = [&]() {
+        float n = 0.f;
+#pragma unroll
+        for (int m = 0; m < NP; ++m) n = fmaf(v[m], v[m], n);
+        return n;
+    };
     reduce(acc, mx);
-    {
-        const float y = adjoint([&]() {
-            beta = bnorm = phibar = sqrt(cta_sum());
-            us = 1.0 / beta;
-            S.ls[2] = (float)us;
-            S.lsi = beta == 0.0;
-        });
-        if (S.lsi) return leave(0);
-        if (mine) v = sF * (y * S.ls[2]);
-    }
-    reduce(fmaf(v, v, 0.f), 0.f);
+    float y[NP];
+    adjoint(y, [&]() {
+        beta = bnorm = phibar = sqrt(cta_sum());
+        us = 1.0 / beta;
+        S.ls[2] = (float)us;
+        S.lsi = beta == 0.0;
+    });
+    if (S.lsi) return leave(0);
+#pragma unroll
+    for (int m = 0; m < NP; ++m)
+        if (mine[m]) v[m] = sF[m] * (y[m] * S.ls[2]);
+    reduce(norm_v(), 0.f);
     if (w0) {
         alpha = rhobar = sqrt(cta_sum());
         S.ls[5] = (float)(1.0 / alpha);
@@ -1234,10 +1298,16 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
     }
     __syncthreads();
     if (S.lsi) return leave(0);
-    v *= S.ls[5];
-    w = v;
-    wt[j] = sF * v;
-    reduce(0.f, fabsf(sF * v));
+    mx = 0.f;
+#pragma unroll
+    for (int m = 0; m < NP; ++m) {
+        v[m] *= S.ls[5];
+        w[m] = v[m];
+        const float wj = sF[m] * v[m];
+        if (mine[m]) wt[threadIdx.x + m * kThreads] = wj;
+        mx = fmaxf(mx, fabsf(wj));
+    }
+    reduce(0.f, mx);
     const int maxit = J.lsqr_maxit > 0 ? J.lsqr_maxit : 4 * f + 20;
     const double atol = J.lsqr_atol, btol = J.lsqr_btol;
     const uint32_t fdesc = idesc_f16_mn(N, BF ? 1 : 0);
@@ -1254,12 +1324,19 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
             const int ngrp = (f + kResRows - 1) / kResRows;
             for (int g = 0; g < ngrp; ++g) {
                 const int b = g & 1, r0 = g * kResRows, ks = (min(kResRows, f - r0) + 15) / 16;
+                const int xb = (r0 / kTcM) & 1;
                 unsigned char *st = T.Bhi() + b * (2 * 2 * kResRows * 128);
                 if (g >= 2) {
                     T.wait(b);
                     tc_fence_after();
                 }
-                res_stage_rows<BF>(T, st, r0, 16 * ks, f, wt, sW);
+                // groups up to g - 2 are done: an odd one ended its tile
+                if (stream && (g & 1) && g >= 3 && (g + 1) / 2 < ntiles && threadIdx.x == 32) load_tile((g + 1) / 2);
+                if (NP > 1 && g >= 4 && !(g & 1)) {
+                    wait_tile(xb);
+                    ldph ^= 1u << xb;
+                }
+                res_stage_rows<BF>(T, st, xb, r0, 16 * ks, f, wt, sW);
                 fence_async_smem();
                 __syncthreads();
                 if (g == 0) {
@@ -1270,9 +1347,8 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
                 if (threadIdx.x == 0) {
                     tc_fence_after();
                     const uint32_t ah = smem_u32(st), al = ah + 2 * kResRows * 128;
-                    const int tile = r0 / kTcM;
                     const uint32_t bo = (uint32_t)((r0 % kTcM) / 8) * 1024;
-                    const uint32_t bh = smem_u32(T.Xhi(tile)) + bo, bl = smem_u32(T.Xlo(tile)) + bo;
+                    const uint32_t bh = smem_u32(T.Xhi(xb)) + bo, bl = smem_u32(T.Xlo(xb)) + bo;
                     const uint32_t d = T.tmem + (uint32_t)(2 * N);
                     constexpr uint32_t alb = kResRows * 128, blb = kTcM * 128;
                     for (int s = 0; s < ks; ++s) {
@@ -1286,10 +1362,7 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
                 }
             }
             if (stop) break;
-            for (int g = max(0, ngrp - 2); g < ngrp; ++g) {
-                const int b = g & 1;
-                T.wait(b);
-            }
+            for (int g = max(0, ngrp - 2); g < ngrp; ++g) T.wait(g & 1);
             tc_fence_after();
             inv = 1.f / (sX * sX * sW);
             const long long c1 = clock64();
@@ -1336,7 +1409,11 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     float2 &t = tr[k0 + q];
-                    if (gram)
+                    // (f > 256: alpha u is not rounded on its own, as in
+                    // lsqr_cta, which took those sizes before)
+                    if (gram && stream)
+                        t = make_float2(__fmaf_rn(-fa, t.x, kv[q].x * inv), __fmaf_rn(-fa, t.y, kv[q].y * inv));
+                    else if (gram)
                         t = make_float2(__fmaf_rn(kv[q].x, inv, -__fmul_rn(fa, t.x)),
                                         __fmaf_rn(kv[q].y, inv, -__fmul_rn(fa, t.y)));
                     else
@@ -1351,7 +1428,7 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
         cyc.aux[2] += c3 - c2;
         cyc.fwd += c3 - c0;
         // v <- M^H u - beta v
-        const float y = adjoint([&]() {
+        adjoint(y, [&]() {
             beta = sqrt(cta_sum());
             us = beta > 0.0 ? 1.0 / beta : 0.0;
             S.ls[1] = (float)beta;
@@ -1365,9 +1442,11 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
             phi = cs * phibar;
             phibar = sn * phibar;
         });
-        if (mine) v = __fmaf_rn(sF, __fmul_rn(y, S.ls[2]), -__fmul_rn(S.ls[1], v));
+#pragma unroll
+        for (int m = 0; m < NP; ++m)
+            if (mine[m]) v[m] = __fmaf_rn(sF[m], __fmul_rn(y[m], S.ls[2]), -__fmul_rn(S.ls[1], v[m]));
         cyc.adj += clock64() - c3;
-        reduce(mine ? fmaf(v, v, 0.f) : 0.f, 0.f);
+        reduce(norm_v(), 0.f);
         if (w0) {
             // lanes 0..2: the coefficients of x and w, 1/alpha
             alpha = sqrt(cta_sum());
@@ -1380,17 +1459,19 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
         __syncthreads();
         acc = 0.f;
         mx = 0.f;
-        if (mine) {
+#pragma unroll
+        for (int m = 0; m < NP; ++m) {
+            if (!mine[m]) continue;
             const float t1 = S.ls[3], t2 = S.ls[4], ia = S.ls[5];
-            const float vj = __fmul_rn(v, ia);          // v <- v / alpha
-            v = vj;
-            const float xj = __fmaf_rn(t1, w, x);
-            x = xj;
-            w = __fmaf_rn(t2, w, vj);
-            acc = fmaf(xj, xj, 0.f);
-            const float wj = sF * vj;
-            wt[j] = wj;
-            mx = fabsf(wj);
+            const float vj = __fmul_rn(v[m], ia);       // v <- v / alpha
+            v[m] = vj;
+            const float xj = __fmaf_rn(t1, w[m], x[m]);
+            x[m] = xj;
+            w[m] = __fmaf_rn(t2, w[m], vj);
+            acc = fmaf(xj, xj, acc);
+            const float wj = sF[m] * vj;
+            wt[threadIdx.x + m * kThreads] = wj;
+            mx = fmaxf(mx, fabsf(wj));
         }
         reduce(acc, mx);
         if (w0) {
@@ -1452,6 +1533,11 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
     TcWork T{};
     if constexpr (MODE != 0) {
         tc_carve(T, dyn, p);
+        if (threadIdx.x == 0) {
+            mbar_init(&S.ldbar[0], 1);
+            mbar_init(&S.ldbar[1], 1);
+            S.ldph = 0;
+        }
         tc_setup(T, tc_bar, &tc_slot, p);
     }
     if constexpr (PREP) {
@@ -1522,10 +1608,10 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
                 info.op_flops += flops_fwd(p, nu);
                 const long long t0 = clock64();
                 int its;
-                if (MODE != 0 && f <= kResF) {
+                if (MODE != 0 && f <= (T.Kp == 64 ? kResMaxF : kResF)) {
                     TcWork Tl = T;            // by reference only here: T stays in registers
                     SolveCycles cl;
-                    its = lsqr_resident<MODE>(J, f, Tl, cl);
+                    its = f <= kResF ? lsqr_resident<MODE, 1>(J, f, Tl, cl) : lsqr_resident<MODE, 2>(J, f, Tl, cl);
                     T.phase = Tl.phase;
                     T.timeouts = Tl.timeouts;
                     cyc.fwd += cl.fwd;
