@@ -562,7 +562,7 @@ img_status img_psi(img_ctx *c, const double *x, double *Kout, int on_device) {
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
             CK(cudaMalloc(&c->fwd_part, img::psi_wide_part_floats(sms) * sizeof(float)));
         }
-        const img::FwdIn in{on_device ? x : nullptr, nullptr, nullptr, c->wx, c->hj.opmax + img::kOpMax};
+        const img::FwdIn in{on_device ? x : nullptr, c->wx, c->hj.opmax + img::kOpMax, 0};
         CK(img::launch_psi_wide(c->dj, in, c->fwd_part, Q, p, c->prm.n_l, c->prm.n_m, om,
                                 on_device ? Kout : reinterpret_cast<double *>(c->Z), nullptr, c->stream));
     } else {
@@ -589,7 +589,7 @@ img_status img_psi_adj(img_ctx *c, const double *U, double *out, int on_device) 
             CK(cudaMemcpyAsync(c->Z, U, (size_t)p * p * sizeof(double2), cudaMemcpyHostToDevice, c->stream));
             Ud = c->Z;
         }
-        CK(img::launch_psi_adj_wide(c->dj, Ud, true, on_device ? out : c->outd, Q, p, om,
+        CK(img::launch_psi_adj_wide(c->dj, Ud, true, 0, on_device ? out : c->outd, Q, p, om,
                                     c->stream));
         if (on_device == 2) return IMG_OK;
         if (on_device) return sync(c);
@@ -718,6 +718,7 @@ img_status img_snapshot_ls_image(img_ctx *const *snap, int K, int maxit, double 
     double *yk = reinterpret_cast<double *>(take((size_t)Q * sizeof(double)));
     double *sig = reinterpret_cast<double *>(take((size_t)Q * sizeof(double)));
     b.sc = reinterpret_cast<double *>(take(img::kLsScalars * sizeof(double)));
+    b.wmax = c0->hj.opmax + img::kOpMax;
 
     img::SnapPtrs sp{};
     img::LsSnap s;
@@ -763,7 +764,7 @@ img_status img_snapshot_ls_image(img_ctx *const *snap, int K, int maxit, double 
         }
     }
     if (it > lim) it = lim;
-    CK(img::ls_finish(s.hj[0], b, on_device ? sigma : sig, nullptr, stream));
+    CK(img::ls_finish(s.hj[0], b, on_device ? sigma : sig, stream));
     if (!on_device) CK(cudaMemcpyAsync(sigma, sig, (size_t)Q * sizeof(double), cudaMemcpyDeviceToHost, stream));
     CK(cudaStreamSynchronize(stream));
     const double secs = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
@@ -830,6 +831,7 @@ img_status img_ls_image(img_ctx *c, int maxit, double *sigma, img_solve_info *in
     b.y = reinterpret_cast<double *>(take((size_t)Q * sizeof(double)));
     double *sig = reinterpret_cast<double *>(take((size_t)Q * sizeof(double)));
     b.sc = reinterpret_cast<double *>(take(img::kLsScalars * sizeof(double)));
+    b.wmax = c->hj.opmax + img::kOpMax;
     const auto t0 = std::chrono::steady_clock::now();
     CK(img::ls_begin(c->dj, c->hj, b, mode, c->stream));
     const int lim = maxit > 0 ? maxit : 200;
@@ -875,7 +877,7 @@ img_status img_ls_image(img_ctx *c, int maxit, double *sigma, img_solve_info *in
         }
     }
     if (it > lim) it = lim;
-    CK(img::ls_finish(c->hj, b, on_device ? sigma : sig, nullptr, c->stream));
+    CK(img::ls_finish(c->hj, b, on_device ? sigma : sig, c->stream));
     if (!on_device) CK(cudaMemcpyAsync(sigma, sig, (size_t)Q * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     const double secs = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();

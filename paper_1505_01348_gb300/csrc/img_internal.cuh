@@ -114,18 +114,26 @@ cudaError_t launch_psi(const JobDev *job_dev, const float *wx, float2 *part, int
 // Bounded-wait self-test (one CTA; *status: IMG_OK or IMG_ETIMEOUT).
 cudaError_t launch_wait_selftest(unsigned polls, int arrive, int *status, cudaStream_t st);
 
+// CTAs that leave per-CTA maxima of an operand (JobDev::opmax).
+constexpr int kOpMax = 256;
+
 // Full-image LSQR (all pixels free): device vectors and FP64 scalars
 // (kLsScalars doubles, indexed by kLs*); Q floats v, w, x, wx,
 // Q doubles y; p x p complex u, Mv, T1, Uw (FP32) and Kd (FP64).
-constexpr int kLsScalars = 16;
-enum : int { kLsSsU = 0, kLsSsV, kLsAlpha, kLsBeta, kLsRhobar, kLsPhibar, kLsAnorm2, kLsT1, kLsT2, kLsIa,
-             kLsBnorm, kLsRnorm, kLsArnorm, kLsUs, kLsXnorm2, kLsCount };
-static_assert(kLsCount <= kLsScalars, "LSQR scalar block");
+// kLsRedU, kLsRedV: 32 partial sums of ||u||^2, ||v||^2 (or ||x||^2) each.  The
+// scalars are in two sets, each written by a kernel that reads the other, so
+// that every CTA of either can form what it needs itself.
+enum : int { kLsAlpha = 0, kLsRhobar, kLsPhibar, kLsAnorm2, kLsRnorm, kLsArnorm,              // with v
+             kLsBeta, kLsUs, kLsBnorm, kLsRho, kLsC, kLsSn, kLsPhi, kLsPhibarU, kLsAnorm2U,   // with u
+             kLsXnorm2, kLsCount, kLsRedU = 32, kLsRedV = 64 };
+constexpr int kLsScalars = 96;
+static_assert(kLsCount <= kLsRedU, "LSQR scalar block");
 struct LsBufs {
     float2 *u, *Mv, *T1, *Uw;
     double2 *Kd;
     float *v, *w, *x, *wx;
     double *y, *sc;
+    float *wmax;               // per-CTA maxima of wx (kOpMax floats)
 };
 // u = b / ||b||, v = M^H u / alpha, w = v, x = 0 (eq. initbeta, eq. initu).
 cudaError_t ls_begin(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, cudaStream_t st);
@@ -134,8 +142,8 @@ cudaError_t ls_begin(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, cu
 // 1/2: tensor-core operators (fwd_part scratch).
 cudaError_t ls_iterate(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, float *fwd_part, float2 *part,
                        int nparts, cudaStream_t st);
-// sigma = scale o x (device, Q doubles); *xnorm2 (device) = ||x||^2 if given.
-cudaError_t ls_finish(const JobDev &hj, LsBufs &b, double *sigma, double *xnorm2, cudaStream_t st);
+// sigma = scale o x (device, Q doubles); ls_xnorm2: *out (device) = ||x||^2.
+cudaError_t ls_finish(const JobDev &hj, LsBufs &b, double *sigma, cudaStream_t st);
 cudaError_t ls_xnorm2(const JobDev &hj, LsBufs &b, double *out, cudaStream_t st);
 
 // Per-snapshot arrays for the K-snapshot dirty images (passed by value).
@@ -164,15 +172,14 @@ cudaError_t ls_snap_iterate(const LsSnap &s, LsBufs &b, cudaStream_t st);
 cudaError_t launch_snap_scale(const SnapPtrs &sp, int K, int Q, int pwls, double C, float *scale, cudaStream_t st);
 
 // Tensor-core forward K = Psi w (p <= 384, mode 1 or 2).  The pixel weights w
-// (Q floats) are made here from x (FP64), or as sc o xf (FP32), or taken as
-// they are (x and sc null); wmax: kOpMax floats of scratch.  part: a scratch of
+// (Q floats) are made here from x (FP64) or taken as they are (x null); wmax:
+// kOpMax floats of scratch, or (nmax > 0) the first nmax hold the maxima.  part: a scratch of
 // psi_wide_part_floats(SMs) floats; K (p x p, interleaved complex) to K64 or,
 // when that is null, K32.
-constexpr int kOpMax = 256;
 struct FwdIn {
     const double *x;
-    const float *sc, *xf;
     float *w, *wmax;
+    int nmax;
 };
 size_t psi_wide_part_floats(int sms);
 cudaError_t launch_psi_wide(const JobDev *job_dev, const FwdIn &in, float *part, int Q, int p, int n_l, int n_m, int mode,
@@ -180,8 +187,9 @@ cudaError_t launch_psi_wide(const JobDev *job_dev, const FwdIn &in, float *part,
 // Wide tensor-core adjoint (64 < p <= 256, mode 1 or 2) from U in FP32
 // (u64 false) or FP64 complex (converted while the operand image is
 // written).
-cudaError_t launch_psi_adj_wide(const JobDev *job_dev, const void *U, bool u64, double *out, int Q, int p, int mode,
-                                cudaStream_t st);
+// nmax > 0: the job's opmax already holds nmax per-CTA maxima of |U|.
+cudaError_t launch_psi_adj_wide(const JobDev *job_dev, const void *U, bool u64, int nmax, double *out, int Q, int p,
+                                int mode, cudaStream_t st);
 cudaError_t launch_psi_adj(const JobDev *job_dev, const float2 *U, double *out, int Q, int p,
                            int mode, cudaStream_t st);
 cudaError_t launch_z2c(const double2 *src, float2 *dst, int n, cudaStream_t st);

@@ -312,14 +312,13 @@ struct FwdMap {
     int idx[6][3];      // 2 Kp <= 768 features: 6 row blocks of 128, 3 column blocks of 256
 };
 
-// Pixel weights of a forward as FP32, w = x (FP64), w = s o x (FP32), or w as
-// it is (x null), and their maximum, one value per CTA.
-__global__ void k_fwd_weights(const double *x, const float *sc, const float *xf, float *w, int Q, float *wmax) {
+// Pixel weights of a forward as FP32, w = x (FP64) or as they are (x null),
+// and their maximum, one value per CTA.
+__global__ void k_fwd_weights(const double *x, float *w, int Q, float *wmax) {
     float mx = 0.f;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Q; i += gridDim.x * blockDim.x) {
         float v;
         if (x) w[i] = v = (float)x[i];
-        else if (sc) w[i] = v = sc[i] * xf[i];
         else v = w[i];
         mx = fmaxf(mx, fabsf(v));
     }
@@ -401,59 +400,45 @@ __global__ void __launch_bounds__(256) k_fwd_assemble(int p, const float *part, 
 // one-CTA reductions in a fixed order, and a one-thread kernel for the FP64
 // scalar recurrences, whose results later kernels read from device memory.
 
-// out = sum of squares of n floats (complex: 2n floats), one CTA, fixed order.
-__global__ void k_sumsq(const float *x, int n, double *out) {
-    __shared__ double red[32];
+// Sums of squares in the order of one CTA of 1024 threads: virtual thread t
+// takes entries t, t + 1024, ..., its warp's butterfly gives one of 32 partial
+// sums, which are added in warp order (ls_sum32).  The virtual warps are 32
+// CTAs of one warp each: on one SM the FP64 additions alone took 15 us for
+// 32,768 entries.
+constexpr int kLsWarps = 32;
+template <class F>
+__device__ __forceinline__ void ls_sumsq_warp(int n, double *red, F value) {
     double acc = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) acc = fma((double)x[i], (double)x[i], acc);
+    int i = blockIdx.x * 32 + threadIdx.x;
+    constexpr int st = 32 * kLsWarps, U = 8;
+    for (; i + (U - 1) * st < n; i += U * st) {
+        float x[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) x[q] = value(i + q * st);
+#pragma unroll
+        for (int q = 0; q < U; ++q) acc = fma((double)x[q], (double)x[q], acc);
+    }
+    for (; i < n; i += st) {
+        const float x = value(i);
+        acc = fma((double)x, (double)x, acc);
+    }
     for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        *out = s;
-    }
+    if (threadIdx.x == 0) red[blockIdx.x] = acc;
 }
-
-// FP64 scalars (one thread).  phase 0: beta of b; 1: alpha of the first v;
-// 2: beta of an iteration; 3: alpha, rotation and update coefficients.
-__global__ void k_ls_scalar(double *sc, int phase) {
-    if (threadIdx.x != 0) return;
-    if (phase == 0) {
-        const double beta = sqrt(sc[kLsSsU]);
-        sc[kLsBeta] = beta;
-        sc[kLsBnorm] = beta;
-        sc[kLsUs] = beta > 0.0 ? 1.0 / beta : 0.0;
-    } else if (phase == 1) {
-        const double alpha = sqrt(sc[kLsSsV]);
-        sc[kLsAlpha] = alpha;
-        sc[kLsIa] = alpha > 0.0 ? 1.0 / alpha : 1.0;
-        sc[kLsPhibar] = sc[kLsBeta];
-        sc[kLsRhobar] = alpha;
-        sc[kLsAnorm2] = 0.0;
-        sc[kLsRnorm] = sc[kLsBeta];
-        sc[kLsArnorm] = alpha * sc[kLsBeta];
-    } else if (phase == 2) {
-        const double beta = sqrt(sc[kLsSsU]), alpha = sc[kLsAlpha];
-        sc[kLsBeta] = beta;
-        sc[kLsUs] = beta > 0.0 ? 1.0 / beta : 0.0;
-        sc[kLsAnorm2] += alpha * alpha + beta * beta;
-    } else {
-        const double alpha = sqrt(sc[kLsSsV]), beta = sc[kLsBeta];
-        const double rhobar = sc[kLsRhobar], phibar = sc[kLsPhibar];
-        const double rho = hypot(rhobar, beta);
-        const double c = rhobar / rho, s = beta / rho;
-        const double theta = s * alpha, phi = c * phibar;
-        sc[kLsAlpha] = alpha;
-        sc[kLsIa] = alpha > 0.0 ? 1.0 / alpha : 1.0;
-        sc[kLsRhobar] = -c * alpha;
-        sc[kLsPhibar] = s * phibar;
-        sc[kLsT1] = phi / rho;
-        sc[kLsT2] = -theta / rho;
-        sc[kLsRnorm] = s * phibar;
-        sc[kLsArnorm] = s * phibar * alpha * fabs(c);
-    }
+// Sum of the partial sums in order; one warp, every lane.
+__device__ __forceinline__ double ls_sum32(const double *red) {
+    const double r = red[threadIdx.x & 31];
+    double s = 0.0;
+#pragma unroll 8
+    for (int w = 0; w < kLsWarps; ++w) s += __shfl_sync(0xffffffffu, r, w);
+    return s;
+}
+__global__ void k_sumsq(const float *x, int n, double *red) {
+    ls_sumsq_warp(n, red, [&](int i) { return x[i]; });
+}
+__global__ void k_sum32(const double *red, double *out) {
+    const double s = ls_sum32(red);
+    if (threadIdx.x == 0) *out = s;
 }
 
 // u = b: vect(R_hat) (CLS) or vect(I) (PWLS, W vect(R_hat) = vect(L^-1 R L^-H)).
@@ -463,45 +448,125 @@ __global__ void k_ls_init_u(const float2 *R32, int p, int pwls, float2 *u) {
         u[e] = pwls ? make_float2(i == j ? 1.f : 0.f, 0.f) : R32[e];
     }
 }
-// u *= us (u = t / beta).
-__global__ void k_ls_scale_u(float2 *u, int pp, const double *sc) {
-    const float us = (float)sc[kLsUs];
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < pp; e += gridDim.x * blockDim.x)
-        u[e] = make_float2(u[e].x * us, u[e].y * us);
-}
-// u = Mv - alpha u.
-__global__ void k_ls_u(float2 *u, const float2 *Mv, int pp, const double *sc) {
+// u = Mv - alpha u (n floats) and the partial sums of ||u||^2.
+__global__ void k_ls_u(float *u, const float *Mv, int n, double *sc) {
     const float a = (float)sc[kLsAlpha];
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < pp; e += gridDim.x * blockDim.x) {
-        const float2 m = Mv[e], o = u[e];
-        u[e] = make_float2(m.x - a * o.x, m.y - a * o.y);
+    ls_sumsq_warp(n, sc + kLsRedU, [&](int i) {
+        const float t = __fmaf_rn(-a, u[i], Mv[i]);
+        u[i] = t;
+        return t;
+    });
+}
+// beta = ||u||, u /= beta (n complex), and max |u| per CTA into umax; CTA 0
+// also leaves the scalars that go with u: beta and 1 / beta, and (not first)
+// ||B||^2 and the plane rotation's part that needs no alpha.
+__global__ void k_ls_scale_u(float2 *u, int n, double *sc, int first, float *umax) {
+    __shared__ float s_us;
+    const int lane = threadIdx.x & 31;
+    const bool w0 = threadIdx.x < 32;
+    double beta = 0.0, us = 0.0;
+    if (w0) {
+        beta = sqrt(ls_sum32(sc + kLsRedU));
+        us = beta > 0.0 ? 1.0 / beta : 0.0;
+        if (lane == 0) s_us = (float)us;
     }
+    __syncthreads();
+    const float f = s_us;
+    float mx = 0.f;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+        const float2 t = make_float2(u[e].x * f, u[e].y * f);
+        u[e] = t;
+        mx = fmaxf(mx, fmaxf(fabsf(t.x), fabsf(t.y)));
+    }
+    mx = cta_max_t0(mx);
+    if (threadIdx.x == 0) umax[blockIdx.x] = mx;
+    if (blockIdx.x != 0 || !w0) return;
+    double anorm2 = sc[kLsAnorm2], rho = 0.0, c = 0.0, sn = 0.0;
+    if (!first) {
+        const double alpha = sc[kLsAlpha], rhobar = sc[kLsRhobar];
+        anorm2 += alpha * alpha + beta * beta;
+        rho = hypot(rhobar, beta);
+        const double q = (lane == 0 ? rhobar : beta) / rho;
+        c = __shfl_sync(0xffffffffu, q, 0);
+        sn = __shfl_sync(0xffffffffu, q, 1);
+    }
+    if (lane != 0) return;
+    sc[kLsBeta] = beta;
+    sc[kLsUs] = us;
+    if (first) {
+        sc[kLsBnorm] = beta;
+        return;
+    }
+    const double phibar = sc[kLsPhibar];
+    sc[kLsAnorm2U] = anorm2;
+    sc[kLsRho] = rho;
+    sc[kLsC] = c;
+    sc[kLsSn] = sn;
+    sc[kLsPhi] = c * phibar;
+    sc[kLsPhibarU] = sn * phibar;
 }
-// wx = scale o v (the forward's pixel weights, D^-1 v for PWLS).
-__global__ void k_ls_weights(const float *scale, const float *v, float *wx, int Q) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Q; i += gridDim.x * blockDim.x) wx[i] = scale[i] * v[i];
-}
-// v = scale o y - beta v (first = true: v = scale o y).
-__global__ void k_ls_v(float *v, const double *y, const float *scale, int Q, const double *sc, int first) {
+// v = scale o y - beta v (first: v = scale o y) and the partial sums of ||v||^2.
+__global__ void k_ls_v(float *v, const double *y, const float *scale, int Q, double *sc, int first) {
     const float b = first ? 0.f : (float)sc[kLsBeta];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Q; i += gridDim.x * blockDim.x)
-        v[i] = scale[i] * (float)y[i] - (first ? 0.f : b * v[i]);
+    ls_sumsq_warp(Q, sc + kLsRedV, [&](int i) {
+        const float t = __fmaf_rn(scale[i], (float)y[i], first ? 0.f : -__fmul_rn(b, v[i]));
+        v[i] = t;
+        return t;
+    });
 }
-// v /= alpha; first: w = v, x = 0; else x += t1 w, w = v + t2 w.
-__global__ void k_ls_xw(float *x, float *w, float *v, int Q, const double *sc, int first) {
-    const float ia = (float)sc[kLsIa], t1 = (float)sc[kLsT1], t2 = (float)sc[kLsT2];
+// alpha = ||v||, v /= alpha; first: w = v, x = 0; else x += t1 w, w = v + t2 w;
+// the next forward's pixel weights wx = scale o v and their maximum per CTA;
+// CTA 0 leaves the scalars that go with v.
+__global__ void k_ls_xw(float *x, float *w, float *v, int Q, double *sc, int first, const float *scale, float *wx,
+                        float *wmax) {
+    __shared__ float s_c[3];                        // t1, t2, 1 / alpha
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x & 31;
+        const double alpha = sqrt(ls_sum32(sc + kLsRedV));
+        const double rho = first ? 1.0 : sc[kLsRho], c = sc[kLsC], sn = sc[kLsSn], phi = sc[kLsPhi];
+        const double theta = sn * alpha;
+        const double q = (lane == 0 ? phi : lane == 1 ? -theta : 1.0) / (lane == 2 ? alpha : rho);
+        if (lane < 2) s_c[lane] = first ? 0.f : (float)q;
+        if (lane == 2) s_c[2] = alpha > 0.0 ? (float)q : 1.f;
+        if (blockIdx.x == 0 && lane == 0) {
+            const double beta = sc[kLsBeta];
+            sc[kLsAlpha] = alpha;
+            if (first) {
+                sc[kLsPhibar] = beta;
+                sc[kLsRhobar] = alpha;
+                sc[kLsAnorm2] = 0.0;
+                sc[kLsRnorm] = beta;
+                sc[kLsArnorm] = alpha * beta;
+            } else {
+                const double phibar = sc[kLsPhibarU];
+                sc[kLsPhibar] = phibar;
+                sc[kLsRhobar] = -c * alpha;
+                sc[kLsAnorm2] = sc[kLsAnorm2U];
+                sc[kLsRnorm] = phibar;
+                sc[kLsArnorm] = phibar * alpha * fabs(c);
+            }
+        }
+    }
+    __syncthreads();
+    const float t1 = s_c[0], t2 = s_c[1], ia = s_c[2];
+    float mx = 0.f;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Q; i += gridDim.x * blockDim.x) {
-        const float vi = v[i] * ia;
+        const float vi = __fmul_rn(v[i], ia);
         v[i] = vi;
         if (first) {
             w[i] = vi;
             x[i] = 0.f;
         } else {
             const float wi = w[i];
-            x[i] += t1 * wi;
-            w[i] = vi + t2 * wi;
+            x[i] = __fmaf_rn(t1, wi, x[i]);
+            w[i] = __fmaf_rn(t2, wi, vi);
         }
+        const float wv = scale[i] * vi;
+        wx[i] = wv;
+        mx = fmaxf(mx, fabsf(wv));
     }
+    mx = cta_max_t0(mx);
+    if (threadIdx.x == 0) wmax[blockIdx.x] = mx;
 }
 __global__ void k_ls_sigma(const float *x, const float *scale, double *sigma, int Q) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Q; i += gridDim.x * blockDim.x)
@@ -513,15 +578,21 @@ __global__ void k_d2c(const double2 *src, float2 *dst, int n) {
 }
 
 // C = op(A) op(B), p x p complex FP32 column-major; op 0: as is, 1: conjugate
-// transpose.  32 x 32 output tiles, 256 threads (2 x 2 outputs each).
-__global__ void k_cgemm(int p, const float2 *A, int opA, const float2 *B, int opB, float2 *C) {
-    __shared__ float2 As[32][33], Bs[32][33];
-    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+// transpose.  16 x 16 output tiles, 64 threads (2 x 2 outputs each): small
+// tiles, because p = 128 makes only 16 of 32 x 32 (13.6 us, a chain of shared
+// loads on 16 SMs).  cmax (may be null): max |C| per CTA.
+__global__ void __launch_bounds__(64) k_cgemm(int p, const float2 *A, int opA, const float2 *B, int opB, float2 *C,
+                                              float *cmax) {
+    constexpr int kT = 16, kK = 32;
+    __shared__ float2 As[kT][kK + 1], Bs[kK][kT + 1];
+    const int i0 = blockIdx.x * kT, j0 = blockIdx.y * kT;
+    const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
     float2 acc[2][2] = {};
-    for (int k0 = 0; k0 < p; k0 += 32) {
-        for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
-            const int r = e & 31, c = e >> 5;           // As[r][c] = op(A)[i0 + r, k0 + c]
+    for (int k0 = 0; k0 < p; k0 += kK) {
+#pragma unroll
+        for (int e = threadIdx.x; e < kT * kK; e += 64) {
+            // consecutive threads along the memory's fast index
+            const int r = opA ? e / kK : e % kT, c = opA ? e % kK : e / kT;    // As[r][c] = op(A)[i0 + r, k0 + c]
             const int i = i0 + r, k = k0 + c;
             float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
             if (i < p && k < p) {
@@ -529,16 +600,17 @@ __global__ void k_cgemm(int p, const float2 *A, int opA, const float2 *B, int op
                 if (opA) a.y = -a.y;
             }
             As[r][c] = a;
-            const int kk = k0 + r, j = j0 + c;          // Bs[r][c] = op(B)[k0 + r, j0 + c]
+            const int rb = opB ? e / kT : e % kK, cb = opB ? e % kT : e / kK;  // Bs[rb][cb] = op(B)[k0 + rb, j0 + cb]
+            const int kk = k0 + rb, j = j0 + cb;
             if (kk < p && j < p) {
                 b = opB ? B[(size_t)kk * p + j] : B[(size_t)j * p + kk];
                 if (opB) b.y = -b.y;
             }
-            Bs[r][c] = b;
+            Bs[rb][cb] = b;
         }
         __syncthreads();
 #pragma unroll 8
-        for (int kk = 0; kk < 32; ++kk) {
+        for (int kk = 0; kk < kK; ++kk) {
 #pragma unroll
             for (int a = 0; a < 2; ++a)
 #pragma unroll
@@ -546,13 +618,19 @@ __global__ void k_cgemm(int p, const float2 *A, int opA, const float2 *B, int op
         }
         __syncthreads();
     }
+    float mx = 0.f;
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
             const int i = i0 + 2 * ty + a, j = j0 + 2 * tx + b;
-            if (i < p && j < p) C[(size_t)j * p + i] = acc[a][b];
+            if (i >= p || j >= p) continue;
+            C[(size_t)j * p + i] = acc[a][b];
+            mx = fmaxf(mx, fmaxf(fabsf(acc[a][b].x), fabsf(acc[a][b].y)));
         }
+    if (!cmax) return;
+    mx = cta_max_t0(mx);
+    if (threadIdx.x == 0) cmax[blockIdx.y * gridDim.x + blockIdx.x] = mx;
 }
 
 // ---------------------------------------------------------------- failure detection
@@ -2105,8 +2183,11 @@ cudaError_t launch_psi_wide(const JobDev *job_dev, const FwdIn &in, float *part,
     const int sms = num_sms();
     const int nblk = fwd_nblocks(n_l, n_m);
     const int S = max(1, min(nblk, sms / map.np));
-    const int nmax = max(1, min(min(sms, kOpMax), (Q + 4 * kThreads - 1) / (4 * kThreads)));
-    k_fwd_weights<<<nmax, kThreads, 0, st>>>(in.x, in.sc, in.xf, in.w, Q, in.wmax);
+    int nmax = in.nmax;
+    if (nmax == 0) {
+        nmax = max(1, min(min(sms, kOpMax), (Q + 4 * kThreads - 1) / (4 * kThreads)));
+        k_fwd_weights<<<nmax, kThreads, 0, st>>>(in.x, in.w, Q, in.wmax);
+    }
     const size_t sm = fwd_smem_bytes();
     cudaError_t e = (mode == 1) ? ensure_smem((const void *)k_fwd_wide<1>, sm) : ensure_smem((const void *)k_fwd_wide<2>, sm);
     if (e != cudaSuccess) return e;
@@ -2122,78 +2203,85 @@ cudaError_t launch_psi_wide(const JobDev *job_dev, const FwdIn &in, float *part,
 
 // ---------------------------------------------------------------- full-image LSQR launchers
 static inline int ls_grid(int n) { return max(1, min(4 * num_sms(), (n + kThreads - 1) / kThreads)); }
+// Grid of the kernels that leave per-CTA maxima.
+static inline int ls_max_grid(int n) { return max(1, min(kOpMax, (n + kThreads - 1) / kThreads)); }
 
+// M v from the pixel weights wx that the vector step left.
 cudaError_t ls_forward(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, float *fwd_part, float2 *part,
                        int nparts, cudaStream_t st) {
     const int Q = hj.Q, p = hj.p, pp = p * p;
     cudaError_t e;
     if (mode != 0) {
-        // pixel weights D^-1 v; K straight to FP32
-        const FwdIn in{nullptr, hj.scale, b.v, b.wx, hj.opmax + kOpMax};
+        const FwdIn in{nullptr, b.wx, b.wmax, ls_max_grid(Q)};
         e = launch_psi_wide(jd, in, fwd_part, Q, p, hj.n_l, hj.n_m, mode, nullptr, reinterpret_cast<float *>(b.Mv), st);
     } else {
-        k_ls_weights<<<ls_grid(Q), kThreads, 0, st>>>(hj.scale, b.v, b.wx, Q);
         e = launch_psi(jd, b.wx, part, nparts, Q, p, 0, b.Kd, st);
         if (e == cudaSuccess) k_d2c<<<ls_grid(pp), kThreads, 0, st>>>(b.Kd, b.Mv, pp);
     }
     if (e != cudaSuccess) return e;
     if (hj.cost == IMG_COST_PWLS) {
         // W vect(K) = vect(L^-1 K L^-H)
-        const dim3 g((p + 31) / 32, (p + 31) / 32);
-        k_cgemm<<<g, kThreads, 0, st>>>(p, b.Mv, 0, hj.Li32, 1, b.T1);
-        k_cgemm<<<g, kThreads, 0, st>>>(p, hj.Li32, 0, b.T1, 0, b.Mv);
+        const dim3 g((p + 15) / 16, (p + 15) / 16);
+        k_cgemm<<<g, 64, 0, st>>>(p, b.Mv, 0, hj.Li32, 1, b.T1, nullptr);
+        k_cgemm<<<g, 64, 0, st>>>(p, hj.Li32, 0, b.T1, 0, b.Mv, nullptr);
     }
     return cudaGetLastError();
 }
 
-cudaError_t ls_adjoint(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, cudaStream_t st) {
+// b.y = M^H u.  numax: per-CTA maxima of |u| in the job's opmax (CLS; 0 when
+// they are not there).
+cudaError_t ls_adjoint(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, int numax, cudaStream_t st) {
     const int Q = hj.Q, p = hj.p;
     const float2 *U = b.u;
     if (hj.cost == IMG_COST_PWLS) {
         // W^H vect(u) = vect(L^-H u L^-1)
-        const dim3 g((p + 31) / 32, (p + 31) / 32);
-        k_cgemm<<<g, kThreads, 0, st>>>(p, b.u, 0, hj.Li32, 0, b.T1);
-        k_cgemm<<<g, kThreads, 0, st>>>(p, hj.Li32, 1, b.T1, 0, b.Uw);
+        const dim3 g((p + 15) / 16, (p + 15) / 16);
+        const bool fits = (int)(g.x * g.y) <= kOpMax;
+        k_cgemm<<<g, 64, 0, st>>>(p, b.u, 0, hj.Li32, 0, b.T1, nullptr);
+        k_cgemm<<<g, 64, 0, st>>>(p, hj.Li32, 1, b.T1, 0, b.Uw, fits ? hj.opmax : nullptr);
         U = b.Uw;
+        numax = fits ? (int)(g.x * g.y) : 0;
     }
-    cudaError_t e = mode != 0 ? launch_psi_adj_wide(jd, U, false, b.y, Q, p, mode, st)
+    cudaError_t e = mode != 0 ? launch_psi_adj_wide(jd, U, false, numax, b.y, Q, p, mode, st)
                               : launch_psi_adj(jd, U, b.y, Q, p, 0, st);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
+// beta, u / beta (n complex); then v, alpha and the vector updates once b.y
+// holds M^H u.
+static void ls_u_step(const JobDev &hj, LsBufs &b, int n, int first, cudaStream_t st) {
+    k_ls_scale_u<<<ls_max_grid(n), kThreads, 0, st>>>(b.u, n, b.sc, first, hj.opmax);
+}
+static void ls_v_step(const JobDev &hj, LsBufs &b, int first, cudaStream_t st) {
+    const int Q = hj.Q;
+    k_ls_v<<<kLsWarps, 32, 0, st>>>(b.v, b.y, hj.scale, Q, b.sc, first);
+    k_ls_xw<<<ls_max_grid(Q), kThreads, 0, st>>>(b.x, b.w, b.v, Q, b.sc, first, hj.scale, b.wx, b.wmax);
+}
+
 cudaError_t ls_begin(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, cudaStream_t st) {
-    const int Q = hj.Q, p = hj.p, pp = p * p;
+    const int p = hj.p, pp = p * p;
     k_ls_init_u<<<ls_grid(pp), kThreads, 0, st>>>(hj.R32, p, hj.cost == IMG_COST_PWLS, b.u);
-    k_sumsq<<<1, 1024, 0, st>>>(reinterpret_cast<const float *>(b.u), 2 * pp, b.sc + kLsSsU);
-    k_ls_scalar<<<1, 32, 0, st>>>(b.sc, 0);
-    k_ls_scale_u<<<ls_grid(pp), kThreads, 0, st>>>(b.u, pp, b.sc);
-    cudaError_t e = ls_adjoint(jd, hj, b, mode, st);
+    k_sumsq<<<kLsWarps, 32, 0, st>>>(reinterpret_cast<const float *>(b.u), 2 * pp, b.sc + kLsRedU);
+    ls_u_step(hj, b, pp, 1, st);
+    cudaError_t e = ls_adjoint(jd, hj, b, mode, ls_max_grid(pp), st);
     if (e != cudaSuccess) return e;
-    k_ls_v<<<ls_grid(Q), kThreads, 0, st>>>(b.v, b.y, hj.scale, Q, b.sc, 1);
-    k_sumsq<<<1, 1024, 0, st>>>(b.v, Q, b.sc + kLsSsV);
-    k_ls_scalar<<<1, 32, 0, st>>>(b.sc, 1);
-    k_ls_xw<<<ls_grid(Q), kThreads, 0, st>>>(b.x, b.w, b.v, Q, b.sc, 1);
+    ls_v_step(hj, b, 1, st);
     return cudaGetLastError();
 }
 
 cudaError_t ls_iterate(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, float *fwd_part, float2 *part,
                        int nparts, cudaStream_t st) {
-    const int Q = hj.Q, pp = hj.p * hj.p;
+    const int pp = hj.p * hj.p;
     // u <- M v - alpha u, beta = ||u||, u <- u / beta
     cudaError_t e = ls_forward(jd, hj, b, mode, fwd_part, part, nparts, st);
     if (e != cudaSuccess) return e;
-    k_ls_u<<<ls_grid(pp), kThreads, 0, st>>>(b.u, b.Mv, pp, b.sc);
-    k_sumsq<<<1, 1024, 0, st>>>(reinterpret_cast<const float *>(b.u), 2 * pp, b.sc + kLsSsU);
-    k_ls_scalar<<<1, 32, 0, st>>>(b.sc, 2);
-    k_ls_scale_u<<<ls_grid(pp), kThreads, 0, st>>>(b.u, pp, b.sc);
+    k_ls_u<<<kLsWarps, 32, 0, st>>>(reinterpret_cast<float *>(b.u), reinterpret_cast<const float *>(b.Mv), 2 * pp, b.sc);
+    ls_u_step(hj, b, pp, 0, st);
     // v <- M^H u - beta v, alpha = ||v||, rotation, x and w updates
-    e = ls_adjoint(jd, hj, b, mode, st);
+    e = ls_adjoint(jd, hj, b, mode, ls_max_grid(pp), st);
     if (e != cudaSuccess) return e;
-    k_ls_v<<<ls_grid(Q), kThreads, 0, st>>>(b.v, b.y, hj.scale, Q, b.sc, 0);
-    k_sumsq<<<1, 1024, 0, st>>>(b.v, Q, b.sc + kLsSsV);
-    k_ls_scalar<<<1, 32, 0, st>>>(b.sc, 3);
-    k_ls_xw<<<ls_grid(Q), kThreads, 0, st>>>(b.x, b.w, b.v, Q, b.sc, 0);
+    ls_v_step(hj, b, 0, st);
     return cudaGetLastError();
 }
 
@@ -2235,7 +2323,8 @@ static cudaError_t snap_adjoint(const LsSnap &s, LsBufs &b, cudaStream_t st) {
     const int Q = s.hj[0].Q;
     for (int k = 0; k < s.K; ++k) {
         LsBufs bk = snap_bufs(s, b, k);
-        cudaError_t e = ls_adjoint(s.jd[k], s.hj[k], bk, s.mode[k], st);
+        // the maxima of the K blocks of u together are no block's own
+        cudaError_t e = ls_adjoint(s.jd[k], s.hj[k], bk, s.mode[k], 0, st);
         if (e != cudaSuccess) return e;
         k_ls_accum<<<ls_grid(Q), kThreads, 0, st>>>(b.y, s.yk, Q, k == 0);
     }
@@ -2253,47 +2342,38 @@ static cudaError_t snap_forward(const LsSnap &s, LsBufs &b, cudaStream_t st) {
 }
 
 cudaError_t ls_snap_begin(const LsSnap &s, LsBufs &b, cudaStream_t st) {
-    const int Q = s.hj[0].Q, p = s.hj[0].p, pp = p * p, n = s.K * pp;
+    const int p = s.hj[0].p, pp = p * p, n = s.K * pp;
     const int pwls = s.hj[0].cost == IMG_COST_PWLS;
     for (int k = 0; k < s.K; ++k)
         k_ls_init_u<<<ls_grid(pp), kThreads, 0, st>>>(s.hj[k].R32, p, pwls, b.u + (size_t)k * pp);
-    k_sumsq<<<1, 1024, 0, st>>>(reinterpret_cast<const float *>(b.u), 2 * n, b.sc + kLsSsU);
-    k_ls_scalar<<<1, 32, 0, st>>>(b.sc, 0);
-    k_ls_scale_u<<<ls_grid(n), kThreads, 0, st>>>(b.u, n, b.sc);
+    k_sumsq<<<kLsWarps, 32, 0, st>>>(reinterpret_cast<const float *>(b.u), 2 * n, b.sc + kLsRedU);
+    ls_u_step(s.hj[0], b, n, 1, st);
     cudaError_t e = snap_adjoint(s, b, st);
     if (e != cudaSuccess) return e;
-    k_ls_v<<<ls_grid(Q), kThreads, 0, st>>>(b.v, b.y, s.hj[0].scale, Q, b.sc, 1);
-    k_sumsq<<<1, 1024, 0, st>>>(b.v, Q, b.sc + kLsSsV);
-    k_ls_scalar<<<1, 32, 0, st>>>(b.sc, 1);
-    k_ls_xw<<<ls_grid(Q), kThreads, 0, st>>>(b.x, b.w, b.v, Q, b.sc, 1);
+    ls_v_step(s.hj[0], b, 1, st);
     return cudaGetLastError();
 }
 
 cudaError_t ls_snap_iterate(const LsSnap &s, LsBufs &b, cudaStream_t st) {
-    const int Q = s.hj[0].Q, pp = s.hj[0].p * s.hj[0].p, n = s.K * pp;
+    const int pp = s.hj[0].p * s.hj[0].p, n = s.K * pp;
     cudaError_t e = snap_forward(s, b, st);
     if (e != cudaSuccess) return e;
-    k_ls_u<<<ls_grid(n), kThreads, 0, st>>>(b.u, b.Mv, n, b.sc);
-    k_sumsq<<<1, 1024, 0, st>>>(reinterpret_cast<const float *>(b.u), 2 * n, b.sc + kLsSsU);
-    k_ls_scalar<<<1, 32, 0, st>>>(b.sc, 2);
-    k_ls_scale_u<<<ls_grid(n), kThreads, 0, st>>>(b.u, n, b.sc);
+    k_ls_u<<<kLsWarps, 32, 0, st>>>(reinterpret_cast<float *>(b.u), reinterpret_cast<const float *>(b.Mv), 2 * n, b.sc);
+    ls_u_step(s.hj[0], b, n, 0, st);
     e = snap_adjoint(s, b, st);
     if (e != cudaSuccess) return e;
-    k_ls_v<<<ls_grid(Q), kThreads, 0, st>>>(b.v, b.y, s.hj[0].scale, Q, b.sc, 0);
-    k_sumsq<<<1, 1024, 0, st>>>(b.v, Q, b.sc + kLsSsV);
-    k_ls_scalar<<<1, 32, 0, st>>>(b.sc, 3);
-    k_ls_xw<<<ls_grid(Q), kThreads, 0, st>>>(b.x, b.w, b.v, Q, b.sc, 0);
+    ls_v_step(s.hj[0], b, 0, st);
     return cudaGetLastError();
 }
 
-cudaError_t ls_finish(const JobDev &hj, LsBufs &b, double *sigma, double *xnorm2, cudaStream_t st) {
+cudaError_t ls_finish(const JobDev &hj, LsBufs &b, double *sigma, cudaStream_t st) {
     k_ls_sigma<<<ls_grid(hj.Q), kThreads, 0, st>>>(b.x, hj.scale, sigma, hj.Q);
-    if (xnorm2) k_sumsq<<<1, 1024, 0, st>>>(b.x, hj.Q, xnorm2);
     return cudaGetLastError();
 }
 
 cudaError_t ls_xnorm2(const JobDev &hj, LsBufs &b, double *out, cudaStream_t st) {
-    k_sumsq<<<1, 1024, 0, st>>>(b.x, hj.Q, out);
+    k_sumsq<<<kLsWarps, 32, 0, st>>>(b.x, hj.Q, b.sc + kLsRedV);
+    k_sum32<<<1, 32, 0, st>>>(b.sc + kLsRedV, out);
     return cudaGetLastError();
 }
 
@@ -2309,15 +2389,16 @@ static cudaError_t launch_psi_adj_tc_t(const JobDev *job_dev, const float2 *U, d
 }
 
 template <int MODE>
-static cudaError_t launch_psi_adj_wide_t(const JobDev *job_dev, const void *U, bool u64, double *out, int Q, int p,
-                                         cudaStream_t st) {
+static cudaError_t launch_psi_adj_wide_t(const JobDev *job_dev, const void *U, bool u64, int nmax, double *out, int Q,
+                                         int p, cudaStream_t st) {
     const dim3 eg(wide_nk(p), 2 * wide_kp(p) / kEmbRows);
-    const int nmax = min(16, (p * p + kThreads - 1) / kThreads);
+    const bool have = nmax > 0;
+    if (!have) nmax = min(16, (p * p + kThreads - 1) / kThreads);
     if (u64) {
-        k_emb_max_one<double2><<<nmax, kThreads, 0, st>>>(job_dev, static_cast<const double2 *>(U));
+        if (!have) k_emb_max_one<double2><<<nmax, kThreads, 0, st>>>(job_dev, static_cast<const double2 *>(U));
         k_emb_one<MODE, double2><<<eg, kThreads, 0, st>>>(job_dev, static_cast<const double2 *>(U), nmax);
     } else {
-        k_emb_max_one<float2><<<nmax, kThreads, 0, st>>>(job_dev, static_cast<const float2 *>(U));
+        if (!have) k_emb_max_one<float2><<<nmax, kThreads, 0, st>>>(job_dev, static_cast<const float2 *>(U));
         k_emb_one<MODE, float2><<<eg, kThreads, 0, st>>>(job_dev, static_cast<const float2 *>(U), nmax);
     }
     cudaError_t e = cudaGetLastError();
@@ -2330,11 +2411,11 @@ static cudaError_t launch_psi_adj_wide_t(const JobDev *job_dev, const void *U, b
     return cudaGetLastError();
 }
 
-cudaError_t launch_psi_adj_wide(const JobDev *job_dev, const void *U, bool u64, double *out, int Q, int p, int mode,
-                                cudaStream_t st) {
+cudaError_t launch_psi_adj_wide(const JobDev *job_dev, const void *U, bool u64, int nmax, double *out, int Q, int p,
+                                int mode, cudaStream_t st) {
     if (p < 1 || p > kMaxWideP || (mode != 1 && mode != 2)) return cudaErrorInvalidValue;
-    if (mode == 1) return launch_psi_adj_wide_t<1>(job_dev, U, u64, out, Q, p, st);
-    return launch_psi_adj_wide_t<2>(job_dev, U, u64, out, Q, p, st);
+    if (mode == 1) return launch_psi_adj_wide_t<1>(job_dev, U, u64, nmax, out, Q, p, st);
+    return launch_psi_adj_wide_t<2>(job_dev, U, u64, nmax, out, Q, p, st);
 }
 
 cudaError_t launch_psi_adj(const JobDev *job_dev, const float2 *U, double *out, int Q, int p, int mode,
