@@ -1036,7 +1036,8 @@ img_status img_solve_batch(img_ctx *const *ctxs, int n, double *const *sigma, im
     }
     // wide jobs (64 < p <= 384 on tensor cores) run their solve graphs, each
     // on its context's stream after the batch's factor and bounds; the other
-    // jobs run the one-CTA solver, one launch per arithmetic group
+    // jobs run the one-CTA solver on the batch's stream, one launch per
+    // arithmetic group
     std::vector<int> wide;
     for (int j = 0; j < n; ++j)
         if (wide_of(ctxs[j])) {
@@ -1044,19 +1045,15 @@ img_status img_solve_batch(img_ctx *const *ctxs, int n, double *const *sigma, im
             if (st != IMG_OK) return st;
             wide.push_back(j);
         }
+    cudaEvent_t ready = nullptr;
     if (!wide.empty()) {
-        cudaEvent_t ready = nullptr;
         CK(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
         CK(cudaEventRecord(ready, s));
-        for (int j : wide) {
-            img_ctx *c = ctxs[j];
-            if (!c->ev) CK(cudaEventCreateWithFlags(&c->ev, cudaEventDisableTiming));
-            CK(cudaStreamWaitEvent(c->stream, ready, 0));
-            CK(img::ws_launch(c->ws, c->stream));
-            CK(cudaEventRecord(c->ev, c->stream));
-        }
-        CK(cudaEventDestroy(ready));
     }
+    // The one-CTA launches go first: streams share the hardware's queues, and
+    // in a queue behind a solve graph they would wait for the whole graph
+    // (16 channels of 48, 64 and 96 antennas with 8 queues: 388 ms instead of
+    // 215), while a graph behind them waits only until their CTAs are placed.
     if (on_device)
         CK(cudaMemcpyAsync(g_ws.sig, outs.data(), n * sizeof(double *), cudaMemcpyHostToDevice, s));
     for (int m = 0; m < kGroups; ++m) {
@@ -1073,6 +1070,16 @@ img_status img_solve_batch(img_ctx *const *ctxs, int n, double *const *sigma, im
                 CK(img::launch_solve(g_ws.jobs + q, 1, ctxs[g.order[q]]->prm.p, Groups::solve_mode(m), g_ws.infos + q,
                                      on_device ? g_ws.sig + q : nullptr, s));
         }
+    }
+    if (ready) {
+        for (int j : wide) {
+            img_ctx *c = ctxs[j];
+            if (!c->ev) CK(cudaEventCreateWithFlags(&c->ev, cudaEventDisableTiming));
+            CK(cudaStreamWaitEvent(c->stream, ready, 0));
+            CK(img::ws_launch(c->ws, c->stream));
+            CK(cudaEventRecord(c->ev, c->stream));
+        }
+        CK(cudaEventDestroy(ready));
     }
     for (int j : wide) CK(cudaStreamWaitEvent(s, ctxs[j]->ev, 0));
     std::vector<DevInfo> d(n);
