@@ -1,5 +1,6 @@
 // Host side of the C ABI declared in include/img.h: validation, device
 // memory layout of a job, and the launch sequence of every call.
+#include <atomic>
 #include <chrono>
 #include <cstdio>
 #include <cmath>
@@ -141,6 +142,7 @@ size_t carve(img_ctx *c, char *base) {
     J.Bscale = cv.take<float>(2);
     J.opmax = cv.take<float>(2 * img::kOpMax);
     J.vmax = cv.take<unsigned long long>(1);
+    J.cmd = cv.take<int>(2 + 2 * img::kSolveCtas);
     J.info = cv.take<DevInfo>(1);
     J.flags = cv.take<int>(4);
     c->dj = cv.take<JobDev>(1);
@@ -240,6 +242,32 @@ img_status copy_out_float(img_ctx *c, const float *src, double *dst, size_t n, i
     CK(img::launch_to_double(src, c->outd, (int)n, c->stream));
     return copy_out_double(c, c->outd, dst, n, 0);
 }
+
+// CTAs per job of a one-CTA-solver launch of n jobs: a cluster of up to 8
+// shares each gradient while SMs are free.  All launches in flight together
+// take at most kMaxHelpers extra CTAs, about a third of a GB300's SMs: with
+// more jobs than that at once, the SMs are better spent on one job each.  The
+// images do not depend on it.  Held until the solve has been waited for.
+constexpr int kMaxHelpers = 56;
+std::atomic<int> g_helpers{0};
+struct SolveCtas {
+    int ctas = 1, held = 0;
+    explicit SolveCtas(int n) {
+        for (int c = img::kSolveCtas; c > 1; c /= 2) {
+            const int want = n * (c - 1);
+            if (want > kMaxHelpers) continue;
+            if (g_helpers.fetch_add(want) + want <= kMaxHelpers) {
+                ctas = c;
+                held = want;
+                return;
+            }
+            g_helpers.fetch_sub(want);
+        }
+    }
+    ~SolveCtas() { g_helpers.fetch_sub(held); }
+    SolveCtas(const SolveCtas &) = delete;
+    SolveCtas &operator=(const SolveCtas &) = delete;
+};
 
 // Batch workspace shared by img_solve_batch calls (grown on demand).
 struct BatchWs {
@@ -499,12 +527,13 @@ img_status img_solve(img_ctx *c, double *sigma, img_solve_info *info, int on_dev
     if (!c || !sigma) return IMG_EINVAL;
     img_status st = prepare(c);
     if (st != IMG_OK) return st;
+    const SolveCtas share(wide_of(c) ? 0 : 1);
     if (wide_of(c)) {
         st = wide_ready(c);
         if (st != IMG_OK) return st;
         CK(img::ws_launch(c->ws, c->stream));
     } else {
-        CK(img::launch_solve(c->djp, 1, c->prm.p, mode_of(c), nullptr, nullptr, c->stream));
+        CK(img::launch_solve(c->djp, 1, c->prm.p, mode_of(c), share.ctas, nullptr, nullptr, c->stream));
     }
     DevInfo d{};
     CK(cudaMemcpyAsync(&d, c->hj.info, sizeof(DevInfo), cudaMemcpyDeviceToHost, c->stream));
@@ -1054,6 +1083,7 @@ img_status img_solve_batch(img_ctx *const *ctxs, int n, double *const *sigma, im
     // in a queue behind a solve graph they would wait for the whole graph
     // (16 channels of 48, 64 and 96 antennas with 8 queues: 388 ms instead of
     // 215), while a graph behind them waits only until their CTAs are placed.
+    const SolveCtas share(n - (int)wide.size());
     if (on_device)
         CK(cudaMemcpyAsync(g_ws.sig, outs.data(), n * sizeof(double *), cudaMemcpyHostToDevice, s));
     for (int m = 0; m < kGroups; ++m) {
@@ -1063,11 +1093,12 @@ img_status img_solve_batch(img_ctx *const *ctxs, int n, double *const *sigma, im
         if (idx.empty()) continue;
         const bool contiguous = (int)idx.size() == g.end[m] - g.begin[m];
         if (contiguous) {
-            CK(img::launch_solve(g_ws.jobs + g.begin[m], (int)idx.size(), g.max_p[m], Groups::solve_mode(m),
+            CK(img::launch_solve(g_ws.jobs + g.begin[m], (int)idx.size(), g.max_p[m], Groups::solve_mode(m), share.ctas,
                                  g_ws.infos + g.begin[m], on_device ? g_ws.sig + g.begin[m] : nullptr, s));
         } else {
             for (int q : idx)
-                CK(img::launch_solve(g_ws.jobs + q, 1, ctxs[g.order[q]]->prm.p, Groups::solve_mode(m), g_ws.infos + q,
+                CK(img::launch_solve(g_ws.jobs + q, 1, ctxs[g.order[q]]->prm.p, Groups::solve_mode(m), share.ctas,
+                                     g_ws.infos + q,
                                      on_device ? g_ws.sig + q : nullptr, s));
         }
     }
@@ -1345,7 +1376,7 @@ struct img_server {
                 CK(img::launch_factor(jp, nb, max_p, sl.s));
                 CK(img::launch_bounds(jp, nb, max_tiles, max_p, Groups::bounds_mode(md), sl.s));
                 CK(img::launch_finalize(jp, nb, max_tiles, sl.s, nullptr));
-                CK(img::launch_solve(jp, nb, max_p, Groups::solve_mode(md), sl.infos + q0, nullptr, sl.s));
+                CK(img::launch_solve(jp, nb, max_p, Groups::solve_mode(md), 1, sl.infos + q0, nullptr, sl.s));
             }
             return IMG_OK;
         };

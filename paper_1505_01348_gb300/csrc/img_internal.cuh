@@ -87,6 +87,7 @@ struct JobDev {
     float *evv;
     int ev_cap;
     int *ev_count;
+    int *cmd;              // words that the CTAs of one solve's cluster exchange
     // status and report
     DevInfo *info;
     int *flags;            // [0]: factor status, [1]: bounds valid, [2]: timeout, [3]: bad pivot
@@ -103,8 +104,10 @@ cudaError_t launch_bounds(JobDev *const *jobs, int n, int max_tiles, int max_p, 
                           cudaStream_t st);
 // max_tiles: most 64-pixel tiles of any job
 cudaError_t launch_finalize(JobDev *const *jobs, int n, int max_tiles, cudaStream_t st, int *batch_status);
-// mode: 0 CUDA-core FP32 operators, 1 tensor cores FP16x3, 2 tensor cores BF16x3
-cudaError_t launch_solve(JobDev *const *jobs, int n, int max_p, int mode, DevInfo *batch_info,
+// mode: 0 CUDA-core FP32 operators, 1 tensor cores FP16x3, 2 tensor cores BF16x3;
+// ctas: CTAs per job (1, 2, 4 or kSolveCtas: a cluster that shares the gradients)
+constexpr int kSolveCtas = 8;
+cudaError_t launch_solve(JobDev *const *jobs, int n, int max_p, int mode, int ctas, DevInfo *batch_info,
                          double *const *sigma_out, cudaStream_t st);
 // Factor, bounds and solve of each job inside its own CTA (one launch).
 cudaError_t launch_job(JobDev *const *jobs, int n, int max_p, int mode, DevInfo *batch_info,

@@ -862,17 +862,17 @@ __device__ void adjoint_list(const JobDev &J, const float2 *U, const int *pos, i
 }
 
 // Full-image adjoint with generated steering vectors: epi(i, Re(a_i^H U a_i))
-// for every pixel, on one thread per pixel.  SQ: epi(i, ||V a_i||^2) with V
+// for every pixel of tiles t0, t0 + dt, ..., on one thread per pixel.  SQ: epi(i, ||V a_i||^2) with V
 // = U on CUDA cores (U column-major) and V = U^H on tensor cores (the B
 // operand's convention), i.e. U = L^-1 resp. L^-H for the whitened MVDR
 // denominator.
 template <int MODE, bool SQ = false, class Epi, class Pre>
 __device__ void adjoint_full(const JobDev &J, const float2 *U, float2 *A, TcWork &T, float *red,
-                             double *dbuf, Epi epi, Pre pre) {
+                             double *dbuf, int t0, int dt, Epi epi, Pre pre) {
     const int Q = J.Q;
     if constexpr (MODE == 0) {
         const int ntiles = (Q + kTile - 1) / kTile;
-        for (int t = 0; t < ntiles; ++t) {
+        for (int t = t0; t < ntiles; t += dt) {
             const int pix0 = t * kTile;
             const int np = min(kTile, Q - pix0);
             fill_steer_adj(J, pix0, np, A);
@@ -890,20 +890,21 @@ __device__ void adjoint_full(const JobDev &J, const float2 *U, float2 *A, TcWork
         const float sX = tc_steer_scale(J.p);
         const float inv = SQ ? 1.f / ((sX * sB) * (sX * sB)) : 1.f / (sX * sX * sB);
         const uint32_t idesc = idesc_f16(2 * T.Kp, BF ? 1 : 0);
+        const int ntiles = tc_num_tiles(J.n_l, J.n_m);
         tc_run_tiles(
-            T, tc_num_tiles(J.n_l, J.n_m), idesc,
-            [&](int t, int b) { tc_gen_X_steer<BF>(J, T, b, t, sX); },
-            [&](int t, int b) {
+            T, t0 < ntiles ? (ntiles - 1 - t0) / dt + 1 : 0, idesc,
+            [&](int k, int b) { tc_gen_X_steer<BF>(J, T, b, t0 + k * dt, sX); },
+            [&](int k, int b) {
                 tc_epilogue<BF, SQ>(T, b, red);
                 if (threadIdx.x < kTcM) {
-                    const int i = tc_tile_pixel(t, threadIdx.x, J.n_l, J.n_m);
+                    const int i = tc_tile_pixel(t0 + k * dt, threadIdx.x, J.n_l, J.n_m);
                     if (i >= 0) epi(i, red[threadIdx.x] * inv);
                 }
                 __syncthreads();
             },
-            [&](int t) {
+            [&](int k) {
                 if (threadIdx.x < kTcM) {
-                    const int i = tc_tile_pixel(t, threadIdx.x, J.n_l, J.n_m);
+                    const int i = tc_tile_pixel(t0 + k * dt, threadIdx.x, J.n_l, J.n_m);
                     if (i >= 0) pre(i);
                 }
             });
@@ -913,7 +914,7 @@ __device__ void adjoint_full(const JobDev &J, const float2 *U, float2 *A, TcWork
 template <int MODE, bool SQ = false, class Epi>
 __device__ void adjoint_full(const JobDev &J, const float2 *U, float2 *A, TcWork &T, float *red,
                              double *dbuf, Epi epi) {
-    adjoint_full<MODE, SQ>(J, U, A, T, red, dbuf, epi, [](int) {});
+    adjoint_full<MODE, SQ>(J, U, A, T, red, dbuf, 0, 1, epi, [](int) {});
 }
 
 // LSQR (Paige-Saunders) on the free set: min || b - M_F x ||, with
@@ -1589,12 +1590,69 @@ __device__ void supp_remove(const JobDev &J, int i, int &ns) {
     __syncthreads();
 }
 
-// Persistent active-set driver (Table I), one CTA per job.  MODE selects the
-// adjoint's arithmetic (0 CUDA cores FP32, 1 tensor cores FP16x3, 2 BF16x3).
+// Gradient and multiplier test over tiles t0, t0 + dt, ...: lambda_L = g,
+// lambda_U = -g (eq. etaL, eq. etaU), FP32; the smallest lambda below its
+// threshold and its pixel, this thread's share.
+template <int MODE>
+__device__ void gradient_tiles(const JobDev &J, const float2 *Ug, float2 *A, TcWork &T, SolveShared &S, int t0, int dt,
+                               float &bestf, int &bidx) {
+    const float *__restrict__ scale = J.scale;
+    const float *__restrict__ eps = J.eps;
+    const unsigned char *set = J.set;             // through L2: the first CTA of a cluster writes it
+    float *__restrict__ grad = J.grad;
+    // this thread's pixel of the tile: its scale, threshold and set
+    // are loaded before the tile's MMA is awaited
+    float pscale = 0.f, peps = 0.f;
+    unsigned char pset = 0;
+    adjoint_full<MODE>(
+        J, Ug, A, T, S.red, S.dbuf, t0, dt,
+        [&](int i, float val) {
+            const float g = -pscale * val;
+            grad[i] = g;
+            if (pset != IMG_SET_F) {
+                const float lam = pset == IMG_SET_U ? -g : g;
+                if (lam < -peps && (lam < bestf || (lam == bestf && i < bidx))) {
+                    bestf = lam;
+                    bidx = i;
+                }
+            }
+        },
+        [&](int i) {
+            pscale = scale[i];
+            peps = eps[i];
+            pset = __ldcg(set + i);
+        });
+}
+
+// A job's cluster: its first CTA runs the solve, the others wait at the
+// cluster barrier for its gradients and take their share of the tiles (in one
+// CTA they are a quarter to a half of a solve).  J.cmd: [0] the matrix of the
+// next gradient (1: W1, 2: W0; 0: done), [1] waits that ran out, [2 + 2 r], [3
+// + 2 r] rank r's smallest lambda (bits) and pixel.
+enum : int { kCmdDone = 0, kCmdW1 = 1, kCmdW0 = 2 };
+__device__ __forceinline__ int cluster_ctas() {
+    int n;
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n));
+    return n;
+}
+__device__ __forceinline__ int cluster_rank() {
+    int r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Persistent active-set driver (Table I), one CTA or one cluster per job.
+// MODE selects the adjoint's arithmetic (0 CUDA cores FP32, 1 tensor cores
+// FP16x3, 2 BF16x3).
 template <int MODE, bool PREP>
 __global__ void __launch_bounds__(kThreads, 1)
 k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
-    const JobDev &J = *jobs[blockIdx.x];
+    const int nctas = cluster_ctas(), rank = cluster_rank(), job = blockIdx.x / nctas;
+    const JobDev &J = *jobs[job];
     // one 1024-aligned region serves the CUDA-core chunk or the tensor tiles
     unsigned char *dyn = dyn_smem();
     float2 *A = reinterpret_cast<float2 *>(dyn);
@@ -1635,13 +1693,34 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
     }
     if (J.flags[0] != 0 || J.flags[1] != 1) {
         info.status = J.flags[0] != 0 ? J.flags[0] : IMG_EINVAL;
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0 && rank == 0) {
             *J.info = info;
-            if (batch_info) batch_info[blockIdx.x] = info;
+            if (batch_info) batch_info[job] = info;
         }
         if constexpr (MODE != 0) tc_teardown(T, p);
         return;
     }
+    if (rank != 0) {
+        for (;;) {
+            cluster_barrier();
+            const int cmd = *(volatile int *)J.cmd;
+            if (cmd == kCmdDone) break;
+            float bestf = INFINITY;
+            int bidx = 0x7fffffff;
+            gradient_tiles<MODE>(J, cmd == kCmdW1 ? J.W1 : J.W0, A, T, S, rank, nctas, bestf, bidx);
+            double best = bestf;
+            block_argmin(best, bidx, S.vbuf, S.ibuf);
+            if (threadIdx.x == 0) {
+                J.cmd[2 + 2 * rank] = __float_as_int((float)best);
+                J.cmd[3 + 2 * rank] = bidx;
+                if (T.timeouts) J.cmd[1] = 1;
+            }
+            cluster_barrier();
+        }
+        if constexpr (MODE != 0) tc_teardown(T, p);
+        return;
+    }
+    if (threadIdx.x == 0) J.cmd[1] = 0;
     for (int i = threadIdx.x; i < Q; i += blockDim.x) {
         J.x[i] = 0.0;
         J.set[i] = IMG_SET_L;
@@ -1732,41 +1811,28 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
                     Ug = J.W0;
                 }
                 const long long tg = clock64();
-                double best = INFINITY;
                 int bidx = 0x7fffffff;
                 float bestf = INFINITY;
-                {
-                    const float *__restrict__ scale = J.scale;
-                    const float *__restrict__ eps = J.eps;
-                    const unsigned char *__restrict__ set = J.set;
-                    float *__restrict__ grad = J.grad;
-                    // this thread's pixel of the tile: its scale, threshold and set
-                    // are loaded before the tile's MMA is awaited
-                    float pscale = 0.f, peps = 0.f;
-                    unsigned char pset = 0;
-                    adjoint_full<MODE>(
-                        J, Ug, A, T, S.red, S.dbuf,
-                        [&](int i, float val) {
-                            // lambda_L = g, lambda_U = -g (eq. etaL, eq. etaU); g and eps are FP32
-                            const float g = -pscale * val;
-                            grad[i] = g;
-                            if (pset != IMG_SET_F) {
-                                const float lam = pset == IMG_SET_U ? -g : g;
-                                if (lam < -peps && (lam < bestf || (lam == bestf && i < bidx))) {
-                                    bestf = lam;
-                                    bidx = i;
-                                }
-                            }
-                        },
-                        [&](int i) {
-                            pscale = scale[i];
-                            peps = eps[i];
-                            pset = set[i];
-                        });
+                if (nctas > 1) {
+                    if (threadIdx.x == 0) J.cmd[0] = Ug == J.W1 ? kCmdW1 : kCmdW0;
+                    cluster_barrier();
                 }
-                best = bestf;
+                gradient_tiles<MODE>(J, Ug, A, T, S, 0, nctas, bestf, bidx);
+                double best = bestf;
                 info.op_flops += flops_adj(p, Q);
                 block_argmin(best, bidx, S.vbuf, S.ibuf);
+                if (nctas > 1) {
+                    cluster_barrier();
+                    if (__ldcg(J.cmd + 1)) T.timeouts++;
+                    for (int r = 1; r < nctas; ++r) {
+                        const float b = __int_as_float(__ldcg(J.cmd + 2 + 2 * r));
+                        const int i = __ldcg(J.cmd + 3 + 2 * r);
+                        if (b < (float)best || (b == (float)best && i < bidx)) {
+                            best = b;
+                            bidx = i;
+                        }
+                    }
+                }
                 cyc.gradient += clock64() - tg;
                 lam_min = best;
                 if (bidx == 0x7fffffff) {
@@ -1831,12 +1897,16 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
             flag = true;
         }
     }
+    if (nctas > 1) {
+        if (threadIdx.x == 0) J.cmd[0] = kCmdDone;
+        cluster_barrier();
+    }
     if (!converged && info.status == IMG_OK) info.status = IMG_ENOTCONV;
     if constexpr (MODE != 0) {
         if (T.timeouts && info.status == IMG_OK) info.status = IMG_ETIMEOUT;
         tc_teardown(T, p);
     }
-    double *out = sigma_out ? sigma_out[blockIdx.x] : nullptr;
+    double *out = sigma_out ? sigma_out[job] : nullptr;
     int nf = 0, nu = 0;
     for (int i = threadIdx.x; i < Q; i += blockDim.x) {
         const double s = (double)J.scale[i] * J.x[i];
@@ -1862,7 +1932,7 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(info.t_end_ns));
         *J.ev_count = nev;
         *J.info = info;
-        if (batch_info) batch_info[blockIdx.x] = info;
+        if (batch_info) batch_info[job] = info;
     }
 }
 
@@ -2104,20 +2174,33 @@ cudaError_t launch_finalize(JobDev *const *jobs, int n, int max_tiles, cudaStrea
 }
 
 template <int MODE, bool PREP>
-static cudaError_t launch_solve_t(JobDev *const *jobs, int n, size_t sm, DevInfo *batch_info,
+static cudaError_t launch_solve_t(JobDev *const *jobs, int n, size_t sm, int ctas, DevInfo *batch_info,
                                   double *const *sigma_out, cudaStream_t st) {
     cudaError_t e = ensure_smem((const void *)k_solve<MODE, PREP>, sm);
     if (e != cudaSuccess) return e;
+    if (ctas > 1) {
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim = {(unsigned)ctas, 1, 1};
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(n * ctas);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = sm;
+        cfg.stream = st;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, k_solve<MODE, PREP>, jobs, batch_info, sigma_out);
+    }
     k_solve<MODE, PREP><<<n, kThreads, sm, st>>>(jobs, batch_info, sigma_out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_solve(JobDev *const *jobs, int n, int max_p, int mode, DevInfo *batch_info,
+cudaError_t launch_solve(JobDev *const *jobs, int n, int max_p, int mode, int ctas, DevInfo *batch_info,
                          double *const *sigma_out, cudaStream_t st) {
     const size_t sm = solve_smem_bytes(max_p, mode);
-    if (mode == 1) return launch_solve_t<1, false>(jobs, n, sm, batch_info, sigma_out, st);
-    if (mode == 2) return launch_solve_t<2, false>(jobs, n, sm, batch_info, sigma_out, st);
-    return launch_solve_t<0, false>(jobs, n, sm, batch_info, sigma_out, st);
+    if (mode == 1) return launch_solve_t<1, false>(jobs, n, sm, ctas, batch_info, sigma_out, st);
+    if (mode == 2) return launch_solve_t<2, false>(jobs, n, sm, ctas, batch_info, sigma_out, st);
+    return launch_solve_t<0, false>(jobs, n, sm, ctas, batch_info, sigma_out, st);
 }
 
 cudaError_t launch_job(JobDev *const *jobs, int n, int max_p, int mode, DevInfo *batch_info,
@@ -2127,9 +2210,9 @@ cudaError_t launch_job(JobDev *const *jobs, int n, int max_p, int mode, DevInfo 
         const size_t b = bounds_smem_bytes(max_p);
         sm = sm > b ? sm : b;
     }
-    if (mode == 1) return launch_solve_t<1, true>(jobs, n, sm, batch_info, sigma_out, st);
-    if (mode == 2) return launch_solve_t<2, true>(jobs, n, sm, batch_info, sigma_out, st);
-    return launch_solve_t<0, true>(jobs, n, sm, batch_info, sigma_out, st);
+    if (mode == 1) return launch_solve_t<1, true>(jobs, n, sm, 1, batch_info, sigma_out, st);
+    if (mode == 2) return launch_solve_t<2, true>(jobs, n, sm, 1, batch_info, sigma_out, st);
+    return launch_solve_t<0, true>(jobs, n, sm, 1, batch_info, sigma_out, st);
 }
 
 // Psi x over all pixels: nparts CTAs write partial p x p sums into `part`
