@@ -583,6 +583,19 @@ __device__ void ws_fred(const JobDev &J, const WsBufs &B, const UnitGeom &g, int
     for (int tile = rank; tile < nt * nt; tile += ctas) {
         float ss = 0.f;
         const int a0 = (tile % nt) * kRedTile, b0 = (tile / nt) * kRedTile;
+        // what the sums are added to, loaded with the partials (after the
+        // sums, each of the four rows' load waited for the store before it)
+        float2 old[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int a = a0 + tx, b = b0 + ty + 8 * q, e = b * p + a;
+            old[q] = make_float2(0.f, 0.f);
+            if (a >= p || b >= p) continue;
+            if (mode == kRedT) old[q] = dst[e];
+            else if (!pwls) old[q] = J.R32[e];
+            else if (mode == kRedG) old[q] = J.Ri32[e];
+            else if (a == b) old[q] = make_float2(1.f, 0.f);
+        }
         if (n > 0) {
             // the stored blocks are column-major: lanes run along the stored
             // row index (coalesced), i along the column.  Each thread gathers
@@ -635,23 +648,16 @@ __device__ void ws_fred(const JobDev &J, const WsBufs &B, const UnitGeom &g, int
         }
         __syncthreads();
         // outputs K(a, b) at dst[b p + a]: lanes along a (coalesced)
-        for (int j = ty; j < kRedTile; j += 8) {
-            const int a = a0 + tx, b = b0 + j;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int j = ty + 8 * q, a = a0 + tx, b = b0 + j;
             if (a < p && b < p) {
-                const int e = b * p + a;
                 float2 k = make_float2(0.f, 0.f);
                 if (n > 0) k = make_float2((T[0][tx][j] + T[1][tx][j]) * inv, (T[3][tx][j] - T[2][tx][j]) * inv);
-                float2 out;
-                if (mode == kRedT) {
-                    const float2 t = dst[e];
-                    out = make_float2(k.x - fa * t.x, k.y - fa * t.y);
-                } else {
-                    float2 base;
-                    if (mode == kRedB) base = pwls ? make_float2(a == b ? 1.f : 0.f, 0.f) : J.R32[e];
-                    else base = pwls ? J.Ri32[e] : J.R32[e];
-                    out = make_float2(base.x + k.x, base.y + k.y);
-                }
-                dst[e] = out;
+                const float2 o = old[q];
+                const float2 out = mode == kRedT ? make_float2(__fmaf_rn(-fa, o.x, k.x), __fmaf_rn(-fa, o.y, k.y))
+                                                 : make_float2(o.x + k.x, o.y + k.y);
+                dst[b * p + a] = out;
                 mx = fmaxf(mx, fmaxf(fabsf(out.x), fabsf(out.y)));
                 ss = fmaf(out.x, out.x, fmaf(out.y, out.y, ss));
             }
