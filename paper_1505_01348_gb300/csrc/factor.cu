@@ -6,7 +6,7 @@
 // code around them does (the one-CTA form measured 37.6 ms; p = 128: 4.6 ms,
 // p = 64: 0.92 ms; a dirty + MVDR call fell from 38.7 to 2.6 ms at p = 288,
 // 256x256, from 5.04 to 0.90 ms at p = 128, from 1.22 to 0.52 ms at p = 64
-// with this form).  Here the elimination of [R | I] runs in panels of kNb
+// with this form and the panels below).  Here the elimination of [R | I] runs in panels of kNb
 // columns over all SMs:
 //
 //   k_fac_panel  one step of the chain: every CTA factors the kNb x kNb
@@ -31,8 +31,9 @@ namespace {
 // launch and ramp) stay below its chain, narrow enough that the redundant
 // diagonal factor is a tenth of the work when many small jobs share the GPU.
 constexpr int kNb = 16;
-constexpr int kItems = 8;                           // vectors of a panel CTA
-constexpr int kPanelThreads = (kNb + kItems) * kNb;
+constexpr int kItems = 4;                           // vectors of a panel CTA
+constexpr int kPanelWork = (kNb + kItems) * kNb;    // threads on elements, then one warp for divisions
+constexpr int kPanelThreads = kPanelWork + 32;
 constexpr int kTrailR = 16, kTrailC = 8;            // tile of a trailing CTA
 constexpr int kInvT = 8;                            // tile edge of R^-1
 
@@ -57,29 +58,63 @@ __global__ void k_fac_init(JobDev *const *jobs) {
     }
 }
 
+__device__ __forceinline__ void bar_sync(int id, int n) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int n) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
 // Thread (r, k): row r < kNb of the diagonal block, or vector r - kNb of this
-// CTA, and column k.  Step j makes column j: the pivot's root and reciprocal,
-// then the scaled column, then its update of the columns k > j.  The columns
-// of L^-1 (which divide by the pivot) run one step behind, so that their
-// divisions overlap the next pivot's square root.  The factored diagonal
-// block itself is not stored: nothing reads it after its panel, and other
-// CTAs of the launch may still have to read the unfactored one.
+// CTA, and column k.  Step j makes column j: (A) the pivot's root and
+// reciprocal, (B) the scaled column, (C) its update of the columns k > j.  The
+// columns of L^-1, which divide by the pivot, run one step behind; their
+// divisions are one warp's, a component per lane, beside the next pivot's
+// root.  The factored diagonal block itself is not stored: nothing reads it
+// after its panel, and other CTAs of the launch may still have to read the
+// unfactored one.
+//
+// Bound by the FP64 pipe's latency (root 590, reciprocal 550 cycles, 67 per
+// dependent operation) and by its 19 cycles per warp instruction whatever
+// lanes are live: with 8 vectors and each vector's own threads dividing, a
+// panel took 49 us (34 in this form; a dirty + MVDR call of p = 288, 256x256
+// went from 1.71 to 1.44 ms, of p = 64, 128x128 from 315 to 260 us).
 __global__ void __launch_bounds__(kPanelThreads) k_fac_panel(JobDev *const *jobs, int j0) {
     const JobDev &J = *jobs[blockIdx.x];
     const int p = J.p;
     if (j0 >= p || (int)blockIdx.y * kItems >= p) return;
     const int nb = min(kNb, p - j0), below = p - j0 - nb;
-    const int k = threadIdx.x % kNb, r = threadIdx.x / kNb;
-    const int item = blockIdx.y * kItems + r - kNb;          // of p vectors: rows below, then columns of L^-1
+    __shared__ double2 l[kNb][kNb];                          // finished columns of the block: l[row][col]
+    __shared__ double2 xr[kNb + kItems];                     // column j of the rows
+    __shared__ double sd[2][kItems][2], xc[2][kItems][2];    // entry j of the L^-1 columns before / after its
+                                                             // division, by parity of j
+    __shared__ double s_dj[kNb], s_inv;
+    // step of the first bad pivot (a step number, not a flag: the dividing warp
+    // may read it a step late and must not leave before the others do)
+    __shared__ int s_bad;
+    enum { kB1 = 1, kB2 = 2, kDiv = 3 };                     // named barriers
+    if (threadIdx.x == 0) s_bad = J.flags[3] != 0 ? -1 : kNb + 1;
+    if (threadIdx.x < 2 * kItems) sd[0][threadIdx.x >> 1][threadIdx.x & 1] = sd[1][threadIdx.x >> 1][threadIdx.x & 1] = 0.0;
+    __syncthreads();
+    if (s_bad < 0) return;                                   // a pivot of an earlier panel was bad
+    if (threadIdx.x >= kPanelWork) {
+        const int lane = threadIdx.x - kPanelWork, it = (lane >> 1) % kItems, c = lane & 1;
+        for (int j = 0; j <= nb; ++j) {
+            bar_sync(kDiv, kPanelThreads);                   // entry j - 1 is complete
+            if (j > 0) {
+                const double q = sd[(j - 1) & 1][it][c] / s_dj[j - 1];
+                if (lane < 2 * kItems) xc[(j - 1) & 1][it][c] = q;
+            }
+            bar_sync(kB1, kPanelThreads);
+            if (s_bad <= j) break;
+        }
+        return;
+    }
+    const int k = threadIdx.x % kNb, r = threadIdx.x / kNb, v = r - kNb;
+    const int item = blockIdx.y * kItems + v;                // of p vectors: rows below, then columns of L^-1
     const bool diag = r < kNb;
     const bool isrow = !diag && item < below;
     const bool iscol = !diag && !isrow && item < p;
-    __shared__ double2 l[kNb][kNb];                          // finished columns of the block: l[row][col]
-    __shared__ double2 xr[kNb + kItems];                     // column j of the rows
-    __shared__ double2 xc[2][kNb + kItems];                  // entry j - 1 of the L^-1 columns, by parity of j
-    __shared__ double s_dj[kNb], s_inv;
-    __shared__ int s_bad;
-    if (threadIdx.x == 0) s_bad = J.flags[3];
     double2 *src = nullptr;                                  // this thread's element
     if (k < nb) {
         if (diag && r < nb && r >= k) src = J.L64 + (size_t)(j0 + k) * p + j0 + r;
@@ -87,41 +122,49 @@ __global__ void __launch_bounds__(kPanelThreads) k_fac_panel(JobDev *const *jobs
         else if (iscol) src = J.Li64 + (size_t)(item - below) * p + j0 + k;
     }
     double2 a = src ? *src : make_double2(0.0, 0.0);
-    __syncthreads();
-    if (s_bad) return;                                       // a pivot of an earlier panel was bad
-    __syncthreads();
+    if (iscol && k == 0) {
+        sd[0][v][0] = a.x;
+        sd[0][v][1] = a.y;
+    }
+    bar_arrive(kDiv, kPanelThreads);
+    bool bad = false;
     for (int j = 0; j <= nb; ++j) {
         if (j < nb && diag && r == j && k == j) {
             const double d = a.x;
-            if (!(d > 0.0 && isfinite(d))) s_bad = 1;
+            if (!(d > 0.0 && isfinite(d))) s_bad = j;
             const double dj = sqrt(d);
             s_dj[j] = dj;
             s_inv = 1.0 / dj;
         }
-        if (j > 0 && iscol && k == j - 1) {
-            const double dj = s_dj[j - 1];
-            a = make_double2(a.x / dj, a.y / dj);
-            xc[j & 1][r] = a;
-        }
-        __syncthreads();
-        if (s_bad) break;
+        bar_sync(kB1, kPanelThreads);
+        bad = s_bad <= j;
+        if (bad) break;
         if (j < nb && k == j && ((diag && r > j) || isrow)) {
             const double inv = s_inv;
             a = make_double2(a.x * inv, a.y * inv);
             xr[r] = a;
             if (diag) l[r][j] = a;
         }
-        __syncthreads();
+        bar_sync(kB2, kPanelWork);
         if (j < nb && k > j && ((diag && r >= k) || isrow)) {
             const double2 prod = zmulc(xr[r], xr[k]);
             a = make_double2(a.x - prod.x, a.y - prod.y);
         }
-        if (j > 0 && iscol && k >= j && k < nb) {
-            const double2 t = zmul(l[k][j - 1], xc[j & 1][r]);
-            a = make_double2(a.x - t.x, a.y - t.y);
+        if (j > 0 && iscol && k < nb) {
+            const double2 x = make_double2(xc[(j - 1) & 1][v][0], xc[(j - 1) & 1][v][1]);
+            if (k == j - 1) a = x;
+            if (k >= j) {
+                const double2 t = zmul(l[k][j - 1], x);
+                a = make_double2(a.x - t.x, a.y - t.y);
+            }
+            if (k == j) {
+                sd[j & 1][v][0] = a.x;
+                sd[j & 1][v][1] = a.y;
+            }
         }
+        if (j < nb) bar_arrive(kDiv, kPanelThreads);
     }
-    if (s_bad) {
+    if (bad) {
         if (blockIdx.y == 0 && threadIdx.x == 0) J.flags[3] = 1;
         return;
     }
