@@ -578,58 +578,60 @@ __global__ void k_d2c(const double2 *src, float2 *dst, int n) {
 }
 
 // C = op(A) op(B), p x p complex FP32 column-major; op 0: as is, 1: conjugate
-// transpose.  16 x 16 output tiles, 64 threads (2 x 2 outputs each): small
-// tiles, because p = 128 makes only 16 of 32 x 32 (13.6 us, a chain of shared
-// loads on 16 SMs).  cmax (may be null): max |C| per CTA.
-__global__ void __launch_bounds__(64) k_cgemm(int p, const float2 *A, int opA, const float2 *B, int opB, float2 *C,
-                                              float *cmax) {
+// transpose.  16 x 16 output tiles, one output per thread, the next 32 terms'
+// loads in flight behind the current ones: at p = 128 the product is latency,
+// 64 tiles on 64 SMs (32 x 32 tiles, 16 CTAs: 13.6 us; 2 x 2 outputs on 64
+// threads: 21 us).  cmax (may be null): max |C| per CTA.
+__global__ void __launch_bounds__(256) k_cgemm(int p, const float2 *A, int opA, const float2 *B, int opB, float2 *C,
+                                               float *cmax) {
     constexpr int kT = 16, kK = 32;
     __shared__ float2 As[kT][kK + 1], Bs[kK][kT + 1];
     const int i0 = blockIdx.x * kT, j0 = blockIdx.y * kT;
-    const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
-    float2 acc[2][2] = {};
+    float2 ra[2], rb[2];
+    // this thread's entries q of a chunk, consecutive threads along the
+    // memory's fast index: As[r][c] = op(A)[i0 + r, k0 + c], Bs[r][c] = op(B)[k0 + r, j0 + c]
+    auto place = [&](int q, int &ar, int &ac, int &br, int &bc) {
+        const int e = threadIdx.x + 256 * q;
+        ar = opA ? e / kK : e % kT;
+        ac = opA ? e % kK : e / kT;
+        br = opB ? e / kT : e % kK;
+        bc = opB ? e % kT : e / kK;
+    };
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            int ar, ac, br, bc;
+            place(q, ar, ac, br, bc);
+            const int i = i0 + ar, k = k0 + ac, kk = k0 + br, j = j0 + bc;
+            ra[q] = rb[q] = make_float2(0.f, 0.f);
+            if (i < p && k < p) ra[q] = opA ? A[(size_t)i * p + k] : A[(size_t)k * p + i];
+            if (kk < p && j < p) rb[q] = opB ? B[(size_t)kk * p + j] : B[(size_t)j * p + kk];
+            if (opA) ra[q].y = -ra[q].y;
+            if (opB) rb[q].y = -rb[q].y;
+        }
+    };
+    const int ti = threadIdx.x & 15, tj = threadIdx.x >> 4;
+    float2 acc = make_float2(0.f, 0.f);
+    load(0);
     for (int k0 = 0; k0 < p; k0 += kK) {
 #pragma unroll
-        for (int e = threadIdx.x; e < kT * kK; e += 64) {
-            // consecutive threads along the memory's fast index
-            const int r = opA ? e / kK : e % kT, c = opA ? e % kK : e / kT;    // As[r][c] = op(A)[i0 + r, k0 + c]
-            const int i = i0 + r, k = k0 + c;
-            float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
-            if (i < p && k < p) {
-                a = opA ? A[(size_t)i * p + k] : A[(size_t)k * p + i];
-                if (opA) a.y = -a.y;
-            }
-            As[r][c] = a;
-            const int rb = opB ? e / kT : e % kK, cb = opB ? e % kT : e / kK;  // Bs[rb][cb] = op(B)[k0 + rb, j0 + cb]
-            const int kk = k0 + rb, j = j0 + cb;
-            if (kk < p && j < p) {
-                b = opB ? B[(size_t)kk * p + j] : B[(size_t)j * p + kk];
-                if (opB) b.y = -b.y;
-            }
-            Bs[rb][cb] = b;
+        for (int q = 0; q < 2; ++q) {
+            int ar, ac, br, bc;
+            place(q, ar, ac, br, bc);
+            As[ar][ac] = ra[q];
+            Bs[br][bc] = rb[q];
         }
         __syncthreads();
-#pragma unroll 8
-        for (int kk = 0; kk < kK; ++kk) {
+        if (k0 + kK < p) load(k0 + kK);
 #pragma unroll
-            for (int a = 0; a < 2; ++a)
-#pragma unroll
-                for (int b = 0; b < 2; ++b) cfma(acc[a][b], As[2 * ty + a][kk], Bs[kk][2 * tx + b]);
-        }
+        for (int kk = 0; kk < kK; ++kk) cfma(acc, As[ti][kk], Bs[kk][tj]);
         __syncthreads();
     }
-    float mx = 0.f;
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const int i = i0 + 2 * ty + a, j = j0 + 2 * tx + b;
-            if (i >= p || j >= p) continue;
-            C[(size_t)j * p + i] = acc[a][b];
-            mx = fmaxf(mx, fmaxf(fabsf(acc[a][b].x), fabsf(acc[a][b].y)));
-        }
+    const int i = i0 + ti, j = j0 + tj;
+    const bool in = i < p && j < p;
+    if (in) C[(size_t)j * p + i] = acc;
     if (!cmax) return;
-    mx = cta_max_t0(mx);
+    const float mx = cta_max_t0(in ? fmaxf(fabsf(acc.x), fabsf(acc.y)) : 0.f);
     if (threadIdx.x == 0) cmax[blockIdx.y * gridDim.x + blockIdx.x] = mx;
 }
 
@@ -2305,8 +2307,8 @@ cudaError_t ls_forward(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, 
     if (hj.cost == IMG_COST_PWLS) {
         // W vect(K) = vect(L^-1 K L^-H)
         const dim3 g((p + 15) / 16, (p + 15) / 16);
-        k_cgemm<<<g, 64, 0, st>>>(p, b.Mv, 0, hj.Li32, 1, b.T1, nullptr);
-        k_cgemm<<<g, 64, 0, st>>>(p, hj.Li32, 0, b.T1, 0, b.Mv, nullptr);
+        k_cgemm<<<g, 256, 0, st>>>(p, b.Mv, 0, hj.Li32, 1, b.T1, nullptr);
+        k_cgemm<<<g, 256, 0, st>>>(p, hj.Li32, 0, b.T1, 0, b.Mv, nullptr);
     }
     return cudaGetLastError();
 }
@@ -2320,8 +2322,8 @@ cudaError_t ls_adjoint(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, 
         // W^H vect(u) = vect(L^-H u L^-1)
         const dim3 g((p + 15) / 16, (p + 15) / 16);
         const bool fits = (int)(g.x * g.y) <= kOpMax;
-        k_cgemm<<<g, 64, 0, st>>>(p, b.u, 0, hj.Li32, 0, b.T1, nullptr);
-        k_cgemm<<<g, 64, 0, st>>>(p, hj.Li32, 1, b.T1, 0, b.Uw, fits ? hj.opmax : nullptr);
+        k_cgemm<<<g, 256, 0, st>>>(p, b.u, 0, hj.Li32, 0, b.T1, nullptr);
+        k_cgemm<<<g, 256, 0, st>>>(p, hj.Li32, 1, b.T1, 0, b.Uw, fits ? hj.opmax : nullptr);
         U = b.Uw;
         numax = fits ? (int)(g.x * g.y) : 0;
     }
