@@ -199,40 +199,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_bounds_tc(JobDev *const *jobs) 
     tc_teardown(T, J.p);
 }
 
-// Tensor-core Psi^H vect(U) over all pixels of one job.
-template <int MODE>
-__global__ void __launch_bounds__(kThreads, 1) k_psi_adj_tc(const JobDev *Jp, const float2 *U,
-                                                           double *out) {
-    const JobDev &J = *Jp;
-    constexpr bool BF = MODE == 2;
-    unsigned char *dyn = dyn_smem();
-    __shared__ uint64_t bars[2];
-    __shared__ uint32_t slot;
-    __shared__ double dbuf[kThreads / 32];
-    __shared__ float red[2 * kTcM];
-    TcWork T{};
-    tc_carve(T, dyn, J.p);
-    tc_setup(T, bars, &slot, J.p);
-    const float sX = tc_steer_scale(J.p);
-    const uint32_t idesc = idesc_f16(2 * T.Kp, BF ? 1 : 0);
-    const float sB = tc_build_B<BF>(U, J.p, T, dbuf);
-    const float inv = 1.f / (sX * sX * sB);
-    const int ntiles = tc_num_tiles(J.n_l, J.n_m);
-    const int mine = ntiles > (int)blockIdx.x ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    tc_run_tiles(
-        T, mine, idesc,
-        [&](int t, int b) { tc_gen_X_steer<BF>(J, T, b, blockIdx.x + t * gridDim.x, sX); },
-        [&](int t, int b) {
-            tc_epilogue<BF>(T, b, red);
-            if (threadIdx.x < kTcM) {
-                const int i = tc_tile_pixel(blockIdx.x + t * gridDim.x, threadIdx.x, J.n_l, J.n_m);
-                if (i >= 0) out[i] = red[threadIdx.x] * inv;
-            }
-            __syncthreads();
-        });
-    tc_teardown(T, J.p);
-}
-
 // max |entry| of R_hat (blockIdx.y = 0) and L^-H (1) per job, 8 blocks
 // each, into J.opmax[8 w + block].
 constexpr int kBoundsMaxBlocks = 8;
@@ -2463,17 +2429,6 @@ cudaError_t ls_xnorm2(const JobDev &hj, LsBufs &b, double *out, cudaStream_t st)
 }
 
 template <int MODE>
-static cudaError_t launch_psi_adj_tc_t(const JobDev *job_dev, const float2 *U, double *out, int Q, int p,
-                                       cudaStream_t st) {
-    const size_t sm = tc_smem_bytes(p) + 1024;
-    cudaError_t e = ensure_smem((const void *)k_psi_adj_tc<MODE>, sm);
-    if (e != cudaSuccess) return e;
-    const int ntiles = (Q + kTcM - 1) / kTcM;
-    k_psi_adj_tc<MODE><<<min(ntiles, num_sms()), kThreads, sm, st>>>(job_dev, U, out);
-    return cudaGetLastError();
-}
-
-template <int MODE>
 static cudaError_t launch_psi_adj_wide_t(const JobDev *job_dev, const void *U, bool u64, int nmax, double *out, int Q,
                                          int p, cudaStream_t st) {
     const dim3 eg(wide_nk(p), 2 * wide_kp(p) / kEmbRows);
@@ -2505,9 +2460,7 @@ cudaError_t launch_psi_adj_wide(const JobDev *job_dev, const void *U, bool u64, 
 
 cudaError_t launch_psi_adj(const JobDev *job_dev, const float2 *U, double *out, int Q, int p, int mode,
                            cudaStream_t st) {
-    if (mode != 0 && p > kMaxTcP) return cudaErrorInvalidValue;   // wide arrays: launch_psi_adj_wide
-    if (mode == 1) return launch_psi_adj_tc_t<1>(job_dev, U, out, Q, p, st);
-    if (mode == 2) return launch_psi_adj_tc_t<2>(job_dev, U, out, Q, p, st);
+    if (mode != 0) return cudaErrorInvalidValue;   // tensor cores: launch_psi_adj_wide
     const size_t sm = bounds_smem_bytes(p);
     cudaError_t e = ensure_smem((const void *)k_psi_adj, sm);
     if (e != cudaSuccess) return e;
