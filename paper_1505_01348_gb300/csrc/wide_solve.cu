@@ -672,7 +672,11 @@ __device__ void ws_fred(const JobDev &J, const WsBufs &B, const UnitGeom &g, int
     if ((threadIdx.x & 31) == 0) atomicMax(&ctl->mx_t, __float_as_uint(mx));
     if (mode != kRedG && rank == 0 && threadIdx.x == 0) ctl->nsums = nt * nt;
 }
-__global__ void __launch_bounds__(kWsThreads) k_ws_fred(const JobDev *Jp, WsBufs B, int mode) {
+// Two CTAs per SM (128 registers, a few spilled): with the 167 it would take,
+// one image alone is faster (first passes of 256 x 256, p = 288: 182 instead
+// of 191 ms), but a CTA keeps the other images' off its SM, and 16 such
+// images in flight take 5.79 s instead of 5.41 for their first 1600 passes.
+__global__ void __launch_bounds__(kWsThreads, 2) k_ws_fred(const JobDev *Jp, WsBufs B, int mode) {
     ws_count(B.ctl);
     if (B.ctl->stop) return;
     ws_fred(*Jp, B, unit_geom(Jp->p), mode, blockIdx.x, gridDim.x);
