@@ -299,6 +299,7 @@ __device__ int items_adjoint(const JobDev &J, const UnitGeom &g, unsigned char *
                     if (leader) issue_copy(c + 1, s1);
                 }
             }
+            wide_drain(bars, kBEmpty, total, ph, timeouts);
         }
     } else if (warp >= 4) {
         if (LIST) idle(warp);
@@ -402,6 +403,7 @@ __device__ int items_adjoint(const JobDev &J, const UnitGeom &g, unsigned char *
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bars[kXFull + s]);
             }
+            wide_drain(bars, kXEmpty, total, ph, timeouts);
         }
     } else {
         // ---------------- epilogue: one row per thread, the unit's 2 ku
@@ -481,6 +483,10 @@ __device__ int items_adjoint(const JobDev &J, const UnitGeom &g, unsigned char *
     if (timeouts) atomicAdd(&s_timeouts, timeouts);
     tc_fence_before();
     __syncthreads();
+    // the caller may set the words up again (several phases, one CTA); after
+    // a wait that ran out arrivals may still be outstanding
+    if (threadIdx.x == 0 && s_timeouts == 0)
+        for (int q = 0; q < kWideBars; ++q) mbar_inval(&bars[q]);
     return s_timeouts;
 }
 
@@ -607,6 +613,7 @@ __device__ int items_forward(const UnitGeom &g, unsigned char *dyn, uint64_t *ba
                     if (leader) issue_copy(t + 1, s1);
                 }
             }
+            wide_drain(bars, kEmpty, mine, ph, timeouts);
         }
     }
     if (warp < 4) {
@@ -634,6 +641,10 @@ __device__ int items_forward(const UnitGeom &g, unsigned char *dyn, uint64_t *ba
     if (timeouts) atomicAdd(&s_timeouts, timeouts);
     tc_fence_before();
     __syncthreads();
+    // the next task or phase sets the words up again (not after a wait that
+    // ran out: arrivals may still be outstanding)
+    if (threadIdx.x == 0 && s_timeouts == 0)
+        for (int q = 0; q <= kAcc; ++q) mbar_inval(&bars[q]);
     return s_timeouts;
 }
 

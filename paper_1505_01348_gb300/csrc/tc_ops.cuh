@@ -43,6 +43,11 @@ __device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
+// Give a barrier's word back, so that it can be set up again.  No thread
+// waits on it and no arrival (a commit's, a bulk copy's) is outstanding.
+__device__ __forceinline__ void mbar_inval(uint64_t *bar) {
+    asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
 
 // Wait until the barrier's phase with the given parity completes.  Returns
 // false after `limit` polls (kSpinLimit by default; the caller records a

@@ -210,6 +210,15 @@ __device__ __forceinline__ void wide_wait_parity(uint64_t *bars, int slot, uint3
     wide_wait(bars, slot, ph, timeouts);
 }
 
+// The last two of n uses of a pair of stages, whose completions on barriers
+// first, first + 1 the loop over the uses leaves unwaited (use u waits for use
+// u - 2): a commit that is still to arrive must find its barrier, neither set
+// up again nor gone with the CTA's shared memory.
+__device__ __forceinline__ void wide_drain(uint64_t *bars, int first, int n, uint32_t &ph, int &timeouts) {
+    if (n > 1) wide_wait(bars, first + (n & 1), ph, timeouts);
+    if (n > 0) wide_wait(bars, first + ((n - 1) & 1), ph, timeouts);
+}
+
 // out = Re(a_i^H U_s a_i) for npass <= 2 operators s (B images B0, B1,
 // scales sB[s]) over the 2-D tiles t0, t0 + dt, ... (ntiles of them);
 // epi(s, i, v) receives each pixel's value.  Bit s of sq_mask makes pass s
@@ -301,6 +310,7 @@ __device__ int wide_adjoint(const JobDev &J, unsigned char *dyn, uint64_t *bars,
                     }
                 }
             }
+            wide_drain(bars, kBEmpty, units, ph, timeouts);
         }
     } else if (warp >= 4) {
         // ---------------- steering producers: chunk c of tile use T into X stage c & 1.
@@ -403,6 +413,7 @@ __device__ int wide_adjoint(const JobDev &J, unsigned char *dyn, uint64_t *bars,
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[kXFull + s]);
         }
+        wide_drain(bars, kXEmpty, total, ph, timeouts);
     } else {
         // ---------------- epilogue: one pixel row per thread.  Each warp
         // stages, 16 k at a time, the 8 E_l rows and its 4 E_m rows of the
