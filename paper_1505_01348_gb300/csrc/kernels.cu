@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_fwd_wide(const JobDev *Jp, c
                                                             FwdMap map, float *part) {
     const JobDev &J = *Jp;
     unsigned char *dyn = dyn_smem();
-    __shared__ uint64_t bars[5];
+    __shared__ uint64_t bars[kFwdBars];
     __shared__ uint32_t slot;
     const int pr = blockIdx.y, S = gridDim.x;
     wide_forward<MODE == 2>(J, dyn, bars, &slot, w, wmax, nmax, map.m[pr], map.nb[pr], blockIdx.x, S,

@@ -23,6 +23,7 @@
 #include <type_traits>
 
 #include "tc_ops.cuh"
+#include "fwd_ring.cuh"
 
 namespace img {
 
@@ -529,8 +530,9 @@ __device__ int wide_adjoint(const JobDev &J, unsigned char *dyn, uint64_t *bars,
 constexpr int kFwdPix = 64;                                  // pixels per stage
 constexpr size_t kFwdChunk = (size_t)kFwdPix * 128;          // one 64-feature chunk, 8 KB
 constexpr size_t kFwdStage = (2 + 4) * 2 * kFwdChunk;        // A: 2 chunks, B: 4 chunks, hi + lo
-constexpr int kFwdProducers = 15;                            // warps
+constexpr int kFwdProducers = fwd_ring::kProducers;          // warps
 constexpr int kFwdThreads = 32 * (kFwdProducers + 1);
+constexpr int kFwdBars = 2 + fwd_ring::kSlots + 1;           // mbarriers
 __host__ __device__ inline size_t fwd_smem_bytes() { return 2 * kFwdStage + 1024; }
 __host__ __device__ inline int fwd_n_of(int p, int nb) {
     const int n = 2 * wide_kp(p) - 256 * nb;
@@ -570,7 +572,7 @@ __device__ int wide_forward(const JobDev &J, unsigned char *dyn, uint64_t *bars,
     const int mine = nblk > s0 ? (nblk - 1 - s0) / S + 1 : 0;
     const float sX = steer_scale(p);
     const float sW = emb_scale_of(warp_max_of(wmax, nmax));
-    enum { kFull = 0, kEmpty = 2, kAcc = 4 };
+    enum { kFull = 0, kEmpty = 2, kAcc = kEmpty + fwd_ring::kSlots };
     // feature chunks of a stage: A = {2m, 2m+1}, then those of B = {4nb ..}
     // that are not among them
     const int nB = N / 64, ov = 2 * m - 4 * nb;              // A's place in B when 0 <= ov < 4
@@ -581,10 +583,8 @@ __device__ int wide_forward(const JobDev &J, unsigned char *dyn, uint64_t *bars,
     __shared__ int s_timeouts;
     if (threadIdx.x == 0) {
         s_timeouts = 0;
-        for (int q = 0; q < 2; ++q) {
-            mbar_init(&bars[kFull + q], ntask);
-            mbar_init(&bars[kEmpty + q], 1);
-        }
+        for (int q = 0; q < 2; ++q) mbar_init(&bars[kFull + q], ntask);
+        for (int q = 0; q < fwd_ring::kSlots; ++q) mbar_init(&bars[kEmpty + q], 1);
         mbar_init(&bars[kAcc], 1);
     }
     if (warp == 0) tmem_alloc(slot, 256);
@@ -616,9 +616,13 @@ __device__ int wide_forward(const JobDev &J, unsigned char *dyn, uint64_t *bars,
                     mma_f16(tmem, sw128_desc_mn(al + o, kFwdChunk, 1024), sw128_desc_mn(bh + o, kFwdChunk, 1024),
                             idesc, 1u);
                 }
-                mma_commit(&bars[kEmpty + sg]);
+                mma_commit(&bars[kEmpty + fwd_ring::slot(t)]);
                 if (t == mine - 1) mma_commit(&bars[kAcc]);
             }
+            // the last commits find their barriers: the producers have seen
+            // every stage but the last two
+            for (int t = max(0, mine - 2); t < mine; ++t)
+                wide_wait_parity(bars, kEmpty + fwd_ring::slot(t), fwd_ring::parity(t), timeouts);
         }
     } else {
         // ---------------- producers: the stages' tasks in order, warp w those
@@ -694,17 +698,13 @@ __device__ int wide_forward(const JobDev &J, unsigned char *dyn, uint64_t *bars,
                 }
             }
         };
-        // At most two stages' tasks in flight: a warp's next task is then at
-        // most two stages on, where the wait below is for the completion after
-        // one that it knows of (the MMAs finish in order), so that a parity
-        // names it.  Small arrays have as few as 4 tasks per stage.
-        const int np = min(kFwdProducers, 2 * ntask);
+        const int np = fwd_ring::warps(ntask);
         const int total = warp < np ? mine * ntask : 0;
         if (warp < total) load(warp / ntask, warp % ntask);
         for (int id = warp; id < total; id += np) {
             const int t = id / ntask, task = id - t * ntask, sg = t & 1;
             // the MMAs of stage t - 2 are done with the buffer
-            if (t >= 2) wide_wait_parity(bars, kEmpty + sg, ((t >> 1) - 1) & 1, timeouts);
+            if (t >= 2) wide_wait_parity(bars, kEmpty + fwd_ring::slot(t - 2), fwd_ring::parity(t - 2), timeouts);
             unsigned char *st = dyn + sg * kFwdStage;
             const int h = task & 1, c = chunk_of(task >> 1);
             const int part = c * 64 + 2 * lane >= Kp;
