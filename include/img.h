@@ -239,6 +239,11 @@ img_status img_psi_adj(img_ctx *ctx, const double *U, double *out, int on_device
  * device stays usable either way; no fault or trap is involved. */
 img_status img_check_wait(unsigned polls, int arrive);
 
+/* The same with one thread of the CTA waiting alone (thread 0 .. 255; -1: all
+ * of them), as for the solver's tile copies: its count reaches the status by
+ * the same reduction as a solve's.  IMG_EINVAL also for other threads. */
+img_status img_check_wait_thread(unsigned polls, int arrive, int thread);
+
 /* Unconstrained LS / WLS image with every pixel free (Sec. III-B/C: the LS
  * and WLS images; Sec. V-A: LSQR): min ||b - M x|| over all Q pixels with
  * M = Psi, b = vect(R_hat) (IMG_COST_LS) or M = W Psi D^-1, b = W vect(R_hat)

@@ -810,12 +810,14 @@ img_status img_snapshot_ls_image(img_ctx *const *snap, int K, int maxit, double 
     return IMG_OK;
 }
 
-img_status img_check_wait(unsigned polls, int arrive) {
-    if (polls == 0 || polls > (1u << 26)) return IMG_EINVAL;
+img_status img_check_wait(unsigned polls, int arrive) { return img_check_wait_thread(polls, arrive, -1); }
+
+img_status img_check_wait_thread(unsigned polls, int arrive, int thread) {
+    if (polls == 0 || polls > (1u << 26) || thread < -1 || thread >= img::kThreads) return IMG_EINVAL;
     int *d = nullptr;
     CK(cudaMalloc(&d, sizeof(int)));
     int h = -1;
-    cudaError_t e = img::launch_wait_selftest(polls, arrive ? 1 : 0, d, nullptr);
+    cudaError_t e = img::launch_wait_selftest(polls, arrive ? 1 : 0, thread, d, nullptr);
     if (e == cudaSuccess) e = cudaMemcpy(&h, d, sizeof(int), cudaMemcpyDeviceToHost);
     cudaFree(d);
     if (e != cudaSuccess) return IMG_ECUDA;

@@ -114,8 +114,9 @@ cudaError_t launch_job(JobDev *const *jobs, int n, int max_p, int mode, DevInfo 
                        double *const *sigma_out, cudaStream_t st);
 cudaError_t launch_psi(const JobDev *job_dev, const float *wx, float2 *part, int nparts, int Q,
                        int p, int mode, double2 *Kout, cudaStream_t st);
-// Bounded-wait self-test (one CTA; *status: IMG_OK or IMG_ETIMEOUT).
-cudaError_t launch_wait_selftest(unsigned polls, int arrive, int *status, cudaStream_t st);
+// Bounded-wait self-test (one CTA; all its threads wait, or the given one;
+// *status: IMG_OK or IMG_ETIMEOUT).
+cudaError_t launch_wait_selftest(unsigned polls, int arrive, int thread, int *status, cudaStream_t st);
 
 // CTAs that leave per-CTA maxima of an operand (JobDev::opmax).
 constexpr int kOpMax = 256;

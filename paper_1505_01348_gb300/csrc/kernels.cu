@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bounds_tc(JobDev *const *jobs) 
                 __syncthreads();
             });
     }
-    if (T.timeouts && threadIdx.x == 0) J.flags[2] = IMG_ETIMEOUT;
+    if (T.timeouts) J.flags[2] = IMG_ETIMEOUT;
     tc_teardown(T, J.p);
 }
 
@@ -604,32 +604,30 @@ __global__ void __launch_bounds__(256) k_cgemm(int p, const float2 *A, int opA, 
 // ---------------------------------------------------------------- failure detection
 // Self-test of the bounded waits every tensor-core kernel uses: one CTA
 // allocates tensor memory, waits on an mbarrier that receives an arrival only
-// when `arrive` is set, gives up after `polls` polls, frees the tensor memory
-// on its normal exit path and reports through *status (IMG_OK or
-// IMG_ETIMEOUT).  No fault, trap or endless loop is involved.
-__global__ void k_wait_selftest(unsigned polls, int arrive, int *status) {
+// when `arrive` is set - all its threads, or thread `thread` alone -, gives up
+// after `polls` polls, frees the tensor memory on its normal exit path and
+// reports through *status (IMG_OK or IMG_ETIMEOUT).  No fault, trap or endless
+// loop is involved.
+__global__ void k_wait_selftest(unsigned polls, int arrive, int thread, int *status) {
     __shared__ uint64_t bar;
     __shared__ uint32_t slot;
-    __shared__ int timed_out;
-    if (threadIdx.x == 0) {
-        mbar_init(&bar, 1);
-        timed_out = 0;
-    }
+    if (threadIdx.x == 0) mbar_init(&bar, 1);
     if (threadIdx.x < 32) tmem_alloc(&slot, 32);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     if (arrive && threadIdx.x == 0)
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar)) : "memory");
-    if (!mbar_wait(&bar, 0u, polls)) atomicOr(&timed_out, 1);
+    int timeouts = 0;
+    if ((thread < 0 || (int)threadIdx.x == thread) && !mbar_wait(&bar, 0u, polls)) timeouts++;
     tc_fence_before();
-    __syncthreads();
+    const bool late = cta_timed_out(timeouts);
     if (threadIdx.x < 32) tmem_dealloc(slot, 32);
-    if (threadIdx.x == 0) *status = timed_out ? IMG_ETIMEOUT : IMG_OK;
+    if (threadIdx.x == 0) *status = late ? IMG_ETIMEOUT : IMG_OK;
 }
 
-cudaError_t launch_wait_selftest(unsigned polls, int arrive, int *status, cudaStream_t st) {
-    k_wait_selftest<<<1, 64, 0, st>>>(polls, arrive, status);
+cudaError_t launch_wait_selftest(unsigned polls, int arrive, int thread, int *status, cudaStream_t st) {
+    k_wait_selftest<<<1, kThreads, 0, st>>>(polls, arrive, thread, status);
     return cudaGetLastError();
 }
 
@@ -1189,14 +1187,18 @@ __device__ __noinline__ int lsqr_resident(const JobDev &J, int f, TcWork &Tio, S
     if (stream) asm volatile("fence.proxy.async;" ::: "memory");
     uint32_t ldph = S.ldph;                       // parities of the tile loads
     // tile t from the image into its buffer (thread 32, after a barrier that
-    // ended every use of the buffer)
+    // ended every use of the buffer); no more copies once one was late
     auto load_tile = [&](int t) {
+        if (T.timeouts) return;
         uint64_t *bar = &S.ldbar[t & 1];
         mbar_expect_tx(bar, tile_bytes);
         tma_bulk_g2s(T.Xhi(t & 1), J.ximg + (size_t)t * tile_bytes, tile_bytes, bar);
     };
     auto wait_tile = [&](int b) {
-        if (!mbar_wait(&S.ldbar[b], (ldph >> b) & 1u)) T.timeouts++;
+        const uint32_t par = (ldph >> b) & 1u;
+        if (mbar_wait(&S.ldbar[b], par, T.timeouts ? 1u : kSpinLimit)) return;
+        // a late copy may still write the buffer: once more before going on
+        if (T.timeouts++ == 0) mbar_wait(&S.ldbar[b], par);
     };
     if (!gram)
         for (int e = threadIdx.x; e < f * p; e += kThreads) {
@@ -1681,8 +1683,8 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
             if (threadIdx.x == 0) {
                 J.cmd[2 + 2 * rank] = __float_as_int((float)best);
                 J.cmd[3 + 2 * rank] = bidx;
-                if (T.timeouts) J.cmd[1] = 1;
             }
+            if (T.timeouts) J.cmd[1] = 1;       // from any thread
             cluster_barrier();
         }
         if constexpr (MODE != 0) tc_teardown(T, p);
@@ -1747,7 +1749,7 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
                 info.lsqr_iters += its;
                 info.op_flops += (its + 1) * (flops_fwd(p, f) + flops_adj(p, f));
                 // feasibility with the relative tolerance tau, non-strict
-                int bad = 0;
+                int bad = MODE != 0 && T.timeouts ? 1 : 0;
                 const double tau = J.feas_tol;
                 for (int j = threadIdx.x; j < f; j += blockDim.x) {
                     const double z = J.xs[j];
@@ -1755,6 +1757,7 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
                     if (!(z >= -tau * u && z <= (1.0 + tau) * u)) bad = 1;
                 }
                 feasible = __syncthreads_or(bad) == 0;
+                if (MODE != 0 && !feasible && cta_timed_out(T.timeouts)) break;
             }
             if (feasible) {
                 for (int j = threadIdx.x; j < f; j += blockDim.x) {
@@ -1869,11 +1872,11 @@ k_solve(JobDev *const *jobs, DevInfo *batch_info, double *const *sigma_out) {
         if (threadIdx.x == 0) J.cmd[0] = kCmdDone;
         cluster_barrier();
     }
-    if (!converged && info.status == IMG_OK) info.status = IMG_ENOTCONV;
     if constexpr (MODE != 0) {
-        if (T.timeouts && info.status == IMG_OK) info.status = IMG_ETIMEOUT;
+        if (cta_timed_out(T.timeouts)) info.status = IMG_ETIMEOUT;
         tc_teardown(T, p);
     }
+    if (!converged && info.status == IMG_OK) info.status = IMG_ENOTCONV;
     double *out = sigma_out ? sigma_out[job] : nullptr;
     int nf = 0, nu = 0;
     for (int i = threadIdx.x; i < Q; i += blockDim.x) {

@@ -67,6 +67,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, unsign
     return false;
 }
 
+// Whether a wait of any thread of the CTA ran out (each thread counts its
+// own, and some waits are made by one thread only).  All threads call it.
+__device__ __forceinline__ bool cta_timed_out(int timeouts) { return __syncthreads_or(timeouts) != 0; }
+
 // ---------------------------------------------------------------- tcgen05
 __device__ __forceinline__ void tmem_alloc(uint32_t *dst_smem, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -216,9 +220,10 @@ struct TcWork {
     __device__ __forceinline__ unsigned char *Xlo(int b) const { return base + (2 * b + 1) * x_bytes(); }
     __device__ __forceinline__ unsigned char *Bhi() const { return base + 4 * x_bytes(); }
     __device__ __forceinline__ unsigned char *Blo() const { return base + 4 * x_bytes() + b_bytes(); }
-    // Wait for the next completion of barrier b.
+    // Wait for the next completion of barrier b.  After one wait of this thread
+    // has run out, later ones poll once, so that the kernel ends soon.
     __device__ __forceinline__ void wait(int b) {
-        if (!mbar_wait(&bar[b], (phase >> b) & 1u)) timeouts++;
+        if (!mbar_wait(&bar[b], (phase >> b) & 1u, timeouts ? 1u : kSpinLimit)) timeouts++;
         phase ^= 1u << b;
     }
 };

@@ -134,6 +134,12 @@ def test_wait_selftest_range(lib):
     assert lib.img_check_wait((1 << 26) + 1, 1) == L.IMG_EINVAL
 
 
+def test_wait_selftest_thread_range(lib):
+    assert lib.img_check_wait_thread(10, 1, 256) == L.IMG_EINVAL
+    assert lib.img_check_wait_thread(10, 1, -2) == L.IMG_EINVAL
+    assert lib.img_check_wait_thread(0, 1, 32) == L.IMG_EINVAL
+
+
 def test_server_null_arguments(lib):
     sp = L.ServerParams()
     lib.img_server_params_default(C.byref(sp))
