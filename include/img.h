@@ -57,7 +57,8 @@ typedef enum {
     IMG_ENOMEM = 2,     /* device allocation failed or a capacity exceeded   */
     IMG_ENOTPD = 3,     /* R_hat is not positive definite (Cholesky failed)  */
     IMG_ENOTCONV = 4,   /* active-set loop hit max_outer; partial image kept */
-    IMG_ETIMEOUT = 5,   /* a bounded device wait ran out                     */
+    IMG_ETIMEOUT = 5,   /* a bounded device wait ran out (in this call, or in
+                           work that an earlier call queued, on_device = 2)  */
     IMG_ECUDA = 6       /* CUDA runtime error (no device, launch failure)    */
 } img_status;
 
@@ -243,6 +244,11 @@ img_status img_check_wait(unsigned polls, int arrive);
  * of them), as for the solver's tile copies: its count reaches the status by
  * the same reduction as a solve's.  IMG_EINVAL also for other threads. */
 img_status img_check_wait_thread(unsigned polls, int arrive, int thread);
+
+/* The same queued on ctx's stream, reporting as an operator kernel of ctx
+ * does: the call returns IMG_OK without waiting, and when the wait ran out the
+ * next call on ctx that waits for its stream returns IMG_ETIMEOUT (once). */
+img_status img_check_wait_ctx(img_ctx *ctx, unsigned polls, int arrive);
 
 /* Unconstrained LS / WLS image with every pixel free (Sec. III-B/C: the LS
  * and WLS images; Sec. V-A: LSQR): min ||b - M x|| over all Q pixels with

@@ -26,7 +26,7 @@ SET_L, SET_U, SET_F = 0, 1, 2
 EXPORTS = ("img_params_default", "img_create", "img_set_covariance", "img_dirty",
            "img_mvdr_bound", "img_solve", "img_get_sets", "img_get_gradient", "img_get_events",
            "img_psi",
-           "img_psi_adj", "img_ls_image", "img_check_wait", "img_check_wait_thread", "img_snapshot_image", "img_snapshot_ls_image", "img_prepare_batch", "img_solve_batch", "img_psi_noalloc",
+           "img_psi_adj", "img_ls_image", "img_check_wait", "img_check_wait_thread", "img_check_wait_ctx", "img_snapshot_image", "img_snapshot_ls_image", "img_prepare_batch", "img_solve_batch", "img_psi_noalloc",
            "img_server_params_default", "img_server_create", "img_server_reserve", "img_server_submit",
            "img_server_wait", "img_server_destroy", "img_destroy", "img_status_str")
 
@@ -108,6 +108,8 @@ def load(build_if_missing: bool = False) -> C.CDLL:
     lib.img_check_wait.restype = i
     lib.img_check_wait_thread.argtypes = [C.c_uint, i, i]
     lib.img_check_wait_thread.restype = i
+    lib.img_check_wait_ctx.argtypes = [vp, C.c_uint, i]
+    lib.img_check_wait_ctx.restype = i
     lib.img_get_sets.argtypes = [vp, dp]
     lib.img_get_sets.restype = i
     lib.img_get_gradient.argtypes = [vp, dp]

@@ -46,6 +46,7 @@ struct img_ctx {
     cudaGraphExec_t ls_exec = nullptr;   // one LSQR iteration as a CUDA graph (own stream only)
     img::WsHost *ws = nullptr;   // graph-driven wide solver (created on the first wide solve)
     cudaEvent_t ev = nullptr;    // ordering event for batched wide solves
+    int *late = nullptr;         // pinned: a bounded wait of an operator or bounds kernel ran out
 };
 
 namespace {
@@ -203,7 +204,21 @@ bool finite_all(const double *v, size_t n) {
     return true;
 }
 
-img_status sync(img_ctx *c) { return cuda_status(cudaStreamSynchronize(c->stream)); }
+// Whether a wait of the context's operator or bounds kernels has run out since
+// the last call that asked; the context's work has been waited for.
+bool took_late(img_ctx *c) {
+    volatile int *w = c->late;
+    const bool late = *w != 0;
+    if (late) *w = 0;
+    return late;
+}
+
+// Wait for the context's stream.  IMG_ETIMEOUT also for work that an earlier
+// call queued without waiting (on_device = 2).
+img_status sync(img_ctx *c) {
+    const img_status st = cuda_status(cudaStreamSynchronize(c->stream));
+    return st == IMG_OK && took_late(c) ? IMG_ETIMEOUT : st;
+}
 
 // Factor, dirty image, bounds (once per covariance).
 img_status prepare(img_ctx *c) {
@@ -222,7 +237,8 @@ img_status prepare(img_ctx *c) {
     CK(img::launch_finalize(c->djp, 1, ntiles, c->stream, nullptr));
     int flag = 0;
     CK(cudaMemcpyAsync(&flag, c->hj.flags, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
+    const img_status st = sync(c);
+    if (st != IMG_OK) return st;
     c->prepared = true;
     c->prep_status = flag == 0 ? IMG_OK : IMG_ENOTPD;
     return (img_status)c->prep_status;
@@ -437,6 +453,12 @@ img_status img_create(const img_params *prm, img_ctx **out) {
         return IMG_ENOMEM;
     }
     carve(c, reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(c->dmem) + 255) & ~uintptr_t(255)));
+    if (cudaHostAlloc((void **)&c->late, sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostGetDevicePointer((void **)&J.late, c->late, 0) != cudaSuccess) {
+        img_destroy(c);
+        return IMG_ENOMEM;
+    }
+    *c->late = 0;
     img_status st = IMG_OK;
     int init_flags[4] = {-1, 0, 0, 0};
     if (cudaMemcpyAsync((void *)J.ant, c->ant.data(), 3 * P.p * sizeof(double), cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
@@ -781,6 +803,8 @@ img_status img_snapshot_ls_image(img_ctx *const *snap, int K, int maxit, double 
             CK(img::ls_xnorm2(s.hj[0], b, b.sc + img::kLsXnorm2, stream));
             CK(cudaMemcpyAsync(h, b.sc, sizeof(h), cudaMemcpyDeviceToHost, stream));
             CK(cudaStreamSynchronize(stream));
+            for (int k = 0; k < K; ++k)
+                if (took_late(snap[k])) return IMG_ETIMEOUT;
             const double anorm = std::sqrt(h[img::kLsAnorm2]), xnorm = std::sqrt(h[img::kLsXnorm2]);
             if (h[img::kLsRnorm] <= btol * h[img::kLsBnorm] + atol * anorm * xnorm) {
                 istop = 1;
@@ -817,11 +841,16 @@ img_status img_check_wait_thread(unsigned polls, int arrive, int thread) {
     int *d = nullptr;
     CK(cudaMalloc(&d, sizeof(int)));
     int h = -1;
-    cudaError_t e = img::launch_wait_selftest(polls, arrive ? 1 : 0, thread, d, nullptr);
+    cudaError_t e = img::launch_wait_selftest(polls, arrive ? 1 : 0, thread, d, nullptr, nullptr);
     if (e == cudaSuccess) e = cudaMemcpy(&h, d, sizeof(int), cudaMemcpyDeviceToHost);
     cudaFree(d);
     if (e != cudaSuccess) return IMG_ECUDA;
     return h == IMG_OK ? IMG_OK : IMG_ETIMEOUT;
+}
+
+img_status img_check_wait_ctx(img_ctx *c, unsigned polls, int arrive) {
+    if (!c || polls == 0 || polls > (1u << 26)) return IMG_EINVAL;
+    return cuda_status(img::launch_wait_selftest(polls, arrive ? 1 : 0, -1, nullptr, c->dj, c->stream));
 }
 
 img_status img_ls_image(img_ctx *c, int maxit, double *sigma, img_solve_info *info, int on_device) {
@@ -895,7 +924,8 @@ img_status img_ls_image(img_ctx *c, int maxit, double *sigma, img_solve_info *in
             // Paige-Saunders stopping tests on the host, every 10 iterations
             CK(img::ls_xnorm2(c->hj, b, b.sc + img::kLsXnorm2, c->stream));
             CK(cudaMemcpyAsync(h, b.sc, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
-            CK(cudaStreamSynchronize(c->stream));
+            st = sync(c);
+            if (st != IMG_OK) return st;
             const double anorm = std::sqrt(h[img::kLsAnorm2]), xnorm = std::sqrt(h[img::kLsXnorm2]);
             if (h[img::kLsRnorm] <= btol * h[img::kLsBnorm] + atol * anorm * xnorm) {
                 istop = 1;
@@ -1028,7 +1058,9 @@ img_status img_prepare_batch(img_ctx *const *ctxs, int n) {
     img_status first = IMG_OK;
     for (int q = 0; q < n; ++q) {
         img_ctx *c = ctxs[g.order[q]];
-        c->prepared = true;
+        const bool late = took_late(c);
+        if (late) first = IMG_ETIMEOUT;
+        c->prepared = !late;
         c->prep_status = flags[q] == 0 ? IMG_OK : IMG_ENOTPD;
     }
     for (int j = 0; j < n; ++j)
@@ -1134,7 +1166,9 @@ img_status img_solve_batch(img_ctx *const *ctxs, int n, double *const *sigma, im
     for (int q = 0; q < n; ++q) byjob[g.order[q]] = d[q];
     for (size_t k = 0; k < wide.size(); ++k) byjob[wide[k]] = dw[k];
     for (int j = 0; j < n; ++j) {
-        ctxs[j]->prepared = true;
+        const bool late = took_late(ctxs[j]);
+        if (late) byjob[j].status = IMG_ETIMEOUT;
+        ctxs[j]->prepared = !late;
         ctxs[j]->prep_status = byjob[j].status == IMG_ENOTPD ? IMG_ENOTPD : IMG_OK;
         ctxs[j]->solved = true;
         if (infos) fill_info(&infos[j], byjob[j]);
@@ -1147,6 +1181,7 @@ void img_destroy(img_ctx *c) {
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
     if (c->dmem) cudaFree(c->dmem);
+    if (c->late) cudaFreeHost(c->late);
     if (c->fwd_part) cudaFree(c->fwd_part);
     if (c->ls_exec) cudaGraphExecDestroy(c->ls_exec);
     if (c->ls_mem) cudaFree(c->ls_mem);
@@ -1449,6 +1484,7 @@ struct img_server {
             SJob *j = sl.group[q];
             const int Q = j->ctx->hj.Q;
             j->sigma.assign(sl.h_sigma + sl.sigma_off[q], sl.h_sigma + sl.sigma_off[q] + Q);
+            if (took_late(j->ctx)) sl.h_infos[q].status = IMG_ETIMEOUT;
             fill_info(&j->info, sl.h_infos[q]);
             j->st = (img_status)sl.h_infos[q].status;
             j->t_done = t;

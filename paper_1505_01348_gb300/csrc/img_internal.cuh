@@ -90,7 +90,8 @@ struct JobDev {
     int *cmd;              // words that the CTAs of one solve's cluster exchange
     // status and report
     DevInfo *info;
-    int *flags;            // [0]: factor status, [1]: bounds valid, [2]: timeout, [3]: bad pivot
+    int *flags;            // [0]: factor status, [1]: bounds valid, [3]: bad pivot
+    int *late;             // host word (mapped): set by an operator or bounds kernel whose wait ran out
 };
 
 // Kernel launchers (defined in the .cu files, called by the host API).
@@ -115,8 +116,10 @@ cudaError_t launch_job(JobDev *const *jobs, int n, int max_p, int mode, DevInfo 
 cudaError_t launch_psi(const JobDev *job_dev, const float *wx, float2 *part, int nparts, int Q,
                        int p, int mode, double2 *Kout, cudaStream_t st);
 // Bounded-wait self-test (one CTA; all its threads wait, or the given one;
-// *status: IMG_OK or IMG_ETIMEOUT).
-cudaError_t launch_wait_selftest(unsigned polls, int arrive, int thread, int *status, cudaStream_t st);
+// *status (may be null): IMG_OK or IMG_ETIMEOUT; job (may be null): as an
+// operator kernel of that job reports).
+cudaError_t launch_wait_selftest(unsigned polls, int arrive, int thread, int *status, const JobDev *job,
+                                 cudaStream_t st);
 
 // CTAs that leave per-CTA maxima of an operand (JobDev::opmax).
 constexpr int kOpMax = 256;

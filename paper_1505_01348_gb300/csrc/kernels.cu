@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_bounds_tc(JobDev *const *jobs) 
                 __syncthreads();
             });
     }
-    if (T.timeouts) J.flags[2] = IMG_ETIMEOUT;
+    post_late(J, T.timeouts);
     tc_teardown(T, J.p);
 }
 
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bounds_wide(JobDev *const *
     const int to = wide_adjoint<MODE == 2>(J, dyn, bars, &slot, J.Bimg, J.Bimg + wide_B_bytes(J.p), J.Bscale, 2,
                                            blockIdx.x, gridDim.x, mine, 2,
                                            [&](int s, int i, float v) { (s == 0 ? dirty : h)[i] = v; });
-    if (to && threadIdx.x == 0) J.flags[2] = IMG_ETIMEOUT;
+    post_late(J, to);
 }
 
 // max |entry| of one operator U, one value per CTA into the job's opmax, and
@@ -265,8 +265,9 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_psi_adj_wide(const JobDev *
     __shared__ uint32_t slot;
     const int ntiles = tc_num_tiles(J.n_l, J.n_m);
     const int mine = ntiles > (int)blockIdx.x ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    wide_adjoint<MODE == 2>(J, dyn, bars, &slot, J.Bimg, J.Bimg, J.Bscale, 1, blockIdx.x, gridDim.x, mine, 0,
-                            [&](int, int i, float v) { out[i] = v; });
+    const int to = wide_adjoint<MODE == 2>(J, dyn, bars, &slot, J.Bimg, J.Bimg, J.Bscale, 1, blockIdx.x, gridDim.x,
+                                           mine, 0, [&](int, int i, float v) { out[i] = v; });
+    post_late(J, to);
 }
 
 // ---------------------------------------------------------------- wide forward
@@ -300,8 +301,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_fwd_wide(const JobDev *Jp, c
     __shared__ uint64_t bars[kFwdBars];
     __shared__ uint32_t slot;
     const int pr = blockIdx.y, S = gridDim.x;
-    wide_forward<MODE == 2>(J, dyn, bars, &slot, w, wmax, nmax, map.m[pr], map.nb[pr], blockIdx.x, S,
-                            part + ((size_t)pr * S + blockIdx.x) * (kTcM * 256));
+    const int to = wide_forward<MODE == 2>(J, dyn, bars, &slot, w, wmax, nmax, map.m[pr], map.nb[pr], blockIdx.x, S,
+                                           part + ((size_t)pr * S + blockIdx.x) * (kTcM * 256));
+    post_late(J, to);
 }
 
 // K (p x p, column-major, interleaved; FP64 or FP32) from the S partials of the
@@ -606,9 +608,9 @@ __global__ void __launch_bounds__(256) k_cgemm(int p, const float2 *A, int opA, 
 // allocates tensor memory, waits on an mbarrier that receives an arrival only
 // when `arrive` is set - all its threads, or thread `thread` alone -, gives up
 // after `polls` polls, frees the tensor memory on its normal exit path and
-// reports through *status (IMG_OK or IMG_ETIMEOUT).  No fault, trap or endless
-// loop is involved.
-__global__ void k_wait_selftest(unsigned polls, int arrive, int thread, int *status) {
+// reports through *status (IMG_OK or IMG_ETIMEOUT) or as an operator kernel of
+// a job.  No fault, trap or endless loop is involved.
+__global__ void k_wait_selftest(unsigned polls, int arrive, int thread, int *status, const JobDev *job) {
     __shared__ uint64_t bar;
     __shared__ uint32_t slot;
     if (threadIdx.x == 0) mbar_init(&bar, 1);
@@ -623,11 +625,13 @@ __global__ void k_wait_selftest(unsigned polls, int arrive, int thread, int *sta
     tc_fence_before();
     const bool late = cta_timed_out(timeouts);
     if (threadIdx.x < 32) tmem_dealloc(slot, 32);
-    if (threadIdx.x == 0) *status = late ? IMG_ETIMEOUT : IMG_OK;
+    if (status && threadIdx.x == 0) *status = late ? IMG_ETIMEOUT : IMG_OK;
+    if (job) post_late(*job, timeouts);
 }
 
-cudaError_t launch_wait_selftest(unsigned polls, int arrive, int thread, int *status, cudaStream_t st) {
-    k_wait_selftest<<<1, kThreads, 0, st>>>(polls, arrive, thread, status);
+cudaError_t launch_wait_selftest(unsigned polls, int arrive, int thread, int *status, const JobDev *job,
+                                 cudaStream_t st) {
+    k_wait_selftest<<<1, kThreads, 0, st>>>(polls, arrive, thread, status, job);
     return cudaGetLastError();
 }
 

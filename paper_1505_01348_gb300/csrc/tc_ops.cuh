@@ -71,6 +71,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, unsign
 // own, and some waits are made by one thread only).  All threads call it.
 __device__ __forceinline__ bool cta_timed_out(int timeouts) { return __syncthreads_or(timeouts) != 0; }
 
+// Report waits that ran out to the host, from any thread.  The word is host
+// memory, so that the host reads it after its wait without a copy (a copy of
+// 4 bytes would add microseconds to every call that waits).
+__device__ __forceinline__ void post_late(const JobDev &J, int timeouts) {
+    if (timeouts) *J.late = 1;
+}
+
 // ---------------------------------------------------------------- tcgen05
 __device__ __forceinline__ void tmem_alloc(uint32_t *dst_smem, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(

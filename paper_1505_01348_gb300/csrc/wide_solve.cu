@@ -1251,7 +1251,7 @@ __global__ void k_ws_bnd_max(const JobDev *Jp, WsBufs B, const float2 *U, int fi
 __global__ void k_ws_bnd_out(const JobDev *Jp, WsBufs B, float *out) {
     const JobDev &J = *Jp;
     WsCtl *ctl = B.ctl;
-    if (ctl->timeouts && blockIdx.x == 0 && threadIdx.x == 0) J.flags[2] = IMG_ETIMEOUT;
+    if (blockIdx.x == 0 && threadIdx.x == 0) post_late(J, ctl->timeouts);
     if (ctl->stop) return;
     const UnitGeom g = unit_geom(J.p);
     const float s1 = steer_scale(J.p) * kLift * ctl->sB;
@@ -1267,6 +1267,7 @@ __global__ void k_ws_bnd_out(const JobDev *Jp, WsBufs B, float *out) {
 __global__ void k_ws_adj_out(const JobDev *Jp, WsBufs B, double *out) {
     const JobDev &J = *Jp;
     WsCtl *ctl = B.ctl;
+    if (blockIdx.x == 0 && threadIdx.x == 0) post_late(J, ctl->timeouts);
     if (ctl->stop) return;
     const UnitGeom g = unit_geom(J.p);
     const float sc = 1.f / (steer_scale(J.p) * kLift * ctl->sB);
