@@ -76,8 +76,13 @@ __host__ __device__ inline uint32_t sw_row_off(int r, int c16) {
 // ---------------------------------------------------------------- B unit image
 // One 16-byte chunk (8 K columns) of an image: its 8 source vectors' entries,
 // `part` chosen and scaled, split and stored at off (hi) and off + lo_off (lo).
-// The image kernels load several chunks before they store any: one chunk at a
-// time they are a chain of L2 latencies.
+// NC chunks are loaded before any is stored.  Inside the cluster LSQR, whose
+// CTAs have their SM to themselves, 4: one chunk at a time is a chain of L2
+// latencies.  In the kernels that take every SM, 1 (34 and 40 registers): with
+// 4 (95) their CTAs keep other solves' kernels off the SMs, and alone the
+// grid's threads hide the latency as well (256x256, p = 288, NC = 4 -> 1 with
+// whole forward blocks: first 1600 passes of 16 images in flight 5.45 -> 4.97 s,
+// of 4 images 2.46 -> 2.37 s, first 200 of one image 88 -> 87 ms).
 struct ImgChunk {
     float2 w[8];
     // 8 consecutive entries from src (null: zeros), the first n of them live.
@@ -103,24 +108,24 @@ struct ImgChunk {
         *reinterpret_cast<uint4 *>(at + lo_off) = lo;
     }
 };
-constexpr int kImgUnroll = 4;
+constexpr int kImgChunksCluster = 4, kImgChunksGrid = 1;
 
 // B unit image of U (p x p column-major FP32 complex, Hermitian), scaled by
 // sc, by threads t0, t0 + nt, ... of the launch:
 //   B[(Re, kr), (Re, kc)] = B[(Im, kr), (Im, kc)] = Re U(kc, kr)
 //   B[(Re, kr), (Im, kc)] = Im U(kc, kr),  B[(Im, kr), (Re, kc)] = -Im U(kc, kr)
 // so that x^T B x = Re(a^H U a) for x = [Re a; Im a].
-template <bool BF16>
+template <bool BF16, int NC>
 __device__ inline void unit_image(const float2 *U, int p, const UnitGeom &g, float sc, unsigned char *img, int t0,
                                   int nt) {
     const int ku = g.ku, rows = unit_rows(g), total = g.nu * g.nk * rows * 8;
     const bool vec = (p & 1) == 0;
-    for (int e0 = t0; e0 < total; e0 += kImgUnroll * nt) {
-        ImgChunk c[kImgUnroll];
-        unsigned char *at[kImgUnroll];
-        int kind[kImgUnroll];                       // 0: Re U, 1: Im U, 2: -Im U
+    for (int e0 = t0; e0 < total; e0 += NC * nt) {
+        ImgChunk c[NC];
+        unsigned char *at[NC];
+        int kind[NC];                       // 0: Re U, 1: Im U, 2: -Im U
 #pragma unroll
-        for (int q = 0; q < kImgUnroll; ++q) {
+        for (int q = 0; q < NC; ++q) {
             const int e = e0 + q * nt;
             at[q] = nullptr;
             if (e >= total) continue;
@@ -134,7 +139,7 @@ __device__ inline void unit_image(const float2 *U, int p, const UnitGeom &g, flo
             at[q] = img + (size_t)(u * g.nk + kc) * unit_block_bytes(g) + sw_row_off(n, c16);
         }
 #pragma unroll
-        for (int q = 0; q < kImgUnroll; ++q) {
+        for (int q = 0; q < NC; ++q) {
             if (!at[q]) continue;
             float v[8];
 #pragma unroll
@@ -149,17 +154,17 @@ __device__ inline void unit_image(const float2 *U, int p, const UnitGeom &g, flo
 // List image of the n vectors vec[pos[j] * p + k] (row j of the tiles; rows
 // beyond n and the padding chunks are zero), scaled by sX and, when wgt is
 // given, by the row weight wgt[j]; by threads t0, t0 + nt, ... of the launch.
-template <bool BF16>
+template <bool BF16, int NC>
 __device__ inline void list_image(const float2 *vec, const int *pos, const float *wgt, int n, int p, const UnitGeom &g,
                                   float sX, unsigned char *img, int t0, int nt) {
     const int total = (n + kTcM - 1) / kTcM * g.nkA * kTcM * 8;
     const bool v4 = (p & 1) == 0;
-    for (int e0 = t0; e0 < total; e0 += kImgUnroll * nt) {
-        ImgChunk c[kImgUnroll];
-        int sl[kImgUnroll];
-        float sw[kImgUnroll];
+    for (int e0 = t0; e0 < total; e0 += NC * nt) {
+        ImgChunk c[NC];
+        int sl[NC];
+        float sw[NC];
 #pragma unroll
-        for (int q = 0; q < kImgUnroll; ++q) {
+        for (int q = 0; q < NC; ++q) {
             const int e = e0 + q * nt;
             const int r = (e >> 3) % kTcM, r2 = (e >> 3) / kTcM, kc = r2 % g.nkA, j = r2 / g.nkA * kTcM + r;
             const bool live = e < total && j < n && kc < g.nk;
@@ -167,14 +172,14 @@ __device__ inline void list_image(const float2 *vec, const int *pos, const float
             sw[q] = live ? (wgt ? __ldcg(wgt + j) * sX : sX) : 0.f;
         }
 #pragma unroll
-        for (int q = 0; q < kImgUnroll; ++q) {
+        for (int q = 0; q < NC; ++q) {
             const int e = e0 + q * nt;
             const int kc = (e >> 3) / kTcM % g.nkA, col0 = kc * kChunkK + (e & 7) * 8;
             const int k0 = col0 >= g.Kp ? col0 - g.Kp : col0;
             c[q].load(sl[q] >= 0 ? vec + (size_t)sl[q] * p + k0 : nullptr, p - k0, v4);
         }
 #pragma unroll
-        for (int q = 0; q < kImgUnroll; ++q) {
+        for (int q = 0; q < NC; ++q) {
             const int e = e0 + q * nt;
             if (e >= total) break;
             const int r = (e >> 3) % kTcM, r2 = (e >> 3) / kTcM, kc = r2 % g.nkA, t = r2 / g.nkA;

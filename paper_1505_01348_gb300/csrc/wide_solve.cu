@@ -439,7 +439,7 @@ __global__ void k_ws_pass(const JobDev *Jp, WsBufs B, cudaGraphConditionalHandle
 // operand of a forward) into ximgW, scaled by sX sW with sW the power of two
 // of max |wl| (stored for the reduction).
 // CTA `rank` of `ctas` does its share.
-template <bool BF16>
+template <bool BF16, int NC>
 __device__ void ws_listimg(const JobDev &J, const WsBufs &B, const UnitGeom &g, int which, int weighted, int rank,
                            int ctas) {
     WsCtl *ctl = B.ctl;
@@ -455,30 +455,30 @@ __device__ void ws_listimg(const JobDev &J, const WsBufs &B, const UnitGeom &g, 
         sX *= sW;
     }
     const float *wgt = weighted ? B.wl : nullptr;
-    list_image<BF16>(vec, pos, wgt, n, J.p, g, sX, img, rank * blockDim.x + threadIdx.x, ctas * blockDim.x);
+    list_image<BF16, NC>(vec, pos, wgt, n, J.p, g, sX, img, rank * blockDim.x + threadIdx.x, ctas * blockDim.x);
 }
 template <bool BF16>
 __global__ void k_ws_listimg(const JobDev *Jp, WsBufs B, int which, int weighted) {
     ws_count(B.ctl);
     if (B.ctl->stop) return;
-    ws_listimg<BF16>(*Jp, B, unit_geom(Jp->p), which, weighted, blockIdx.x, gridDim.x);
+    ws_listimg<BF16, kImgChunksGrid>(*Jp, B, unit_geom(Jp->p), which, weighted, blockIdx.x, gridDim.x);
 }
 
 // B unit image of the matrix U (W0 for LSQR, W1 for the gradient) with the
 // power-of-two scale of ctl->mx_t.
-template <bool BF16>
+template <bool BF16, int NC>
 __device__ void ws_emb(const JobDev &J, const WsBufs &B, const UnitGeom &g, const float2 *U, int rank, int ctas) {
     WsCtl *ctl = B.ctl;
     const float sc = pow2_scale(__uint_as_float(ctl->mx_t)) * kLift;
     if (rank == 0 && threadIdx.x == 0) ctl->sB = sc;
-    unit_image<BF16>(U, J.p, g, sc, B.bimg, rank * blockDim.x + threadIdx.x, ctas * blockDim.x);
+    unit_image<BF16, NC>(U, J.p, g, sc, B.bimg, rank * blockDim.x + threadIdx.x, ctas * blockDim.x);
 }
 template <bool BF16>
 __global__ void k_ws_emb(const JobDev *Jp, WsBufs B, int grad, const float2 *Um) {
     ws_count(B.ctl);
     const JobDev &J = *Jp;
     if (B.ctl->stop) return;
-    ws_emb<BF16>(J, B, unit_geom(J.p), Um ? Um : (grad ? J.W1 : J.W0), blockIdx.x, gridDim.x);
+    ws_emb<BF16, kImgChunksGrid>(J, B, unit_geom(J.p), Um ? Um : (grad ? J.W1 : J.W0), blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------- operators
@@ -486,9 +486,13 @@ __global__ void k_ws_emb(const JobDev *Jp, WsBufs B, int grad, const float2 *Um)
 // -s_i x_i, cvec) or the support S (weights -s_i x_i, dvec / cvec): Gram
 // blocks from the list's image and its weighted image.  The list's split over
 // tasks (nsplit) fixes the order of the sums; how many of a block's 64-column
-// chunks one task takes does not, so blocks are cut into slices while there
-// are fewer tasks than CTAs.  dyn, bars, tmem: as items_forward.
-template <bool BF16>
+// chunks one task takes does not.  SLICE (the cluster's 8 CTAs): blocks are cut
+// into slices while there are fewer blocks than CTAs.  As a kernel, whose CTAs
+// share the GPU with other solves, whole blocks: each slice copies both A
+// chunks again (16 images of 256x256, p = 288, first 1600 passes 5.05 instead of
+// 4.97 s with slices, 4 images 2.42 instead of 2.37 s, one image the same).
+// dyn, bars, tmem: as items_forward.
+template <bool BF16, bool SLICE>
 __device__ int ws_forward(const WsBufs &B, const UnitGeom &g, int which, int rank, int ctas, unsigned char *dyn,
                           uint64_t *bars, uint32_t tmem) {
     const WsCtl *ctl = B.ctl;
@@ -497,7 +501,7 @@ __device__ int ws_forward(const WsBufs &B, const UnitGeom &g, int which, int ran
     if (n <= 0) return 0;
     const int nsplit = ctl->nsplit;
     const int blocks = B.npairs * nsplit;
-    const int slices = blocks >= 2 * ctas ? 1 : (2 * blocks >= ctas ? 2 : 4), nq = 4 / slices;
+    const int slices = !SLICE || blocks >= 2 * ctas ? 1 : (2 * blocks >= ctas ? 2 : 4), nq = 4 / slices;
     int to = 0;
     for (int task = rank; task < blocks * slices; task += ctas) {
         const int blk = task / slices, q0 = (task - blk * slices) * nq;
@@ -531,7 +535,7 @@ __global__ void __launch_bounds__(kItemsFwdThreads, 1) k_ws_fwd(const JobDev *Jp
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tslot;
-    const int to = ws_forward<BF16>(B, unit_geom(Jp->p), which, blockIdx.x, gridDim.x, dyn, bars, tmem);
+    const int to = ws_forward<BF16, false>(B, unit_geom(Jp->p), which, blockIdx.x, gridDim.x, dyn, bars, tmem);
     tc_fence_before();
     __syncthreads();
     if (threadIdx.x < 32) tmem_dealloc(tmem, 256);
@@ -1018,9 +1022,9 @@ k_ws_lsqr(const JobDev *Jp, WsBufs B) {
     tc_fence_after();
     const uint32_t tmem = tslot;
     // data b = base - sum_U s x c c^H, then M^H b
-    ws_listimg<BF16>(J, B, g, kListF, 0, rank, kLsqrCtas);
-    ws_listimg<BF16>(J, B, g, kListU, 0, rank, kLsqrCtas);
-    ws_listimg<BF16>(J, B, g, kListU, 1, rank, kLsqrCtas);
+    ws_listimg<BF16, kImgChunksCluster>(J, B, g, kListF, 0, rank, kLsqrCtas);
+    ws_listimg<BF16, kImgChunksCluster>(J, B, g, kListU, 0, rank, kLsqrCtas);
+    ws_listimg<BF16, kImgChunksCluster>(J, B, g, kListU, 1, rank, kLsqrCtas);
     cluster_sync();
     for (int it = 0;; ++it) {
         const bool init = it == 0;
@@ -1030,18 +1034,18 @@ k_ws_lsqr(const JobDev *Jp, WsBufs B) {
                 const bool more = vx_more(J, ctl, S, it - 1) && !*(volatile int *)&ctl->stop;
                 if (threadIdx.x == 0) ctl->cond[kCondLsqr] = more;
             }
-            ws_listimg<BF16>(J, B, g, kListF, 1, rank, kLsqrCtas);
+            ws_listimg<BF16, kImgChunksCluster>(J, B, g, kListF, 1, rank, kLsqrCtas);
             cluster_sync();
             if (!*(volatile unsigned *)&ctl->cond[kCondLsqr]) {
                 if (rank == 0 && threadIdx.x == 0) ctl->it = it - 1;
                 break;
             }
         }
-        ws_timeouts(ctl, ws_forward<BF16>(B, g, init ? kListU : kListF, rank, kLsqrCtas, dyn, bars, tmem));
+        ws_timeouts(ctl, ws_forward<BF16, true>(B, g, init ? kListU : kListF, rank, kLsqrCtas, dyn, bars, tmem));
         cluster_sync();
         ws_fred(J, B, g, init ? kRedB : kRedT, rank, kLsqrCtas);
         cluster_sync();
-        ws_emb<BF16>(J, B, g, J.W0, rank, kLsqrCtas);
+        ws_emb<BF16, kImgChunksCluster>(J, B, g, J.W0, rank, kLsqrCtas);
         cluster_sync();
         ws_timeouts(ctl, ws_adj_list<BF16>(J, B, g, rank, kLsqrCtas, dyn, bars, tmem, [&](int warp) {
                         if (rank == 0 && warp == 7) vx_beta(ctl, S, init);
