@@ -3,7 +3,8 @@
 //
 // The Table I loop is a graph WHILE node whose body is one pass (or two:
 // freeing the pixel chosen by the last gradient, then the next subproblem).
-// The subproblem's LSQR is an IF node holding one kernel, whose thread-block
+// The subproblem's LSQR is a SWITCH node: nothing (no free pixel), an
+// initialisation and a WHILE node of iterations, or one kernel whose thread-block
 // cluster iterates until the stopping tests hold; the feasible / infeasible
 // branch is an IF/ELSE node.  Kernels set the conditions from device memory, so
 // a whole solve runs without a host round trip.  Every kernel has a fixed grid
@@ -78,7 +79,10 @@ struct WsCtl {
     double sums[kWsSums];
 };
 
-enum { kCondOuter = 0, kCondLsqrIf = 1, kCondLsqr = 2, kCondFeas = 3 };
+enum { kCondOuter = 0, kCondLsqrForm = 1, kCondLsqr = 2, kCondFeas = 3 };
+// Values of kCondLsqrForm: a pass without free pixels, LSQR as kernels, as one
+// cluster kernel.
+enum : unsigned { kLsqrNone = 0, kLsqrKernels = 1, kLsqrCluster = 2 };
 
 // Set a graph condition (h != 0 inside the solve graph) and mirror it in the
 // control block for the host-driven mode.
@@ -100,6 +104,7 @@ struct WsBufs {
     int npairs, pm[kItemsFwdMaxPairs], pnb[kItemsFwdMaxPairs];
     int max_tasks;              // capacity of pfwd in blocks
     int list_grid;              // CTAs that the free-list adjoint's K groups are chosen for
+    int cluster_f;              // most free pixels of the cluster form of LSQR
     int fwd_per;                // 64-pixel stages per forward task (at least)
     int nrows_adj;              // rows of padj (max(Q, cap))
     int ld_adj;                 // partial dots per row of padj (nu nk)
@@ -378,8 +383,8 @@ __global__ void k_ws_free(const JobDev *Jp, WsBufs B) {
 
 // Then set up the subproblem of the next pass: compact F and U, the U
 // weights -s_i x_i (eq. bsubproblemLS / MVDR), the F scales, the list scales
-// and the LSQR iteration cap; h_lif := (|F| > 0).
-__global__ void k_ws_pass(const JobDev *Jp, WsBufs B, cudaGraphConditionalHandle h_lif) {
+// and the LSQR iteration cap; h_form := the form of LSQR (none when F is empty).
+__global__ void k_ws_pass(const JobDev *Jp, WsBufs B, cudaGraphConditionalHandle h_form) {
     ws_count(B.ctl);
     const JobDev &J = *Jp;
     WsCtl *ctl = B.ctl;
@@ -395,7 +400,7 @@ __global__ void k_ws_pass(const JobDev *Jp, WsBufs B, cudaGraphConditionalHandle
     if (s_skip) {
         if (threadIdx.x == 0) {
             ctl->f = 0;
-            ws_cond(ctl, kCondLsqrIf, h_lif, 0u);
+            ws_cond(ctl, kCondLsqrForm, h_form, kLsqrNone);
         }
         return;
     }
@@ -427,7 +432,7 @@ __global__ void k_ws_pass(const JobDev *Jp, WsBufs B, cudaGraphConditionalHandle
         ctl->maxit = J.lsqr_maxit > 0 ? J.lsqr_maxit : 4 * f + 20;
         ctl->it = 0;
         ctl->op_flops += ws_flops_fwd(J.p, nu);
-        ws_cond(ctl, kCondLsqrIf, h_lif, f > 0 ? 1u : 0u);
+        ws_cond(ctl, kCondLsqrForm, h_form, f == 0 ? kLsqrNone : f <= B.cluster_f ? kLsqrCluster : kLsqrKernels);
     }
 }
 
@@ -741,16 +746,16 @@ __device__ int ws_adj_list(const JobDev &J, const WsBufs &B, const UnitGeom &g, 
 //   B image of t | free-list adjoint | vectors (one CTA)
 //
 // each a few microseconds of work for a list of some hundred pixels.  Two
-// forms of the same phases, chosen by ws_clustered:
+// forms of the same phases, chosen by the length of the list (ws_cluster_f):
 //
-// * small operands: one kernel, a cluster of kLsqrCtas CTAs that walks the
-//   phases, separated by cluster barriers, until the stopping tests hold.
+// * short lists, small operands: one kernel, a cluster of kLsqrCtas CTAs that
+//   walks the phases, separated by cluster barriers, until the stopping tests hold.
 //   As kernels of the solve's graph most of an iteration's ~45 us at p = 100
 //   is launch, ramp and drain between the phases.  Eight CTAs are one portable
 //   cluster: the hardware places them together, so no phase waits for another
 //   solve's CTAs, and 16 solves in flight leave SMs for their gradients.
-// * large operands: a graph WHILE node of one kernel per phase, whose grids
-//   spread the images and the reduction over every SM.
+// * long lists, large operands: a graph WHILE node of one kernel per phase,
+//   whose grids spread the images and the reduction over every SM.
 //
 // Shares and splits follow the list alone (not the CTA count), so every sum
 // has the same order in both.
@@ -1351,7 +1356,6 @@ struct WsHost {
     int device = 0;
     int bf16 = 0;
     int direct = 0;             // host-driven loop instead of the graph
-    int cluster = 0;            // LSQR as one cluster kernel
     int sms = 1;
     unsigned *h_cond = nullptr; // pinned mirror of the conditions
     const JobDev *dj = nullptr;
@@ -1396,12 +1400,18 @@ size_t ws_bytes(const JobDev &hj, int sms, WsBufs *B, char *base) {
     return off + 1024;
 }
 
-// LSQR as one cluster kernel (see there) when the B image has one unit, p <=
-// 128.  Time per iteration, 64x64 pixels, 300 passes (f <= 150), cluster /
-// kernels: p = 70: 34.7 / 40.4 us, 100: 38.3 / 41.2, 128: 39.5 / 42.9, but 130:
-// 54.0 / 40.7, 288: 104 / 48 (the reduction and the B image of 81 and 27 tiles
-// need more than 8 SMs).  16 solves in flight: p = 100: 41 / 61 us each.
-static bool ws_clustered(const UnitGeom &g) { return g.nu == 1; }
+// Most free pixels of LSQR as one cluster kernel (see there): 512 while the B
+// image has one unit (p <= 128), none above that.  us per iteration over passes
+// that free one pixel each (20 iterations per pass), cluster / kernels, one
+// image of p = 100, 72x72 pixels: f = 50 .. 100: 38 / 48, 250 .. 300: 50 / 57,
+// 400 .. 500: 54 / 56, 500 .. 700: 65 / 54, 1000 .. 1500: 87 / 65 (8 SMs walk
+// lists that fill 32 and more); p = 72: 48 / 53 and 56 / 50 to both sides of
+// 500, p = 128: 54 / 57 and 66 / 55.  With 16 images in flight the 8 SMs of a
+// cluster stay ahead for longer (p = 100, f = 500 .. 750: 72 / 78, 750 .. 1000: 84
+// / 88), with 4 the lines cross at 600.  p = 130 at 64x64, f <= 150: 54 / 41, p =
+// 288: 104 / 48 (the reduction and the B image need more than 8 SMs).
+constexpr int kClusterF = 512;
+static int ws_cluster_f(const UnitGeom &g) { return g.nu == 1 ? kClusterF : 0; }
 
 // The launches of LSQR's initialisation and of one iteration as kernels.
 template <bool BF>
@@ -1438,10 +1448,10 @@ static cudaError_t ws_capture(WsHost *w, const JobDev *dj, const JobDev &hj, int
     cudaStreamCreateWithFlags(&c.st, cudaStreamNonBlocking);
     cudaGraph_t G = nullptr;
     c.err = cudaGraphCreate(&G, 0);
-    cudaGraphConditionalHandle h_outer = 0, h_lif = 0, h_lsqr = 0, h_feas = 0;
+    cudaGraphConditionalHandle h_outer = 0, h_form = 0, h_lsqr = 0, h_feas = 0;
     if (c.err == cudaSuccess) c.err = cudaGraphConditionalHandleCreate(&h_outer, G, 1, cudaGraphCondAssignDefault);
-    if (c.err == cudaSuccess) c.err = cudaGraphConditionalHandleCreate(&h_lif, G, 0, 0);
-    if (c.err == cudaSuccess && !w->cluster) c.err = cudaGraphConditionalHandleCreate(&h_lsqr, G, 0, 0);
+    if (c.err == cudaSuccess) c.err = cudaGraphConditionalHandleCreate(&h_form, G, 0, 0);
+    if (c.err == cudaSuccess) c.err = cudaGraphConditionalHandleCreate(&h_lsqr, G, 0, 0);
     if (c.err == cudaSuccess) c.err = cudaGraphConditionalHandleCreate(&h_feas, G, 0, 0);
     const size_t fsm = items_fwd_smem_bytes(), asm_ = items_smem_bytes();
     if (c.err == cudaSuccess) c.err = set_smem(k_ws_fwd<BF>, fsm);
@@ -1468,28 +1478,32 @@ static cudaError_t ws_capture(WsHost *w, const JobDev *dj, const JobDev &hj, int
     c.begin(ob[0], nullptr);
     k_ws_free<<<1, 32, 0, s>>>(dj, B);
     k_ws_cache<<<g_cache, kWsThreads, 0, s>>>(dj, B);
-    k_ws_pass<<<1, kWsThreads, 0, s>>>(dj, B, h_lif);
+    k_ws_pass<<<1, kWsThreads, 0, s>>>(dj, B, h_form);
     c.check();
     cudaGraphNode_t n1 = c.end();
-    cudaGraph_t lb[1] = {};
-    cudaGraphNode_t nif = add_cond(c, ob[0], h_lif, cudaGraphCondTypeIf, 1, n1, lb);
-    // LSQR on F (Sec. V-A)
-    c.begin(lb[0], nullptr);
-    if (w->cluster) {
+    // LSQR on F (Sec. V-A), in the form that k_ws_pass chose: a switch over
+    // kLsqr* (its body 0 is empty), or an IF where there are only kernels
+    cudaGraph_t lb[3] = {};
+    cudaGraphNode_t nif;
+    if (w->B.cluster_f > 0) {
+        nif = add_cond(c, ob[0], h_form, cudaGraphCondTypeSwitch, 3, n1, lb);
+        c.begin(lb[kLsqrCluster], nullptr);
         k_ws_lsqr<BF><<<kLsqrCtas, kThreads, asm_, s>>>(dj, B);
         c.check();
         c.end();
     } else {
-        ws_lsqr_begin<BF>(w, s, h_lsqr);
-        c.check();
-        cudaGraphNode_t n2 = c.end();
-        cudaGraph_t wb[1] = {};
-        add_cond(c, lb[0], h_lsqr, cudaGraphCondTypeWhile, 1, n2, wb);
-        c.begin(wb[0], nullptr);
-        ws_lsqr_iterate<BF>(w, s, h_lsqr);
-        c.check();
-        c.end();
+        nif = add_cond(c, ob[0], h_form, cudaGraphCondTypeIf, 1, n1, lb + kLsqrKernels);
     }
+    c.begin(lb[kLsqrKernels], nullptr);
+    ws_lsqr_begin<BF>(w, s, h_lsqr);
+    c.check();
+    cudaGraphNode_t n2 = c.end();
+    cudaGraph_t wb[1] = {};
+    add_cond(c, lb[kLsqrKernels], h_lsqr, cudaGraphCondTypeWhile, 1, n2, wb);
+    c.begin(wb[0], nullptr);
+    ws_lsqr_iterate<BF>(w, s, h_lsqr);
+    c.check();
+    c.end();
     // feasibility, then the gradient (feasible) or the step (infeasible)
     c.begin(ob[0], nif);
     k_ws_feas<<<1, kWsThreads, 0, s>>>(dj, B, h_feas);
@@ -1549,13 +1563,12 @@ static cudaError_t ws_direct(WsHost *w, cudaStream_t s) {
         k_ws_free<<<1, 32, 0, s>>>(dj, B);
         k_ws_cache<<<g_cache, kWsThreads, 0, s>>>(dj, B);
         k_ws_pass<<<1, kWsThreads, 0, s>>>(dj, B, 0);
-        if (cond(kCondLsqrIf)) {
-            if (w->cluster) {
-                k_ws_lsqr<BF><<<kLsqrCtas, kThreads, asm_, s>>>(dj, B);
-            } else {
-                ws_lsqr_begin<BF>(w, s, 0);
-                while (cond(kCondLsqr)) ws_lsqr_iterate<BF>(w, s, 0);
-            }
+        const unsigned form = cond(kCondLsqrForm);
+        if (form == kLsqrCluster) {
+            k_ws_lsqr<BF><<<kLsqrCtas, kThreads, asm_, s>>>(dj, B);
+        } else if (form == kLsqrKernels) {
+            ws_lsqr_begin<BF>(w, s, 0);
+            while (cond(kCondLsqr)) ws_lsqr_iterate<BF>(w, s, 0);
         }
         k_ws_feas<<<1, kWsThreads, 0, s>>>(dj, B, 0);
         if (cond(kCondFeas)) {
@@ -1614,7 +1627,6 @@ cudaError_t ws_create(const JobDev &hj, const JobDev *dj, int mode, WsHost **out
     w->p = hj.p;
     w->cap = hj.cap;
     w->Q = hj.Q;
-    w->cluster = ws_clustered(w->g);
     {
         const int ntr = (hj.p + kRedTile - 1) / kRedTile;
         w->g_red = std::min(ntr * ntr, kWsSums);
@@ -1631,6 +1643,7 @@ cudaError_t ws_create(const JobDev &hj, const JobDev *dj, int mode, WsHost **out
     }
     char *base = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(w->mem) + 1023) & ~uintptr_t(1023));
     ws_bytes(hj, sms, &w->B, base);
+    w->B.cluster_f = ws_cluster_f(w->g);
     e = w->bf16 ? ws_carveout<true>() : ws_carveout<false>();
     if (e == cudaSuccess) e = set_smem(k_ws_adj<true>, items_smem_bytes());
     if (e == cudaSuccess) e = set_smem(k_ws_adj<false>, items_smem_bytes());

@@ -1,8 +1,9 @@
-"""The cluster form of LSQR (64 < p <= 128) on long free lists: every CTA of
-the cluster takes several forward tasks and several adjoint items per phase,
-phase after phase on the same barriers, for more than a thousand passes.  The
-oracle replays the decisions (ties within 1e-6 of scale); the image is held to
-max(1e-4, 8 cond(M_F) 2^-24), the attainable accuracy of FP32 LSQR vectors."""
+"""LSQR of the wide solver (64 < p <= 128) on long free lists: every CTA of the
+cluster form takes several forward tasks and several adjoint items per phase,
+phase after phase on the same barriers, for about a thousand passes; above 512
+free pixels the kernels take over.  The oracle replays the decisions (ties
+within 1e-6 of scale); the image is held to max(1e-4, 8 cond(M_F) 2^-24), the
+attainable accuracy of FP32 LSQR vectors."""
 import numpy as np
 import pytest
 
@@ -39,3 +40,37 @@ def test_cluster_lsqr_on_a_growing_list_follows_the_oracle(G):
     cond = np.sqrt(np.linalg.cond(np.abs(A[:, F].conj().T @ A[:, F]) ** 2))
     err = np.linalg.norm(sigma - rep.result.sigma) / np.linalg.norm(rep.result.sigma)
     assert err <= max(1e-4, 8.0 * cond * 2.0 ** -24)
+
+
+# one kernel per subproblem in the cluster form, six per iteration otherwise
+@pytest.mark.parametrize("p,prec", [(66, 1), (128, 2)])
+def test_long_lists_leave_the_cluster(G, p, prec):
+    job = synth.custom(940 + p, p, 40, 40, 12, 20000, radius=60.0, snr_db=0.0)
+
+    def run(passes):
+        im = G.Imager.from_job(job, precision=prec, kappa=0.1, lsqr_maxit=20, max_outer=passes)
+        _, info = im.solve()
+        im.close()
+        return info
+
+    a, b, c = run(900), run(960), run(1120)
+    assert a.n_free < b.n_free <= 512 < c.n_free
+    per_it = lambda x, y: (y.cyc_aux[0] - x.cyc_aux[0]) / (y.lsqr_iters - x.lsqr_iters)
+    assert per_it(a, b) < 3.0               # kernels of a pass over its 20 iterations
+    assert per_it(b, c) > 3.0               # most of these passes have more than 512
+
+
+@pytest.mark.parametrize("p,cost", [(72, O.COST_PWLS), (120, O.COST_LS)])
+def test_host_loop_runs_the_same_forms(G, p, cost, monkeypatch):
+    """The solve's graph and the host-driven loop give the same bits on lists
+    to both sides of 512 pixels."""
+    job = synth.custom(950 + p, p, 30, 30, 10, 20000, radius=50.0, snr_db=0.0)
+    out = []
+    for graph in ("1", "0"):
+        monkeypatch.setenv("IMG_SOLVE_GRAPH", graph)
+        im = G.Imager.from_job(job, precision=1, cost=cost, kappa=0.1, lsqr_maxit=20, max_outer=1200)
+        out.append(im.solve())
+        im.close()
+    assert out[0][1].n_free > 512
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    assert out[0][1].lsqr_iters == out[1][1].lsqr_iters
