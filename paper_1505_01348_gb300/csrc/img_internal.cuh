@@ -106,7 +106,8 @@ cudaError_t launch_bounds(JobDev *const *jobs, int n, int max_tiles, int max_p, 
 // max_tiles: most 64-pixel tiles of any job
 cudaError_t launch_finalize(JobDev *const *jobs, int n, int max_tiles, cudaStream_t st, int *batch_status);
 // mode: 0 CUDA-core FP32 operators, 1 tensor cores FP16x3, 2 tensor cores BF16x3;
-// ctas: CTAs per job (1, 2, 4 or kSolveCtas: a cluster that shares the gradients)
+// ctas: CTAs per job (1, 2, 4 or kSolveCtas: a cluster that shares the
+// gradients; fewer where the GPU has no room for it)
 constexpr int kSolveCtas = 8;
 cudaError_t launch_solve(JobDev *const *jobs, int n, int max_p, int mode, int ctas, DevInfo *batch_info,
                          double *const *sigma_out, cudaStream_t st);

@@ -11,6 +11,7 @@
 #include "cta_ops.cuh"
 #include "tc_ops.cuh"
 #include "tc_wide.cuh"
+#include "cluster_fit.cuh"
 
 #include <mutex>
 #include <unordered_map>
@@ -2153,6 +2154,10 @@ static cudaError_t launch_solve_t(JobDev *const *jobs, int n, size_t sm, int cta
                                   double *const *sigma_out, cudaStream_t st) {
     cudaError_t e = ensure_smem((const void *)k_solve<MODE, PREP>, sm);
     if (e != cudaSuccess) return e;
+    if (ctas > 1)
+        ctas = cluster_that_fits(ctas, [&](int c) {
+            return active_clusters((const void *)k_solve<MODE, PREP>, c, kThreads, sm);
+        });
     if (ctas > 1) {
         cudaLaunchAttribute attr{};
         attr.id = cudaLaunchAttributeClusterDimension;

@@ -26,6 +26,7 @@
 
 #include "cta_ops.cuh"
 #include "tc_items.cuh"
+#include "cluster_fit.cuh"
 
 namespace img {
 
@@ -1401,7 +1402,8 @@ size_t ws_bytes(const JobDev &hj, int sms, WsBufs *B, char *base) {
 }
 
 // Most free pixels of LSQR as one cluster kernel (see there): 512 while the B
-// image has one unit (p <= 128), none above that.  us per iteration over passes
+// image has one unit (p <= 128), none above that or where the GPU has no room
+// for the cluster (a partition with fewer SMs).  us per iteration over passes
 // that free one pixel each (20 iterations per pass), cluster / kernels, one
 // image of p = 100, 72x72 pixels: f = 50 .. 100: 38 / 48, 250 .. 300: 50 / 57,
 // 400 .. 500: 54 / 56, 500 .. 700: 65 / 54, 1000 .. 1500: 87 / 65 (8 SMs walk
@@ -1411,7 +1413,12 @@ size_t ws_bytes(const JobDev &hj, int sms, WsBufs *B, char *base) {
 // / 88), with 4 the lines cross at 600.  p = 130 at 64x64, f <= 150: 54 / 41, p =
 // 288: 104 / 48 (the reduction and the B image need more than 8 SMs).
 constexpr int kClusterF = 512;
-static int ws_cluster_f(const UnitGeom &g) { return g.nu == 1 ? kClusterF : 0; }
+template <bool BF>
+static int ws_cluster_f(const UnitGeom &g) {
+    const size_t sm = items_smem_bytes();
+    if (g.nu != 1 || set_smem(k_ws_lsqr<BF>, sm) != cudaSuccess) return 0;
+    return active_clusters((const void *)k_ws_lsqr<BF>, kLsqrCtas, kThreads, sm) > 0 ? kClusterF : 0;
+}
 
 // The launches of LSQR's initialisation and of one iteration as kernels.
 template <bool BF>
@@ -1455,7 +1462,6 @@ static cudaError_t ws_capture(WsHost *w, const JobDev *dj, const JobDev &hj, int
     if (c.err == cudaSuccess) c.err = cudaGraphConditionalHandleCreate(&h_feas, G, 0, 0);
     const size_t fsm = items_fwd_smem_bytes(), asm_ = items_smem_bytes();
     if (c.err == cudaSuccess) c.err = set_smem(k_ws_fwd<BF>, fsm);
-    if (c.err == cudaSuccess) c.err = set_smem(k_ws_lsqr<BF>, asm_);
     if (c.err == cudaSuccess) c.err = set_smem(k_ws_adj_list<BF>, asm_);
     if (c.err == cudaSuccess) c.err = set_smem(k_ws_adj<BF>, asm_);
     const int g_grad = std::min((hj.Q + kWsThreads - 1) / kWsThreads, 4 * sms);
@@ -1643,7 +1649,7 @@ cudaError_t ws_create(const JobDev &hj, const JobDev *dj, int mode, WsHost **out
     }
     char *base = reinterpret_cast<char *>((reinterpret_cast<uintptr_t>(w->mem) + 1023) & ~uintptr_t(1023));
     ws_bytes(hj, sms, &w->B, base);
-    w->B.cluster_f = ws_cluster_f(w->g);
+    w->B.cluster_f = w->bf16 ? ws_cluster_f<true>(w->g) : ws_cluster_f<false>(w->g);
     e = w->bf16 ? ws_carveout<true>() : ws_carveout<false>();
     if (e == cudaSuccess) e = set_smem(k_ws_adj<true>, items_smem_bytes());
     if (e == cudaSuccess) e = set_smem(k_ws_adj<false>, items_smem_bytes());
@@ -1657,10 +1663,8 @@ cudaError_t ws_create(const JobDev &hj, const JobDev *dj, int mode, WsHost **out
             // the attributes the graph build would set
             e = set_smem(k_ws_fwd<true>, items_fwd_smem_bytes());
             if (e == cudaSuccess) e = set_smem(k_ws_fwd<false>, items_fwd_smem_bytes());
-            if (e == cudaSuccess) e = set_smem(k_ws_lsqr<true>, items_smem_bytes());
             if (e == cudaSuccess) e = set_smem(k_ws_adj_list<true>, items_smem_bytes());
             if (e == cudaSuccess) e = set_smem(k_ws_adj<true>, items_smem_bytes());
-            if (e == cudaSuccess) e = set_smem(k_ws_lsqr<false>, items_smem_bytes());
             if (e == cudaSuccess) e = set_smem(k_ws_adj_list<false>, items_smem_bytes());
             if (e == cudaSuccess) e = set_smem(k_ws_adj<false>, items_smem_bytes());
         }
