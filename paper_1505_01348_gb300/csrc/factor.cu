@@ -269,8 +269,14 @@ __global__ void __launch_bounds__(kInvT * kInvT) k_fac_out(JobDev *const *jobs) 
 
 }  // namespace
 
-// Factor n jobs of at most max_p antennas: two launches per kNb columns.
+// Factor n jobs of at most max_p antennas: two launches per kNb columns, or,
+// while the launches cost more than one SM's FP64 pipe, one CTA per job in one
+// launch.  A call of set_covariance + dirty image (64 pixels to 256, FP32),
+// panels / one CTA: p = 2: 67 / 61 us, 4: 73 / 66, 6: 79 / 76, 8: 88 / 87, 10: 92
+// / 98, 12: 97 / 106, 16: 106 / 136.
+constexpr int kOneCtaP = 8;
 cudaError_t launch_factor(JobDev *const *jobs, int n, int max_p, cudaStream_t st) {
+    if (max_p <= kOneCtaP) return launch_factor_one(jobs, n, st);
     k_fac_init<<<dim3(n, (max_p * max_p + 1023) / 1024), 256, 0, st>>>(jobs);
     const int cols = (max_p + kTrailC - 1) / kTrailC;
     for (int j0 = 0; j0 < max_p; j0 += kNb) {

@@ -99,6 +99,7 @@ struct JobDev {
 cudaError_t launch_tables(JobDev *const *jobs, int n, cudaStream_t st);
 // Cholesky factor, L^-1, R^-1 (factor.cu); max_p: most antennas of any job.
 cudaError_t launch_factor(JobDev *const *jobs, int n, int max_p, cudaStream_t st);
+cudaError_t launch_factor_one(JobDev *const *jobs, int n, cudaStream_t st);
 // mode 1/2 use tensor cores: the shared-memory operator for p <= 64, the
 // streamed (wide) operator for 64 < p <= 256.
 cudaError_t launch_bounds(JobDev *const *jobs, int n, int max_tiles, int max_p, int mode,

@@ -2,7 +2,7 @@
 //
 //   k_tables    separable steering tables (FP64 phase reduction + sincospi)
 //   factor_job  Cholesky R = L L^H, L^-1 and R^-1 in FP64 by one CTA (the
-//               fused server kernel; all other paths: factor.cu)
+//               fused server kernel, p <= 8; all other paths: factor.cu)
 //   k_bounds    dirty image a^H R a and a^H R^-1 a over all pixels (many CTAs
 //               per job), the adjoint operator with U = R_hat and R_hat^-1
 //   k_finalize  MVDR bound, D, thresholds (Sec. III-D, Appendix A)
@@ -130,6 +130,17 @@ __device__ void factor_job(const JobDev &J) {
         J.R32[e] = make_float2((float)J.R64[e].x, (float)J.R64[e].y);
     }
     if (threadIdx.x == 0) J.flags[0] = 0;
+}
+
+// The smallest jobs' factor (launch_factor).
+__global__ void k_factor_one(JobDev *const *jobs) {
+    const JobDev &J = *jobs[blockIdx.x];
+    if (threadIdx.x == 0) *J.vmax = 0ull;            // (k_finalize)
+    factor_job(J);
+}
+cudaError_t launch_factor_one(JobDev *const *jobs, int n, cudaStream_t st) {
+    k_factor_one<<<n, kThreads, 0, st>>>(jobs);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- bounds
@@ -710,6 +721,12 @@ __global__ void k_finalize(JobDev *const *jobs, int *batch_status) {
         mx = fmax(mx, finalize_pixel(J, k, i));
     mx = block_max_pos(mx, sbuf);
     if (threadIdx.x == 0 && mx > 0.0) atomicMax(J.vmax, (unsigned long long)__double_as_longlong(mx));
+}
+// The smallest jobs: both in one launch.
+__global__ void k_finalize_one(JobDev *const *jobs, int *batch_status) {
+    const JobDev &J = *jobs[blockIdx.x];
+    if (batch_status && threadIdx.x == 0) batch_status[blockIdx.x] = J.flags[0];
+    if (J.flags[0] == 0) finalize_job(J);
 }
 __global__ void k_eps_floor(JobDev *const *jobs) {
     const JobDev &J = *jobs[blockIdx.x];
@@ -2140,10 +2157,18 @@ cudaError_t launch_bounds(JobDev *const *jobs, int n, int max_tiles, int max_p, 
     return cudaGetLastError();
 }
 
+// Up to 512 pixels one CTA per job in one launch (set_covariance + dirty image
+// at p = 16, two launches / one: 256 pixels: 105 / 103 us, 400: 106 / 103, 576: 106
+// / 107, 1024: 108 / 115; p = 4, 64 pixels: 73 / 67).
+constexpr int kFinalizeOne = 2;              // thread blocks of pixels
 cudaError_t launch_finalize(JobDev *const *jobs, int n, int max_tiles, cudaStream_t st, int *batch_status) {
     // one pixel per thread while the CTAs of all jobs stay within a few waves
     const int need = (max_tiles * kTile + kThreads - 1) / kThreads;
-    const dim3 grid(n, max(1, min(need, 8 * num_sms() / n)));
+    if (need <= kFinalizeOne) {
+        k_finalize_one<<<n, kThreads, 0, st>>>(jobs, batch_status);
+        return cudaGetLastError();
+    }
+    const dim3 grid(n, min(need, max(1, 8 * num_sms() / n)));
     k_finalize<<<grid, kThreads, 0, st>>>(jobs, batch_status);
     k_eps_floor<<<grid, kThreads, 0, st>>>(jobs);
     return cudaGetLastError();

@@ -57,3 +57,33 @@ def test_bad_pivot_is_reported(G, p, k):
     im.set_covariance(job.R, job.N)
     assert _mvdr_error(im.mvdr_bound(), job) <= 1e-5
     im.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("p", [2, 5, 8])
+def test_small_jobs_take_the_same_bits_from_either_form(G, p, prec):
+    """Alone, a small job is factored by one CTA; in a batch with a larger job
+    it goes through the panels and the larger job's pixel grid."""
+    small = synth.custom(760 + p, p, 13, 17, 2, 8 * p + 50, radius=4.0)
+    large = synth.custom(770, 40, 33, 20, 2, 400, radius=4.0)
+    a = G.Imager.from_job(small, precision=prec)
+    b, c = G.Imager.from_job(small, precision=prec), G.Imager.from_job(large, precision=prec)
+    G.prepare_batch([b, c])
+    np.testing.assert_array_equal(a.dirty(), b.dirty())
+    np.testing.assert_array_equal(a.mvdr_bound(), b.mvdr_bound())
+    np.testing.assert_array_equal(a.solve()[0], b.solve()[0])
+    for im in (a, b, c):
+        im.close()
+
+
+@pytest.mark.parametrize("p", [16, 45, 64])
+def test_server_factor_takes_the_same_bits(G, p):
+    """The server's fused kernel factors in one CTA, img_solve over panels."""
+    job = synth.custom(780 + p, p, 18, 15, 3, 8 * p + 50, radius=6.0)
+    im = G.Imager.from_job(job, precision=1, kappa=3.0)
+    alone, _ = im.solve()
+    im.close()
+    srv = G.Server()
+    image, _, _ = srv.wait(srv.submit_job(job, precision=1, kappa=3.0))
+    srv.close()
+    np.testing.assert_array_equal(alone, image)
