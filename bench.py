@@ -159,13 +159,16 @@ def measured_peaks():
 
 
 def prepare_launches(p: int, B: int, precision: str) -> int:
-    """Kernels of one prepare_batch call on B jobs of p antennas in one
-    arithmetic: the factor's start, its panels of 16 columns with a trailing
-    update after each but the last, and its products; the bounds (one launch
-    for all jobs, above p = 256 on the tensor cores eleven per job); two for
-    the thresholds."""
-    factor = 2 + 2 * (-(-p // 16)) - 1
-    bounds = 11 * B if p > 256 and precision != "fp32" else 1
+    """Kernels of one prepare_batch call on B jobs of p antennas, more than
+    512 pixels each, in one arithmetic: the factor's start, its panels of 16
+    columns with a trailing update after each but the last, and its products
+    (one kernel up to p = 8); the bounds (one kernel for all jobs; on the
+    tensor cores three for 64 < p <= 256 - maxima, operand images, operators -
+    and eleven per job above); two for the thresholds."""
+    factor = 1 if p <= 8 else 2 + 2 * (-(-p // 16)) - 1
+    bounds = 1
+    if precision != "fp32" and p > 64:
+        bounds = 3 if p <= 256 else 11 * B
     return factor + bounds + 2
 
 

@@ -59,3 +59,16 @@ def test_unit_kp(p, kp):
     assert bench.unit_kp(p) == kp
     if p > 256:
         assert any(kp % nu == 0 and (kp // nu) % 16 == 0 and kp // nu <= 128 for nu in range(1, 9))
+
+
+@pytest.mark.parametrize("p,B,precision,kernels", [
+    (64, 304, "f16x3", 9 + 1 + 2),          # 4 panels, 3 updates, start and products
+    (64, 304, "fp32", 9 + 1 + 2),
+    (65, 4, "f16x3", 11 + 3 + 2),           # maxima, operand images, operators
+    (256, 4, "bf16x3", 33 + 3 + 2),
+    (256, 4, "fp32", 33 + 1 + 2),
+    (288, 16, "f16x3", 37 + 11 * 16 + 2),   # work items, job by job
+    (8, 1, "f16x3", 1 + 1 + 2),
+])
+def test_kernels_of_a_prepare_call(p, B, precision, kernels):
+    assert bench.prepare_launches(p, B, precision) == kernels
