@@ -71,3 +71,28 @@ def test_clusters_of_ctas_do_not_change_the_image(G):
             np.testing.assert_array_equal(o, one)
         for im in ims:
             im.close()
+
+
+def test_growing_free_set_in_bf16x3(G):
+    """The split tiles streamed from global memory with BF16 parts (three and
+    four tiles).  Products keep about 16 bits: decisions are admitted within the
+    operators' tolerance (1e-4 of scale), the image is held to
+    max(1e-3, 8 cond(M_F) 2^-16)."""
+    job = synth.custom(905, 48, 26, 22, 8, 20000, radius=30.0, snr_db=0.0)
+    prm = O.Params(cost=O.COST_LS, kappa=0.5, eps_floor=1e-6, feas_tol=1e-4, lsqr_atol=1e-6, lsqr_btol=1e-6)
+    im = G.Imager.from_job(job, cost=O.COST_LS, kappa=0.5, eps_floor=1e-6, feas_tol=1e-4, precision=G.PREC_BF16X3)
+    sigma, info = im.solve()
+    log = [(k, q) for k, q, _ in im.events()]
+    sets = im.sets()
+    im.close()
+    assert info.converged == 1
+    assert np.cumsum([1 if k == 0 else -1 for k, _ in log]).max() > 384
+    A = O.steering_matrix(job.ant_xyz, job.l, job.m, job.lam)
+    bnd = O.bounds(A, None, job.R, job.N, prm)
+    rep = O.active_set_follow(O.cost_problem(A, None, job.R, bnd, O.COST_LS), bnd.eps, prm, log, tol=1e-4)
+    assert not rep.violations, (rep.violations[:3], rep.max_margin)
+    np.testing.assert_array_equal(sets, rep.result.sets)
+    F = np.nonzero(sets == O.SET_F)[0]
+    cond = np.sqrt(np.linalg.cond(np.abs(A[:, F].conj().T @ A[:, F]) ** 2))
+    err = np.linalg.norm(sigma - rep.result.sigma) / np.linalg.norm(rep.result.sigma)
+    assert err <= max(1e-3, 8.0 * cond * 2.0 ** -16)
