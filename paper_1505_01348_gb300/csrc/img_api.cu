@@ -618,7 +618,7 @@ img_status img_psi(img_ctx *c, const double *x, double *Kout, int on_device) {
                                 on_device ? Kout : reinterpret_cast<double *>(c->Z), nullptr, c->stream));
     } else {
         if (on_device) CK(img::launch_d2f(x, c->wx, Q, c->stream));
-        CK(img::launch_psi(c->dj, c->wx, c->part, c->nparts, Q, p, mode_of(c), c->Z, c->stream));
+        CK(img::launch_psi(c->dj, c->wx, c->part, c->nparts, Q, p, c->Z, c->stream));
     }
     if (om == 0 || !on_device)
         CK(cudaMemcpyAsync(Kout, c->Z, (size_t)p * p * sizeof(double2),
@@ -655,7 +655,7 @@ img_status img_psi_adj(img_ctx *c, const double *U, double *out, int on_device) 
         if (st != IMG_OK) return st;
         CK(img::ws_psi_adj(c->ws, c->hj, c->U32, on_device ? out : c->outd, c->stream));
     } else {
-        CK(img::launch_psi_adj(c->dj, c->U32, on_device ? out : c->outd, Q, p, op_mode_of(c), c->stream));
+        CK(img::launch_psi_adj(c->dj, c->U32, on_device ? out : c->outd, Q, p, c->stream));
     }
     if (on_device == 2) return IMG_OK;           // stream-ordered, no host wait
     if (on_device) return sync(c);

@@ -116,7 +116,7 @@ cudaError_t launch_solve(JobDev *const *jobs, int n, int max_p, int mode, int ct
 cudaError_t launch_job(JobDev *const *jobs, int n, int max_p, int mode, DevInfo *batch_info,
                        double *const *sigma_out, cudaStream_t st);
 cudaError_t launch_psi(const JobDev *job_dev, const float *wx, float2 *part, int nparts, int Q,
-                       int p, int mode, double2 *Kout, cudaStream_t st);
+                       int p, double2 *Kout, cudaStream_t st);
 // Bounded-wait self-test (one CTA; all its threads wait, or the given one;
 // *status (may be null): IMG_OK or IMG_ETIMEOUT; job (may be null): as an
 // operator kernel of that job reports).
@@ -199,8 +199,7 @@ cudaError_t launch_psi_wide(const JobDev *job_dev, const FwdIn &in, float *part,
 // nmax > 0: the job's opmax already holds nmax per-CTA maxima of |U|.
 cudaError_t launch_psi_adj_wide(const JobDev *job_dev, const void *U, bool u64, int nmax, double *out, int Q, int p,
                                 int mode, cudaStream_t st);
-cudaError_t launch_psi_adj(const JobDev *job_dev, const float2 *U, double *out, int Q, int p,
-                           int mode, cudaStream_t st);
+cudaError_t launch_psi_adj(const JobDev *job_dev, const float2 *U, double *out, int Q, int p, cudaStream_t st);
 cudaError_t launch_z2c(const double2 *src, float2 *dst, int n, cudaStream_t st);
 cudaError_t launch_c2z(const float2 *src, double2 *dst, int n, cudaStream_t st);
 cudaError_t launch_d2f(const double *src, float *dst, int n, cudaStream_t st);

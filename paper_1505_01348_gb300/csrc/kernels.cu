@@ -836,7 +836,6 @@ __device__ void adjoint_list(const JobDev &J, const float2 *U, const int *pos, i
             [&](int t, int b) {
                 const int j0 = t * kTcM;
                 tc_gen_X_cache<BF>(J, T, b, pos, j0, min(kTcM, n - j0), sXl);
-                
             },
             [&](int t, int b) {
                 const int j0 = t * kTcM;
@@ -1113,7 +1112,7 @@ __device__ __forceinline__ void bar_arrive(int id, int n) {
 template <bool BF16>
 __device__ __forceinline__ void res_build_B(const TcWork &T, int p, float sc) {
     constexpr int kNt = kThreads - 32, kMax = 3;             // 64 x 8 chunks over 224 threads
-    const int Kp = T.Kp, N = 2 * Kp, nc8 = Kp / 8, items = Kp * nc8;
+    const int Kp = T.Kp, nc8 = Kp / 8, items = Kp * nc8;
     const float2 *t = reinterpret_cast<const float2 *>(T.Bhi());
     const int tid = threadIdx.x - 32;
     const bool vec = (p & 1) == 0;
@@ -1998,29 +1997,6 @@ __global__ void k_psi_partial(const JobDev *Jp, const float *wx, float2 *part, i
     }
 }
 
-// Tensor-core Psi x: CTA b accumulates pixels [b*per, (b+1)*per) into its
-// partial matrix part[b] (Kp = 64).
-template <int MODE>
-__global__ void __launch_bounds__(kThreads, 1) k_psi_partial_tc(const JobDev *Jp, const float *wx, float2 *part,
-                                                               int per) {
-    const JobDev &J = *Jp;
-    constexpr bool BF = MODE == 2;
-    unsigned char *dyn = dyn_smem();
-    __shared__ uint64_t bars[2];
-    __shared__ uint32_t slot;
-    __shared__ double dbuf[kThreads / 32];
-    TcWork T{};
-    tc_carve(T, dyn, J.p);
-    tc_setup(T, bars, &slot, J.p);
-    const int i0 = blockIdx.x * per;
-    const int n = max(0, min(per, J.Q - i0));
-    const float sX = tc_steer_scale(J.p);
-    tc_forward<BF>(T, J.p, n, wx + i0, sX,
-                   [&](int t, int np) { tc_gen_X_range<BF>(J, T, 0, i0 + t * kTcM, np, sX); },
-                   nullptr, false, part + (size_t)blockIdx.x * J.p * J.p, dbuf);
-    tc_teardown(T, J.p);
-}
-
 __global__ void k_psi_reduce(const float2 *part, int nparts, int pp, double2 *Kout) {
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < pp; e += gridDim.x * blockDim.x) {
         double sx = 0.0, sy = 0.0;
@@ -2220,29 +2196,10 @@ cudaError_t launch_job(JobDev *const *jobs, int n, int max_p, int mode, DevInfo 
     return launch_solve_t<0, true>(jobs, n, sm, 1, batch_info, sigma_out, st);
 }
 
-// Psi x over all pixels: nparts CTAs write partial p x p sums into `part`
+// Psi x over all pixels on CUDA cores: nparts CTAs write partial p x p sums into `part`
 // (nparts * p * p float2 of scratch), reduced in a fixed order in FP64.
-template <int MODE>
-static cudaError_t launch_psi_tc_t(const JobDev *job_dev, const float *wx, float2 *part, int nparts, int Q,
-                                   int p, double2 *Kout, cudaStream_t st) {
-    const size_t sm = tc_smem_bytes(p) + 1024;
-    cudaError_t e = ensure_smem((const void *)k_psi_partial_tc<MODE>, sm);
-    if (e != cudaSuccess) return e;
-    int per = (Q + nparts - 1) / nparts;
-    per = ((per + kTcM - 1) / kTcM) * kTcM;
-    const int used = (Q + per - 1) / per;
-    k_psi_partial_tc<MODE><<<used, kThreads, sm, st>>>(job_dev, wx, part, per);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_psi_reduce<<<(p * p + 255) / 256, 256, 0, st>>>(part, used, p * p, Kout);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_psi(const JobDev *job_dev, const float *wx, float2 *part, int nparts, int Q,
-                       int p, int mode, double2 *Kout, cudaStream_t st) {
-    const int Kp = (p + 31) / 32 * 32;
-    if (mode == 1 && Kp == 64) return launch_psi_tc_t<1>(job_dev, wx, part, nparts, Q, p, Kout, st);
-    if (mode == 2 && Kp == 64) return launch_psi_tc_t<2>(job_dev, wx, part, nparts, Q, p, Kout, st);
+                       int p, double2 *Kout, cudaStream_t st) {
     const size_t sm = (size_t)p * kTile * sizeof(float2);
     cudaError_t e = ensure_smem((const void *)k_psi_partial, sm);
     if (e != cudaSuccess) return e;
@@ -2303,7 +2260,7 @@ cudaError_t ls_forward(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, 
         const FwdIn in{nullptr, b.wx, b.wmax, ls_max_grid(Q)};
         e = launch_psi_wide(jd, in, fwd_part, Q, p, hj.n_l, hj.n_m, mode, nullptr, reinterpret_cast<float *>(b.Mv), st);
     } else {
-        e = launch_psi(jd, b.wx, part, nparts, Q, p, 0, b.Kd, st);
+        e = launch_psi(jd, b.wx, part, nparts, Q, p, b.Kd, st);
         if (e == cudaSuccess) k_d2c<<<ls_grid(pp), kThreads, 0, st>>>(b.Kd, b.Mv, pp);
     }
     if (e != cudaSuccess) return e;
@@ -2331,7 +2288,7 @@ cudaError_t ls_adjoint(const JobDev *jd, const JobDev &hj, LsBufs &b, int mode, 
         numax = fits ? (int)(g.x * g.y) : 0;
     }
     cudaError_t e = mode != 0 ? launch_psi_adj_wide(jd, U, false, numax, b.y, Q, p, mode, st)
-                              : launch_psi_adj(jd, U, b.y, Q, p, 0, st);
+                              : launch_psi_adj(jd, U, b.y, Q, p, st);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -2495,9 +2452,8 @@ cudaError_t launch_psi_adj_wide(const JobDev *job_dev, const void *U, bool u64, 
     return launch_psi_adj_wide_t<2>(job_dev, U, u64, nmax, out, Q, p, st);
 }
 
-cudaError_t launch_psi_adj(const JobDev *job_dev, const float2 *U, double *out, int Q, int p, int mode,
-                           cudaStream_t st) {
-    if (mode != 0) return cudaErrorInvalidValue;   // tensor cores: launch_psi_adj_wide
+// On CUDA cores (tensor cores: launch_psi_adj_wide).
+cudaError_t launch_psi_adj(const JobDev *job_dev, const float2 *U, double *out, int Q, int p, cudaStream_t st) {
     const size_t sm = bounds_smem_bytes(p);
     cudaError_t e = ensure_smem((const void *)k_psi_adj, sm);
     if (e != cudaSuccess) return e;

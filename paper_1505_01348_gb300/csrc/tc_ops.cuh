@@ -502,37 +502,6 @@ __device__ inline void tc_gen_X_steer(const JobDev &J, TcWork &T, int b, int t, 
     }
 }
 
-// X tile of the consecutive pixels pix0 .. pix0+np-1 (forward over all
-// pixels, where every pixel's weight comes from a linear array).
-template <bool BF16>
-__device__ inline void tc_gen_X_range(const JobDev &J, TcWork &T, int b, int pix0, int np, float sX) {
-    const int p = J.p, Kp = T.Kp, nc8 = Kp / 8, nl = J.n_l;
-    unsigned char *xh = T.Xhi(b), *xl = T.Xlo(b);
-    for (int it = threadIdx.x; it < kTcM * nc8; it += blockDim.x) {
-        const int r = it / nc8, c8 = it - r * nc8;
-        float re[8], im[8];
-        const int i = pix0 + r;
-        const int mm = i / nl, ll = i - mm * nl;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int k = c8 * 8 + q;
-            float2 a = make_float2(0.f, 0.f);
-            if (r < np && k < p) a = steer(J, ll, mm, k);
-            re[q] = a.x * sX;
-            im[q] = a.y * sX;
-        }
-        uint4 hi, lo;
-        split8<BF16>(re, hi, lo);
-        uint32_t off = sw128_off(r, c8, kTcM);
-        *reinterpret_cast<uint4 *>(xh + off) = hi;
-        *reinterpret_cast<uint4 *>(xl + off) = lo;
-        split8<BF16>(im, hi, lo);
-        off = sw128_off(r, nc8 + c8, kTcM);
-        *reinterpret_cast<uint4 *>(xh + off) = hi;
-        *reinterpret_cast<uint4 *>(xl + off) = lo;
-    }
-}
-
 // X tile from cached vectors cvec[pos[j0 + r]] (pos == nullptr: j0 + r),
 // scaled by sX (a power of two keeping every entry within unit range).
 template <bool BF16>

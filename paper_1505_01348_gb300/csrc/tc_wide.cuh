@@ -110,7 +110,6 @@ __device__ __forceinline__ float cta_max_t0(float mx) {
 // share (grid-stride over blocks `b` of `nb`); thread 0 has the result.
 template <class TC>
 __device__ inline float emb_absmax(const TC *U, int p, int b, int nb) {
-    __shared__ float sred[32];
     const int n2 = p * p, stride = nb * blockDim.x;
     float mx = 0.f;
     int e = b * blockDim.x + threadIdx.x;
