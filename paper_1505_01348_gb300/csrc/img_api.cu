@@ -1258,12 +1258,15 @@ struct SSlot {                           // one launch stream and its workspace
     }
 };
 
-using ShapeKey = std::tuple<int, int, int, int>;   // p, n_l, n_m, support cap
+// p, n_l, n_m, support cap, and the arithmetic of a wide solver's graph (0: a
+// context without one, which serves every arithmetic)
+using ShapeKey = std::tuple<int, int, int, int, int>;
 
 ShapeKey key_of(const img_params &p) {
     const int Q = p.n_l * p.n_m;
     const int cap = p.support_cap > 0 ? std::min(p.support_cap, Q) : std::min(Q, 16384);
-    return ShapeKey(p.p, p.n_l, p.n_m, cap);
+    const bool wide = p.precision != IMG_PREC_FP32 && p.p > img::kMaxTcP && p.p <= img::kMaxWideSolveP;
+    return ShapeKey(p.p, p.n_l, p.n_m, cap, wide ? p.precision : 0);
 }
 
 // Load a job's parameters, geometry and covariance into a pooled context of
