@@ -117,10 +117,10 @@ def make_jobs(seeds, workload: str = "large"):
 def default_batch(workload: str, steps: int, sms: int) -> int:
     """Images per step.  mid: two per SM (one CTA each).  large: each image
     is a graph of kernels spread over the GPU, and the solves in flight
-    overlap: 8 give 0.42 images/s, 16 give 0.54, 24 give 0.55 and 32 fall
-    back to 0.49 (their working sets no longer share L2); the batch shrinks
-    (to 4 at least) when many steps are asked for, to keep the timed region
-    near a minute."""
+    overlap: 4 give 0.29 images/s, 8 give 0.43, 16 give 0.55, 24 give 0.56 and
+    32 fall back to 0.50 (their working sets no longer share L2); the batch
+    shrinks (to 4 at least) when many steps are asked for, to keep the timed
+    region near a minute."""
     if workload == "mid":
         return 2 * sms
     return max(4, min(16, 48 // max(steps, 1)))

@@ -255,7 +255,7 @@ img_status img_check_wait_ctx(img_ctx *ctx, unsigned polls, int arrive);
  * M = Psi, b = vect(R_hat) (IMG_COST_LS) or M = W Psi D^-1, b = W vect(R_hat)
  * (IMG_COST_PWLS, W = conj(L^-1) kron L^-1), cold start x0 = 0, no bounds.
  * The bidiagonalisation runs on the device (operators as in img_psi /
- * img_psi_adj, FP64 scalar recurrences in a one-thread kernel); the
+ * img_psi_adj, FP64 scalar recurrences beside the vector updates); the
  * Paige-Saunders stopping tests with the context's lsqr_atol / lsqr_btol are
  * checked every 10 iterations.  maxit <= 0: 200 iterations at most.
  * sigma[0..Q) receives the image (host or device per on_device); info (may

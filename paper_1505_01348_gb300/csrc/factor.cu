@@ -4,10 +4,10 @@
 // What bounds it: GB300's FP64 pipe takes about two lanes per clock and SM,
 // so the ~96 M lane instructions of p = 288 cost 25 ms on one SM whatever the
 // code around them does (the one-CTA form measured 37.6 ms; p = 128: 4.6 ms,
-// p = 64: 0.92 ms; a dirty + MVDR call fell from 38.7 to 2.6 ms at p = 288,
-// 256x256, from 5.04 to 0.90 ms at p = 128, from 1.22 to 0.52 ms at p = 64
-// with this form and the panels below).  Here the elimination of [R | I] runs in panels of kNb
-// columns over all SMs:
+// p = 64: 0.92 ms; a dirty + MVDR call takes 1.45 instead of 38.7 ms at p =
+// 288, 256x256, 0.67 instead of 5.04 ms at p = 128, 0.26 instead of 1.22 ms at
+// p = 64 with this form and the thresholds over all SMs).  Here the elimination
+// of [R | I] runs in panels of kNb columns over all SMs:
 //
 //   k_fac_panel  one step of the chain: every CTA factors the kNb x kNb
 //                diagonal block for itself (sqrt, reciprocal: the serial part;
@@ -19,9 +19,10 @@
 //   k_fac_out    FP32 copies, and R^-1 = L^-H L^-1 for the jobs that use it.
 //
 // Every element is computed by the same operations in the same order as in
-// the one-CTA form that the fused server kernel keeps (factor_job): the
-// panels only group the subtractions, which each element takes in ascending
-// column order either way.  Both give the same bits.
+// the one-CTA form that the fused server kernel and the smallest jobs keep
+// (factor_job): the panels only group the subtractions, which each element
+// takes in ascending column order either way.  Both give the same bits
+// (tests/test_gpu_factor.py).
 #include "cta_ops.cuh"
 
 namespace img {

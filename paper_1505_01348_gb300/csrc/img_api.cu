@@ -904,7 +904,7 @@ img_status img_ls_image(img_ctx *c, int maxit, double *sigma, img_solve_info *in
         } else {
             CK(img::ls_iterate(c->dj, c->hj, b, mode, c->fwd_part, c->part, c->nparts, c->stream));
             if (c->own_stream) {
-                // the iteration is a fixed sequence of ~15 launches on buffers the
+                // the iteration is a fixed sequence of 12 launches (PWLS) on buffers the
                 // context keeps: record it once as a graph and replay it (the
                 // first, direct iteration has set every kernel attribute)
                 cudaGraph_t g = nullptr;

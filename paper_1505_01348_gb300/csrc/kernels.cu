@@ -376,9 +376,12 @@ __global__ void __launch_bounds__(256) k_fwd_assemble(int p, const float *part, 
 // Unconstrained LS / WLS image with every pixel free: LSQR (Sec. V-A) on
 // M = Psi (CLS) or W Psi D^-1 (PWLS, W = conj(L^-1) kron L^-1), b = vect(R_hat)
 // or W vect(R_hat) = vect(I).  The bidiagonalisation runs as a stream of
-// kernels: the operators above, complex p x p products for the whitening,
-// one-CTA reductions in a fixed order, and a one-thread kernel for the FP64
-// scalar recurrences, whose results later kernels read from device memory.
+// kernels, 12 per iteration for PWLS: the operators above, complex p x p
+// products for the whitening, and the vector updates with their norms' partial
+// sums (32 CTAs, a fixed order).  The FP64 scalars of the recurrences are in
+// two sets, each written by CTA 0 of the one kernel (k_ls_scale_u, k_ls_xw)
+// whose other CTAs read only the other set and the partial sums, so that every
+// CTA forms the factors it needs itself.
 
 // Sums of squares in the order of one CTA of 1024 threads: virtual thread t
 // takes entries t, t + 1024, ..., its warp's butterfly gives one of 32 partial

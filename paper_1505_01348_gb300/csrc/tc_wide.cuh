@@ -507,7 +507,7 @@ __device__ int wide_adjoint(const JobDev &J, unsigned char *dyn, uint64_t *bars,
 
 
 // ================================================================ forward
-// Psi x for 64 < p <= 256 on tensor cores: K = sum_i w_i a_i a_i^H from the
+// Psi x for p <= 384 on tensor cores: K = sum_i w_i a_i a_i^H from the
 // real Gram matrix G = sum_i w_i x_i x_i^T (2Kp x 2Kp), K = (G_rr + G_ii) +
 // j (G_ir - G_ri).  G is tiled in blocks of 128 rows (features 128m ..) by up
 // to 256 columns (features 256nb ..); only blocks that reach the upper

@@ -682,10 +682,10 @@ __device__ void ws_fred(const JobDev &J, const WsBufs &B, const UnitGeom &g, int
     if ((threadIdx.x & 31) == 0) atomicMax(&ctl->mx_t, __float_as_uint(mx));
     if (mode != kRedG && rank == 0 && threadIdx.x == 0) ctl->nsums = nt * nt;
 }
-// Two CTAs per SM (128 registers, a few spilled): with the 167 it would take,
-// one image alone is faster (first passes of 256 x 256, p = 288: 182 instead
-// of 191 ms), but a CTA keeps the other images' off its SM, and 16 such
-// images in flight take 5.79 s instead of 5.41 for their first 1600 passes.
+// Two CTAs per SM (128 registers, 248 bytes spilled): with the 166 it would
+// take, few images are faster (256x256, p = 288: first 200 passes of one 84
+// instead of 87 ms, first 1600 of four 2.33 instead of 2.37 s), but a CTA keeps
+// the other images' off its SM, and 16 in flight take 5.42 s instead of 4.97.
 __global__ void __launch_bounds__(kWsThreads, 2) k_ws_fred(const JobDev *Jp, WsBufs B, int mode) {
     ws_count(B.ctl);
     if (B.ctl->stop) return;
